@@ -3611,6 +3611,159 @@ struct LastOnlyArgs {
     int32_t* order; int32_t* uncached; int64_t* ttft; int64_t* completion; int32_t* n_skipped;
 };
 
+// First index in [0, n) where a and b differ, or n, for short strings: one warp-wide minimum per 128 tokens instead of
+// a ballot per 32 of them.  Warp-cooperative: every lane calls it with the same arguments and gets the result.
+__device__ __forceinline__ int32_t first_mismatch_short(const int32_t* __restrict__ a, const int32_t* __restrict__ b, int32_t n, int lane) {
+    for (int32_t base = 0; base < n; base += 128) {
+        unsigned at = 0xffffffffu;
+#pragma unroll
+        for (int r = 3; r >= 0; --r) {
+            const int32_t i = base + r * 32 + lane;
+            if (i < n && __ldg(a + i) != __ldg(b + i)) at = (unsigned)i;
+        }
+        const unsigned m = __reduce_min_sync(FULL_MASK, at);
+        if (m != 0xffffffffu) return (int32_t)m;
+    }
+    return n;
+}
+
+// A queue of at most 32 prompts (every queue of the Monte-Carlo): lane i keeps prompt i in registers from the first
+// decision to the last, and the results leave in four coalesced stores at the end.
+//   * The two orders a pick goes by -- (arrival, index) and (priority, arrival, index) -- are turned into ranks once, so
+//     a pick is one or two warp reductions instead of a five-step tournament over 64-bit tuples.
+//   * Overlaps come from one comparison per prompt instead of one or two per decision and candidate: prompts with the
+//     same first token form a class, and each of them is compared once with the class's first prompt (the pivot), which
+//     gives e = overlap with the pivot and the token that follows.  Two members with different e overlap in the smaller
+//     one; with equal e and different next tokens in exactly e.  Only members that leave the pivot at the same place
+//     with the same token (`twin`, rare) still have to be compared with each other, from e on.
+// What bounds it: the issue rate (about 50 warp instructions per decision, 32 comparisons of 128 tokens); the tokens are
+// read from HBM once.  65,536 queues of 32 prompts of 128 tokens: 395 us (2.97 TB/s, 5.3 G decisions/s); two passes over
+// the queue and two token comparisons per decision, as longer queues still do it, took 1,482 us.
+// Every warp-wide operation below is executed by all 32 lanes: lanes beyond the queue's length take part with values
+// that never win.
+__device__ __forceinline__ void last_only_small(const LastOnlyArgs& A, int32_t q0, int32_t n, int lane) {
+    const long long INF = 0x7fffffffffffffffLL;
+    const bool in = lane < n;
+    long long t = INF, pr = 0;
+    int32_t len = 0;
+    const int32_t* x = A.tok;
+    if (in) {
+        t = __ldg(A.arrival + q0 + lane);
+        const int64_t lo = __ldg(A.off + q0 + lane);
+        len = (int32_t)(__ldg(A.off + q0 + lane + 1) - lo);
+        x += lo;
+        if (A.prio) pr = __ldg(A.prio + q0 + lane);
+    }
+    const bool full = len > 0;
+    const int32_t first = full ? __ldg(x) : 0;
+    const unsigned nonempty = __ballot_sync(FULL_MASK, full);
+    const unsigned same = __match_any_sync(FULL_MASK, first) & nonempty;
+    const int pivot = full ? __ffs(same) - 1 : 32 + lane;     // (an empty prompt is in no class)
+    // ---- overlap with the class's pivot (the pivot's own is its length)
+    int32_t e = len;
+    for (unsigned todo = __ballot_sync(FULL_MASK, full && pivot != lane); todo; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1, p = __shfl_sync(FULL_MASK, pivot, src);
+        const int32_t* xs = (const int32_t*)__shfl_sync(FULL_MASK, (unsigned long long)x, src);
+        const int32_t* xp = (const int32_t*)__shfl_sync(FULL_MASK, (unsigned long long)x, p);
+        const int32_t ls = __shfl_sync(FULL_MASK, len, src), lp = __shfl_sync(FULL_MASK, len, p);
+        const int32_t ee = first_mismatch_short(xs, xp, ls < lp ? ls : lp, lane);
+        if (lane == src) e = ee;
+    }
+    const bool ended = e >= len;                              // nothing follows: agrees with the pivot to its own end
+    const int32_t ntok = ended ? 0 : __ldg(x + e);
+    const unsigned goes_on = __ballot_sync(FULL_MASK, !ended);
+    const unsigned alike = __match_any_sync(FULL_MASK, ((unsigned long long)(unsigned)ntok << 32) | (unsigned)e) & same & goes_on;
+    const bool twin = !ended && (alike & (alike - 1)) != 0;   // another member leaves the pivot at the same place with the same token
+    const bool twins = __any_sync(FULL_MASK, twin);
+    // ---- ranks in the two orders, the lane in the low bits: (rank << 5) | lane
+    int rank_f = 0, rank_l = 0;
+    const int t_hi = (int)(t >> 32), p_hi = (int)(pr >> 32);
+    const int t_hi0 = __shfl_sync(FULL_MASK, t_hi, 0), p_hi0 = __shfl_sync(FULL_MASK, p_hi, 0);
+    if (__all_sync(FULL_MASK, !in || (t_hi == t_hi0 && p_hi == p_hi0))) {      // the high words agree: the low ones decide
+        const unsigned t32 = (unsigned)t, p32 = (unsigned)pr;
+        for (int s = 0; s < n; ++s) {
+            const unsigned ts = __shfl_sync(FULL_MASK, t32, s), ps = __shfl_sync(FULL_MASK, p32, s);
+            const bool before = ts < t32 || (ts == t32 && s < lane);
+            rank_f += before;
+            rank_l += ps < p32 || (ps == p32 && before);
+        }
+    } else {
+        for (int s = 0; s < n; ++s) {
+            const long long ts = __shfl_sync(FULL_MASK, t, s), ps = __shfl_sync(FULL_MASK, pr, s);
+            const bool before = ts < t || (ts == t && s < lane);
+            rank_f += before;
+            rank_l += ps < pr || (ps == pr && before);
+        }
+    }
+    rank_f = rank_f << 5 | lane;
+    rank_l = rank_l << 5 | lane;
+    const long long cost_per = A.c_den + A.c_num * (long long)len;     // per uncached token (Definition 2)
+    long long now = A.start_tick, my_R = 0;
+    bool left = in, arrived = false;                          // not processed yet; everybody has arrived
+    int32_t my_order = 0, my_m = 0, until_f = 0;
+    int last = -1;
+    for (int32_t c = 0; c < n; ++c) {
+        // ---- who is waiting; if nobody, idle until the next arrival
+        bool wait = left;
+        if (!arrived) {                                       // (uniform)
+            wait = left && t <= now;
+            if (!__any_sync(FULL_MASK, wait)) {
+                long long tmin = left ? t : INF;
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) { const long long o = __shfl_xor_sync(FULL_MASK, tmin, d); tmin = o < tmin ? o : tmin; }
+                now = tmin;
+                wait = left && t <= now;
+            }
+            arrived = __all_sync(FULL_MASK, wait == left);
+        }
+        bool fcfs_turn = A.policy == KLPM_POLICY_FCFS;
+        if (A.policy == KLPM_POLICY_KLPM) { fcfs_turn = until_f == 0; until_f = fcfs_turn ? A.k - 1 : until_f - 1; }
+        // ---- overlap with the prompt processed last
+        int32_t score = 0;
+        if (last >= 0) {
+            const int32_t e_l = __shfl_sync(FULL_MASK, e, last), p_l = __shfl_sync(FULL_MASK, pivot, last);
+            if (pivot == p_l) score = e < e_l ? e : e_l;
+            if (twins) {                                      // (uniform)
+                const int32_t n_l = __shfl_sync(FULL_MASK, ntok, last);
+                const bool t_l = __shfl_sync(FULL_MASK, (int)twin, last) != 0;
+                unsigned tm = __ballot_sync(FULL_MASK, wait && twin && t_l && pivot == p_l && e == e_l && ntok == n_l);
+                if (tm) {                                     // they share more than e: compare from there on
+                    const int32_t* xl = (const int32_t*)__shfl_sync(FULL_MASK, (unsigned long long)x, last);
+                    const int32_t len_l = __shfl_sync(FULL_MASK, len, last);
+                    for (; tm; tm &= tm - 1) {
+                        const int src = __ffs(tm) - 1;
+                        const int32_t* xs = (const int32_t*)__shfl_sync(FULL_MASK, (unsigned long long)x, src);
+                        const int32_t ls = __shfl_sync(FULL_MASK, len, src);
+                        const int32_t ee = e_l + first_mismatch_short(xs + e_l, xl + e_l, (ls < len_l ? ls : len_l) - e_l, lane);
+                        if (lane == src) score = ee;
+                    }
+                }
+            }
+        }
+        // ---- the pick: oldest, or largest overlap and then smallest (priority, arrival, index)
+        unsigned r = 0xffffffffu;
+        if (fcfs_turn) {
+            if (wait) r = (unsigned)rank_f;
+        } else {
+            const unsigned best = __reduce_max_sync(FULL_MASK, wait ? (unsigned)score : 0u);
+            if (wait && (unsigned)score == best) r = (unsigned)rank_l;
+        }
+        const int j = (int)(__reduce_min_sync(FULL_MASK, r) & 31u);     // (somebody is waiting)
+        // ---- charge by Definition 2 (the pick has arrived, so it begins at once); x_j is the cached prompt now
+        const long long cost = cost_per * (long long)(len - score);
+        now += __shfl_sync(FULL_MASK, cost, j);
+        if (lane == j) { my_m = score; my_R = now; left = false; }
+        if (lane == c) my_order = j;
+        last = j;
+    }
+    if (in) {
+        A.order[q0 + lane] = my_order;
+        A.uncached[q0 + lane] = len - my_m;
+        A.ttft[q0 + lane] = my_R - t;
+        if (A.completion) A.completion[q0 + lane] = my_R;
+    }
+}
+
 __global__ void __launch_bounds__(32 * KLPM_LAST_ONLY_WARPS)
 last_only_batch_kernel(LastOnlyArgs A) {
     __shared__ unsigned s_done[KLPM_LAST_ONLY_WARPS][KLPM_LAST_ONLY_MAX_QUEUE / 32];
@@ -3623,6 +3776,7 @@ last_only_batch_kernel(LastOnlyArgs A) {
         if (lane == 0 && A.n_skipped) atomicAdd(A.n_skipped, 1);
         return;
     }
+    if (n <= 32) { last_only_small(A, q0, n, lane); return; }
     unsigned* done = s_done[warp];
     for (int32_t w = lane; w < KLPM_LAST_ONLY_MAX_QUEUE / 32; w += 32) done[w] = 0u;
     __syncwarp();
@@ -3709,7 +3863,8 @@ last_only_batch_kernel(LastOnlyArgs A) {
         const int32_t len = (int32_t)(__ldg(A.off + q0 + j + 1) - lo);
         const int32_t* x = A.tok + lo;
         int32_t m = 0;
-        if (last >= 0) m = first_mismatch<true, 1>(x, last_x, len < last_len ? len : last_len);
+        if (!fcfs_turn) m = b_score;                          // the overlap it was picked by
+        else if (last >= 0) m = first_mismatch<true, 1>(x, last_x, len < last_len ? len : last_len);
         const int32_t unc = len - m;
         const long long tj = __ldg(A.arrival + q0 + j);
         const long long begin = now > tj ? now : tj;

@@ -114,3 +114,31 @@ def test_ragged_random_queues_with_arrival_gaps_and_c_attn(K, seed):
             want = oracle_queue(queues[q], arrivals[q], policy, k, None, 1, 3, 2)
             for g, w_ in zip(out[q], want):
                 assert np.array_equal(g, w_), (q, policy)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33])
+def test_queue_lengths_around_one_warp(K, n):
+    """Queues of up to 32 prompts are held in registers, longer ones are not: lengths on both sides of that line, nested
+    prefixes over two tokens and long prompts (several comparison chunks, members that leave the first prompt of their
+    class at the same place with the same token), random priorities, every policy."""
+    rng = np.random.RandomState(n)
+    queues, arrivals, prios = [], [], []
+    for q in range(64):
+        vocab, max_len = (2, 12) if q % 2 else (3, 400)
+        prompts, arr = W.random_small_queue(500 * n + q, n, vocab=vocab, max_len=max_len, min_len=0, max_gap=40)
+        if q % 4 == 0:                       # a shared stem in front of most of them
+            stem = [1] * 300
+            prompts = [stem[:int(rng.randint(100, 301))] + p if rng.randint(0, 4) else p for p in prompts]
+        if q % 8 == 1:                       # arrivals and priorities beyond 32 bits
+            arr = [t * (1 << 31) for t in arr]
+            prios.append((rng.randint(-2, 3, size=n).astype(np.int64) * (1 << 32)).tolist())
+        else:
+            prios.append(rng.randint(0, 3, size=n).tolist())
+        queues.append(prompts); arrivals.append(arr)
+    for policy, k in ((K.POLICY_KLPM, 2), (K.POLICY_KLPM, 5), (K.POLICY_LPM, 1), (K.POLICY_FCFS, 1)):
+        out, skipped = run_batch(K, queues, arrivals, policy, k, prios, 1, 3, 1)
+        assert skipped == 0
+        for q in range(len(queues)):
+            want = oracle_queue(queues[q], arrivals[q], policy, k, np.asarray(prios[q], dtype=np.int64), 1, 3, 1)
+            for g, w_ in zip(out[q], want):
+                assert np.array_equal(g, w_), (q, policy, k)
