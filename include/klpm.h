@@ -110,7 +110,7 @@ typedef struct { int64_t w[4]; } klpm_match_state;
  * (rt_insert, klpm_replay, klpm_run*, rt_rollback), (b) d_q_tokens / d_q_offsets / nq are the ones passed here
  * and their contents have not changed, and (c) no later rt_match_batch_ex with a state buffer was made on this
  * tree.  On a tree with a budget the records are written but klpm_run_ex does not use them (the tree changes
- * under the loop).  Batches of 2,048 queries or more are taken in an order bucketed by first token, for which
+ * under the loop).  Large batches (more than 16,384 queries) are taken in an order bucketed by first token, for which
  * the first such call allocates scratch (synchronously); results do not depend on the order. */
 rt_status rt_match_batch_ex(rt_tree* tree, const int32_t* d_q_tokens, const int64_t* d_q_offsets, int32_t nq,
                             int32_t* d_match_len, int32_t* d_term_node, int32_t* d_term_off,

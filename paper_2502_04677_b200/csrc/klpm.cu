@@ -107,8 +107,8 @@ __device__ __forceinline__ void set_status(TreeState* st, int code, int detail =
 
 // A child lookup that probed every slot of the table without meeting the key or an empty slot gives up; the
 // walk then reports a shorter match, and the status word says that it is not to be trusted.
-__device__ __noinline__ void probe_limit(const TreeDev& T) {
-    if ((threadIdx.x & 31) == 0) set_status(T.st, RT_ERR_LIMIT, 106);
+__device__ __noinline__ void probe_limit(TreeState* st) {       // (a pointer: a reference to T would put the kernel's copy of it on the stack)
+    if ((threadIdx.x & 31) == 0) set_status(st, RT_ERR_LIMIT, 106);
 }
 
 // First index in [0, n) where a and b differ, or n.  Warp-cooperative: every lane gets the result.
@@ -160,7 +160,7 @@ __device__ Term walk(const TreeDev& T, const int32_t* __restrict__ q, int32_t le
         unsigned long long probes = 0;
         while (c.key != key) {
             if (c.key == 0ULL) return t;
-            if (++probes > T.table_mask) { probe_limit(T); return t; }      // no empty slot: cannot happen below load 1
+            if (++probes > T.table_mask) { probe_limit(T.st); return t; }      // no empty slot: cannot happen below load 1
             slot = (slot + 1) & T.table_mask;
             c = ld_entry<RO>(T.table + slot);
         }
@@ -361,7 +361,7 @@ __device__ __forceinline__ int32_t walk_chain(const TreeDev& T, const int32_t* _
         unsigned long long probes = 0;
         while (c.key != key) {
             if (c.key == 0ULL) return m;
-            if (++probes > T.table_mask) { probe_limit(T); return m; }      // no empty slot: cannot happen below load 1
+            if (++probes > T.table_mask) { probe_limit(T.st); return m; }      // no empty slot: cannot happen below load 1
             slot = (slot + 1) & T.table_mask;
             c = ld_entry<true>(T.table + slot);
         }
@@ -564,9 +564,9 @@ __device__ void insert_serial(const TreeDev& T, const int32_t* x, int32_t len, i
 // One warp per query, queries handed out by an atomic counter (persistent grid).
 // Trees without a budget: stream along contiguous pool runs.
 //
-// Queries are taken in the order of `perm` when it is given: the host buckets them by their first token first, so
-// that queries which start down the same root child -- and therefore read the same pool tokens -- are in flight
-// at the same time and all but the first of them find those tokens in L2.
+// Queries are taken in the order of `perm`: the host buckets them by their first token first, so that queries which
+// start down the same root child -- and therefore read the same pool tokens -- are in flight at the same time and all
+// but the first of them find those tokens in L2.
 //
 // With STATE the kernel also records, per query, what the scheduling loop needs to start from this match instead
 // of walking the query again (MatchState: where the match ended, the run that position lies in, the next token).
@@ -592,7 +592,7 @@ match_chain_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* _
         if (lane == 0) c = atomicAdd(counter, 1ULL);
         c = __shfl_sync(FULL_MASK, c, 0);
         if (c >= (unsigned long long)nq) return;
-        const int64_t i = perm ? (int64_t)__ldg(perm + c) : (int64_t)c;
+        const int64_t i = __ldg(perm + c);
         const int64_t lo = __ldg(qoff + i);
         int64_t len = __ldg(qoff + i + 1) - lo;
         if (len < 0 || len > 0x7fffffffLL) { if (lane == 0) set_status(T.st, RT_ERR_INVALID); len = 0; }
@@ -675,7 +675,7 @@ match_batch_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* _
         if (lane == 0) c = atomicAdd(counter, 1ULL);
         c = __shfl_sync(FULL_MASK, c, 0);
         if (c >= (unsigned long long)nq) return;
-        const int64_t i = perm ? (int64_t)__ldg(perm + c) : (int64_t)c;
+        const int64_t i = __ldg(perm + c);
         const int64_t lo = __ldg(qoff + i), hi = __ldg(qoff + i + 1);
         int64_t len = hi - lo;
         if (len < 0 || len > 0x7fffffffLL) { if (lane == 0) set_status(T.st, RT_ERR_INVALID); len = 0; }
@@ -690,6 +690,101 @@ match_batch_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* _
                 r.pos = t.pos; r.chain_end = t.node; r.m = t.m; r.ntok = t.m < (int32_t)len ? __ldg(qtok + lo + t.m) : 0; r.tag = tag;
                 state[i] = r;
             }
+        }
+    }
+}
+
+// The batched match for few queries: one CTA per query, every warp of it walks (redundantly: the lookups are
+// broadcasts) and compares its own 512 tokens of the stretch at hand, so a long edge costs one memory latency per
+// 512 x warps tokens instead of one per 512 (match_batch_kernel) or 128 (match_chain_kernel).  With few queries that
+// latency is all there is: no batch order, no work counter to clear, the grid is the batch.  CHAIN: streams along
+// contiguous pool runs (trees without a budget), otherwise hop by hop.
+// 32 queries of 1,024 to 8,192 tokens, caches cold: 10 us (match_batch_kernel 21), on a tree without a budget 12 us
+// (match_chain_kernel 33).
+__device__ __forceinline__ int32_t wide_mismatch(const int32_t* __restrict__ a, const int32_t* __restrict__ b, int32_t n,
+                                                 int32_t* s_min, unsigned& phase) {
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    if (nwarps == 1) return first_mismatch<true>(a, b, n);
+    for (int32_t base = 0; base < n; base += nwarps * 512) {     // (n is the same in every thread of the CTA)
+        const int32_t lo = base + warp * 512;
+        const unsigned p = phase % 3u, q = (phase + 1u) % 3u;    // three words in turn: the next one is reset a barrier ahead
+        ++phase;
+        if (lo < n) {
+            const int32_t seg = n - lo < 512 ? n - lo : 512;
+            const int32_t r = first_mismatch<true>(a + lo, b + lo, seg);
+            if (r < seg && (threadIdx.x & 31) == 0) atomicMin(s_min + p, lo + r);
+        }
+        if (threadIdx.x == 0) s_min[q] = 0x7fffffff;
+        __syncthreads();
+        const int32_t m = s_min[p];
+        if (m != 0x7fffffff) return m;
+    }
+    return n;
+}
+
+template <bool CHAIN>
+__global__ void __launch_bounds__(256, 4)
+match_wide_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* __restrict__ qoff, int32_t* __restrict__ mlen,
+                  int32_t* __restrict__ tnode, int32_t* __restrict__ toff, MatchState* __restrict__ state, unsigned long long tag) {
+    __shared__ int32_t s_min[3];
+    if (threadIdx.x < 3) s_min[threadIdx.x] = 0x7fffffff;
+    __syncthreads();
+    unsigned phase = 0;
+    const int64_t i = blockIdx.x;
+    const int64_t lo = __ldg(qoff + i);
+    int64_t len64 = __ldg(qoff + i + 1) - lo;
+    if (len64 < 0 || len64 > 0x7fffffffLL) { if (threadIdx.x == 0) set_status(T.st, RT_ERR_INVALID); len64 = 0; }
+    const int32_t len = (int32_t)len64;
+    const int32_t* q = qtok + lo;
+    const EndIndex X = end_index(T);
+    const long long n_nodes = CHAIN ? *reinterpret_cast<const volatile long long*>(&T.st->n_nodes) : 0;
+    int32_t m = 0, cur = 0, node = 0, off = 0;
+    int64_t pos = -1, cend = 0;
+    while (m < len) {
+        const unsigned long long key = make_key(cur, __ldg(q + m));
+        unsigned long long slot = hash_key(key) & T.table_mask;
+        Entry c = ld_entry<true>(T.table + slot);
+        unsigned long long probes = 0;
+        bool found = true;
+        while (c.key != key) {
+            if (c.key == 0ULL) { found = false; break; }
+            if (++probes > T.table_mask) { probe_limit(T.st); found = false; break; }      // no empty slot: cannot happen below load 1
+            slot = (slot + 1) & T.table_mask;
+            c = ld_entry<true>(T.table + slot);
+        }
+        if (!found || c.child < 0) break;
+        int64_t run = CHAIN ? c.chain_end - c.span_off : (int64_t)c.span_len;
+        if (run > (int64_t)(len - m)) run = len - m;
+        const int32_t x = wide_mismatch(q + m, T.pool + c.span_off, (int32_t)run, s_min, phase);     // x >= 1: the first token is the key
+        m += x;
+        pos = c.span_off + x - 1;
+        if (CHAIN) {
+            cend = c.chain_end;
+            const int32_t e = node_ending_at(X, pos, n_nodes);
+            if (e < 0) {                                          // stopped inside an edge
+                if (tnode || toff) {
+                    const int32_t f = node_after(X, pos, cend);
+                    if (f >= 0) { node = f; off = m - __ldg(T.depth_start + f); }
+                }
+                break;
+            }
+            node = e;
+            if (tnode || toff) off = __ldg(T.span_len + e);
+            cur = e;
+        } else {
+            node = c.child; off = x; cend = c.child;              // (trees with a budget: the record carries the node)
+            if (x < c.span_len) break;
+            cur = c.child;
+        }
+    }
+    if (threadIdx.x == 0) {
+        if (mlen) mlen[i] = m;
+        if (tnode) tnode[i] = node;
+        if (toff) toff[i] = off;
+        if (state) {
+            MatchState r;
+            r.pos = pos; r.chain_end = cend; r.m = m; r.ntok = m < len ? __ldg(q + m) : 0; r.tag = tag;
+            state[i] = r;
         }
     }
 }
@@ -4346,30 +4441,45 @@ rt_status bulk_insert(rt_tree* t, const int32_t* d_tokens, const int64_t* d_offs
     return RT_OK;
 }
 
-#define KLPM_ORDER_MIN 2048       // smaller batches are matched in index order (three launches saved)
+// Batches up to these sizes go to match_wide_kernel.  Cold caches, wide against the ordered persistent kernels:
+//   with a budget (hop by hop): 32 queries 10 / 21 us, 4,736 32 / 54, 14,000 56 / 77, 48,000 140 / 159
+//   without (along runs), medium tree: 32 queries 12 / 33 us, 4,736 34 / 62, 14,000 69 / 89, 48,000 184 / 187; deep edges
+//   (adversarial): 32 queries 27 / 96, 4,736 111 / 153, 14,000 201 / 218, 24,000 307 / 288: there every query of a trunk
+//   reads the trunk from HBM again unless they are taken together.
+#define KLPM_WIDE_MAX_CHAIN 16384
+#define KLPM_WIDE_MAX_HOPS 65536
 std::atomic<unsigned long long> g_match_tag{0};
 
 // The batched match: the order in which the queries are taken, then the kernel.  `state` (nullable) receives the
 // per-query records, stamped with `tag`.
 rt_status launch_match(rt_tree* t, const int32_t* d_q_tokens, const int64_t* d_q_offsets, int32_t nq, int32_t* d_match_len,
                        int32_t* d_term_node, int32_t* d_term_off, MatchState* state, unsigned long long tag, cudaStream_t s) {
-    const int32_t* perm = nullptr;
-    if (nq >= KLPM_ORDER_MIN) {
-        if (nq > t->match_cap) {
-            cudaFree(t->match_perm); cudaFree(t->match_bucket);
-            t->match_perm = nullptr; t->match_bucket = nullptr; t->match_cap = 0;
-            rt_status st;
-            if ((st = dalloc(&t->match_perm, nq)) || (st = dalloc(&t->match_bucket, nq))) return st;
-            t->match_cap = nq;
-        }
-        if (!t->match_hist) { rt_status st = dalloc(&t->match_hist, KLPM_ORDER_BUCKETS); if (st) return st; }
-        const unsigned qb = (unsigned)((nq + 255) / 256);
-        CK(cudaMemsetAsync(t->match_hist, 0, KLPM_ORDER_BUCKETS * sizeof(unsigned int), s));
-        order_hist_kernel<<<qb, 256, 0, s>>>(d_q_tokens, d_q_offsets, nq, t->match_hist, t->match_bucket);
-        order_scan_kernel<<<1, 1024, 0, s>>>(t->match_hist);
-        order_scatter_kernel<<<qb, 256, 0, s>>>(t->match_bucket, nq, t->match_hist, t->match_perm);
-        perm = t->match_perm;
+    if (nq <= (t->cfg.budget_tokens == 0 ? KLPM_WIDE_MAX_CHAIN : KLPM_WIDE_MAX_HOPS)) {
+        // as many warps per query (a power of two, 8 at most) as leave every query of the batch resident at once
+        const long long resident = (long long)t->num_sms * 32;
+        int warps = 8;
+        while (warps > 1 && (long long)nq * warps > resident) warps >>= 1;
+        if (t->cfg.budget_tokens == 0) match_wide_kernel<true><<<(unsigned)nq, warps * 32, 0, s>>>(t->dev, d_q_tokens, d_q_offsets, d_match_len,
+                                                                                                  d_term_node, d_term_off, state, tag);
+        else match_wide_kernel<false><<<(unsigned)nq, warps * 32, 0, s>>>(t->dev, d_q_tokens, d_q_offsets, d_match_len, d_term_node,
+                                                                          d_term_off, state, tag);
+        CK(cudaGetLastError());
+        return RT_OK;
     }
+    if (nq > t->match_cap) {
+        cudaFree(t->match_perm); cudaFree(t->match_bucket);
+        t->match_perm = nullptr; t->match_bucket = nullptr; t->match_cap = 0;
+        rt_status st;
+        if ((st = dalloc(&t->match_perm, nq)) || (st = dalloc(&t->match_bucket, nq))) return st;
+        t->match_cap = nq;
+    }
+    if (!t->match_hist) { rt_status st = dalloc(&t->match_hist, KLPM_ORDER_BUCKETS); if (st) return st; }
+    const unsigned qb = (unsigned)((nq + 255) / 256);
+    CK(cudaMemsetAsync(t->match_hist, 0, KLPM_ORDER_BUCKETS * sizeof(unsigned int), s));
+    order_hist_kernel<<<qb, 256, 0, s>>>(d_q_tokens, d_q_offsets, nq, t->match_hist, t->match_bucket);
+    order_scan_kernel<<<1, 1024, 0, s>>>(t->match_hist);
+    order_scatter_kernel<<<qb, 256, 0, s>>>(t->match_bucket, nq, t->match_hist, t->match_perm);
+    const int32_t* perm = t->match_perm;
     CK(cudaMemsetAsync(t->match_counter, 0, sizeof(unsigned long long), s));
     const int threads = 256, warps_per_block = threads / 32;
     long long blocks = ((long long)nq + warps_per_block - 1) / warps_per_block;

@@ -1,0 +1,88 @@
+"""Calls of the sizes an online scheduler makes: few queries per batched match, short queues per selection."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2502_04677_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SMS = 148                                        # the batch sizes at which a B200 takes fewer warps per query
+
+
+@pytest.fixture(scope="module")
+def K():
+    from paper_2502_04677_b200 import binding
+    return binding
+
+
+def long_edges():
+    """Cached prompts that cut two trunks at many depths, and queries that leave them around every comparison boundary (512 tokens per
+    warp, 4,096 per CTA), inside edges and at node ends, at every 16-byte phase."""
+    rng = np.random.RandomState(3)
+    trunks = [rng.randint(0, 1000, size=9000).tolist() for _ in range(2)]
+    cached = [trunks[0], trunks[1][:5000] + [1001] * 40]
+    for cut in (1, 511, 512, 513, 3000, 4096, 4100, 8190):
+        cached.append(trunks[0][:cut] + [1002] + trunks[1][:700])
+    queries = [[], [2000], trunks[0], trunks[0] + [7], trunks[1], trunks[0][:512], trunks[0][:4096]]
+    for d in [1, 2, 127, 128, 510, 511, 512, 513, 514, 1023, 1024, 1025, 3583, 3584, 3585, 4094, 4095, 4096, 4097, 4608, 4609, 8189, 8190, 8191,
+              8192, 8193, 8999]:
+        queries.append(trunks[0][:d] + [1003, 5])
+        queries.append(trunks[0][:d] + [1002] + trunks[1][:d // 2] + [1003])
+        queries.append(trunks[1][:d])
+    return cached, queries
+
+
+@pytest.mark.parametrize("budget", [0, 60_000])
+@pytest.mark.parametrize("n", [1, 4 * SMS, 4 * SMS + 1, 8 * SMS + 1, 16 * SMS + 1, 32 * SMS, 32 * SMS + 1])
+def test_match_of_few_queries(K, n, budget):
+    cached, queries = long_edges()
+    ct, co = W.to_csr(cached)
+    tree = K.rt_create(max_nodes=4 * len(cached) + 16, max_pool_tokens=ct.numel() + 8 * len(cached) + 16, budget_tokens=budget,
+                       max_clock=len(cached) + 16)
+    K.rt_insert(tree, ct.cuda(), co.cuda())
+    ot = oracle.OracleTree(budget)
+    ot.insert(ct.numpy(), co.numpy())
+    which = [(5 * i + 2) % len(queries) for i in range(n)]
+    lens = np.array([len(queries[w]) for w in which], dtype=np.int64)
+    pad = 3                                      # the first query starts off a 16-byte boundary
+    off = np.zeros(n + 1, dtype=np.int64)
+    off[0] = pad
+    off[1:] = pad + np.cumsum(lens)
+    flat = [torch.tensor(q, dtype=torch.int32) for q in queries]
+    tok = torch.cat([torch.zeros(pad, dtype=torch.int32)] + [flat[w] for w in which] + [torch.zeros(8, dtype=torch.int32)]).cuda()
+    m, node, at = (torch.full((n,), -7, dtype=torch.int32, device="cuda") for _ in range(3))
+    K.rt_match_batch(tree, tok, torch.from_numpy(off).cuda(), m, node, at)
+    assert K.rt_sync_status(tree) == 0
+    qt, qo = W.to_csr(queries)
+    want_m, want_at, want_depth = (np.asarray(x)[which] for x in ot.match_pos(qt.numpy(), qo.numpy()))
+    assert np.array_equal(m.cpu().numpy(), want_m)
+    assert np.array_equal(at.cpu().numpy(), want_at)
+    assert np.array_equal((m - at).cpu().numpy(), want_depth)
+    assert np.array_equal((node == 0).cpu().numpy(), want_m == 0)
+    if n > 1:                                    # the records of the same match carry a whole schedule (trees without a budget use them)
+        state = K.match_state_buffer(n, "cuda")
+        K.rt_match_batch_ex(tree, tok, torch.from_numpy(off).cuda(), m, node, at, state)
+        assert np.array_equal(m.cpu().numpy(), want_m)
+
+
+@pytest.mark.parametrize("n", [16_384, 16_385])
+def test_match_around_the_ordered_batches(K, n):
+    """Trees without a budget: the last batch size that is taken in index order and the first that is ordered."""
+    cached, queries = long_edges()
+    queries = [q[:900] for q in queries]
+    ct, co = W.to_csr(cached)
+    tree = K.rt_build(ct.cuda(), co.cuda(), max_nodes=4 * len(cached) + 16, max_pool_tokens=ct.numel() + 8 * len(cached) + 16)
+    qt, qo = W.to_csr(queries)
+    want = oracle.OracleTree(0)
+    want.insert(ct.numpy(), co.numpy())
+    want_m = want.match_pos(qt.numpy(), qo.numpy())[0]
+    reps = -(-n // len(queries))
+    tok = qt.repeat(reps).cuda()
+    lens = np.tile(np.diff(qo.numpy()), reps)
+    off = np.concatenate([[0], np.cumsum(lens)])[:n + 1]
+    m = torch.full((n,), -7, dtype=torch.int32, device="cuda")
+    K.rt_match_batch(tree, tok, torch.from_numpy(off).cuda(), m)
+    assert K.rt_sync_status(tree) == 0
+    assert np.array_equal(m.cpu().numpy(), np.tile(want_m, reps)[:n])
