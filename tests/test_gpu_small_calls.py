@@ -86,3 +86,25 @@ def test_match_around_the_ordered_batches(K, n):
     K.rt_match_batch(tree, tok, torch.from_numpy(off).cuda(), m)
     assert K.rt_sync_status(tree) == 0
     assert np.array_equal(m.cpu().numpy(), np.tile(want_m, reps)[:n])
+
+
+@pytest.mark.parametrize("n", [0, 1, 31, 33, 1023, 1025, 8191, 8192, 8193])
+def test_selection_on_both_sides_of_the_one_cta_kernel(K, n):
+    """One pick and the 64 best of queues around a warp, a thread per query and the largest queue that one CTA holds: few distinct
+    values (ties), negative and large arrivals, queues with fewer than 64 waiting."""
+    g = torch.Generator().manual_seed(n)
+    m = torch.randint(0, 7, (n,), generator=g, dtype=torch.int32)
+    t = torch.randint(-2, 3, (n,), generator=g, dtype=torch.int64) * ((1 << 33) + 1)
+    for waiting in (torch.ones(n, dtype=torch.uint8), (torch.randint(0, 200, (n,), generator=g) == 0).to(torch.uint8), torch.zeros(n, dtype=torch.uint8)):
+        d = m.cuda(), t.cuda(), waiting.cuda()
+        for policy, k, c in ((K.POLICY_KLPM, 3, 6), (K.POLICY_KLPM, 3, 7), (K.POLICY_FCFS, 1, 1), (K.POLICY_LPM, 1, 0)):
+            pick, same = torch.full((1,), -7, dtype=torch.int32, device="cuda"), torch.full((1,), -7, dtype=torch.int32, device="cuda")
+            K.klpm_select(*d, c, K.make_params(policy, k), pick)
+            K.klpm_select_noalloc(*d, c, K.make_params(policy, k), same)
+            want = oracle.select(m.numpy(), t.numpy(), waiting.numpy(), c, policy, k) if n else -1
+            assert int(pick) == want and int(same) == want
+        out = torch.full((64,), -7, dtype=torch.int32, device="cuda")
+        K.klpm_select_topk(*d, out)
+        idx = np.nonzero(waiting.numpy())[0]
+        best = sorted(idx.tolist(), key=lambda i: (-int(m[i]), int(t[i]), i))[:64]
+        assert out.tolist() == best + [-1] * (64 - len(best))
