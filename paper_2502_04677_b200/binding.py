@@ -104,20 +104,22 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
-def _dev(t: Optional[torch.Tensor], dtype, name: str, nullable: bool = False):
+def _dev(t: Optional[torch.Tensor], dtype, name: str, nullable: bool = False) -> Optional[int]:
     if t is None:
         if nullable:
             return None
         raise ValueError("%s must not be None" % name)
     if not t.is_cuda:
         raise ValueError("%s must be a CUDA tensor (this library has no CPU path)" % name)
-    if t.dtype != dtype or not t.is_contiguous():
+    if t.dtype is not dtype or not t.is_contiguous():
         raise ValueError("%s must be a contiguous %s tensor" % (name, dtype))
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    """The current stream's handle.  (Without a torch.cuda.Stream object around it: that object costs more than the
+    launches of a small call.)"""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _check(code: int, where: str) -> None:
