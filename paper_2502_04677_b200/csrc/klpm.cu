@@ -756,6 +756,7 @@ match_wide_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* __
         int64_t run = CHAIN ? c.chain_end - c.span_off : (int64_t)c.span_len;
         if (run > (int64_t)(len - m)) run = len - m;
         const int32_t x = wide_mismatch(q + m, T.pool + c.span_off, (int32_t)run, s_min, phase);     // x >= 1: the first token is the key
+        if (x <= 0) { probe_limit(T.st); break; }                 // (an entry that does not lead to its token: cannot happen)
         m += x;
         pos = c.span_off + x - 1;
         if (CHAIN) {
@@ -1560,6 +1561,10 @@ struct alignas(32) FStat {    // constant during the loop; the first 16 bytes ar
     int32_t pad;
 };
 
+// Trees with a budget: what the loop reads of a node, in one 32-byte sector (the tree's arrays are packed into these
+// records before the loop and written back after it).  nchild < 0: evicted.
+struct alignas(32) LNode { int32_t parent, depth, len, nchild; long long last, off; };
+
 struct FastPost {
     int32_t c0; int32_t pad; long long now0;    // first decision made in list mode; the time it was made at
     // what the loop did (rt_debug_counters): careful steps, dissolves by the whole CTA, fallback scans, slots that fell
@@ -1598,6 +1603,8 @@ struct FastArgs {
     int32_t lru;                  // 1: the tree has a budget
     int32_t mem_cap;              // entries of the member array (groups formed by evictions are appended behind the first n)
     TreeDev T;
+    LNode* node;                  // the tree's node arrays, one record per node, while the loop runs
+    const long long* sorted_t;    // per slot: arrival, side by side
     int32_t* parked;              // per node: unprocessed slots whose hint is that node
     int32_t* hintc;               // per slot: the hint once more, side by side (what the scan after an eviction reads)
     int2* leaf_run;               // per node: the member run that holds every slot whose hint is that node (y < 0: no such run is known)
@@ -1652,6 +1659,25 @@ __device__ __forceinline__ FStat ld_stat(const FStat* p) {
     s.soff = (long long)(((unsigned long long)(unsigned)b.y << 32) | (unsigned)b.x);
     s.rank = b.z; s.pad = 0;
     return s;
+}
+__device__ __forceinline__ LNode ld_node(const LNode* p) {
+    const int4* q = reinterpret_cast<const int4*>(p);
+    const int4 a = q[0], b = q[1];
+    LNode r;
+    r.parent = a.x; r.depth = a.y; r.len = a.z; r.nchild = a.w;
+    r.last = (long long)(((unsigned long long)(unsigned)b.y << 32) | (unsigned)b.x);
+    r.off = (long long)(((unsigned long long)(unsigned)b.w << 32) | (unsigned)b.z);
+    return r;
+}
+__device__ __forceinline__ void st_node(LNode* p, const LNode& r) {
+    int4* q = reinterpret_cast<int4*>(p);
+    q[0] = make_int4(r.parent, r.depth, r.len, r.nchild);
+    q[1] = make_int4((int)(unsigned)(unsigned long long)r.last, (int)(unsigned)((unsigned long long)r.last >> 32),
+                     (int)(unsigned)(unsigned long long)r.off, (int)(unsigned)((unsigned long long)r.off >> 32));
+}
+__device__ __forceinline__ void named_arrive(int id, int nthreads) {      // does not wait; what was written before is seen by whoever the barrier releases
+    __threadfence_block();
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 __device__ __forceinline__ void named_bar(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -1779,6 +1805,35 @@ struct FastTour {
 };
 // A word of one of the loop's bitmaps: shared memory, or global memory read through L2 (other warps set bits with atomics).
 __device__ __forceinline__ unsigned bm_ld(const unsigned int* p, long long i, int g) { return g ? __ldcg(p + i) : p[i]; }
+
+// The first unprocessed slot after `head` (which is processed); n if there is none.  One warp.
+__device__ __forceinline__ int32_t next_head(const unsigned int* s_done, int gdone, int32_t nwords, int32_t n, int32_t head, int lane) {
+    if (head + 1 < n) {                                     // the usual cases: the next slot, or one of the next 32 to 63
+        const int32_t h1 = head + 1, wi = h1 >> 5;
+        const unsigned f0 = ~bm_ld(s_done, wi, gdone) & ~((1u << (h1 & 31)) - 1u);
+        if (f0) { head = wi * 32 + __ffs(f0) - 1; return head > n ? n : head; }
+        if (wi + 1 < nwords) {
+            const unsigned f1 = ~bm_ld(s_done, wi + 1, gdone);
+            if (f1) { head = (wi + 1) * 32 + __ffs(f1) - 1; return head > n ? n : head; }
+        }
+    }
+    int32_t w0 = head >> 5;
+    for (;;) {
+        const int32_t wi = w0 + lane;
+        unsigned w = 0u;                                      // past the end: "unprocessed", so the search stops
+        if (wi < nwords) w = bm_ld(s_done, wi, gdone);
+        if (wi == (head >> 5)) w |= (1u << (head & 31)) - 1u;
+        const unsigned bal = __ballot_sync(FULL_MASK, w != 0xffffffffu);
+        if (bal) {
+            const int src = __ffs(bal) - 1;
+            const unsigned fw = ~__shfl_sync(FULL_MASK, w, src);
+            head = (w0 + src) * 32 + __ffs(fw) - 1;
+            break;
+        }
+        w0 += 32;
+    }
+    return head > n ? n : head;
+}
 
 // Recompute the ancestors of leaf block b; returns the root.  One warp.
 __device__ __forceinline__ unsigned long long tour_update(const FastTour& R, int32_t b, int lane) {
@@ -1952,6 +2007,35 @@ __device__ __forceinline__ unsigned long long fast_member(const FastArgs& A, con
     }
     if (!live) return KLPM_FAST_NOGROUP;
     return d.m < s.len ? group_hash(d.pos, d.ntok) : single_hash(r);
+}
+
+// Small groups are handled by the sequencer warp alone, unless several long compares are better spread over the CTA.
+__device__ __forceinline__ bool dissolve_is_small(int32_t gcount, int32_t unc) { return gcount <= 32 && !(gcount > 2 && unc > 512); }
+
+// The sequencer warp dissolves a group of at most 32 members and regroups it inside its run; returns the tournament's root.
+__device__ __forceinline__ unsigned long long dissolve_small(const FastArgs& A, const FastPick& P, const FastTour& R, unsigned long long root, int lane) {
+    const int32_t r = lane < P.gcount ? __ldcg(A.mem + P.gstart + lane) : -1;
+    bool touched;
+    const unsigned long long h = fast_member(A, P, R, r, lane, &touched);
+    int32_t rank = 0, start = 0, cnt = 0;
+    for (int k2i = 0; k2i < 32; ++k2i) {
+        const unsigned long long hk = __shfl_sync(FULL_MASK, h, k2i);
+        const bool lt = hk < h, eq = hk == h;
+        start += lt; cnt += eq; rank += (lt || (eq && k2i < lane));
+    }
+    if (h != KLPM_FAST_NOGROUP) {
+        __stcg(A.mem + P.gstart + rank, r);
+        st_dyn_group(A.dyn + r, P.gstart + start, cnt);
+        set_grouped(R, r, cnt > 1);
+    }
+    __syncwarp();
+    unsigned tm = __ballot_sync(FULL_MASK, touched);
+    while (tm) {
+        const int src = __ffs(tm) - 1; tm &= tm - 1;
+        const int32_t bb = __shfl_sync(FULL_MASK, r >> A.lb_shift, src);
+        root = tour_update(R, bb, lane);
+    }
+    return root;
 }
 
 // The warp-wide step of list mode (see fast_run_kernel) with the whole CTA: 1,024 list entries and 8,192 bitmap slots
@@ -2332,6 +2416,7 @@ __device__ void admit_blocks(const FastArgs& A, const FastTour& R, int32_t a0, i
 }
 
 // Work the whole CTA shares; every thread calls it with the same job.  Ends with t2 recomputed from t1.
+template <bool LRU>
 __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J, unsigned long long* sh, int32_t* sr, int* s_cnt,
                          int32_t* s_memcur) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -2340,6 +2425,7 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
         // slots [a0, a1) have arrived: the largest key of every leaf block they fall into
         admit_blocks(A, R, J.a0, J.a1);
     } else if (J.type == FAST_JOB_FALLBACK) {
+      if constexpr (LRU) {
         // Trees with a budget: a leaf in which queries were parked has been evicted.  Every unprocessed slot whose hint
         // is a dead node walks up to the node its match ends in now; the slots that lose matched tokens that way (the
         // match ended inside an evicted leaf) end at the end of a live node's edge, get their new state and key, and
@@ -2355,7 +2441,7 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
 #pragma unroll
             for (int u = 0; u < 4; ++u) { const int32_t r = r0 + u * nthr; hh[u] = r < A.n ? __ldcg(A.hintc + r) : 0; }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) dd[u] = hh[u] != 0 && __ldcg(A.T.dead + hh[u]) != 0;
+            for (int u = 0; u < 4; ++u) dd[u] = hh[u] != 0 && __ldcg(&A.node[hh[u]].nchild) < 0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int32_t r = r0 + u * nthr, h = hh[u];
@@ -2364,11 +2450,10 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
                 const int32_t m0 = __ldcg(dp + 2);
                 int32_t m = m0, a = h;
                 while (a != 0) {
-                    const bool dead = __ldcg(A.T.dead + a) != 0;
-                    const int32_t ds = __ldcg(A.T.depth_start + a);
-                    if (dead) { if (ds < m) m = ds; }
-                    else if (m > ds) break;
-                    a = __ldcg(A.T.parent + a);
+                    const LNode w = ld_node(A.node + a);
+                    if (w.nchild < 0) { if (w.depth < m) m = w.depth; }
+                    else if (m > w.depth) break;
+                    a = w.parent;
                 }
                 st_dyn_hint(A.dyn + r, a);
                 __stcg(A.hintc + r, a);
@@ -2376,7 +2461,8 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
                 A.leaf_run[a].y = -1;                        // slots from elsewhere are parked in a now: no one run holds them all
                 if (m != m0) {
                     const FStat s = ld_stat(A.stat + r);
-                    const long long pos = a == 0 ? -1 : __ldcg(A.T.span_off + a) + (long long)(m - __ldcg(A.T.depth_start + a)) - 1;
+                    long long pos = -1;
+                    if (a != 0) { const LNode w = ld_node(A.node + a); pos = w.off + (long long)(m - w.depth) - 1; }
                     const int32_t ntok = __ldg(A.tok + s.soff + m);                 // m < m0 <= length
                     st_dyn_state(A.dyn + r, pos, m, ntok);
                     __stcg(A.key + r, fast_key(m, s.len, s.rank, A.score_mode));
@@ -2420,6 +2506,7 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
                 admit_blocks_one(A, R, b, lo_slot, J.a1, lane);
             }
         }
+      }
     } else if (J.type == FAST_JOB_REBUILD) {
         // entering list mode (32-slot leaf blocks): the tournament keeps only the unprocessed slots whose key has changed
         for (int32_t b = warp; b < A.nb; b += nwarps) {
@@ -2466,7 +2553,7 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
                     const long long pos2 = P.vleaf + e - 1;
                     const int32_t ntok2 = m2 < s.len ? __ldg(qq + m2) : 0;
                     st_dyn_state(A.dyn + r, pos2, m2, ntok2);
-                    if (A.lru) lru_move(A, r, __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 6), P.leaf);
+                    if (LRU) lru_move(A, r, __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 6), P.leaf);
                     const unsigned long long key = fast_key(m2, s.len, s.rank, A.score_mode);
                     __stcg(A.key + r, key);
                     if (R.skip) atomicOr(R.skip + (r >> 5), 1u << (r & 31));
@@ -2518,10 +2605,7 @@ fast_run_kernel(FastArgs A) {
     __shared__ int32_t s_H[32], s_E[32];      // a batch's oldest-first and longest-match picks, by rank
     __shared__ FastBatchIO s_bio;             // a CTA-wide batch: what the sequencer hands over and gets back
     __shared__ int32_t s_scan[KLPM_FAST_THREADS / 32];
-    __shared__ TreeState s_st;                // trees with a budget: the tree's counters while the loop runs
-    __shared__ int32_t s_memcur;              // trees with a budget: first free entry of the member array
-    __shared__ unsigned int s_dirty[256];
-    if (A.lru && *reinterpret_cast<const volatile int32_t*>(A.skip)) return;       // the capacity check said no: nothing is touched
+    __shared__ int32_t s_memcur;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t n = A.n;
     const int32_t nb1p = (A.nb + 31) & ~31, n2 = nb1p >> 5, n2p = (n2 + 31) & ~31, n3 = n2p >> 5;
@@ -2540,12 +2624,12 @@ fast_run_kernel(FastArgs A) {
     R.done = A.done_in_smem ? s_bits : A.done;
     R.skip = !A.list_mode ? nullptr : A.bits_in_smem ? s_bits + nwords : A.gskip;
     R.gb = !A.list_mode ? nullptr : A.bits_in_smem ? s_bits + 2 * nwords : A.gbits;
-    R.dirty = s_dirty;
+    R.dirty = nullptr;
     unsigned int* const s_done = R.done;
     if (!G) { R.g_done = 0; R.g_bits = 0; }
     const int gdone = G ? R.g_done : 0, gbits = G ? R.g_bits : 0;
     for (int32_t i = threadIdx.x; i < nb1p + n2p + 32; i += blockDim.x) R.t1[i] = 0ULL;
-    if (threadIdx.x == 0) { s_memcur = A.lru ? 2 * n : n; if (A.lru) s_st = *A.st; }
+    if (threadIdx.x == 0) s_memcur = n;
     if (A.done_in_smem) for (int32_t i = threadIdx.x; i < nwords; i += blockDim.x) s_bits[i] = 0u;
     if (A.list_mode && A.bits_in_smem) for (int32_t i = threadIdx.x; i < nwords; i += blockDim.x) { R.skip[i] = 0u; R.gb[i] = __ldcg(A.gbits + i); }
     __syncthreads();
@@ -2556,7 +2640,7 @@ fast_run_kernel(FastArgs A) {
             const FastJob J = s_job;
             if (J.type == FAST_JOB_EXIT) return;
             if (J.type == FAST_JOB_BATCH) { fast_batch_job<G>(A, R, &s_bio, sr, sr + 1024, sr + 2048, reinterpret_cast<int32_t*>(sh), s_scan, nwords); continue; }
-            fast_job(A, R, J, sh, sr, &s_cnt, &s_memcur);
+            fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
         }
     }
 
@@ -2566,39 +2650,12 @@ fast_run_kernel(FastArgs A) {
     int32_t head = 0, admitted = 0;
     long long next_t = __ldg(&A.stat[0].t);
     unsigned long long root = 0;
-    long long n_careful = 0, n_cta_dissolve = 0, n_scan = 0, n_evict = 0, cy_tree = 0, cy_scan = 0, cy_dissolve = 0;
+    long long n_careful = 0, n_cta_dissolve = 0, cy_dissolve = 0;
     int32_t cyc = 0;                                        // c mod k
     int32_t c = 0;
     bool failed = false;
 
-    // first unprocessed slot at or after `head` (which is processed)
-    auto advance_head = [&]() {
-        if (head + 1 < n) {                                 // the usual cases: the next slot, or one of the next 32 to 63
-            const int32_t h1 = head + 1, wi = h1 >> 5;
-            const unsigned f0 = ~bm_ld(s_done, wi, gdone) & ~((1u << (h1 & 31)) - 1u);
-            if (f0) { head = wi * 32 + __ffs(f0) - 1; if (head > n) head = n; return; }
-            if (wi + 1 < nwords) {
-                const unsigned f1 = ~bm_ld(s_done, wi + 1, gdone);
-                if (f1) { head = (wi + 1) * 32 + __ffs(f1) - 1; if (head > n) head = n; return; }
-            }
-        }
-        int32_t w0 = head >> 5;
-        for (;;) {
-            const int32_t wi = w0 + lane;
-            unsigned w = 0u;                                  // past the end: "unprocessed", so the search stops
-            if (wi < nwords) w = bm_ld(s_done, wi, gdone);
-            if (wi == (head >> 5)) w |= (1u << (head & 31)) - 1u;
-            const unsigned bal = __ballot_sync(FULL_MASK, w != 0xffffffffu);
-            if (bal) {
-                const int src = __ffs(bal) - 1;
-                const unsigned fw = ~__shfl_sync(FULL_MASK, w, src);
-                head = (w0 + src) * 32 + __ffs(fw) - 1;
-                break;
-            }
-            w0 += 32;
-        }
-        if (head > n) head = n;
-    };
+    auto advance_head = [&]() { head = next_head(s_done, gdone, nwords, n, head, lane); };
     // slot j is processed from now on (every lane performs the same shared-memory stores)
     auto mark_done = [&](int32_t j) {
         if (!gdone) s_done[j >> 5] |= 1u << (j & 31);
@@ -2628,279 +2685,13 @@ fast_run_kernel(FastArgs A) {
         // the new leaf's positions: unique per decision, above every real pool index
         const long long vleaf = A.vbase + ((long long)c << 32);
         ++c;
-        int32_t leaf = -1;
         ++n_careful;
-        if (A.lru) {
-            const long long t_tree = clock64();
-            // ---- the tree's node arrays follow the decision (what insert_serial does, minus the child table and the
-            //      tokens, which the pass after the loop writes for the nodes that are still alive then)
-            const TreeDev& T = A.T;
-            if (lane == 0) atomicSub(A.parked + d.hint, 1);
-            if (s_st.clock + 1 >= T.max_clock || s_st.n_nodes + 2 > T.max_nodes) {        // (the check before the loop rules this out)
-                if (lane == 0) set_status(A.st, RT_ERR_CAPACITY, 114);
-                failed = true; return;
-            }
-            const long long clock = s_st.clock + 1;
-            // Two chains of dependent loads are started side by side: the node the match ends in (hint, then up), and
-            // the least recently used leaf (the cursor's next 32 clock values, their owners' fields) -- most decisions
-            // evict, and which leaf goes does not depend on the pick, except that the node stamped below is safe.
-            const long long cur0 = s_st.lru_cursor;
-            int32_t a = d.hint;
-            int32_t ds = T.depth_start[a], sl = T.span_len[a], pa = T.parent[a];
-            const long long pre_cc = cur0 + lane;
-            const int32_t pre_v = pre_cc < clock ? T.clock_owner[pre_cc] : 0;
-            bool pre_ok = false;
-            int32_t pre_P = 0, pre_len = 0, pre_parked = 0;
-            if (pre_v > 0) {
-                pre_ok = !T.dead[pre_v] && T.last_access[pre_v] == pre_cc && T.nchild[pre_v] == 0;
-                pre_P = T.parent[pre_v]; pre_len = T.span_len[pre_v]; pre_parked = __ldcg(A.parked + pre_v);
-            }
-            while (a != 0 && m <= ds) { a = pa; ds = T.depth_start[a]; sl = T.span_len[a]; pa = T.parent[a]; }
-            const int32_t o = a == 0 ? 0 : m - ds;
-            int32_t end = a;
-            bool cut = false;
-            long long n_nodes = s_st.n_nodes, live_nodes = s_st.live_nodes, tokens_live = s_st.tokens_live, evictions = s_st.evictions;
-            if (a != 0 && o < sl) {                         // node boundary inside a's edge: a new node takes the upper part
-                const int32_t u = (int32_t)n_nodes++;
-                ++live_nodes;
-                cut = true;
-                if (lane == 0) {
-                    const int64_t so = T.span_off[a];
-                    T.parent[u] = pa; T.depth_start[u] = ds; T.span_off[u] = so; T.span_len[u] = o;
-                    T.nchild[u] = 1; T.dead[u] = 0; T.last_access[u] = T.last_access[a];
-                    T.span_off[a] = so + o; T.span_len[a] = sl - o; T.depth_start[a] = ds + o; T.parent[a] = u;
-                }
-                end = u;
-            }
-            if (end != 0 && lane == 0) { T.last_access[end] = clock; T.clock_owner[clock] = end; }
-            __syncwarp();
-            // least recently used leaves go until the prompt's uncached tokens fit (the node just stamped is safe)
-            bool scan = false;
-            int32_t small_v[8];                             // evicted leaves whose parked queries this warp looks after itself
-            int n_small = 0;
-            long long cur = cur0;
-            // The leaves of the window that was loaded ahead are taken one after the other while the window's view of who
-            // is a leaf holds: it ends when an eviction turns a parent into a leaf (that parent may be the next to go).
-            bool first = true, win_ok = true;
-            unsigned win = 0;
-            while (tokens_live + unc > T.budget) {
-                int32_t victim = -1, P = 0, vlen = 0, vparked = 0;
-                if (win_ok) {
-                    if (first) { win = __ballot_sync(FULL_MASK, pre_ok && pre_v != end); first = false; }      // (the node stamped above has moved on)
-                    if (win) {
-                        const int src = __ffs(win) - 1;
-                        win &= win - 1;
-                        victim = __shfl_sync(FULL_MASK, pre_v, src); P = __shfl_sync(FULL_MASK, pre_P, src);
-                        vlen = __shfl_sync(FULL_MASK, pre_len, src); vparked = __shfl_sync(FULL_MASK, pre_parked, src);
-                        cur = cur0 + src;
-                        if (cut && victim == a) { P = T.parent[victim]; vlen = T.span_len[victim]; }      // the lower part of the edge just cut
-                    } else {
-                        cur = cur0 + 32;
-                        win_ok = false;
-                    }
-                }
-                if (victim < 0) {
-                    while (cur < clock) {                   // 32 clock values at a time
-                        const long long cc = cur + lane;
-                        const int32_t v = cc < clock ? T.clock_owner[cc] : 0;
-                        const bool ok = v > 0 && !T.dead[v] && T.last_access[v] == cc && T.nchild[v] == 0;
-                        const unsigned bal = __ballot_sync(FULL_MASK, ok);
-                        if (bal) { const int src = __ffs(bal) - 1; victim = __shfl_sync(FULL_MASK, v, src); cur += src; break; }
-                        cur += 32;
-                    }
-                    if (victim >= 0) { P = T.parent[victim]; vlen = T.span_len[victim]; vparked = __ldcg(A.parked + victim); }
-                }
-                if (victim < 0) {
-                    if (lane == 0) set_status(A.st, RT_ERR_BUDGET);
-                    failed = true; break;
-                }
-                tokens_live -= vlen;
-                --live_nodes; ++evictions; ++n_evict;
-                if (vparked > 0) {
-                    // Queries are parked in the evicted leaf.  If one run of the member array is known to hold every slot
-                    // whose hint is this leaf, the warp looks after them itself below (up to 8 such leaves and 32 slots
-                    // that fall back per decision); otherwise the whole CTA scans the unprocessed slots.
-                    const int2 lr = __ldcg(A.leaf_run + victim);
-                    if (lr.y > 0 && lr.y <= 1024 && n_small < 8) { small_v[n_small] = victim; ++n_small; }
-                    else scan = true;
-                }
-                int new_leaf = 0;
-                if (lane == 0) {
-                    T.dead[victim] = 1;
-                    const int32_t nc = T.nchild[P] - 1;
-                    T.nchild[P] = nc;
-                    const long long stamp = T.last_access[victim];
-                    if (P != 0 && stamp >= T.last_access[P]) { T.last_access[P] = stamp; T.clock_owner[stamp] = P; }
-                    new_leaf = nc == 0 && P != 0;
-                }
-                __syncwarp();
-                if (win_ok && __shfl_sync(FULL_MASK, new_leaf, 0)) win_ok = false;
-            }
-            if (cur > clock) cur = clock;
-            if (!failed && unc > 0) {
-                leaf = (int32_t)n_nodes++;
-                ++live_nodes;
-                tokens_live += unc;
-                if (lane == 0) {
-                    T.parent[leaf] = end; T.depth_start[leaf] = m; T.span_off[leaf] = vleaf; T.span_len[leaf] = unc;
-                    T.nchild[leaf] = 0; T.dead[leaf] = 0; T.last_access[leaf] = clock; T.clock_owner[clock] = leaf;
-                    T.nchild[end]++;
-                    A.leaf_run[leaf] = make_int2(d.gstart, d.gcount);     // whoever gets parked in it is a member of the pick's group
-                }
-            }
-            __syncwarp();
-            if (lane == 0) {
-                s_st.clock = clock; s_st.n_nodes = n_nodes; s_st.live_nodes = live_nodes; s_st.tokens_live = tokens_live;
-                s_st.evictions = evictions; s_st.lru_cursor = cur;
-            }
-            __syncwarp();
-            // ---- evicted leaves whose parked queries sit in known member runs: the warp moves them itself.  All leaves of
-            //      this decision are taken together: two of them, one above the other, send their queries to one group.
-            if (n_small > 0 && !scan && !failed) {
-                // first pass: how many slots fall back (more than 32: leave it to the scan)
-                int32_t n_fall = 0;
-                for (int sv = 0; sv < n_small; ++sv) {
-                    const int32_t v = small_v[sv];
-                    const int2 lr = __ldcg(A.leaf_run + v);
-                    const int32_t ds_v = T.depth_start[v];
-                    for (int32_t base = 0; base < lr.y; base += 32) {
-                        const int32_t r = base + lane < lr.y ? __ldcg(A.mem + lr.x + base + lane) : -1;
-                        bool hit = r >= 0 && !slot_done(R, A, r) && __ldcg(A.hintc + r) == v;
-                        if (hit) hit = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2) > ds_v;
-                        const unsigned same = __match_any_sync(FULL_MASK, hit ? r : -1 - lane);       // a slot can be listed twice in a run
-                        if (hit && (int)(__ffs(same) - 1) != lane) hit = false;
-                        n_fall += __popc(__ballot_sync(FULL_MASK, hit));
-                    }
-                }
-                if (n_fall > 32) scan = true;
-            }
-            if (n_small > 0 && !scan && !failed) {
-                // second pass: every member whose hint is a dead leaf walks up; those that lose tokens are collected
-                int32_t f_slot = -1;                        // lane k holds the k-th slot that fell back
-                unsigned long long f_hash = KLPM_FAST_NOGROUP;
-                int32_t n_f = 0;
-                for (int sv = 0; sv < n_small; ++sv) {
-                    const int32_t v = small_v[sv];
-                    const int2 lr = __ldcg(A.leaf_run + v);
-                    for (int32_t base = 0; base < lr.y; base += 32) {
-                        const int32_t r = base + lane < lr.y ? __ldcg(A.mem + lr.x + base + lane) : -1;
-                        bool hit = r >= 0 && !slot_done(R, A, r) && __ldcg(A.hintc + r) == v;
-                        const unsigned same = __match_any_sync(FULL_MASK, hit ? r : -1 - lane);
-                        if (hit && (int)(__ffs(same) - 1) != lane) hit = false;
-                        bool fell = false;
-                        unsigned long long h = KLPM_FAST_NOGROUP;
-                        if (hit) {
-                            const int32_t m0 = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2);
-                            int32_t mm = m0, a = v;
-                            while (a != 0) {
-                                const bool dead = T.dead[a] != 0;
-                                const int32_t dsa = T.depth_start[a];
-                                if (dead) { if (dsa < mm) mm = dsa; }
-                                else if (mm > dsa) break;
-                                a = T.parent[a];
-                            }
-                            st_dyn_hint(A.dyn + r, a);
-                            __stcg(A.hintc + r, a);
-                            atomicAdd(A.parked + a, 1);
-                            A.leaf_run[a].y = -1;
-                            if (mm != m0) {
-                                const FStat fs = ld_stat(A.stat + r);
-                                const long long pos = a == 0 ? -1 : T.span_off[a] + (long long)(mm - T.depth_start[a]) - 1;
-                                const int32_t ntok = __ldg(A.tok + fs.soff + mm);
-                                st_dyn_state(A.dyn + r, pos, mm, ntok);
-                                __stcg(A.key + r, fast_key(mm, fs.len, fs.rank, A.score_mode));
-                                h = group_hash(pos, ntok);
-                                fell = true;
-                            }
-                        }
-                        const unsigned fb = __ballot_sync(FULL_MASK, fell);
-                        const int32_t my = n_f + __popc(fb & ((1u << lane) - 1u));
-                        for (unsigned bits = fb; bits; bits &= bits - 1) {      // hand each fallen slot to the lane that keeps it
-                            const int src = __ffs(bits) - 1;
-                            const int32_t dst = __shfl_sync(FULL_MASK, my, src);
-                            const int32_t rr = __shfl_sync(FULL_MASK, r, src);
-                            const unsigned long long hh = __shfl_sync(FULL_MASK, h, src);
-                            if (lane == dst) { f_slot = rr; f_hash = hh; }
-                        }
-                        n_f += __popc(fb);
-                        __syncwarp();
-                    }
-                }
-                if (n_f > 0) {
-                    // the fallen slots are grouped afresh in a run appended to the member array (ranked by shuffles)
-                    const int32_t base = s_memcur;
-                    if ((long long)base + n_f > (long long)A.mem_cap) {
-                        if (lane == 0) set_status(A.st, RT_ERR_CAPACITY, 113);
-                        failed = true;
-                    } else {
-                        int32_t rank = 0, start = 0, cnt = 0;
-                        for (int k2i = 0; k2i < 32; ++k2i) {
-                            const unsigned long long hk = __shfl_sync(FULL_MASK, f_hash, k2i);
-                            const bool lt = hk < f_hash, eq = hk == f_hash;
-                            start += lt; cnt += eq; rank += (lt || (eq && k2i < lane));
-                        }
-                        if (f_slot >= 0) {
-                            __stcg(A.mem + base + rank, f_slot);
-                            st_dyn_group(A.dyn + f_slot, base + start, cnt);
-                            set_grouped(R, f_slot, cnt > 1);
-                        }
-                        if (lane == 0) s_memcur = base + n_f;
-                        __syncwarp();
-                        // their keys went down: the leaf blocks of the arrived ones are recomputed
-                        for (int k2i = 0; k2i < n_f; ++k2i) {
-                            const int32_t rr = __shfl_sync(FULL_MASK, f_slot, k2i);
-                            if (rr < admitted) {
-                                const int32_t bb = rr >> A.lb_shift;
-                                admit_blocks_one(A, R, bb, bb << A.lb_shift, admitted, lane);
-                                __syncwarp();
-                                root = tour_update(R, bb, lane);
-                            }
-                        }
-                    }
-                }
-            }
-            cy_tree += clock64() - t_tree;
-            if (scan) {                                     // somebody was parked in an evicted leaf
-                const long long t_scan = clock64();
-                ++n_scan;
-                if (lane == 0) { s_job.type = FAST_JOB_FALLBACK; s_job.a0 = head < slot ? head : slot; s_job.a1 = admitted; }
-                __threadfence_block();
-                __syncwarp();
-                named_bar(1, KLPM_FAST_THREADS);
-                const FastJob J = s_job;
-                fast_job(A, R, J, sh, sr, &s_cnt, &s_memcur);
-                root = tour_top(R, lane);
-                cy_scan += clock64() - t_scan;
-            }
-            if (failed) return;
-        }
         if (unc > 0 && d.gcount > 1) {
             FastPick P;
             P.slot = slot; P.m = m; P.len = len; P.ntok = d.ntok; P.x = A.tok + s.soff; P.pos = d.pos; P.vleaf = vleaf;
-            P.admitted = admitted; P.gstart = d.gstart; P.gcount = d.gcount; P.leaf = leaf;
-            // small groups are handled by this warp alone, unless several long compares are better spread over the CTA
-            if (d.gcount <= 32 && !(d.gcount > 2 && unc > 512)) {
-                const int32_t r = lane < d.gcount ? __ldcg(A.mem + d.gstart + lane) : -1;
-                bool touched;
-                const unsigned long long h = fast_member(A, P, R, r, lane, &touched);
-                int32_t rank = 0, start = 0, cnt = 0;       // regroup inside the run
-                for (int k2i = 0; k2i < 32; ++k2i) {
-                    const unsigned long long hk = __shfl_sync(FULL_MASK, h, k2i);
-                    const bool lt = hk < h, eq = hk == h;
-                    start += lt; cnt += eq; rank += (lt || (eq && k2i < lane));
-                }
-                if (h != KLPM_FAST_NOGROUP) {
-                    __stcg(A.mem + d.gstart + rank, r);
-                    st_dyn_group(A.dyn + r, d.gstart + start, cnt);
-                    set_grouped(R, r, cnt > 1);
-                }
-                __syncwarp();
-                unsigned tm = __ballot_sync(FULL_MASK, touched);
-                while (tm) {
-                    const int src = __ffs(tm) - 1; tm &= tm - 1;
-                    const int32_t bb = __shfl_sync(FULL_MASK, r >> A.lb_shift, src);
-                    root = tour_update(R, bb, lane);
-                }
+            P.admitted = admitted; P.gstart = d.gstart; P.gcount = d.gcount; P.leaf = -1;
+            if (dissolve_is_small(d.gcount, unc)) {
+                root = dissolve_small(A, P, R, root, lane);
             } else {
                 const long long t_dis = clock64();
                 ++n_cta_dissolve;
@@ -2908,7 +2699,7 @@ fast_run_kernel(FastArgs A) {
                 __syncwarp();
                 named_bar(1, KLPM_FAST_THREADS);
                 const FastJob J = s_job;
-                fast_job(A, R, J, sh, sr, &s_cnt, &s_memcur);
+                fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
                 root = tour_top(R, lane);
                 cy_dissolve += clock64() - t_dis;
             }
@@ -2967,7 +2758,7 @@ fast_run_kernel(FastArgs A) {
                 __syncwarp();
                 named_bar(1, KLPM_FAST_THREADS);
                 const FastJob J = s_job;
-                fast_job(A, R, J, sh, sr, &s_cnt, &s_memcur);
+                fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
                 root = tour_top(R, lane);
             }
             admitted = a1;
@@ -3005,7 +2796,7 @@ fast_run_kernel(FastArgs A) {
         named_bar(1, KLPM_FAST_THREADS);
         {
             const FastJob J = s_job;
-            fast_job(A, R, J, sh, sr, &s_cnt, &s_memcur);
+            fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
         }
         root = tour_top(R, lane);
         // the sorted list, 32 entries at a time: lane l holds entry (cur & ~31) + l, the next 32 are on their way
@@ -3163,7 +2954,9 @@ fast_run_kernel(FastArgs A) {
         // a batch that was cut short stopped before a decision only the one-at-a-time path can take: that one comes
         // next, without another attempt that would find it again
         bool one_next = false;
+        long long iters = 0;                                // every iteration makes a decision or gives up an attempt for a while
         while (c < n && !failed) {
+            if (++iters > 64LL * n + 4096) { if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 118); failed = true; break; }      // cannot happen
             // first choice: the whole CTA makes up to 1,024 decisions (the sort scratch is free between dissolves)
             if (!one_next && cb_wait <= 0 && calm >= KLPM_FAST_CALM && c >= cb_until && n - c >= KLPM_FAST_CTA_MIN) {
                 if (lane == 0) {
@@ -3284,17 +3077,519 @@ fast_run_kernel(FastArgs A) {
     __syncwarp();
     if (lane == 0) {
         long long* cn = A.post->counters;
-        cn[0] = n_careful; cn[1] = n_cta_dissolve; cn[2] = n_scan; cn[3] = s_memcur - (A.lru ? 2 * n : n); cn[4] = n_evict;
-        cn[5] = cy_tree; cn[6] = cy_scan; cn[7] = cy_dissolve;
-    }
-    if (A.lru && lane == 0) {                               // the tree's counters go back (a status recorded meanwhile stays)
-        TreeState out = s_st;
-        out.status = *reinterpret_cast<const volatile int*>(&A.st->status);
-        out.detail = *reinterpret_cast<const volatile int*>(&A.st->detail);
-        *A.st = out;
+        cn[0] = n_careful; cn[1] = n_cta_dissolve; cn[2] = 0; cn[3] = 0; cn[4] = 0; cn[5] = 0; cn[6] = 0; cn[7] = cy_dissolve;
     }
     if (lane == 0) s_job.type = FAST_JOB_EXIT;
     __syncwarp();
+    named_bar(1, KLPM_FAST_THREADS);
+}
+
+// The loop on a tree with a budget (and klpm_replay on one).  Every decision is a careful step, and a step has two
+// halves that need little of each other, so two warps share it:
+//   * warp 0 decides: admits who has arrived, picks, charges, and dissolves the pick's group;
+//   * warp 1 keeps the tree: brings the node records up to date as insert_serial would -- cut the edge the match ends
+//     in, stamp its node, evict least-recently-used leaves until the uncached tokens fit, add the leaf.  It keeps a
+//     window of 32 clock values and who owns them in registers from one decision to the next (lane i: the owner of
+//     value wbase + i, and whether it is a leaf that may go).
+// While warp 1 works on decision c, warp 0 prepares decision c + 1: admission, the likely pick's records and its leaf
+// block's keys are all asked for at once.  Only then does it wait for warp 1; nothing of c + 1 is committed before.  An
+// eviction that shortens matches (queries parked in the evicted leaf) is handed back: warp 0 moves those queries and
+// prepares the decision afresh.  A pick whose group has other members waits for its new leaf's id before the group is
+// dissolved.  The other warps join for work that is worth sharing; so does warp 1, which is idle then.
+// The two hand over through named barriers 2 (a job for warp 1) and 3 (its answer), helpers wait at barrier 1.
+// What bounds it: @@LRU@@
+struct LruJob { int32_t type; int32_t hint, m, len, gstart, gcount; long long vleaf; };
+struct LruAnswer { int32_t failed, scan, n_small, leaf; int32_t small_v[8]; };
+enum { LRU_JOB_EXIT = 0, LRU_JOB_STEP = 1, LRU_JOB_JOIN = 2 };
+
+// Warp 1.  Returns when the loop is over; *out receives the tree's counters.
+__device__ __forceinline__ void lru_tree_warp(const FastArgs& A, const FastTour& R, const LruJob* s_tj, LruAnswer* s_ta, const FastJob* s_job,
+                                              unsigned long long* sh, int32_t* sr, int* s_cnt, int32_t* s_memcur, int lane) {
+    const TreeDev& T = A.T;
+    TreeState st = *A.st;
+    const long long evictions0 = st.evictions;
+    long long wbase = st.lru_cursor, wend = wbase;          // the window's clock values: [wbase, wend)
+    int32_t wv = 0;                                         // this lane's owner
+    bool wok = false;                                       // it is a leaf and its stamp is this clock value
+    for (;;) {
+        named_bar(2, 64);
+        const LruJob J = *s_tj;
+        if (J.type != LRU_JOB_STEP) {
+            if (J.type == LRU_JOB_EXIT) break;
+            named_bar(1, KLPM_FAST_THREADS);
+            const FastJob F = *s_job;
+            fast_job<true>(A, R, F, sh, sr, s_cnt, s_memcur);
+            continue;
+        }
+        LruAnswer ans;
+        ans.failed = 0; ans.scan = 0; ans.n_small = 0; ans.leaf = -1;
+        const int32_t unc = J.len - J.m;
+        if (st.clock + 1 >= T.max_clock || st.n_nodes + 2 > T.max_nodes) {           // (the check before the loop rules this out)
+            if (lane == 0) { set_status(A.st, RT_ERR_CAPACITY, 114); s_ta->failed = 1; s_ta->scan = 0; s_ta->n_small = 0; s_ta->leaf = -1; }
+            __syncwarp();
+            named_arrive(3, 64);
+            continue;
+        }
+        const long long clock = ++st.clock;
+        // the node the match ends in, and beside it the next leaf to go
+        LNode ra = ld_node(A.node + J.hint);
+        int32_t v0 = -1, pk0 = 0;
+        LNode rv; rv.parent = 0; rv.depth = 0; rv.len = 0; rv.nchild = 0; rv.last = 0; rv.off = 0;
+        if (st.tokens_live + unc > T.budget) {
+            const unsigned okm = __ballot_sync(FULL_MASK, wok);
+            if (okm) {
+                v0 = __shfl_sync(FULL_MASK, wv, __ffs(okm) - 1);
+                rv = ld_node(A.node + v0);
+                pk0 = __ldcg(A.parked + v0);
+            }
+        }
+        if (lane == 0) atomicSub(A.parked + J.hint, 1);
+        int32_t a = J.hint;
+        while (a != 0 && J.m <= ra.depth) { a = ra.parent; ra = ld_node(A.node + a); }
+        const int32_t o = a == 0 ? 0 : J.m - ra.depth;
+        int32_t end = a;                                    // the node that ends where the match ends; its record, stored below
+        LNode e = ra;
+        const bool cut = a != 0 && o < ra.len;
+        if (cut) {                                          // a new node takes the upper part of a's edge
+            end = (int32_t)st.n_nodes++;
+            ++st.live_nodes;
+            e.len = o; e.nchild = 1;
+            ra.parent = end; ra.depth += o; ra.len -= o; ra.off += o;
+            if (lane == 0) st_node(A.node + a, ra);
+        }
+        if (end != 0) e.last = clock;
+        if (wv == end) wok = false;                         // (the node stamped here is safe)
+        __syncwarp();
+        while (st.tokens_live + unc > T.budget) {
+            unsigned okm = __ballot_sync(FULL_MASK, wok);
+            while (!okm && wend < clock) {                  // the next 32 clock values
+                wbase = wend;
+                const long long cc = wbase + lane;
+                wv = cc < clock ? T.clock_owner[cc] : 0;
+                wend = wbase + 32 < clock ? wbase + 32 : clock;
+                wok = false;
+                if (wv > 0 && wv != end) { const LNode w = ld_node(A.node + wv); wok = w.nchild == 0 && w.last == cc; }
+                okm = __ballot_sync(FULL_MASK, wok);
+            }
+            if (!okm) {
+                if (lane == 0) set_status(A.st, RT_ERR_BUDGET);
+                ans.failed = 1; break;
+            }
+            const int src = __ffs(okm) - 1;
+            const int32_t victim = __shfl_sync(FULL_MASK, wv, src);
+            const long long stamp = wbase + src;
+            if (victim != v0) { rv = ld_node(A.node + victim); pk0 = __ldcg(A.parked + victim); }
+            if (cut && victim == a) { rv.parent = end; rv.len = ra.len; }      // the lower part of the edge just cut
+            v0 = -1;
+            st.tokens_live -= rv.len;
+            --st.live_nodes; ++st.evictions;
+            if (pk0 > 0) {
+                // Queries are parked in the evicted leaf.  If one run of the member array is known to hold every slot whose
+                // hint is this leaf, warp 0 looks after them itself (up to 8 such leaves and 32 slots that fall back per
+                // decision); otherwise the whole CTA scans the unprocessed slots.
+                const int2 lr = __ldcg(A.leaf_run + victim);
+                if (lr.y > 0 && lr.y <= 1024 && ans.n_small < 8) { if (lane == 0) s_ta->small_v[ans.n_small] = victim; ++ans.n_small; }
+                else ans.scan = 1;
+            }
+            if (lane == src) wok = false;
+            const int32_t P = rv.parent;
+            if (lane == 0) A.node[victim].nchild = -1;
+            if (P == end) --e.nchild;                       // (its stamp is newer)
+            else {
+                LNode rp = ld_node(A.node + P);
+                const int32_t nc = rp.nchild - 1;
+                if (P != 0 && stamp >= rp.last) {           // the stamp goes to the parent if newer
+                    rp.last = stamp;
+                    if (lane == 0) { A.node[P].last = stamp; T.clock_owner[stamp] = P; }
+                }
+                if (lane == 0) A.node[P].nchild = nc;
+                // a parent that has become a leaf may be the next to go
+                if (nc == 0 && P != 0 && rp.last >= wbase && rp.last < wend && lane == (int)(rp.last - wbase)) { wv = P; wok = true; }
+            }
+            __syncwarp();
+        }
+        if (!ans.failed && unc > 0) {
+            ans.leaf = (int32_t)st.n_nodes++;
+            ++st.live_nodes;
+            st.tokens_live += unc;
+            ++e.nchild;
+            if (lane == 0) {
+                LNode l;
+                l.parent = end; l.depth = J.m; l.len = unc; l.nchild = 0; l.last = clock; l.off = J.vleaf;
+                st_node(A.node + ans.leaf, l);
+                T.clock_owner[clock] = ans.leaf;
+                A.leaf_run[ans.leaf] = make_int2(J.gstart, J.gcount);     // whoever gets parked in it is a member of the pick's group
+            }
+        } else if (end != 0 && lane == 0) T.clock_owner[clock] = end;
+        if (lane == 0) {
+            st_node(A.node + end, e);
+            s_ta->failed = ans.failed; s_ta->scan = ans.scan; s_ta->n_small = ans.n_small; s_ta->leaf = ans.leaf;
+        }
+        __syncwarp();
+        named_arrive(3, 64);
+    }
+    if (lane == 0) {                                        // the tree's counters go back (a status recorded meanwhile stays)
+        st.lru_cursor = wbase;
+        TreeState* S = A.st;
+        S->n_nodes = st.n_nodes; S->tokens_live = st.tokens_live; S->live_nodes = st.live_nodes; S->clock = st.clock;
+        S->lru_cursor = st.lru_cursor; S->evictions = st.evictions;
+        A.post->counters[4] = st.evictions - evictions0;
+    }
+    __syncwarp();
+    named_bar(1, KLPM_FAST_THREADS);                        // (the helpers are told to leave)
+}
+
+// Warp 0: the queries parked in leaves that the last decision evicted, when known member runs hold them all.  All leaves
+// are taken together: two of them, one above the other, send their queries to one group.  Returns false, nothing changed,
+// if more than 32 slots lose matched tokens (the caller has the CTA scan for them); *failed if there is no room.
+__device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTour& R, const int32_t* small_v, int n_small, int32_t admitted,
+                                                 int32_t* s_memcur, unsigned long long* root, bool* failed, int lane) {
+    int32_t n_fall = 0;
+    for (int sv = 0; sv < n_small; ++sv) {
+        const int32_t v = small_v[sv];
+        const int2 lr = __ldcg(A.leaf_run + v);
+        const int32_t ds_v = A.node[v].depth;
+        for (int32_t base = 0; base < lr.y; base += 32) {
+            const int32_t r = base + lane < lr.y ? __ldcg(A.mem + lr.x + base + lane) : -1;
+            bool hit = r >= 0 && !slot_done(R, A, r) && __ldcg(A.hintc + r) == v;
+            if (hit) hit = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2) > ds_v;
+            const unsigned same = __match_any_sync(FULL_MASK, hit ? r : -1 - lane);       // a slot can be listed twice in a run
+            if (hit && (int)(__ffs(same) - 1) != lane) hit = false;
+            n_fall += __popc(__ballot_sync(FULL_MASK, hit));
+        }
+    }
+    if (n_fall > 32) return false;
+    // every member whose hint is a dead leaf walks up; those that lose tokens are collected
+    int32_t f_slot = -1;                                    // lane k holds the k-th slot that fell back
+    unsigned long long f_hash = KLPM_FAST_NOGROUP;
+    int32_t n_f = 0;
+    for (int sv = 0; sv < n_small; ++sv) {
+        const int32_t v = small_v[sv];
+        const int2 lr = __ldcg(A.leaf_run + v);
+        for (int32_t base = 0; base < lr.y; base += 32) {
+            const int32_t r = base + lane < lr.y ? __ldcg(A.mem + lr.x + base + lane) : -1;
+            bool hit = r >= 0 && !slot_done(R, A, r) && __ldcg(A.hintc + r) == v;
+            const unsigned same = __match_any_sync(FULL_MASK, hit ? r : -1 - lane);
+            if (hit && (int)(__ffs(same) - 1) != lane) hit = false;
+            bool fell = false;
+            unsigned long long h = KLPM_FAST_NOGROUP;
+            if (hit) {
+                const int32_t m0 = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2);
+                int32_t mm = m0, a = v;
+                LNode w = ld_node(A.node + a);
+                while (a != 0) {
+                    if (w.nchild < 0) { if (w.depth < mm) mm = w.depth; }
+                    else if (mm > w.depth) break;
+                    a = w.parent;
+                    w = ld_node(A.node + a);
+                }
+                st_dyn_hint(A.dyn + r, a);
+                __stcg(A.hintc + r, a);
+                atomicAdd(A.parked + a, 1);
+                A.leaf_run[a].y = -1;
+                if (mm != m0) {
+                    const FStat fs = ld_stat(A.stat + r);
+                    const long long pos = a == 0 ? -1 : w.off + (long long)(mm - w.depth) - 1;
+                    const int32_t ntok = __ldg(A.tok + fs.soff + mm);
+                    st_dyn_state(A.dyn + r, pos, mm, ntok);
+                    __stcg(A.key + r, fast_key(mm, fs.len, fs.rank, A.score_mode));
+                    h = group_hash(pos, ntok);
+                    fell = true;
+                }
+            }
+            const unsigned fb = __ballot_sync(FULL_MASK, fell);
+            const int32_t my = n_f + __popc(fb & ((1u << lane) - 1u));
+            for (unsigned bits = fb; bits; bits &= bits - 1) {      // hand each fallen slot to the lane that keeps it
+                const int src = __ffs(bits) - 1;
+                const int32_t dst = __shfl_sync(FULL_MASK, my, src);
+                const int32_t rr = __shfl_sync(FULL_MASK, r, src);
+                const unsigned long long hh = __shfl_sync(FULL_MASK, h, src);
+                if (lane == dst) { f_slot = rr; f_hash = hh; }
+            }
+            n_f += __popc(fb);
+            __syncwarp();
+        }
+    }
+    if (n_f > 0) {
+        // the fallen slots are grouped afresh in a run appended to the member array (ranked by shuffles)
+        const int32_t base = *s_memcur;
+        if ((long long)base + n_f > (long long)A.mem_cap) {
+            if (lane == 0) set_status(A.st, RT_ERR_CAPACITY, 113);
+            *failed = true;
+        } else {
+            int32_t rank = 0, start = 0, cnt = 0;
+            for (int k2i = 0; k2i < 32; ++k2i) {
+                const unsigned long long hk = __shfl_sync(FULL_MASK, f_hash, k2i);
+                const bool lt = hk < f_hash, eq = hk == f_hash;
+                start += lt; cnt += eq; rank += (lt || (eq && k2i < lane));
+            }
+            if (f_slot >= 0) {
+                __stcg(A.mem + base + rank, f_slot);
+                st_dyn_group(A.dyn + f_slot, base + start, cnt);
+            }
+            __syncwarp();
+            if (lane == 0) *s_memcur = base + n_f;
+            __syncwarp();
+            // their keys went down: the leaf blocks of the arrived ones are recomputed
+            for (int k2i = 0; k2i < n_f; ++k2i) {
+                const int32_t rr = __shfl_sync(FULL_MASK, f_slot, k2i);
+                if (rr < admitted) {
+                    const int32_t bb = rr >> A.lb_shift;
+                    admit_blocks_one(A, R, bb, bb << A.lb_shift, admitted, lane);
+                    __syncwarp();
+                    *root = tour_update(R, bb, lane);
+                }
+            }
+        }
+    }
+    return true;
+}
+
+// G: the bitmap of processed slots lives in global memory (queues too long for shared memory).
+template <bool G>
+__global__ void __launch_bounds__(KLPM_FAST_THREADS, 1)
+lru_run_kernel(const __grid_constant__ FastArgs A) {
+    extern __shared__ __align__(16) unsigned char fast_smem[];
+    __shared__ FastJob s_job;
+    __shared__ LruJob s_tj;
+    __shared__ LruAnswer s_ta;
+    __shared__ int s_cnt;
+    __shared__ int32_t s_memcur;              // first free entry of the member array
+    __shared__ unsigned int s_dirty[256];
+    if (*reinterpret_cast<const volatile int32_t*>(A.skip)) return;       // the capacity check said no: nothing is touched
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t n = A.n;
+    const int32_t nb1p = (A.nb + 31) & ~31, n2 = nb1p >> 5, n2p = (n2 + 31) & ~31, n3 = n2p >> 5;
+    const int32_t nwords = (n + 31) >> 5;
+    FastTour R;
+    R.t1 = reinterpret_cast<unsigned long long*>(fast_smem);
+    R.t2 = R.t1 + nb1p;
+    R.t3 = R.t2 + n2p;
+    R.n2 = n2; R.n3 = n3;
+    unsigned long long* sh = R.t3 + 32;
+    int32_t* sr = reinterpret_cast<int32_t*>(sh + KLPM_FAST_SORT_CAP);
+    unsigned int* s_bits = reinterpret_cast<unsigned int*>(sr + KLPM_FAST_SORT_CAP);
+    R.g_done = G ? 1 : 0;
+    R.g_bits = 0;
+    R.done = G ? A.done : s_bits;
+    R.skip = nullptr; R.gb = nullptr;
+    R.dirty = s_dirty;
+    for (int32_t i = threadIdx.x; i < nb1p + n2p + 32; i += blockDim.x) R.t1[i] = 0ULL;
+    if (threadIdx.x == 0) s_memcur = 2 * n;
+    if (!G) for (int32_t i = threadIdx.x; i < nwords; i += blockDim.x) s_bits[i] = 0u;
+    __syncthreads();
+
+    if (warp == 1) { lru_tree_warp(A, R, &s_tj, &s_ta, &s_job, sh, sr, &s_cnt, &s_memcur, lane); return; }
+    if (warp > 1) {
+        for (;;) {
+            named_bar(1, KLPM_FAST_THREADS);
+            const FastJob J = s_job;
+            if (J.type == FAST_JOB_EXIT) return;
+            fast_job<true>(A, R, J, sh, sr, &s_cnt, &s_memcur);
+        }
+    }
+
+    // ---------------------------------------------------------------- warp 0
+    const long long INF = 0x7fffffffffffffffLL;
+    const bool fixed = A.fixed != nullptr;
+    const int32_t n_dec = fixed ? *reinterpret_cast<const volatile int32_t*>(A.n_fixed) : n;
+    const int LB = 1 << A.lb_shift;
+    long long now = A.start_tick;
+    int32_t head = 0, admitted = 0, cyc = 0, c = 0;
+    unsigned long long root = 0;
+    long long n_cta_dissolve = 0, n_scan = 0, cy_wait = 0, cy_scan = 0, cy_dissolve = 0;
+    bool failed = false;
+    bool busy = false;                                      // warp 1 works on decision c - 1
+    bool regroup = false;                                   // decision c - 1's group has other members: dissolve it once its leaf is known
+    FastPick P;
+    P.slot = 0; P.m = 0; P.len = 0; P.ntok = 0; P.x = A.tok; P.pos = 0; P.vleaf = 0; P.admitted = 0; P.gstart = 0; P.gcount = 0; P.leaf = -1;
+
+    auto cta_job = [&]() {                                  // lane 0 has filled s_job; warp 1 is idle
+        if (lane == 0) s_tj.type = LRU_JOB_JOIN;
+        __syncwarp();
+        named_arrive(2, 64);
+        named_bar(1, KLPM_FAST_THREADS);
+        const FastJob J = s_job;
+        fast_job<true>(A, R, J, sh, sr, &s_cnt, &s_memcur);
+        root = tour_top(R, lane);
+    };
+    // Waits for warp 1 and finishes decision c - 1: queries that fell back out of evicted leaves, then the pick's group.
+    // True if anything that the next decision is prepared from may have changed.
+    auto finish = [&]() -> bool {
+        const long long t0 = clock64();
+        named_bar(3, 64);
+        cy_wait += clock64() - t0;
+        busy = false;
+        const int32_t n_small = s_ta.n_small;
+        bool scan = s_ta.scan != 0, changed = false;
+        const int32_t leaf = s_ta.leaf;
+        if (s_ta.failed) { failed = true; return true; }
+        if (n_small > 0 || scan) {
+            changed = true;
+            if (!scan) scan = !lru_fall_back_small(A, R, s_ta.small_v, n_small, admitted, &s_memcur, &root, &failed, lane);
+            if (scan) {                                     // somebody was parked in an evicted leaf
+                const long long t1 = clock64();
+                ++n_scan;
+                if (lane == 0) { s_job.type = FAST_JOB_FALLBACK; s_job.a0 = fixed ? 0 : head; s_job.a1 = admitted; }
+                cta_job();
+                cy_scan += clock64() - t1;
+            }
+        }
+        if (regroup && !failed) {
+            changed = true;
+            P.leaf = leaf; P.admitted = admitted;
+            if (dissolve_is_small(P.gcount, P.len - P.m)) root = dissolve_small(A, P, R, root, lane);
+            else {
+                const long long t1 = clock64();
+                ++n_cta_dissolve;
+                if (lane == 0) { s_job.type = FAST_JOB_DISSOLVE; s_job.pick = P; }
+                cta_job();
+                cy_dissolve += clock64() - t1;
+            }
+        }
+        regroup = false;
+        __syncwarp();
+        return changed;
+    };
+    auto slot_of_root = [&]() -> int32_t {
+        const unsigned rk = 0xffffffffu - (unsigned)(root & 0xffffffffULL);
+        return A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
+    };
+
+    while (c < n_dec && !failed) {
+        if (busy && regroup) { finish(); if (failed) break; }
+        FDyn pd; FStat ps;
+        int32_t slot, b = 0;
+        unsigned long long bm = 0;
+        if (fixed) {                                        // a given order (klpm_replay): no admission, no pick; slots are the queries in index order
+            slot = __ldg(A.fixed + c);
+            pd = ld_dyn(A.dyn + slot);
+            ps = ld_stat(A.stat + slot);
+            if (busy && finish()) continue;
+        } else {
+            const bool fcfs_turn = A.policy == KLPM_POLICY_FCFS || (A.policy == KLPM_POLICY_KLPM && cyc == 0);
+            // ---- everything this decision is likely to need, asked for at once: the likely pick's records and its leaf
+            //      block's keys, the coming arrivals and their keys
+            int32_t guess = head < n ? head : n - 1;
+            if (!fcfs_turn && head < admitted) guess = slot_of_root();
+            if (guess < 0 || guess >= n) guess = 0;         // (never picked: see the check below)
+            const int32_t ra = admitted + lane;
+            const long long tw = ra < n ? __ldg(A.sorted_t + ra) : INF;
+            const unsigned long long ak = ra < n ? __ldcg(A.key + ra) : 0ULL;
+            const long long r0 = (((long long)guess >> A.lb_shift) << A.lb_shift) + lane;
+            unsigned long long kk = r0 < n ? __ldcg(A.key + r0) : 0ULL;
+            pd = ld_dyn(A.dyn + guess);
+            ps = ld_stat(A.stat + guess);
+            // ---- time and arrivals: idle until somebody has arrived, then admit everybody who has
+            const long long next_t = __shfl_sync(FULL_MASK, tw, 0);
+            if (head == admitted && next_t > now) now = next_t;
+            if (next_t <= now) {
+                const unsigned bal = __ballot_sync(FULL_MASK, tw <= now);      // (past the end: INF; arrivals are sorted)
+                const int cnt = bal == FULL_MASK ? 32 : __ffs(~bal) - 1;
+                int32_t a1 = admitted + cnt;
+                if (cnt == 32 && a1 < n) {                 // a full window: gallop, then bisect (lane 0)
+                    long long lo = a1, hi = n;
+                    if (lane == 0 && __ldg(A.sorted_t + lo) <= now) {
+                        long long step = 1;
+                        ++lo;
+                        while (lo + step <= hi && __ldg(A.sorted_t + lo + step - 1) <= now) { lo += step; step <<= 1; }
+                        if (lo + step < hi) hi = lo + step;
+                        while (lo < hi) { const long long mid = (lo + hi) >> 1; if (__ldg(A.sorted_t + mid) <= now) lo = mid + 1; else hi = mid; }
+                    }
+                    a1 = (int32_t)__shfl_sync(FULL_MASK, lo, 0);
+                }
+                if (a1 > n) a1 = n;
+                if (a1 - admitted <= 32) {
+                    // keys only come in: every level above takes the larger of what it holds and the newcomers (one or two leaf blocks)
+                    const int32_t b0 = admitted >> A.lb_shift, b1 = (a1 - 1) >> A.lb_shift;
+                    for (int32_t bb = b0; bb <= b1; ++bb) {
+                        const unsigned long long km = warp_max64r(ra < a1 && (ra >> A.lb_shift) == bb ? ak : 0ULL);
+                        const unsigned long long o1 = R.t1[bb], o2 = R.t2[bb >> 5], o3 = R.t3[bb >> 10];
+                        __syncwarp();
+                        R.t1[bb] = km > o1 ? km : o1; R.t2[bb >> 5] = km > o2 ? km : o2; R.t3[bb >> 10] = km > o3 ? km : o3;
+                        root = km > root ? km : root;
+                        __syncwarp();
+                    }
+                    admitted = a1;
+                } else {
+                    if (busy) { finish(); if (failed) break; }
+                    if (lane == 0) { s_job.type = FAST_JOB_ADMIT; s_job.a0 = admitted; s_job.a1 = a1; }
+                    cta_job();
+                    admitted = a1;
+                    continue;                               // (what was asked for above may be out of date)
+                }
+            }
+            // ---- pick
+            slot = fcfs_turn ? head : slot_of_root();
+            if (slot < 0 || slot >= admitted || slot_done(R, A, slot)) {
+                if (busy) { finish(); if (!failed) continue; break; }              // (prepared from a tournament that is being corrected)
+                if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 105);
+                failed = true; break;                       // cannot happen
+            }
+            b = slot >> A.lb_shift;
+            if (slot != guess) {
+                const long long r = ((long long)b << A.lb_shift) + lane;
+                kk = r < n ? __ldcg(A.key + r) : 0ULL;
+                pd = ld_dyn(A.dyn + slot);
+                ps = ld_stat(A.stat + slot);
+            }
+            {   // its leaf block's largest key without it
+                const long long r = ((long long)b << A.lb_shift) + lane;
+                if (r < admitted && r != slot && lane < LB && !slot_done(R, A, r)) bm = kk;
+                for (int32_t u = lane + 32; u < LB; u += 32) {
+                    const long long r2 = ((long long)b << A.lb_shift) + u;
+                    if (r2 < admitted && r2 != slot && !slot_done(R, A, r2)) { const unsigned long long k2 = __ldcg(A.key + r2); if (k2 > bm) bm = k2; }
+                }
+                bm = warp_max64r(bm);
+            }
+            // ---- nothing has been committed yet: the decision before must be finished first
+            if (busy && finish()) continue;                 // (or failed: the loop ends)
+            if (++cyc == A.k) cyc = 0;
+            root = tour_set(R, b, bm, lane);
+        }
+        // ---- the pick is processed: charge it (Definition 2), hand the tree its part
+        if (!G) R.done[slot >> 5] |= 1u << (slot & 31);
+        else if (lane == 0) __stcg(R.done + (slot >> 5), __ldcg(R.done + (slot >> 5)) | (1u << (slot & 31)));
+        const int32_t unc = ps.len - pd.m;
+        const long long vleaf = A.vbase + ((long long)c << 32);               // positions in its new leaf: unique per decision, above every real pool index
+        {
+            const long long begin = now > ps.t ? now : ps.t;
+            now = begin + (A.c_den + A.c_num * (long long)ps.len) * (long long)unc;
+        }
+        if (lane == 0) {
+            s_tj.type = LRU_JOB_STEP; s_tj.hint = pd.hint; s_tj.m = pd.m; s_tj.len = ps.len; s_tj.gstart = pd.gstart; s_tj.gcount = pd.gcount;
+            s_tj.vleaf = vleaf;
+        }
+        __syncwarp();
+        named_arrive(2, 64);
+        busy = true;
+        if (lane == 0) {
+            if (A.order) A.order[c] = ps.ord;
+            A.uncached[ps.ord] = unc; A.ttft[ps.ord] = now - ps.t;
+            if (A.completion) A.completion[ps.ord] = now;
+        }
+        ++c;
+        regroup = unc > 0 && pd.gcount > 1;
+        if (regroup) {
+            P.slot = slot; P.m = pd.m; P.len = ps.len; P.ntok = pd.ntok; P.x = A.tok + ps.soff; P.pos = pd.pos; P.vleaf = vleaf;
+            P.gstart = pd.gstart; P.gcount = pd.gcount;
+        }
+        if (!fixed && slot == head) head = next_head(R.done, G ? 1 : 0, nwords, n, head, lane);
+        __syncwarp();
+    }
+    if (busy) { named_bar(3, 64); }
+    if (lane == 0) {
+        A.post->c0 = n;                                     // list mode never began: nothing is left to charge
+        A.post->now0 = now;
+        long long* cn = A.post->counters;
+        cn[0] = c; cn[1] = n_cta_dissolve; cn[2] = n_scan; cn[3] = s_memcur - 2 * n;
+        cn[5] = cy_wait; cn[6] = cy_scan; cn[7] = cy_dissolve;
+        for (int i = 8; i < 16; ++i) cn[i] = 0;
+        s_job.type = FAST_JOB_EXIT;
+        s_tj.type = LRU_JOB_EXIT;
+    }
+    __syncwarp();
+    named_arrive(2, 64);
     named_bar(1, KLPM_FAST_THREADS);
 }
 
@@ -3723,7 +4018,7 @@ bulk_rounds_kernel(TreeDev T, BulkArgs A, BulkSync* g, long long n_total, const 
         for (unsigned long long p0 = (unsigned long long)warp0 * 32ULL; p0 < n_apply; p0 += (unsigned long long)nwarps * 32ULL)
             bulk_apply_warp(T, R, p0, n_apply, lane, &s_live_nodes, &s_live_tokens);
         if (!bulk_barrier(g, S, limit_ns, [&] {
-                const bool stop = *(volatile int*)&S->status != 0 || r > 100000000u;
+                const bool stop = *(volatile int*)&S->status != 0 || (long long)r > 4 * n_total + 64;      // (every round stores a prompt)
                 g->go = stop ? 0u : *(volatile unsigned*)&g->cnt_a[par];
             })) break;
         count = __ldcg(&g->go);
@@ -4101,6 +4396,27 @@ lru_tokens_kernel(TreeDev T, const int32_t* __restrict__ order, const int32_t* _
     }
 }
 
+// The node arrays as records for the loop, and back.
+__global__ void lru_pack_kernel(TreeDev T, LNode* node, const LruInfo* info) {
+    if (info->skip) return;
+    const long long n = T.st->n_nodes, step = (long long)gridDim.x * blockDim.x;
+    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += step) {
+        LNode r;
+        r.parent = T.parent[v]; r.depth = T.depth_start[v]; r.len = T.span_len[v]; r.nchild = T.dead[v] ? -1 : T.nchild[v];
+        r.last = T.last_access[v]; r.off = T.span_off[v];
+        st_node(node + v, r);
+    }
+}
+__global__ void lru_unpack_kernel(TreeDev T, const LNode* __restrict__ node, const LruInfo* info) {
+    if (info->skip) return;
+    const long long n = T.st->n_nodes, step = (long long)gridDim.x * blockDim.x;
+    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += step) {
+        const LNode r = ld_node(node + v);
+        T.parent[v] = r.parent; T.depth_start[v] = r.depth; T.span_len[v] = r.len; T.nchild[v] = r.nchild < 0 ? 0 : r.nchild;
+        T.dead[v] = r.nchild < 0; T.last_access[v] = r.last; T.span_off[v] = r.off;
+    }
+}
+
 __global__ void table_clear_kernel(TreeDev T, const LruInfo* info) {
     if (info->skip) return;
     int4* p = reinterpret_cast<int4*>(T.table);
@@ -4325,7 +4641,7 @@ struct rt_tree {
     long long fast_mem_cap;  // entries of fast_mem
     int32_t* lru_parked; LruInfo* lru_info;     // grouped loop on a tree with a budget
     int32_t* lru_hintc; long long lru_hintc_cap;
-    int2* lru_leaf_run;
+    int2* lru_leaf_run; LNode* lru_node;
     ReplayInfo* replay_info;
     int run_path;           // which loop the last klpm_run took: 0 none yet, 1 one by one, 2 grouped
     int num_sms;
@@ -4368,7 +4684,7 @@ void free_tree(rt_tree* t) {
     cudaFree(t->fast_dyn); cudaFree(t->fast_stat); cudaFree(t->fast_key_arr); cudaFree(t->fast_mem);
     cudaFree(t->fast_gh); cudaFree(t->fast_gidx); cudaFree(t->fast_done); cudaFree(t->fast_counter);
     cudaFree(t->fast_lk); cudaFree(t->fast_ls); cudaFree(t->fast_post); cudaFree(t->fast_bsum);
-    cudaFree(t->lru_parked); cudaFree(t->lru_info); cudaFree(t->lru_hintc); cudaFree(t->lru_leaf_run); cudaFree(t->replay_info);
+    cudaFree(t->lru_parked); cudaFree(t->lru_info); cudaFree(t->lru_hintc); cudaFree(t->lru_leaf_run); cudaFree(t->lru_node); cudaFree(t->replay_info);
     cudaFree(t->claim);
     cudaFree(t->bulk_pend_a); cudaFree(t->bulk_pend_b); cudaFree(t->bulk_pm); cudaFree(t->bulk_pnode); cudaFree(t->bulk_poff);
     cudaFree(t->bulk_sync);
@@ -5011,6 +5327,8 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             f.hintc = tree->lru_hintc;
             if (!tree->lru_leaf_run && (st = dalloc(&tree->lru_leaf_run, tree->dev.max_nodes))) return st;
             f.leaf_run = tree->lru_leaf_run;
+            if (!tree->lru_node && (st = dalloc(&tree->lru_node, tree->dev.max_nodes))) return st;
+            f.node = tree->lru_node; f.sorted_t = tree->run_key;
             f.pk = tree->fast_lk; f.pi = tree->fast_ls;      // (the key list of list mode is not used on these trees)
             CK(cudaMemsetAsync(tree->lru_leaf_run, 0xff, (size_t)tree->dev.max_nodes * sizeof(int2), s));
             f.lru = 1; f.T = tree->dev; f.parked = tree->lru_parked; f.skip = &tree->lru_info->skip;
@@ -5021,6 +5339,7 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             if (d_fixed) lru_sum_order_kernel<<<(unsigned)((n_fixed + 255) / 256), 256, 0, s>>>(d_q_offsets, d_fixed, n_fixed, n, tree->lru_info);
             else lru_sum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d_q_offsets, n, tree->lru_info);
             lru_check_kernel<<<1, 1, 0, s>>>(tree->dev, d_fixed ? n_fixed : n, tree->lru_info);
+            lru_pack_kernel<<<(unsigned)tree->num_sms * 4, 256, 0, s>>>(tree->dev, tree->lru_node, tree->lru_info);
         }
         f.tok = d_q_tokens; f.n = n; f.policy = params->policy; f.k = params->k; f.score_mode = score_mode;
         f.c_num = params->c_num; f.c_den = params->c_den; f.start_tick = params->start_tick;
@@ -5088,7 +5407,13 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             sort_pairs(tree->fast_lk, tree->fast_ls, np2, s);
         }
         CK(cudaGetLastError());
-        if (f.done_in_smem && (f.bits_in_smem || !f.list_mode)) {
+        if (lru && f.done_in_smem) {
+            CK(cudaFuncSetAttribute(lru_run_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            lru_run_kernel<false><<<1, KLPM_FAST_THREADS, smem, s>>>(f);
+        } else if (lru) {
+            CK(cudaFuncSetAttribute(lru_run_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            lru_run_kernel<true><<<1, KLPM_FAST_THREADS, smem, s>>>(f);
+        } else if (f.done_in_smem && (f.bits_in_smem || !f.list_mode)) {
             CK(cudaFuncSetAttribute(fast_run_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             fast_run_kernel<false><<<1, KLPM_FAST_THREADS, smem, s>>>(f);
         } else {
@@ -5108,6 +5433,7 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         if (lru) {
             // the nodes that are alive after the loop get their tokens, and the child table is written afresh
             const TreeDev& d = tree->dev;
+            lru_unpack_kernel<<<(unsigned)tree->num_sms * 4, 256, 0, s>>>(d, tree->lru_node, tree->lru_info);
             lru_tokens_kernel<<<(unsigned)tree->num_sms * 8, 256, 0, s>>>(d, d_fixed ? d_fixed : d_order, d_q_tokens, d_q_offsets, f.vbase, tree->lru_info);
             table_clear_kernel<<<(unsigned)tree->num_sms * 8, 256, 0, s>>>(d, tree->lru_info);
             lru_table_kernel<<<(unsigned)((d.max_nodes + 255) / 256), 256, 0, s>>>(d, f.vbase, tree->lru_info);
