@@ -1643,6 +1643,14 @@ __device__ __forceinline__ FDyn ld_dyn(const FDyn* p) {
     d.m = a.z; d.ntok = a.w; d.gstart = b.x; d.gcount = b.y; d.hint = b.z; d.pad = 0;
     return d;
 }
+__device__ __forceinline__ FDyn ld_dyn_l1(const FDyn* p) {      // a plain load: served by L1 if another warp of the CTA has read it before
+    const int4* q = reinterpret_cast<const int4*>(p);
+    const int4 a = q[0], b = q[1];
+    FDyn d;
+    d.pos = (long long)(((unsigned long long)(unsigned)a.y << 32) | (unsigned)a.x);
+    d.m = a.z; d.ntok = a.w; d.gstart = b.x; d.gcount = b.y; d.hint = b.z; d.pad = 0;
+    return d;
+}
 __device__ __forceinline__ void st_dyn_state(FDyn* p, long long pos, int32_t m, int32_t ntok) {
     __stcg(reinterpret_cast<int4*>(p), make_int4((int)(unsigned)(unsigned long long)pos, (int)(unsigned)((unsigned long long)pos >> 32), m, ntok));
 }
@@ -3098,7 +3106,7 @@ fast_run_kernel(FastArgs A) {
 // dissolved.  The other warps join for work that is worth sharing; so does warp 1, which is idle then.
 // The two hand over through named barriers 2 (a job for warp 1) and 3 (its answer), helpers wait at barrier 1.
 // What bounds it: @@LRU@@
-struct LruJob { int32_t type; int32_t hint, m, len, gstart, gcount; long long vleaf; };
+struct LruJob { int32_t type; int32_t hint, m, len, gstart, gcount; int32_t moved; long long vleaf; };   // moved: queries have been parked elsewhere since the last job
 struct LruAnswer { int32_t failed, scan, n_small, leaf; int32_t small_v[8]; };
 enum { LRU_JOB_EXIT = 0, LRU_JOB_STEP = 1, LRU_JOB_JOIN = 2 };
 
@@ -3111,7 +3119,22 @@ __device__ __forceinline__ void lru_tree_warp(const FastArgs& A, const FastTour&
     long long wbase = st.lru_cursor, wend = wbase;          // the window's clock values: [wbase, wend)
     int32_t wv = 0;                                         // this lane's owner
     bool wok = false;                                       // it is a leaf and its stamp is this clock value
+    // the next leaf to go, its record, its parent's record and how many queries are parked in it: read between two jobs
+    int32_t v0 = -1, pk0 = 0;
+    LNode rv, rp0;
+    rv.parent = 0; rv.depth = 0; rv.len = 0; rv.nchild = 0; rv.last = 0; rv.off = 0;
+    rp0 = rv;
     for (;;) {
+        {
+            const unsigned okm = __ballot_sync(FULL_MASK, wok);
+            v0 = -1;
+            if (okm) {
+                v0 = __shfl_sync(FULL_MASK, wv, __ffs(okm) - 1);
+                rv = ld_node(A.node + v0);
+                pk0 = __ldcg(A.parked + v0);
+                rp0 = ld_node(A.node + rv.parent);
+            }
+        }
         named_bar(2, 64);
         const LruJob J = *s_tj;
         if (J.type != LRU_JOB_STEP) {
@@ -3131,18 +3154,8 @@ __device__ __forceinline__ void lru_tree_warp(const FastArgs& A, const FastTour&
             continue;
         }
         const long long clock = ++st.clock;
-        // the node the match ends in, and beside it the next leaf to go
-        LNode ra = ld_node(A.node + J.hint);
-        int32_t v0 = -1, pk0 = 0;
-        LNode rv; rv.parent = 0; rv.depth = 0; rv.len = 0; rv.nchild = 0; rv.last = 0; rv.off = 0;
-        if (st.tokens_live + unc > T.budget) {
-            const unsigned okm = __ballot_sync(FULL_MASK, wok);
-            if (okm) {
-                v0 = __shfl_sync(FULL_MASK, wv, __ffs(okm) - 1);
-                rv = ld_node(A.node + v0);
-                pk0 = __ldcg(A.parked + v0);
-            }
-        }
+        LNode ra = ld_node(A.node + J.hint);                // the node the match ends in (its hint; then up)
+        if (J.moved && v0 >= 0) pk0 = __ldcg(A.parked + v0);
         if (lane == 0) atomicSub(A.parked + J.hint, 1);
         int32_t a = J.hint;
         while (a != 0 && J.m <= ra.depth) { a = ra.parent; ra = ld_node(A.node + a); }
@@ -3178,8 +3191,10 @@ __device__ __forceinline__ void lru_tree_warp(const FastArgs& A, const FastTour&
             const int src = __ffs(okm) - 1;
             const int32_t victim = __shfl_sync(FULL_MASK, wv, src);
             const long long stamp = wbase + src;
+            bool have_parent = victim == v0;
             if (victim != v0) { rv = ld_node(A.node + victim); pk0 = __ldcg(A.parked + victim); }
             if (cut && victim == a) { rv.parent = end; rv.len = ra.len; }      // the lower part of the edge just cut
+            if (cut && rv.parent == a) have_parent = false;                    // (its parent's record has changed)
             v0 = -1;
             st.tokens_live -= rv.len;
             --st.live_nodes; ++st.evictions;
@@ -3196,7 +3211,8 @@ __device__ __forceinline__ void lru_tree_warp(const FastArgs& A, const FastTour&
             if (lane == 0) A.node[victim].nchild = -1;
             if (P == end) --e.nchild;                       // (its stamp is newer)
             else {
-                LNode rp = ld_node(A.node + P);
+                LNode rp = rp0;
+                if (!have_parent) rp = ld_node(A.node + P);
                 const int32_t nc = rp.nchild - 1;
                 if (P != 0 && stamp >= rp.last) {           // the stamp goes to the parent if newer
                     rp.last = stamp;
@@ -3237,6 +3253,63 @@ __device__ __forceinline__ void lru_tree_warp(const FastArgs& A, const FastTour&
     }
     __syncwarp();
     named_bar(1, KLPM_FAST_THREADS);                        // (the helpers are told to leave)
+}
+
+struct LruTouch { int32_t seq, join; int32_t slot0, admitted; unsigned long long root; };
+
+// Warp 2, between the jobs of the whole CTA: reads ahead.  Each time warp 0 has committed a decision it says who is oldest
+// and what the tournament's root is; one of the two is nearly always the next pick.  This warp loads their records, their
+// leaf blocks' keys, the keys of the coming arrivals and then the node records that warp 1 will walk, for no other
+// purpose than to have them in this SM's L1.  It decides nothing, so it may be late or wrong.  Returns when warp 0 calls
+// for a job of the whole CTA (or after a bounded number of polls, after which it only takes part in such jobs).
+__device__ __forceinline__ int32_t touch(const void* p) {
+    int32_t v;
+    asm volatile("ld.global.ca.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void lru_touch_warp(const FastArgs& A, const LruTouch* s_touch, int32_t joined, int32_t n, int32_t fixed_n, int lane) {
+    int32_t seen = 0;
+    for (unsigned polls = 0; polls < (1u << 28); ++polls) {
+        if (*(const volatile int32_t*)&s_touch->join != joined) return;
+        const int32_t seq = *(const volatile int32_t*)&s_touch->seq;
+        if (seq == seen) { __nanosleep(20); continue; }
+        seen = seq;
+        __threadfence_block();
+        int32_t a = *(const volatile int32_t*)&s_touch->slot0, b = -1;
+        const int32_t adm = *(const volatile int32_t*)&s_touch->admitted;
+        const unsigned long long root = *(const volatile unsigned long long*)&s_touch->root;
+        if (A.fixed) {
+            a = a >= 0 && a < fixed_n ? __ldg(A.fixed + a) : -1;               // (slot0 is the number of the decision here)
+            if (a >= n) a = -1;
+        } else if (root != 0) {
+            const unsigned rk = 0xffffffffu - (unsigned)(root & 0xffffffffULL);
+            if (rk < (unsigned)n) b = A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
+        }
+        // lanes 0-9: the oldest, 10-19: the root's slot (state with its hint, constant record, eight sectors of its block's keys), 20-27: keys of arrivals
+        const int u = lane < 10 ? lane : lane - 10;
+        const int32_t s = lane < 10 ? a : b;
+        const void* p = nullptr;
+        if (lane < 20 && s >= 0 && s < n) {
+            if (u == 0) p = reinterpret_cast<const int32_t*>(A.dyn + s) + 6;
+            else if (u == 1) p = A.stat + s;
+            else if (!A.fixed) {
+                const long long r = (((long long)s >> A.lb_shift) << A.lb_shift) + 4 * (u - 2);
+                if (r < n) p = A.key + r;
+            }
+        } else if (lane >= 20 && lane < 28 && !A.fixed) {
+            const long long r = (long long)(adm & ~3) + 4 * (lane - 20);
+            if (r < n) p = A.key + r;
+        }
+        int32_t v = p ? touch(p) : 0;
+        // the node the match ends in is the hint's or above it
+        bool chain = u == 0 && lane < 20 && p != nullptr;
+#pragma unroll 1
+        for (int d = 0; d < 3 && chain; ++d) {
+            if (v <= 0 || v >= A.T.max_nodes) chain = false;
+            else v = touch(&A.node[v].parent);
+        }
+        __syncwarp();
+    }
 }
 
 // Warp 0: the queries parked in leaves that the last decision evicted, when known member runs hold them all.  All leaves
@@ -3353,6 +3426,7 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
     __shared__ FastJob s_job;
     __shared__ LruJob s_tj;
     __shared__ LruAnswer s_ta;
+    __shared__ LruTouch s_touch;
     __shared__ int s_cnt;
     __shared__ int32_t s_memcur;              // first free entry of the member array
     __shared__ unsigned int s_dirty[256];
@@ -3375,13 +3449,16 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
     R.skip = nullptr; R.gb = nullptr;
     R.dirty = s_dirty;
     for (int32_t i = threadIdx.x; i < nb1p + n2p + 32; i += blockDim.x) R.t1[i] = 0ULL;
-    if (threadIdx.x == 0) s_memcur = 2 * n;
+    if (threadIdx.x == 0) { s_memcur = 2 * n; s_touch.seq = 0; s_touch.join = 0; }
     if (!G) for (int32_t i = threadIdx.x; i < nwords; i += blockDim.x) s_bits[i] = 0u;
     __syncthreads();
 
+    const int32_t fixed_n = A.fixed ? *reinterpret_cast<const volatile int32_t*>(A.n_fixed) : 0;
     if (warp == 1) { lru_tree_warp(A, R, &s_tj, &s_ta, &s_job, sh, sr, &s_cnt, &s_memcur, lane); return; }
     if (warp > 1) {
+        int32_t joined = 0;
         for (;;) {
+            if (warp == 2) lru_touch_warp(A, &s_touch, joined++, n, fixed_n, lane);
             named_bar(1, KLPM_FAST_THREADS);
             const FastJob J = s_job;
             if (J.type == FAST_JOB_EXIT) return;
@@ -3392,7 +3469,7 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
     // ---------------------------------------------------------------- warp 0
     const long long INF = 0x7fffffffffffffffLL;
     const bool fixed = A.fixed != nullptr;
-    const int32_t n_dec = fixed ? *reinterpret_cast<const volatile int32_t*>(A.n_fixed) : n;
+    const int32_t n_dec = fixed ? fixed_n : n;
     const int LB = 1 << A.lb_shift;
     long long now = A.start_tick;
     int32_t head = 0, admitted = 0, cyc = 0, c = 0;
@@ -3400,12 +3477,14 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
     long long n_cta_dissolve = 0, n_scan = 0, cy_wait = 0, cy_scan = 0, cy_dissolve = 0;
     bool failed = false;
     bool busy = false;                                      // warp 1 works on decision c - 1
+    bool moved = false;                                     // queries have been parked elsewhere since warp 1's last job
     bool regroup = false;                                   // decision c - 1's group has other members: dissolve it once its leaf is known
     FastPick P;
     P.slot = 0; P.m = 0; P.len = 0; P.ntok = 0; P.x = A.tok; P.pos = 0; P.vleaf = 0; P.admitted = 0; P.gstart = 0; P.gcount = 0; P.leaf = -1;
 
+    int32_t told = 0, joins = 0;                            // messages to warp 2
     auto cta_job = [&]() {                                  // lane 0 has filled s_job; warp 1 is idle
-        if (lane == 0) s_tj.type = LRU_JOB_JOIN;
+        if (lane == 0) { s_tj.type = LRU_JOB_JOIN; __threadfence_block(); *(volatile int32_t*)&s_touch.join = ++joins; }
         __syncwarp();
         named_arrive(2, 64);
         named_bar(1, KLPM_FAST_THREADS);
@@ -3425,7 +3504,7 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
         const int32_t leaf = s_ta.leaf;
         if (s_ta.failed) { failed = true; return true; }
         if (n_small > 0 || scan) {
-            changed = true;
+            changed = true; moved = true;
             if (!scan) scan = !lru_fall_back_small(A, R, s_ta.small_v, n_small, admitted, &s_memcur, &root, &failed, lane);
             if (scan) {                                     // somebody was parked in an evicted leaf
                 const long long t1 = clock64();
@@ -3436,7 +3515,7 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
             }
         }
         if (regroup && !failed) {
-            changed = true;
+            changed = true; moved = true;
             P.leaf = leaf; P.admitted = admitted;
             if (dissolve_is_small(P.gcount, P.len - P.m)) root = dissolve_small(A, P, R, root, lane);
             else {
@@ -3456,96 +3535,108 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
         return A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
     };
 
+    auto fcfs_next = [&]() -> bool { return A.policy == KLPM_POLICY_FCFS || (A.policy == KLPM_POLICY_KLPM && cyc == 0); };
+    // warp 2 is told which slots come next: it brings what the two warps are about to read into L1
+    auto tell = [&]() {
+        if (lane == 0) {
+            s_touch.slot0 = fixed ? c : head; s_touch.root = root; s_touch.admitted = admitted;
+            __threadfence_block();
+            *(volatile int32_t*)&s_touch.seq = ++told;
+        }
+    };
+    long long tw = INF, next_t = INF;                       // 32 coming arrivals (lane i: slot wb + i); the next one
+    int32_t wb = 0;
+    if (!fixed) { tw = lane < n ? __ldg(A.sorted_t + lane) : INF; next_t = __shfl_sync(FULL_MASK, tw, 0); }
+    tell();
+
     while (c < n_dec && !failed) {
         if (busy && regroup) { finish(); if (failed) break; }
+        int32_t slot = 0, b = 0;
+        unsigned long long bm = 0, o1 = 0, o2 = 0, o3 = 0;
         FDyn pd; FStat ps;
-        int32_t slot, b = 0;
-        unsigned long long bm = 0;
         if (fixed) {                                        // a given order (klpm_replay): no admission, no pick; slots are the queries in index order
             slot = __ldg(A.fixed + c);
-            pd = ld_dyn(A.dyn + slot);
+            pd = ld_dyn_l1(A.dyn + slot);
             ps = ld_stat(A.stat + slot);
             if (busy && finish()) continue;
         } else {
-            const bool fcfs_turn = A.policy == KLPM_POLICY_FCFS || (A.policy == KLPM_POLICY_KLPM && cyc == 0);
-            // ---- everything this decision is likely to need, asked for at once: the likely pick's records and its leaf
-            //      block's keys, the coming arrivals and their keys
-            int32_t guess = head < n ? head : n - 1;
-            if (!fcfs_turn && head < admitted) guess = slot_of_root();
-            if (guess < 0 || guess >= n) guess = 0;         // (never picked: see the check below)
-            const int32_t ra = admitted + lane;
-            const long long tw = ra < n ? __ldg(A.sorted_t + ra) : INF;
-            const unsigned long long ak = ra < n ? __ldcg(A.key + ra) : 0ULL;
-            const long long r0 = (((long long)guess >> A.lb_shift) << A.lb_shift) + lane;
-            unsigned long long kk = r0 < n ? __ldcg(A.key + r0) : 0ULL;
-            pd = ld_dyn(A.dyn + guess);
-            ps = ld_stat(A.stat + guess);
             // ---- time and arrivals: idle until somebody has arrived, then admit everybody who has
-            const long long next_t = __shfl_sync(FULL_MASK, tw, 0);
             if (head == admitted && next_t > now) now = next_t;
-            if (next_t <= now) {
-                const unsigned bal = __ballot_sync(FULL_MASK, tw <= now);      // (past the end: INF; arrivals are sorted)
-                const int cnt = bal == FULL_MASK ? 32 : __ffs(~bal) - 1;
-                int32_t a1 = admitted + cnt;
-                if (cnt == 32 && a1 < n) {                 // a full window: gallop, then bisect (lane 0)
-                    long long lo = a1, hi = n;
-                    if (lane == 0 && __ldg(A.sorted_t + lo) <= now) {
+            while (next_t <= now && !failed) {
+                const int off = admitted - wb;
+                const int cnt = __popc(__ballot_sync(FULL_MASK, lane >= off && tw <= now));      // (arrivals are sorted; past the end: INF)
+                const int32_t a1 = admitted + cnt, ra = wb + lane;
+                if (off + cnt == 32 && a1 + 64 < n && __ldg(A.sorted_t + a1 + 64) <= now) {
+                    // a crowd: gallop, then bisect (lane 0), and the whole CTA admits them
+                    long long lo = a1 + 65, hi = n;
+                    if (lane == 0) {
                         long long step = 1;
-                        ++lo;
                         while (lo + step <= hi && __ldg(A.sorted_t + lo + step - 1) <= now) { lo += step; step <<= 1; }
                         if (lo + step < hi) hi = lo + step;
                         while (lo < hi) { const long long mid = (lo + hi) >> 1; if (__ldg(A.sorted_t + mid) <= now) lo = mid + 1; else hi = mid; }
                     }
-                    a1 = (int32_t)__shfl_sync(FULL_MASK, lo, 0);
-                }
-                if (a1 > n) a1 = n;
-                if (a1 - admitted <= 32) {
+                    const int32_t all = (int32_t)__shfl_sync(FULL_MASK, lo, 0);
+                    if (busy) finish();
+                    if (failed) break;
+                    if (lane == 0) { s_job.type = FAST_JOB_ADMIT; s_job.a0 = admitted; s_job.a1 = all; }
+                    cta_job();
+                    admitted = all;
+                } else {
                     // keys only come in: every level above takes the larger of what it holds and the newcomers (one or two leaf blocks)
+                    const unsigned long long ak = ra >= admitted && ra < a1 ? *(A.key + ra) : 0ULL;
                     const int32_t b0 = admitted >> A.lb_shift, b1 = (a1 - 1) >> A.lb_shift;
                     for (int32_t bb = b0; bb <= b1; ++bb) {
-                        const unsigned long long km = warp_max64r(ra < a1 && (ra >> A.lb_shift) == bb ? ak : 0ULL);
-                        const unsigned long long o1 = R.t1[bb], o2 = R.t2[bb >> 5], o3 = R.t3[bb >> 10];
+                        const unsigned long long km = warp_max64r((ra >> A.lb_shift) == bb ? ak : 0ULL);
+                        const unsigned long long p1 = R.t1[bb], p2 = R.t2[bb >> 5], p3 = R.t3[bb >> 10];
                         __syncwarp();
-                        R.t1[bb] = km > o1 ? km : o1; R.t2[bb >> 5] = km > o2 ? km : o2; R.t3[bb >> 10] = km > o3 ? km : o3;
+                        R.t1[bb] = km > p1 ? km : p1; R.t2[bb >> 5] = km > p2 ? km : p2; R.t3[bb >> 10] = km > p3 ? km : p3;
                         root = km > root ? km : root;
                         __syncwarp();
                     }
                     admitted = a1;
-                } else {
-                    if (busy) { finish(); if (failed) break; }
-                    if (lane == 0) { s_job.type = FAST_JOB_ADMIT; s_job.a0 = admitted; s_job.a1 = a1; }
-                    cta_job();
-                    admitted = a1;
-                    continue;                               // (what was asked for above may be out of date)
                 }
+                if (admitted >= wb + 32) {
+                    wb = admitted;
+                    tw = wb + lane < n ? __ldg(A.sorted_t + wb + lane) : INF;
+                }
+                next_t = __shfl_sync(FULL_MASK, tw, admitted - wb);
             }
+            if (failed) break;
             // ---- pick
-            slot = fcfs_turn ? head : slot_of_root();
+            slot = fcfs_next() ? head : slot_of_root();
             if (slot < 0 || slot >= admitted || slot_done(R, A, slot)) {
-                if (busy) { finish(); if (!failed) continue; break; }              // (prepared from a tournament that is being corrected)
+                if (busy) { finish(); continue; }           // (prepared from a tournament that is being corrected)
                 if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 105);
                 failed = true; break;                       // cannot happen
             }
+            // ---- its records; its leaf block's largest key without it, and the largest beside its blocks on the levels above
             b = slot >> A.lb_shift;
-            if (slot != guess) {
-                const long long r = ((long long)b << A.lb_shift) + lane;
-                kk = r < n ? __ldcg(A.key + r) : 0ULL;
-                pd = ld_dyn(A.dyn + slot);
-                ps = ld_stat(A.stat + slot);
-            }
-            {   // its leaf block's largest key without it
-                const long long r = ((long long)b << A.lb_shift) + lane;
+            const long long r = ((long long)b << A.lb_shift) + lane;
+            const unsigned long long kk = r < n ? *(A.key + r) : 0ULL;
+            pd = ld_dyn_l1(A.dyn + slot);
+            ps = ld_stat(A.stat + slot);
+            {
+                const int32_t i2 = b >> 5, i3 = i2 >> 5;
+                const unsigned long long x1 = lane == (b & 31) ? 0ULL : R.t1[(i2 << 5) + lane];
+                const unsigned long long x2 = lane == (i2 & 31) ? 0ULL : R.t2[(i3 << 5) + lane];
+                const unsigned long long x3 = lane == i3 ? 0ULL : R.t3[lane];
                 if (r < admitted && r != slot && lane < LB && !slot_done(R, A, r)) bm = kk;
                 for (int32_t u = lane + 32; u < LB; u += 32) {
                     const long long r2 = ((long long)b << A.lb_shift) + u;
-                    if (r2 < admitted && r2 != slot && !slot_done(R, A, r2)) { const unsigned long long k2 = __ldcg(A.key + r2); if (k2 > bm) bm = k2; }
+                    if (r2 < admitted && r2 != slot && !slot_done(R, A, r2)) { const unsigned long long k2 = *(A.key + r2); if (k2 > bm) bm = k2; }
                 }
+                o1 = warp_max64r(x1); o2 = warp_max64r(x2); o3 = warp_max64r(x3);
                 bm = warp_max64r(bm);
             }
             // ---- nothing has been committed yet: the decision before must be finished first
             if (busy && finish()) continue;                 // (or failed: the loop ends)
             if (++cyc == A.k) cyc = 0;
-            root = tour_set(R, b, bm, lane);
+            {
+                const unsigned long long v2 = bm > o1 ? bm : o1, v3 = v2 > o2 ? v2 : o2;
+                const int32_t i2 = b >> 5;
+                R.t1[b] = bm; R.t2[i2] = v2; R.t3[i2 >> 5] = v3;       // (every lane stores the same)
+                root = v3 > o3 ? v3 : o3;
+            }
         }
         // ---- the pick is processed: charge it (Definition 2), hand the tree its part
         if (!G) R.done[slot >> 5] |= 1u << (slot & 31);
@@ -3558,8 +3649,9 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
         }
         if (lane == 0) {
             s_tj.type = LRU_JOB_STEP; s_tj.hint = pd.hint; s_tj.m = pd.m; s_tj.len = ps.len; s_tj.gstart = pd.gstart; s_tj.gcount = pd.gcount;
-            s_tj.vleaf = vleaf;
+            s_tj.vleaf = vleaf; s_tj.moved = moved ? 1 : 0;
         }
+        moved = false;
         __syncwarp();
         named_arrive(2, 64);
         busy = true;
@@ -3574,8 +3666,9 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
             P.slot = slot; P.m = pd.m; P.len = ps.len; P.ntok = pd.ntok; P.x = A.tok + ps.soff; P.pos = pd.pos; P.vleaf = vleaf;
             P.gstart = pd.gstart; P.gcount = pd.gcount;
         }
-        if (!fixed && slot == head) head = next_head(R.done, G ? 1 : 0, nwords, n, head, lane);
         __syncwarp();
+        if (!fixed && slot == head) head = next_head(R.done, G ? 1 : 0, nwords, n, head, lane);
+        tell();
     }
     if (busy) { named_bar(3, 64); }
     if (lane == 0) {
@@ -3587,6 +3680,8 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
         for (int i = 8; i < 16; ++i) cn[i] = 0;
         s_job.type = FAST_JOB_EXIT;
         s_tj.type = LRU_JOB_EXIT;
+        __threadfence_block();
+        *(volatile int32_t*)&s_touch.join = ++joins;
     }
     __syncwarp();
     named_arrive(2, 64);
