@@ -616,7 +616,8 @@ match_chain_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* _
 }
 
 // The order in which the batched match takes the queries: bucketed by first token (counting sort over a hash of
-// it; the order inside a bucket is whatever the atomics give -- results do not depend on it).
+// it; the order inside a bucket is whatever the atomics give -- results do not depend on it).  One addition per warp and
+// bucket: where a few system prompts start every query, one per query took 40 us per kernel for 65,536 queries, now 6.
 #define KLPM_ORDER_BUCKETS 8192
 __device__ __forceinline__ unsigned order_bucket(const int32_t* __restrict__ qtok, const int64_t* __restrict__ qoff, int32_t i) {
     const int64_t lo = __ldg(qoff + i);
@@ -627,10 +628,11 @@ __device__ __forceinline__ unsigned order_bucket(const int32_t* __restrict__ qto
 __global__ void order_hist_kernel(const int32_t* __restrict__ qtok, const int64_t* __restrict__ qoff, int32_t nq,
                                   unsigned* __restrict__ hist, unsigned short* __restrict__ bucket) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned b = i < nq ? order_bucket(qtok, qoff, i) : 0xffffffffu;
+    const unsigned same = __match_any_sync(FULL_MASK, b);
     if (i >= nq) return;
-    const unsigned b = order_bucket(qtok, qoff, i);
     bucket[i] = (unsigned short)b;
-    atomicAdd(hist + b, 1u);
+    if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(hist + b, (unsigned)__popc(same));
 }
 // hist[b] <- number of queries in buckets below b (one CTA of 1,024 threads, 8 buckets each)
 __global__ void __launch_bounds__(1024) order_scan_kernel(unsigned* hist) {
@@ -659,8 +661,14 @@ __global__ void __launch_bounds__(1024) order_scan_kernel(unsigned* hist) {
 __global__ void order_scatter_kernel(const unsigned short* __restrict__ bucket, int32_t nq, unsigned* __restrict__ cursor,
                                      int32_t* __restrict__ perm) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nq) return;
-    perm[atomicAdd(cursor + bucket[i], 1u)] = i;
+    const int lane = threadIdx.x & 31;
+    const unsigned b = i < nq ? (unsigned)bucket[i] : 0xffffffffu;
+    const unsigned same = __match_any_sync(FULL_MASK, b);
+    const int lead = __ffs(same) - 1;
+    unsigned at = 0;
+    if (i < nq && lane == lead) at = atomicAdd(cursor + b, (unsigned)__popc(same));
+    at = __shfl_sync(FULL_MASK, at, lead) + (unsigned)__popc(same & ((1u << lane) - 1u));
+    if (i < nq) perm[at] = i;
 }
 
 // Trees with a budget (evicted children break the runs): hop by hop.
@@ -1742,7 +1750,9 @@ __global__ void fast_state_kernel(FastArgs A, const MatchState* __restrict__ sta
     }
     st_dyn_state(A.dyn + r, pos, m, ntok);
     if (A.lru) {
-        st_dyn_hint(A.dyn + r, hint); A.hintc[r] = hint; atomicAdd(A.parked + hint, 1);
+        st_dyn_hint(A.dyn + r, hint); A.hintc[r] = hint;
+        const unsigned on = __activemask(), same = __match_any_sync(on, hint);      // (on an empty tree every query is parked at the root)
+        if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(A.parked + hint, __popc(same));
         A.pk[r] = hint; A.pi[r] = (int32_t)r;
     }
     A.key[r] = fast_key(m, s.len, s.rank, A.score_mode);
@@ -2085,7 +2095,7 @@ __device__ __forceinline__ unsigned long long dissolve_small(const FastArgs& A, 
     bool touched;
     const unsigned long long h = fast_member(A, P, R, r, lane, &touched);
     int32_t rank = 0, start = 0, cnt = 0;
-    for (int k2i = 0; k2i < 32; ++k2i) {
+    for (int k2i = 0; k2i < P.gcount; ++k2i) {              // (at most 32)
         const unsigned long long hk = __shfl_sync(FULL_MASK, h, k2i);
         const bool lt = hk < h, eq = hk == h;
         start += lt; cnt += eq; rank += (lt || (eq && k2i < lane));
@@ -2763,7 +2773,7 @@ fast_run_kernel(FastArgs A) {
                 if (A.completion) A.completion[s.ord] = Rj;
             }
         } else if (lane == 0) {
-            A.order[c] = slot;                              // list mode: the charge pass after the loop does the rest
+            if (A.order) A.order[c] = slot;                 // list mode: the charge pass after the loop does the rest
         }
         // the new leaf's positions: unique per decision, above every real pool index
         const long long vleaf = A.vbase + ((long long)c << 32);
@@ -2791,15 +2801,27 @@ fast_run_kernel(FastArgs A) {
     };
 
     // ================================================================ a given order (klpm_replay): no admission, no pick
+    // A decision matters to another one only if both are in one of the starting groups, so the loop runs through the order
+    // and makes the decisions of grouped slots; the charge pass does everything else.
     if (A.fixed) {
         const int32_t nfix = *reinterpret_cast<const volatile int32_t*>(A.n_fixed);
-        while (c < nfix && !failed) {
-            const int32_t slot = __ldg(A.fixed + c);        // slots are the queries in index order here
-            const FDyn pd = ld_dyn(A.dyn + slot);
-            const FStat ps = ld_stat(A.stat + slot);
-            mark_done(slot);
-            careful(slot, true, pd, ps);                     // (head stays 0 and nobody is admitted: scans cover every slot)
-            __syncwarp();
+        for (int32_t c1 = 0; c1 < nfix && !failed; c1 += 128) {
+            int32_t j[4]; bool g[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { const int32_t x = c1 + u * 32 + lane; j[u] = x < nfix ? __ldg(A.fixed + x) : -1; }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) g[u] = j[u] >= 0 && ((__ldcg(A.gbits + (j[u] >> 5)) >> (j[u] & 31)) & 1u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                for (unsigned bal = __ballot_sync(FULL_MASK, g[u]); bal; bal &= bal - 1) {
+                    const int src = __ffs(bal) - 1;
+                    const int32_t slot = __shfl_sync(FULL_MASK, j[u], src);      // slots are the queries in index order here
+                    c = c1 + u * 32 + src;
+                    mark_done(slot);
+                    careful(slot, false, ld_dyn(A.dyn + slot), ld_stat(A.stat + slot));
+                    __syncwarp();
+                }
+            }
         }
         c = n;                                               // nothing is left for the policy loops below
     }
@@ -3154,7 +3176,7 @@ fast_run_kernel(FastArgs A) {
             cn[14] = cy_cta; cn[15] = cy_warp;
         }
     } else if (lane == 0) {
-        A.post->c0 = n;                                     // list mode never began: nothing is left to charge
+        A.post->c0 = A.fixed ? 0 : n;                       // list mode never began: nothing is left to charge (a given order: everything)
         A.post->now0 = now;
         for (int i = 8; i < 16; ++i) A.post->counters[i] = 0;
     }
@@ -3393,8 +3415,9 @@ __device__ __forceinline__ void lru_touch_warp(const FastArgs& A, const LruTouch
 // if more than 32 slots lose matched tokens (the caller has the CTA scan for them); *failed if there is no room.
 __device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTour& R, const int32_t* small_v, int n_small, int32_t admitted,
                                                  int32_t* s_memcur, unsigned long long* root, bool* failed, int lane) {
-    int32_t n_fall = 0;
-    for (int sv = 0; sv < n_small; ++sv) {
+    int32_t n_fall = 0, listed = 0;
+    for (int sv = 0; sv < n_small; ++sv) listed += __ldcg(A.leaf_run + small_v[sv]).y;
+    for (int sv = 0; sv < n_small && listed > 32; ++sv) {   // (up to 32 slots in the runs: no need to count first)
         const int32_t v = small_v[sv];
         const int2 lr = __ldcg(A.leaf_run + v);
         const int32_t ds_v = A.node[v].depth;
@@ -3467,7 +3490,7 @@ __device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTo
             *failed = true;
         } else {
             int32_t rank = 0, start = 0, cnt = 0;
-            for (int k2i = 0; k2i < 32; ++k2i) {
+            for (int k2i = 0; k2i < n_f; ++k2i) {           // (at most 32)
                 const unsigned long long hk = __shfl_sync(FULL_MASK, f_hash, k2i);
                 const bool lt = hk < f_hash, eq = hk == f_hash;
                 start += lt; cnt += eq; rank += (lt || (eq && k2i < lane));
@@ -3765,76 +3788,117 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
     named_bar(1, KLPM_FAST_THREADS);
 }
 
-// The charge pass after the loop: the decisions made in list mode, c0 .. n-1, are in `order` as slots.  Nobody waited
-// for an arrival there, so completion times are the time list mode began plus a running sum of the costs
-// (Definition 2 with R_prev >= t_j).  Three small kernels: per decision its uncached tokens and cost (and the query
-// index put in `order`), a scan of the per-block sums, and the completion times and TTFTs.
+// The charge pass after the loop: the decisions made in list mode, c0 .. n-1, are in `order` as slots (of a given order,
+// klpm_replay, all decisions, and slots are queries).  Definition 2: R = max(R_prev, t) + cost.  As a function of R_prev
+// that is x -> max(x + a, b) with a = cost, b = t + cost, and such functions compose to one of the same form, so the
+// completion times are a prefix scan.  Three small kernels: per decision its uncached tokens and cost (and the query
+// index put in `order`), a scan of the blocks, and the completion times and TTFTs.
 #define KLPM_CHARGE_THREADS 256
+struct ChargeFn { long long a, b; };
+__device__ __forceinline__ ChargeFn charge_none() { ChargeFn f; f.a = 0; f.b = -0x4000000000000000LL; return f; }
+__device__ __forceinline__ ChargeFn charge_then(const ChargeFn& f, const ChargeFn& g) {      // first f, then g
+    ChargeFn r;
+    r.a = f.a + g.a;
+    const long long x = f.b + g.a;
+    r.b = x > g.b ? x : g.b;
+    return r;
+}
+__device__ __forceinline__ long long charge_at(const ChargeFn& f, long long x) { return x + f.a > f.b ? x + f.a : f.b; }
+// inclusive scan over the warp
+__device__ __forceinline__ ChargeFn charge_warp_scan(ChargeFn f, int lane) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        ChargeFn o;
+        o.a = __shfl_up_sync(FULL_MASK, f.a, d); o.b = __shfl_up_sync(FULL_MASK, f.b, d);
+        if (lane >= d) f = charge_then(o, f);
+    }
+    return f;
+}
+__device__ __forceinline__ int32_t charge_end(const FastArgs& A) { return A.fixed ? *A.n_fixed : A.n; }
+
 // `ipt` consecutive decisions per thread: at most 1,024 blocks whatever the queue's length.
 __global__ void __launch_bounds__(KLPM_CHARGE_THREADS)
-charge_cost_kernel(FastArgs A, long long* cost, long long* bsum, int32_t ipt) {
-    __shared__ long long s_w[KLPM_CHARGE_THREADS / 32];
+charge_cost_kernel(FastArgs A, long long* cost, ChargeFn* bsum, int32_t ipt) {
+    __shared__ ChargeFn s_w[KLPM_CHARGE_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long i0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * ipt;
-    long long x = 0;
+    const long long c0 = A.post->c0;
+    const int32_t end = charge_end(A);
+    ChargeFn f = charge_none();
     for (int32_t u = 0; u < ipt; ++u) {
-        const long long i = i0 + u, c = A.post->c0 + i;
-        if (c < A.n) {
-            const int32_t slot = A.order[c];
+        const long long i = i0 + u, c = c0 + i;
+        if (c < end) {
+            const int32_t slot = A.fixed ? __ldg(A.fixed + c) : A.order[c];
             const int4 s = __ldg(reinterpret_cast<const int4*>(A.stat + slot));     // arrival, length, query index
             const int32_t len = s.z, ord = s.w, unc = len - A.dyn[slot].m;
-            const long long y = (A.c_den + A.c_num * (long long)len) * (long long)unc;
-            A.order[c] = ord;
+            const long long t = (long long)(((unsigned long long)(unsigned)s.y << 32) | (unsigned)s.x);
+            ChargeFn g;
+            g.a = (A.c_den + A.c_num * (long long)len) * (long long)unc;
+            g.b = t + g.a;
+            if (A.order) A.order[c] = ord;
             A.uncached[ord] = unc;
-            cost[i] = y;
-            x += y;
+            cost[i] = g.a;
+            f = charge_then(f, g);
         }
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) x += __shfl_down_sync(FULL_MASK, x, d);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = x;
+    f = charge_warp_scan(f, lane);
+    if (lane == 31) s_w[warp] = f;
     __syncthreads();
     if (threadIdx.x == 0) {
-        long long sum = 0;
-        for (int w = 0; w < KLPM_CHARGE_THREADS / 32; ++w) sum += s_w[w];
+        ChargeFn sum = s_w[0];
+        for (int w = 1; w < KLPM_CHARGE_THREADS / 32; ++w) sum = charge_then(sum, s_w[w]);
         bsum[blockIdx.x] = sum;
     }
 }
-// bsum[b] <- time at which block b's first decision starts (at most 1,024 blocks)
+// bsum[b].a <- time at which block b's first decision may start (at most 1,024 blocks)
 __global__ void __launch_bounds__(1024)
-charge_scan_kernel(FastArgs A, long long* bsum, int32_t nblocks) {
-    __shared__ long long s[1024];
-    const int u = threadIdx.x;
-    const long long v = u < nblocks ? bsum[u] : 0;
-    s[u] = v;
+charge_scan_kernel(FastArgs A, ChargeFn* bsum, int32_t nblocks) {
+    __shared__ ChargeFn s_w[32];
+    const int u = threadIdx.x, lane = u & 31, warp = u >> 5;
+    ChargeFn f = u < nblocks ? bsum[u] : charge_none();
+    f = charge_warp_scan(f, lane);
+    if (lane == 31) s_w[warp] = f;
     __syncthreads();
-    for (int d = 1; d < 1024; d <<= 1) {
-        const long long o = u >= d ? s[u - d] : 0;
-        __syncthreads();
-        s[u] += o;
-        __syncthreads();
-    }
-    if (u < nblocks) bsum[u] = A.post->now0 + s[u] - v;
+    if (warp == 0) { ChargeFn g = charge_warp_scan(s_w[lane], lane); __syncwarp(); s_w[lane] = g; }
+    __syncthreads();
+    ChargeFn before;                                        // everything before this block
+    before.a = __shfl_up_sync(FULL_MASK, f.a, 1); before.b = __shfl_up_sync(FULL_MASK, f.b, 1);
+    if (lane == 0) before = charge_none();
+    if (warp > 0) before = charge_then(s_w[warp - 1], before);
+    if (u < nblocks) bsum[u].a = charge_at(before, A.post->now0);
 }
 __global__ void __launch_bounds__(KLPM_CHARGE_THREADS)
-charge_apply_kernel(FastArgs A, const long long* cost, const long long* bsum, int32_t ipt) {
-    __shared__ long long s_w[KLPM_CHARGE_THREADS / 32];
+charge_apply_kernel(FastArgs A, const long long* cost, const ChargeFn* bsum, int32_t ipt) {
+    __shared__ ChargeFn s_w[KLPM_CHARGE_THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long i0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * ipt;
-    long long mine = 0;                                     // cost of this thread's decisions
-    for (int32_t u = 0; u < ipt; ++u) { const long long c = A.post->c0 + i0 + u; if (c < A.n) mine += cost[i0 + u]; }
-    long long x = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) { const long long o = __shfl_up_sync(FULL_MASK, x, d); if (lane >= d) x += o; }
-    if (lane == 31) s_w[warp] = x;
-    __syncthreads();
-    long long run = bsum[blockIdx.x] + x - mine;            // time at which this thread's first decision starts
-    for (int w = 0; w < warp; ++w) run += s_w[w];
+    const long long c0 = A.post->c0;
+    const int32_t end = charge_end(A);
+    ChargeFn f = charge_none();                             // this thread's decisions
     for (int32_t u = 0; u < ipt; ++u) {
-        const long long i = i0 + u, c = A.post->c0 + i;
-        if (c < A.n) {
-            const int32_t ord = A.order[c];
-            run += cost[i];
-            A.ttft[ord] = run - A.arrival[ord];
+        const long long c = c0 + i0 + u;
+        if (c < end) {
+            ChargeFn g;
+            g.a = cost[i0 + u];
+            g.b = A.arrival[A.fixed ? __ldg(A.fixed + c) : A.order[c]] + g.a;
+            f = charge_then(f, g);
+        }
+    }
+    f = charge_warp_scan(f, lane);
+    if (lane == 31) s_w[warp] = f;
+    __syncthreads();
+    long long run = bsum[blockIdx.x].a;                     // time at which this thread's first decision may start
+    for (int w = 0; w < warp; ++w) run = charge_at(s_w[w], run);
+    ChargeFn before;
+    before.a = __shfl_up_sync(FULL_MASK, f.a, 1); before.b = __shfl_up_sync(FULL_MASK, f.b, 1);
+    if (lane > 0) run = charge_at(before, run);
+    for (int32_t u = 0; u < ipt; ++u) {
+        const long long i = i0 + u, c = c0 + i;
+        if (c < end) {
+            const int32_t ord = A.fixed ? __ldg(A.fixed + c) : A.order[c];
+            const long long t = A.arrival[ord];
+            run = (run > t ? run : t) + cost[i];
+            A.ttft[ord] = run - t;
             if (A.completion) A.completion[ord] = run;
         }
     }
@@ -4810,7 +4874,7 @@ struct rt_tree {
     FDyn* fast_dyn; FStat* fast_stat; unsigned long long* fast_key_arr; int32_t* fast_mem;
     long long* fast_gh; int32_t* fast_gidx; unsigned int* fast_done; unsigned long long* fast_counter;
     long long* fast_lk; int32_t* fast_ls;
-    FastPost* fast_post; long long* fast_bsum;
+    FastPost* fast_post; ChargeFn* fast_bsum;
     long long fast_mem_cap;  // entries of fast_mem
     int32_t* lru_parked; LruInfo* lru_info;     // grouped loop on a tree with a budget
     int32_t* lru_hintc; long long lru_hintc_cap;
@@ -5602,10 +5666,11 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             CK(cudaFuncSetAttribute(fast_run_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             fast_run_kernel<true><<<1, KLPM_FAST_THREADS, smem, s>>>(f);
         }
-        if (f.list_mode) {           // the decisions made in list mode are charged here (none if list mode never began)
-            const int32_t ipt = (int32_t)(((long long)n + 1024LL * KLPM_CHARGE_THREADS - 1) / (1024LL * KLPM_CHARGE_THREADS));
+        if (!lru) {                  // the decisions made in list mode are charged here (none if list mode never began), or a given order
+            const long long nc = d_fixed ? n_fixed : n;
+            const int32_t ipt = (int32_t)((nc + 1024LL * KLPM_CHARGE_THREADS - 1) / (1024LL * KLPM_CHARGE_THREADS));
             const int32_t per_block = KLPM_CHARGE_THREADS * ipt;
-            const int32_t cblocks = (n + per_block - 1) / per_block;                          // at most 1,024
+            const int32_t cblocks = (int32_t)((nc + per_block - 1) / per_block);              // at most 1,024
             charge_cost_kernel<<<cblocks, KLPM_CHARGE_THREADS, 0, s>>>(f, tree->fast_gh, tree->fast_bsum, ipt);
             charge_scan_kernel<<<1, 1024, 0, s>>>(f, tree->fast_bsum, cblocks);
             charge_apply_kernel<<<cblocks, KLPM_CHARGE_THREADS, 0, s>>>(f, tree->fast_gh, tree->fast_bsum, ipt);
