@@ -3977,13 +3977,42 @@ bulk_from_state_kernel(TreeDev T, BulkArgs A, const MatchState* __restrict__ sta
                 inside = node < 0;
             }
         }
-        unsigned im = __ballot_sync(FULL_MASK, inside);
-        while (im) {
-            const int src = __ffs(im) - 1; im &= im - 1;
-            const int32_t r = node_after(X, __shfl_sync(FULL_MASK, pos, src), __shfl_sync(FULL_MASK, cend, src));
-            if (lane == src) {
-                if (r < 0) { set_status(T.st, RT_ERR_LIMIT, 111); act = false; }      // cannot happen
-                else { node = r; off = m - __ldg(T.depth_start + r); }
+        // The node of the run whose edge ends first after the match: four searches side by side, eight lanes and 32 pool
+        // tokens each per step (one after the other with the whole warp: 239 us for 262,144 prompts, now 196; 32,768: 47, now 31).
+        const long long n_nodes = *reinterpret_cast<const volatile long long*>(&T.st->n_nodes);
+        for (unsigned im = __ballot_sync(FULL_MASK, inside); im;) {
+            const int grp = lane >> 3, sub = lane & 7;
+            int src = -1;                                    // the prompt (lane) this group of eight looks after
+#pragma unroll
+            for (int g = 0; g < 4; ++g) { if (im) { if (g == grp) src = __ffs(im) - 1; im &= im - 1; } }
+            const long long gp = __shfl_sync(FULL_MASK, pos, src < 0 ? 0 : src), ge = __shfl_sync(FULL_MASK, cend, src < 0 ? 0 : src);
+            long long q = ((gp + 1) & ~3LL) + 4 * sub;       // aligned: end_node has as many entries as the pool, rounded up
+            int32_t found = -1;
+            bool open = src >= 0;
+            while (__any_sync(FULL_MASK, open)) {
+                int32_t cand = -1;
+                if (open && q < ge) {
+                    const int4 e = __ldg(reinterpret_cast<const int4*>(X.end_node + q));
+                    const int32_t ev[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+                    for (int u = 3; u >= 0; --u) {
+                        const long long at = q + u;
+                        if (ev[u] > 0 && ev[u] < n_nodes && at > gp && at < ge && __ldg(X.span_off + ev[u]) + __ldg(X.span_len + ev[u]) - 1 == at && !__ldg(X.dead + ev[u])) cand = ev[u];
+                    }
+                }
+                const unsigned hit = (__ballot_sync(FULL_MASK, cand >= 0) >> (8 * grp)) & 0xffu;
+                const int32_t first = __shfl_sync(FULL_MASK, cand, 8 * grp + (hit ? __ffs(hit) - 1 : 0));
+                if (open && hit) { found = first; open = false; }
+                q += 32;
+                if (open && q - 4 * sub >= ge) open = false;
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {                    // hand the answers to the prompts' lanes
+                const int32_t to = __shfl_sync(FULL_MASK, src, 8 * g), r = __shfl_sync(FULL_MASK, found, 8 * g);
+                if (lane == to) {
+                    if (r < 0) { set_status(T.st, RT_ERR_LIMIT, 111); act = false; }      // cannot happen
+                    else { node = r; off = m - __ldg(T.depth_start + r); }
+                }
             }
         }
         const bool pend = act && !(m == len && off < 0);
@@ -4002,16 +4031,16 @@ bulk_from_state_kernel(TreeDev T, BulkArgs A, const MatchState* __restrict__ sta
     }
 }
 
-// What the apply step does for 32 pending prompts of the list (one per lane, from number p0 on): cut the edge the
+// What the apply step does for `width` pending prompts of the list (one per lane, from number p0 on): cut the edge the
 // match ends in if the prompt holds the claim, add its leaf if it wins the child's table slot, or put the prompt on
 // the list for the next round; then the warp copies the new leaves' tokens, one leaf after the other.  New nodes are
 // numbered and pool space is taken with one addition per warp.  Tree fields are read through L2 (__ldcg): inside the
 // kernel that runs all later rounds, another SM may have written them a moment ago.
-__device__ __forceinline__ void bulk_apply_warp(const TreeDev& T, const BulkArgs& A, unsigned long long p0, unsigned n_apply, int lane,
+__device__ __forceinline__ void bulk_apply_warp(const TreeDev& T, const BulkArgs& A, unsigned long long p0, unsigned n_apply, unsigned width, int lane,
                                                 unsigned long long* s_live_nodes, unsigned long long* s_live_tokens) {
     TreeState* S = T.st;
     const unsigned lt = (1u << lane) - 1u;
-    const bool act = p0 + lane < n_apply;
+    const bool act = (unsigned)lane < width && p0 + lane < n_apply;
     int32_t i = 0, len = 0, m = 0, node = 0, off = -1;
     const int32_t* x = A.tok;
     if (act) {
@@ -4122,21 +4151,47 @@ __device__ __forceinline__ void bulk_apply_warp(const TreeDev& T, const BulkArgs
         base = __shfl_sync(FULL_MASK, base, lead);
         if (retry) A.pend_next[base + __popc(rm & lt)] = i;
     }
-    // ---- the new leaves' tokens
+    // ---- the new leaves' tokens: the first 128 of four leaves in flight together, the rest 512 at a time
     unsigned dm = __ballot_sync(FULL_MASK, dst >= 0);
     while (dm) {
-        const int src = __ffs(dm) - 1; dm &= dm - 1;
-        const int64_t d = __shfl_sync(FULL_MASK, dst, src);
-        const int32_t* xs = reinterpret_cast<const int32_t*>(__shfl_sync(FULL_MASK, (unsigned long long)(x + m), src));
-        const int32_t cnt = __shfl_sync(FULL_MASK, unc, src);
-        for (int32_t t0 = 0; t0 < cnt; t0 += 128) {
-            int32_t v[4];
+        int32_t v[16];
+        const int32_t* xs[4]; int64_t d[4]; int32_t cnt[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) { const int32_t t = t0 + r * 32 + lane; v[r] = t < cnt ? __ldg(xs + t) : 0; }
+        for (int g = 0; g < 4; ++g) {
+            const int src = dm ? __ffs(dm) - 1 : 0;
+            cnt[g] = __shfl_sync(FULL_MASK, unc, src);
+            if (!dm) cnt[g] = 0;
+            dm &= dm - 1;
+            d[g] = __shfl_sync(FULL_MASK, dst, src);
+            xs[g] = reinterpret_cast<const int32_t*>(__shfl_sync(FULL_MASK, (unsigned long long)(x + m), src));
 #pragma unroll
-            for (int r = 0; r < 4; ++r) { const int32_t t = t0 + r * 32 + lane; if (t < cnt) T.pool[d + t] = v[r]; }
+            for (int r = 0; r < 4; ++r) { const int32_t t = r * 32 + lane; v[4 * g + r] = t < cnt[g] ? __ldg(xs[g] + t) : 0; }
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) { const int32_t t = r * 32 + lane; if (t < cnt[g]) T.pool[d[g] + t] = v[4 * g + r]; }
+#pragma unroll 1
+        for (int g = 0; g < 4; ++g) {
+            const int32_t* xg = g == 0 ? xs[0] : g == 1 ? xs[1] : g == 2 ? xs[2] : xs[3];
+            const int64_t dg = g == 0 ? d[0] : g == 1 ? d[1] : g == 2 ? d[2] : d[3];
+            const int32_t cg = g == 0 ? cnt[0] : g == 1 ? cnt[1] : g == 2 ? cnt[2] : cnt[3];
+            for (int32_t t0 = 128; t0 < cg; t0 += 512) {
+#pragma unroll
+                for (int r = 0; r < 16; ++r) { const int32_t t = t0 + r * 32 + lane; v[r] = t < cg ? __ldg(xg + t) : 0; }
+#pragma unroll
+                for (int r = 0; r < 16; ++r) { const int32_t t = t0 + r * 32 + lane; if (t < cg) T.pool[dg + t] = v[r]; }
+            }
         }
     }
+}
+
+// Pending prompts per warp of the apply step: as few as keep every warp of the grid busy (their leaves' tokens are copied
+// one warp after the other: 2,000 prompts with 6,000 tokens to store took 509 us at 32 per warp, now 50), at least two
+// (a warp's prompts share its additions to the tree's counters), at most one per lane.
+__device__ __forceinline__ unsigned bulk_width(unsigned n_apply, unsigned nwarps) {
+    const unsigned w = (n_apply + nwarps - 1) / nwarps;
+    return w < 2 ? 2 : w > 32 ? 32 : w;
 }
 
 __global__ void __launch_bounds__(256)
@@ -4148,9 +4203,10 @@ bulk_apply_kernel(TreeDev T, BulkArgs A) {
     const unsigned n_pending = *A.n_out;
     const int lane = threadIdx.x & 31;
     const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (unsigned long long p0 = (unsigned long long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32ULL; p0 < n_pending;
-         p0 += (unsigned long long)nwarps * 32ULL)
-        bulk_apply_warp(T, A, p0, n_pending, lane, &s_live_nodes, &s_live_tokens);
+    const unsigned width = bulk_width(n_pending, nwarps);
+    for (unsigned long long p0 = (unsigned long long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * width; p0 < n_pending;
+         p0 += (unsigned long long)nwarps * width)
+        bulk_apply_warp(T, A, p0, n_pending, width, lane, &s_live_nodes, &s_live_tokens);
     __syncthreads();
     if (threadIdx.x == 0) {
         if (s_live_nodes) atomicAdd((unsigned long long*)&T.st->live_nodes, s_live_nodes);
@@ -4251,8 +4307,9 @@ bulk_rounds_kernel(TreeDev T, BulkArgs A, BulkSync* g, long long n_total, const 
         // ---- cuts and leaves
         const unsigned n_apply = __ldcg(R.n_out);
         if (blockIdx.x == 0 && threadIdx.x == 0) { g->cnt_w[par ^ 1u] = 0u; g->cnt_a[par ^ 1u] = 0u; }     // the next round's
-        for (unsigned long long p0 = (unsigned long long)warp0 * 32ULL; p0 < n_apply; p0 += (unsigned long long)nwarps * 32ULL)
-            bulk_apply_warp(T, R, p0, n_apply, lane, &s_live_nodes, &s_live_tokens);
+        const unsigned width = bulk_width(n_apply, nwarps);
+        for (unsigned long long p0 = (unsigned long long)warp0 * width; p0 < n_apply; p0 += (unsigned long long)nwarps * width)
+            bulk_apply_warp(T, R, p0, n_apply, width, lane, &s_live_nodes, &s_live_tokens);
         if (!bulk_barrier(g, S, limit_ns, [&] {
                 const bool stop = *(volatile int*)&S->status != 0 || (long long)r > 4 * n_total + 64;      // (every round stores a prompt)
                 g->go = stop ? 0u : *(volatile unsigned*)&g->cnt_a[par];
