@@ -1586,6 +1586,7 @@ struct FastArgs {
     const int32_t* tok;
     int32_t n;
     int32_t policy, k, score_mode;
+    unsigned recip_k1;            // 2^32 / (k - 1) rounded up: x / (k - 1) = high half of x * recip_k1, exact while x (k - 1) < 2^32; 0 if k - 1 is 1 or larger than any x it is used for
     long long c_num, c_den, start_tick;
     int32_t* order; int32_t* uncached; int64_t* ttft; int64_t* completion;
     FDyn* dyn; FStat* stat;
@@ -2003,6 +2004,7 @@ __device__ __forceinline__ unsigned long long changed_block_max(const FastArgs& 
 
 // What the sequencer hands to a CTA-wide batch of decisions, and what it gets back.
 struct FastBatchIO {
+    int32_t per;                      // in: list entries per thread, 4 (1,024 decisions at most) or 1 (256: cheaper where batches end early)
     int32_t cur, head, c, cyc;        // in: list cursor, oldest unprocessed slot, decisions made, c mod k
     unsigned long long root;          // in: largest key in the tournament
     int32_t B, consumed, hmax;        // out: decisions made (0: none), list entries passed, last slot taken by an oldest-first turn
@@ -2013,12 +2015,16 @@ struct FastBatchIO {
     int32_t colPhi[32], colRk[32], remH[32], remE[32];
     int32_t hard;                     // out: the batch stopped before a decision that needs the one-at-a-time path
     int32_t Braw;                     // out: decisions the batch could have made (it makes none below KLPM_FAST_CTA_MIN)
+    int32_t wide;                     // in: look at as many slots and entries as the scratch holds (the last batch had many meetings)
+    int32_t played;                   // out: the batch was played through decision by decision (more than 32 meetings)
+    int32_t played_t, played_u;       // scratch: ranks of the last slot and the last entry taken, -1 if none
     int32_t limB;                     // scratch: the batch must end before this decision (list entries that an oldest-first pick would meet)
 };
 #define KLPM_FAST_CTA_BATCH 1024      // decisions per CTA-wide batch at most (4 list entries per thread)
 #ifndef KLPM_FAST_CTA_MIN
 #define KLPM_FAST_CTA_MIN 32         // smaller batches are left to the warp-wide step (an attempt costs about 10,000 cycles)
 #endif
+#define KLPM_FAST_PLAY 48
 #ifndef KLPM_FAST_CB_MAX
 #define KLPM_FAST_CB_MAX 32           // longest back-off (loop iterations) after CTA-wide attempts that failed
 #endif
@@ -2126,13 +2132,14 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     const int tid = threadIdx.x;
     const int32_t n = A.n, cur = io->cur, head = io->head, c = io->c, cyc = io->cyc;
     const unsigned long long root = io->root;
+    const int32_t per = io->per, most_ = KLPM_FAST_THREADS * per;      // list entries per thread; decisions the batch can make
     // the list entries cur + 4 tid .. + 3 (asked for first: the table below is filled while they travel)
     long long kk[4]; int32_t es[4]; bool ok[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        const long long idx = (long long)cur + tid * 4 + r;
+        const long long idx = (long long)cur + tid * per + r;
         kk[r] = 0; es[r] = 0;
-        if (idx < n) { kk[r] = __ldg(A.lk + idx); es[r] = __ldg(A.ls + idx); }
+        if (r < per && idx < n) { kk[r] = __ldg(A.lk + idx); es[r] = __ldg(A.ls + idx); }
     }
     // sF[x] = oldest-first turns among the next x decisions, x = 0 .. 1,024.  Under k-LPM the first such turn is
     // decision (k - cyc) mod k and then every k-th, which is floor((x + s) / k) with s = (cyc + k - 1) mod k; one
@@ -2154,8 +2161,8 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     int32_t cnt = 0;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        const long long idx = (long long)cur + tid * 4 + r;
-        ok[r] = idx < n && !((bm_ld(R.skip, es[r] >> 5, R.g_bits) >> (es[r] & 31)) & 1u);
+        const long long idx = (long long)cur + tid * per + r;
+        ok[r] = r < per && idx < n && !((bm_ld(R.skip, es[r] >> 5, R.g_bits) >> (es[r] & 31)) & 1u);
         cnt += ok[r];
     }
     // the unprocessed slots from `head` on, one bitmap word per thread
@@ -2176,11 +2183,16 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     int32_t* sP = sF + KLPM_FAST_CTA_BATCH + 8;             // per word: free slots before it
     unsigned* sFr = reinterpret_cast<unsigned*>(sP + KLPM_FAST_THREADS);
     sP[tid] = qk; sFr[tid] = fr;
+    int32_t* sMet = reinterpret_cast<int32_t*>(sFr + KLPM_FAST_THREADS);      // per entry rank: rank of its slot among the oldest-first picks, or -1
+    int32_t* sBack = sMet + KLPM_FAST_CTA_BATCH;            // and the other way round
+    int32_t* sSel = sBack + KLPM_FAST_CTA_BATCH;            // a batch that is played through: the slot of every decision
+    // u / (k - 1) for u up to 2,048: a multiplication by the reciprocal rounded up
+    auto per_k1 = [&](int32_t u) -> int32_t { return A.k == 2 ? u : (int32_t)__umulhi((unsigned)u, A.recip_k1); };
     {   // as many decisions as those entries allow: the largest x with x - f(x) <= avail, every thread trying four values
-        const int32_t hi = n - c < KLPM_FAST_CTA_BATCH ? n - c : KLPM_FAST_CTA_BATCH;
+        const int32_t hi = n - c < most_ ? n - c : most_;
         int32_t best = 0;
-#pragma unroll
-        for (int r = 1; r <= 4; ++r) { const int32_t x = tid * 4 + r; if (x <= hi && x - f(x) <= avail) best = x; }
+#pragma unroll 1
+        for (int r = 1; r <= per; ++r) { const int32_t x = tid * per + r; if (x <= hi && x - f(x) <= avail) best = x; }
         best = __reduce_max_sync(FULL_MASK, best);
         if ((tid & 31) == 0 && best > 0) atomicMax(&io->B0, best);
     }
@@ -2190,8 +2202,9 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     // batch (a slot that is both among the oldest unprocessed and among the next list entries), the side that comes
     // later passes over it and takes one more of its own.
     const bool both_kinds = A.policy == KLPM_POLICY_KLPM && A.k >= 2;       // (k = 1: every turn is an oldest-first turn)
-    const int32_t nFw = both_kinds ? (nF0 + 32 < KLPM_FAST_CTA_BATCH ? nF0 + 32 : KLPM_FAST_CTA_BATCH) : nF0;
-    const int32_t nLw = both_kinds ? (nL0 + 32 < KLPM_FAST_CTA_BATCH ? nL0 + 32 : KLPM_FAST_CTA_BATCH) : nL0;
+    const bool wide = both_kinds && io->wide != 0;
+    const int32_t nFw = wide ? KLPM_FAST_CTA_BATCH : both_kinds ? (nF0 + 32 < KLPM_FAST_CTA_BATCH ? nF0 + 32 : KLPM_FAST_CTA_BATCH) : nF0;
+    const int32_t nLw = wide ? KLPM_FAST_CTA_BATCH : both_kinds ? (nL0 + 32 < KLPM_FAST_CTA_BATCH ? nL0 + 32 : KLPM_FAST_CTA_BATCH) : nL0;
     const int32_t nFa = nfree < nFw ? nfree : nFw;          // oldest-first picks there are slots for
     const int32_t nEa = avail < nLw ? avail : nLw;          // longest-match picks there are entries for
     // the next nFa unprocessed slots in order: a thread per slot, eight words at a time; the slot's rank among the free
@@ -2225,14 +2238,16 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
         for (int r = 0; r < 4; ++r) {
             if (ok[r]) {
                 if (rk < nEa) {
-                    sE[rk] = es[r]; sEpos[rk] = tid * 4 + r;
+                    sE[rk] = es[r]; sEpos[rk] = tid * per + r;
                     const unsigned long long ek = ~((unsigned long long)kk[r] ^ 0x8000000000000000ULL);
+                    int32_t met = -1;
                     if ((((bm_ld(R.gb, es[r] >> 5, R.g_bits) >> (es[r] & 31)) & 1u)) || root > ek) {
                         atomicMin(&io->limL, rk);
                     } else if (es[r] >= head && es[r] <= hmax0) {
-                        int32_t lo = 0, hi = nFa;                        // phi: slots of sH before this one
-                        while (lo < hi) { const int32_t mid = (lo + hi) >> 1; if (sH[mid] < es[r]) lo = mid + 1; else hi = mid; }
-                        const int32_t phi = lo;
+                        // phi: slots of sH before this one (its word is one of those looked at: it lies between head and hmax0)
+                        const int32_t wl = (es[r] >> 5) - w0;
+                        const int32_t phi = sP[wl] + __popc(sFr[wl] & ((1u << (es[r] & 31)) - 1u));
+                        met = phi;
                         // decision of the oldest-first turn of rank phi, and of the longest-match turn of rank rk
                         int32_t xF, xL;
                         if (A.policy == KLPM_POLICY_FCFS) { xF = phi; xL = B0; }
@@ -2242,20 +2257,17 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
                             const long long xF64 = i0 + (long long)phi * A.k;
                             xF = xF64 < 0x3ffffff ? (int32_t)xF64 : 0x3ffffff;
                             xL = rk;                                       // before the first oldest-first turn; after it k - 1 of every k decisions
-                            if (rk >= i0 && A.k >= 2) {
-                                const int32_t u1 = rk - i0, q = u1 / (A.k - 1);
-                                const long long xL64 = i0 + (long long)q * A.k + 1 + (u1 - q * (A.k - 1));
-                                xL = xL64 < 0x3ffffff ? (int32_t)xL64 : 0x3ffffff;
-                            }
+                            if (rk >= i0 && A.k >= 2) { const int32_t u1 = rk - i0; xL = rk + 1 + per_k1(u1); }
                         }
                         // without resolving: the batch would have to end before the later of the two decisions (used
-                        // when there are more such slots than the resolution below takes)
+                        // where there are more such slots than are resolved)
                         atomicMin(&io->limB, xF > xL ? xF : xL);
                         if (both_kinds) {
                             const int32_t ci = atomicAdd(&io->ncol, 1);
                             if (ci < 32) { io->colPhi[ci] = phi; io->colRk[ci] = rk; }
                         }
                     }
+                    if (both_kinds) sMet[rk] = met;
                 }
                 ++rk;
             }
@@ -2281,26 +2293,25 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
                 if (rj < rk) belowRk |= 1u << j;
             }
             const int32_t i0 = cyc == 0 ? 0 : A.k - cyc;    // decisions before the first oldest-first turn
-            const long long FAR = 0x3ffffff;
-            // decision of the longest-match turn of rank u, of the oldest-first turn of rank t
-            auto l_turn = [&](int32_t u) -> long long {
-                if (u < i0) return u;
-                const int32_t u1 = u - i0, q = u1 / (A.k - 1);
-                return i0 + (long long)q * A.k + 1 + (u1 - q * (A.k - 1));
-            };
+            const int32_t FAR = 0x3ffffff;
+            // decision of the longest-match turn of rank u, of the oldest-first turn of rank t (capped)
+            auto l_turn = [&](int32_t u) -> int32_t { return u < i0 ? u : u + 1 + per_k1(u - i0); };
+            auto f_turn = [&](int32_t t) -> int32_t { const long long x = i0 + (long long)t * A.k; return x < FAR ? (int32_t)x : FAR; };
             // no batch gets past the first slot or entry that needs the careful step, whoever passes over what
             const int32_t capF = io->limF < nFa ? io->limF : nFa, capL = io->limL < nEa ? io->limL : nEa;
-            long long bcap = B0;
-            { const long long a1 = i0 + (long long)capF * A.k, a2 = l_turn(capL); if (a1 < bcap) bcap = a1; if (a2 < bcap) bcap = a2; }
-            long long xF = FAR, xL = FAR;
-            if (mine) { xF = i0 + (long long)phi * A.k; xL = l_turn(rk); if (xF > FAR) xF = FAR; }
+            int32_t bcap = B0;
+            { const int32_t a1 = f_turn(capF), a2 = l_turn(capL); if (a1 < bcap) bcap = a1; if (a2 < bcap) bcap = a2; }
+            int32_t xF = FAR, xL = FAR;
+            // oldest-first turns before a longest-match turn of rank u are 1 + u1 / (k - 1): whether u1 is the first of its k - 1
+            int32_t cur_rk = rk;                            // the entry's rank less those this side has passed over below it
+            if (mine) { xF = f_turn(phi); xL = l_turn(rk); }
             unsigned remH = 0, remE = 0, open_ = ncol == 32 ? 0xffffffffu : ((1u << ncol) - 1u);
             while (open_) {
                 unsigned key = 0xffffffffu;
                 const bool l_first = xL < xF;
                 if (mine && ((open_ >> lane) & 1u)) key = ((unsigned)(l_first ? xL : xF) << 5) | (unsigned)lane;
                 const unsigned win = __reduce_min_sync(FULL_MASK, key);
-                if ((long long)(win >> 5) >= bcap) break;   // beyond what the batch can reach: nothing more to settle
+                if ((int32_t)(win >> 5) >= bcap) break;   // beyond what the batch can reach: nothing more to settle
                 const int wl = (int)(win & 31u);
                 const bool wl_first = __shfl_sync(FULL_MASK, (int)l_first, wl) != 0;
                 open_ &= ~(1u << wl);
@@ -2309,16 +2320,93 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
                     if (((belowPhi >> wl) & 1u) && xF < FAR) xF -= A.k;
                 } else {                                    // an oldest-first turn took that entry's slot: later list picks come one turn earlier
                     remE |= 1u << wl;
-                    if ((belowRk >> wl) & 1u) {
-                        long long y = xL - 1;
-                        if (y >= i0 && (y - i0) % A.k == 0) --y;       // (that one is an oldest-first turn)
-                        xL = y;
-                    }
+                    if ((belowRk >> wl) & 1u) { --cur_rk; xL = l_turn(cur_rk); }
                 }
             }
             if (mine && ((remH >> lane) & 1u)) io->remH[__popc(remH & belowPhi)] = phi;
             if (mine && ((remE >> lane) & 1u)) io->remE[__popc(remE & belowRk)] = rk;
             if (lane == 0) { io->nRH = __popc(remH); io->nRE = __popc(remE); }
+        }
+        __syncthreads();
+    }
+    // More meetings than that (two orders that run side by side): the batch is played through decision by decision.  Warp 0
+    // holds one bit per rank of either side (word w in lane w; the word a side is at also in a uniform register): the next
+    // rank whose bit is clear is the pick, and its slot's bit on the other side is set: about 250 cycles a decision, and
+    // far less where the two orders agree, where the one-at-a-time path takes 1,000.  A batch that gets KLPM_FAST_PLAY decisions far without it costs less that way
+    // (9,000 cycles in all).
+    const bool play = both_kinds && ncol > 32 && io->limB < KLPM_FAST_PLAY;
+    if (play) {
+        for (int32_t x = tid; x < nFa; x += KLPM_FAST_THREADS) sBack[x] = -1;
+        __syncthreads();
+        for (int32_t x = tid; x < nEa; x += KLPM_FAST_THREADS) if (sMet[x] >= 0) sBack[sMet[x]] = x;
+        __syncthreads();
+        if (tid < 32) {
+            const int lane = tid;
+            const int32_t capF = io->limF < nFa ? io->limF : nFa, capL = io->limL < nEa ? io->limL : nEa;
+            const int32_t most = n - c < KLPM_FAST_CTA_BATCH ? n - c : KLPM_FAST_CTA_BATCH;      // (wide: both sides in sight beyond the list window)
+            unsigned mh = 0, me = 0;                        // ranks that are taken, of this lane's word
+            unsigned ch = 0, ce = 0;                        // the words the two sides are at
+            int32_t t = 0, u = 0, lt = -1, lu = -1, x = 0, turn = cyc;
+            bool stop_f = false, stop_l = false;            // ran into the end of what is in sight, or into a limit, on which side
+            for (; x < most; ++x) {
+                // Where both sides are at the same slot, that slot is the next pick whichever turn it is, and so on for as
+                // long as the two orders agree: up to 32 decisions at once.
+                {
+                    const unsigned fh = ~ch & (0xffffffffu << (t & 31)), fe = ~ce & (0xffffffffu << (u & 31));
+                    if (fh && fe) {
+                        t = (t & ~31) + __ffs(fh) - 1;
+                        u = (u & ~31) + __ffs(fe) - 1;
+                        const int32_t tt = t + lane, uu = u + lane;
+                        const bool same = tt < capF && uu < capL && x + lane < most && (tt >> 5) == (t >> 5) && !((ch >> (tt & 31)) & 1u) && sMet[uu] == tt;
+                        const unsigned no = ~__ballot_sync(FULL_MASK, same);
+                        const int r = no ? __ffs(no) - 1 : 32;
+                        if (r >= 2) {
+                            if (lane < r) sSel[x + lane] = sH[tt];
+                            const unsigned run = r == 32 ? 0xffffffffu : (1u << r) - 1u;
+                            const unsigned long long runE = (unsigned long long)run << (u & 31);
+                            ch |= run << (t & 31);
+                            if (lane == (t >> 5)) mh |= run << (t & 31);
+                            if (lane == (u >> 5)) me |= (unsigned)runE;
+                            if (lane == (u >> 5) + 1) me |= (unsigned)(runE >> 32);
+                            ce |= (unsigned)runE;
+                            lt = t + r - 1; lu = u + r - 1;
+                            x += r - 1;
+                            turn = (turn + r) % A.k;
+                            continue;
+                        }
+                    }
+                }
+                const bool fcfs_turn = turn == 0;
+                if (++turn == A.k) turn = 0;
+                int32_t other, slot;
+                if (fcfs_turn) {
+                    unsigned free_ = ~ch & (0xffffffffu << (t & 31));
+                    while (!free_ && (t | 31) + 1 < capF) { t = (t | 31) + 1; ch = __shfl_sync(FULL_MASK, mh, t >> 5); free_ = ~ch; }
+                    stop_f = !free_;
+                    if (!stop_f) { t = (t & ~31) + __ffs(free_) - 1; stop_f = t >= capF; }
+                    if (stop_f) break;
+                    slot = sH[t]; other = sBack[t]; lt = t;
+                    ch |= 1u << (t & 31);
+                    if (lane == (t >> 5)) mh |= 1u << (t & 31);
+                    if (other >= 0) { const unsigned bit = 1u << (other & 31); if ((other >> 5) == (u >> 5)) ce |= bit; if (lane == (other >> 5)) me |= bit; }
+                } else {
+                    unsigned free_ = ~ce & (0xffffffffu << (u & 31));
+                    while (!free_ && (u | 31) + 1 < capL) { u = (u | 31) + 1; ce = __shfl_sync(FULL_MASK, me, u >> 5); free_ = ~ce; }
+                    stop_l = !free_;
+                    if (!stop_l) { u = (u & ~31) + __ffs(free_) - 1; stop_l = u >= capL; }
+                    if (stop_l) break;
+                    slot = sE[u]; other = sMet[u]; lu = u;
+                    ce |= 1u << (u & 31);
+                    if (lane == (u >> 5)) me |= 1u << (u & 31);
+                    if (other >= 0) { const unsigned bit = 1u << (other & 31); if ((other >> 5) == (t >> 5)) ch |= bit; if (lane == (other >> 5)) mh |= bit; }
+                }
+                if (lane == 0) sSel[x] = slot;
+            }
+            if (lane == 0) {
+                io->played_t = lt; io->played_u = lu; io->Bmax = x;
+                // stopped by a decision only the one-at-a-time path can take, not by the end of what is in sight?
+                io->hard = (stop_f && io->limF < nFa) || (stop_l && io->limL < nEa) ? 1 : 0;
+            }
         }
         __syncthreads();
     }
@@ -2329,11 +2417,11 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     // rank t among the oldest-first picks -> index of its slot in sH; rank u among the longest-match picks -> index in sE
     auto hI = [&](int32_t t) -> int32_t { for (int32_t j = 0; j < nRH; ++j) { if (io->remH[j] <= t) ++t; else break; } return t; };
     auto eI = [&](int32_t u) -> int32_t { for (int32_t j = 0; j < nRE; ++j) { if (io->remE[j] <= u) ++u; else break; } return u; };
-    {   // the largest x that respects the limits, every thread trying four values
+    if (!play) {   // the largest x that respects the limits, every thread trying four values
         int32_t best = 0;
-#pragma unroll
-        for (int r = 1; r <= 4; ++r) {
-            const int32_t x = tid * 4 + r, nf = f(x), nl = x - nf;
+#pragma unroll 1
+        for (int r = 1; r <= per; ++r) {
+            const int32_t x = tid * per + r, nf = f(x), nl = x - nf;
             if (x <= limB && (nf == 0 || hI(nf - 1) < limF) && (nl == 0 || eI(nl - 1) < limL)) best = x;
         }
         best = __reduce_max_sync(FULL_MASK, best);
@@ -2342,9 +2430,13 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     __syncthreads();
     const int32_t Braw = io->Bmax;
     const int32_t B = Braw >= KLPM_FAST_CTA_MIN ? Braw : 0;     // nothing is changed by a batch too short to pay
-    if (tid == 0) {
+    if (tid == 0) { io->B = B; io->Braw = Braw; io->played = play ? 1 : 0; io->wide = play ? 1 : 0; }
+    if (tid == 0 && play) {
+        io->consumed = io->played_u >= 0 ? sEpos[io->played_u] + 1 : 0;
+        io->hmax = io->played_t >= 0 ? sH[io->played_t] : -1;
+        if (B == 0) io->hard = 0;
+    } else if (tid == 0) {
         const int32_t nF = f(B), nL = B - nF;
-        io->B = B; io->Braw = Braw;
         io->consumed = nL > 0 ? sEpos[eI(nL - 1)] + 1 : 0;
         io->hmax = nF > 0 ? sH[hI(nF - 1)] : -1;
         // stopped by a decision only the one-at-a-time path can take (not by the end of what is in sight, nor by a
@@ -2354,7 +2446,7 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     }
     for (int32_t x = tid; x < B; x += KLPM_FAST_THREADS) {   // thread makes decisions c + x
         const int32_t f0 = f(x);
-        const int32_t slot = f(x + 1) > f0 ? sH[hI(f0)] : sE[eI(x - f0)];
+        const int32_t slot = play ? sSel[x] : f(x + 1) > f0 ? sH[hI(f0)] : sE[eI(x - f0)];
         atomicOr(R.done + (slot >> 5), 1u << (slot & 31));
         atomicOr(R.skip + (slot >> 5), 1u << (slot & 31));
         A.order[c + x] = slot;
@@ -3055,6 +3147,9 @@ fast_run_kernel(FastArgs A) {
         int32_t vb_wait = 0, vb_back = 1;                   // decisions until the next attempt; doubles while attempts fail
         int32_t cb_wait = 0, cb_back = 8;                   // the same for the CTA-wide batch (loop iterations; 8 .. 1,024)
         int32_t cb_until = 0, cb_fail = 0;                  // after an attempt that made no decision: not before decision cb_until; attempts failed in a row
+        if (lane == 0) s_bio.wide = 0;
+        int32_t per_now = 4;
+        int32_t calm_until = 0;
         int32_t calm = KLPM_FAST_CALM;                      // consecutive full warp-wide steps: the CTA-wide batch is tried in calm water only
         long long n_cta_try = 0, n_cta_ok = 0, dec_cta = 0, n_warp_ok = 0, dec_warp = 0, dec_one = 0, cy_cta = 0, cy_warp = 0;
         // a batch that was cut short stopped before a decision only the one-at-a-time path can take: that one comes
@@ -3064,9 +3159,9 @@ fast_run_kernel(FastArgs A) {
         while (c < n && !failed) {
             if (++iters > 64LL * n + 4096) { if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 118); failed = true; break; }      // cannot happen
             // first choice: the whole CTA makes up to 1,024 decisions (the sort scratch is free between dissolves)
-            if (!one_next && cb_wait <= 0 && calm >= KLPM_FAST_CALM && c >= cb_until && n - c >= KLPM_FAST_CTA_MIN) {
+            if (!one_next && cb_wait <= 0 && (calm >= KLPM_FAST_CALM || c >= calm_until) && c >= cb_until && n - c >= KLPM_FAST_CTA_MIN) {
                 if (lane == 0) {
-                    s_bio.cur = cur; s_bio.head = head; s_bio.c = c; s_bio.cyc = cyc; s_bio.root = root; s_bio.B = 0;
+                    s_bio.per = per_now; s_bio.cur = cur; s_bio.head = head; s_bio.c = c; s_bio.cyc = cyc; s_bio.root = root; s_bio.B = 0;
                     s_job.type = FAST_JOB_BATCH;
                 }
                 __syncwarp();
@@ -3079,6 +3174,7 @@ fast_run_kernel(FastArgs A) {
                 cy_cta += cy_this;
                 if (Bc > 0) {
                     ++n_cta_ok; dec_cta += Bc;
+                    per_now = s_bio.wide || Bc >= (per_now == 1 ? 224 : 160) ? 4 : 1;
                     const int32_t consumed = s_bio.consumed, hmax = s_bio.hmax;
                     c += Bc;
                     one_next = s_bio.hard != 0;
@@ -3088,13 +3184,14 @@ fast_run_kernel(FastArgs A) {
                     else if (head < n && ((bm_ld(s_done, head >> 5, gdone) >> (head & 31)) & 1u)) advance_head();
                     // did it pay?  its cycles per decision against what the warp-wide steps have cost per decision so far
                     const long long warp_cpd = dec_warp >= 256 ? cy_warp / dec_warp : 100;
-                    if (cy_this <= (long long)Bc * warp_cpd) { cb_back = 8; cb_fail = 0; continue; }
+                    if (s_bio.played /* the alternative is one at a time */ || cy_this <= (long long)Bc * warp_cpd) { cb_back = 8; cb_fail = 0; continue; }
                     // committed, but too short to have paid for the attempt: warp-wide steps for a while, as after a failure
                     cb_wait = cb_back;
                     cb_back = cb_back < KLPM_FAST_CB_MAX ? cb_back * 2 : KLPM_FAST_CB_MAX;
-                    calm = 0;
+                    calm = 0; calm_until = c + 64;
                     continue;
                 }
+                per_now = 1; calm_until = c + 64;
                 // too few decisions before one that needs the one-at-a-time path: the next attempt waits until that one has
                 // been made (and longer when attempts keep failing: such decisions come in runs)
                 cb_until = c + s_bio.Braw + 1 + (cb_fail > 0 ? (8 << cb_fail) : 0);
@@ -3106,7 +3203,8 @@ fast_run_kernel(FastArgs A) {
                 const long long t_w = clock64();
                 const bool took = try_batch();
                 cy_warp += clock64() - t_w;
-                if (took) { ++n_warp_ok; dec_warp += c - c_was; vb_back = 1; calm = c - c_was == 32 ? calm + 1 : 0; one_next = tb_cut; continue; }
+                if (took) { ++n_warp_ok; dec_warp += c - c_was; vb_back = 1; if (c - c_was == 32) ++calm; else { if (calm > 0) calm_until = c + 64; calm = 0; } one_next = tb_cut; continue; }
+                if (calm > 0) calm_until = c + 64;          // (where warp-wide steps keep failing the whole CTA may do better)
                 calm = 0;
                 vb_wait = vb_back;
                 vb_back = vb_back < 64 ? vb_back * 2 : 64;
@@ -5638,6 +5736,7 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             lru_pack_kernel<<<(unsigned)tree->num_sms * 4, 256, 0, s>>>(tree->dev, tree->lru_node, tree->lru_info);
         }
         f.tok = d_q_tokens; f.n = n; f.policy = params->policy; f.k = params->k; f.score_mode = score_mode;
+        f.recip_k1 = params->k > 2 && params->k <= 4096 ? (unsigned)(((1ULL << 32) + (unsigned long long)(params->k - 2)) / (unsigned long long)(params->k - 1)) : 0u;
         f.c_num = params->c_num; f.c_den = params->c_den; f.start_tick = params->start_tick;
         f.order = d_order; f.uncached = d_uncached; f.ttft = d_ttft; f.completion = d_completion;
         f.dyn = tree->fast_dyn; f.stat = tree->fast_stat; f.key = tree->fast_key_arr; f.mem = tree->fast_mem;
