@@ -1774,20 +1774,53 @@ __global__ void lru_parklist_kernel(FastArgs A) {
     A.leaf_run[node] = make_int2(A.n + i, lo - i);
 }
 
-// after the sort by hash: runs of equal hashes are the groups
-__global__ void fast_group_kernel(FastArgs A) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= A.n) return;
-    const long long h = A.gh[i];
-    int32_t lo = 0, hi = i;                    // first index with gh >= h
-    while (lo < hi) { const int32_t mid = (lo + hi) >> 1; if (A.gh[mid] < h) lo = mid + 1; else hi = mid; }
-    const int32_t first = lo;
-    lo = i + 1; hi = A.n;                      // first index with gh > h
-    while (lo < hi) { const int32_t mid = (lo + hi) >> 1; if (A.gh[mid] <= h) lo = mid + 1; else hi = mid; }
-    const int32_t r = A.gidx[i];
-    A.mem[i] = r;
-    st_dyn_group(A.dyn + r, first, lo - first);
-    if (lo - first > 1) atomicOr(A.gbits + (r >> 5), 1u << (r & 31));
+// The groups the loop starts from: slots with equal hashes, side by side in the member array (in any order).  A hash table
+// counts them -- nothing needs them sorted, which took eight launches and 94 us for 32,768 slots, the three kernels take 20:
+// every slot finds its entry and its number there, one slot per entry takes room in the member array, and every slot
+// writes itself down.
+struct GroupTable { unsigned long long* key; int32_t* cnt; int32_t* off; unsigned mask; int32_t* ent; int32_t* num; unsigned int* used; };
+__global__ void group_count_kernel(FastArgs A, GroupTable H) {
+    const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = r < A.n;
+    unsigned e = 0;
+    if (in) {
+        const unsigned long long h = (unsigned long long)A.gh[r];              // 62 bits
+        const unsigned long long key = h + 1;                                  // 0: empty entry
+        e = (unsigned)(h ^ (h >> 31)) & H.mask;
+        for (unsigned probes = 0; probes <= H.mask; ++probes) {                // (at most half full: an entry is found)
+            const unsigned long long old = atomicCAS(H.key + e, 0ULL, key);
+            if (old == 0ULL || old == key) break;
+            e = (e + 1) & H.mask;
+        }
+    }
+    const int lane = threadIdx.x & 31;
+    const unsigned same = __match_any_sync(FULL_MASK, in ? e : 0xffffffffu);
+    const int lead = __ffs(same) - 1;
+    int32_t at = 0;
+    if (in && lane == lead) at = atomicAdd(H.cnt + e, __popc(same));
+    at = __shfl_sync(FULL_MASK, at, lead) + __popc(same & ((1u << lane) - 1u));
+    if (in) { H.ent[r] = (int32_t)e; H.num[r] = at; }
+}
+__global__ void group_room_kernel(FastArgs A, GroupTable H) {
+    const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const bool first = r < A.n && H.num[r] == 0;
+    const int32_t e = first ? H.ent[r] : 0, cnt = first ? H.cnt[e] : 0;
+    int32_t inc = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const int32_t o = __shfl_up_sync(FULL_MASK, inc, d); if (lane >= d) inc += o; }
+    unsigned base = 0;
+    if (lane == 31 && inc > 0) base = atomicAdd(H.used, (unsigned)inc);
+    base = __shfl_sync(FULL_MASK, base, 31);
+    if (first) H.off[e] = (int32_t)base + inc - cnt;
+}
+__global__ void fast_group_kernel(FastArgs A, GroupTable H) {
+    const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= A.n) return;
+    const int32_t e = H.ent[r], first = H.off[e], cnt = H.cnt[e];
+    A.mem[first + H.num[r]] = r;
+    st_dyn_group(A.dyn + r, first, cnt);
+    if (cnt > 1) atomicOr(A.gbits + (r >> 5), 1u << (r & 31));
 }
 
 // Overlaps inside the groups the loop starts from, worked out by the whole chip before the one CTA of the loop needs them.
@@ -4426,6 +4459,37 @@ bulk_rounds_kernel(TreeDev T, BulkArgs A, BulkSync* g, long long n_total, const 
     }
 }
 
+// Several arrays copied by one launch, 16 bytes at a time (every allocation of the library has room for the last, partial
+// unit).  A rollback was eleven copies of their own, about 2 us each on a small tree.
+#define KLPM_COPY_MAX 12
+struct CopyList { int4* dst[KLPM_COPY_MAX]; const int4* src[KLPM_COPY_MAX]; long long end[KLPM_COPY_MAX]; int32_t n; };      // end: running sum of 16-byte units
+__global__ void __launch_bounds__(512)
+copy_list_kernel(CopyList L) {
+    const long long step = (long long)gridDim.x * blockDim.x;
+    if (L.end[L.n - 1] <= 4 * step) {                       // a small tree: all arrays at once, one latency
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < L.end[L.n - 1]; i += step) {
+            int32_t a = 0;
+            while (i >= L.end[a]) ++a;
+            const long long at = i - (a > 0 ? L.end[a - 1] : 0);
+            L.dst[a][at] = __ldcs(L.src[a] + at);
+        }
+        return;
+    }
+    long long begin = 0;
+    for (int32_t a = 0; a < L.n; ++a) {                     // every array is spread over the whole grid
+        const long long len = L.end[a] - begin;
+        const int4* __restrict__ src = L.src[a];
+        int4* __restrict__ dst = L.dst[a];
+        long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        for (; i + 3 * step < len; i += 4 * step) {
+            const int4 v0 = __ldcs(src + i), v1 = __ldcs(src + i + step), v2 = __ldcs(src + i + 2 * step), v3 = __ldcs(src + i + 3 * step);
+            dst[i] = v0; dst[i + step] = v1; dst[i + 2 * step] = v2; dst[i + 3 * step] = v3;
+        }
+        for (; i < len; i += step) dst[i] = __ldcs(src + i);
+        begin = L.end[a];
+    }
+}
+
 __global__ void bulk_iota_kernel(int32_t* p, int32_t n) {
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) p[i] = i;
@@ -4894,11 +4958,14 @@ __global__ void lru_sum_order_kernel(const int64_t* __restrict__ off, const int3
 }
 
 // slot order: bitonic sort of (arrival, index) pairs, padded to a power of two
-__global__ void rank_init_kernel(const int64_t* __restrict__ arrival, int32_t n, long long np2, long long* key, int32_t* idx) {
+// *unsorted (cleared by the host side): set if the arrivals are not in order yet -- queues mostly are, and their sort then
+// has nothing to do.
+__global__ void rank_init_kernel(const int64_t* __restrict__ arrival, int32_t n, long long np2, long long* key, int32_t* idx, unsigned int* unsorted) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= np2) return;
     key[i] = i < n ? arrival[i] : 0x7fffffffffffffffLL;
     idx[i] = i < n ? (int32_t)i : 0x7fffffff;
+    if (i + 1 < n && arrival[i] > arrival[i + 1]) *unsorted = 1u;
 }
 __global__ void slot_arrays_kernel(const int32_t* __restrict__ ord, const int64_t* __restrict__ off, int32_t n, long long* soff, int32_t* slen) {
     int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -4919,7 +4986,8 @@ __global__ void prio_rank_kernel(const int32_t* __restrict__ pinv, int32_t n, in
     int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r < n) prank[pinv[r]] = r;
 }
-__global__ void bitonic_step_kernel(long long* key, int32_t* idx, long long np2, long long k, long long j) {
+__global__ void bitonic_step_kernel(long long* key, int32_t* idx, long long np2, long long k, long long j, const unsigned int* needed) {
+    if (needed && !*needed) return;
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= np2) return;
     long long l = i ^ j;
@@ -4934,7 +5002,8 @@ __global__ void bitonic_step_kernel(long long* key, int32_t* idx, long long np2,
 
 // Two steps of one stage in one pass (partner distances j and j / 2): a thread holds the four entries that differ in
 // those two bits.
-__global__ void bitonic_step2_kernel(long long* key, int32_t* idx, long long np2, long long k, long long j) {
+__global__ void bitonic_step2_kernel(long long* key, int32_t* idx, long long np2, long long k, long long j, const unsigned int* needed) {
+    if (needed && !*needed) return;
     const long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= (np2 >> 2)) return;
     const long long j2 = j >> 1;
@@ -4959,7 +5028,8 @@ __global__ void bitonic_step2_kernel(long long* key, int32_t* idx, long long np2
 // tile) of the one stage k_lo = k_hi.
 #define KLPM_SORT_TILE 4096
 __global__ void __launch_bounds__(1024)
-bitonic_tile_kernel(long long* key, int32_t* idx, long long np2, long long k_lo, long long k_hi) {
+bitonic_tile_kernel(long long* key, int32_t* idx, long long np2, long long k_lo, long long k_hi, const unsigned int* needed) {
+    if (needed && !*needed) return;
     __shared__ long long sk[KLPM_SORT_TILE];
     __shared__ int32_t si[KLPM_SORT_TILE];
     const int T = np2 < KLPM_SORT_TILE ? (int)np2 : KLPM_SORT_TILE;
@@ -4983,17 +5053,17 @@ bitonic_tile_kernel(long long* key, int32_t* idx, long long np2, long long k_lo,
     for (int u = threadIdx.x; u < T; u += blockDim.x) { key[base + u] = sk[u]; idx[base + u] = si[u]; }
 }
 
-// (key, idx) pairs ascending by key, then idx; np2 a power of two
-void sort_pairs(long long* key, int32_t* idx, long long np2, cudaStream_t s) {
+// (key, idx) pairs ascending by key, then idx; np2 a power of two.  `needed` (nullable, device): 0 = they are in order already
+void sort_pairs(long long* key, int32_t* idx, long long np2, cudaStream_t s, const unsigned int* needed = nullptr) {
     const long long T = np2 < KLPM_SORT_TILE ? np2 : KLPM_SORT_TILE;
     const unsigned tiles = (unsigned)(np2 / T), blocks = (unsigned)((np2 + 255) / 256);
     const unsigned blocks4 = (unsigned)(((np2 >> 2) + 255) / 256);
-    if (T >= 2) bitonic_tile_kernel<<<tiles, 1024, 0, s>>>(key, idx, np2, 2, T);
+    if (T >= 2) bitonic_tile_kernel<<<tiles, 1024, 0, s>>>(key, idx, np2, 2, T, needed);
     for (long long k = T << 1; k <= np2; k <<= 1) {
         long long j = k >> 1;
-        for (; (j >> 1) >= T; j >>= 2) bitonic_step2_kernel<<<blocks4, 256, 0, s>>>(key, idx, np2, k, j);
-        if (j >= T) bitonic_step_kernel<<<blocks, 256, 0, s>>>(key, idx, np2, k, j);
-        bitonic_tile_kernel<<<tiles, 1024, 0, s>>>(key, idx, np2, k, k);
+        for (; (j >> 1) >= T; j >>= 2) bitonic_step2_kernel<<<blocks4, 256, 0, s>>>(key, idx, np2, k, j, needed);
+        if (j >= T) bitonic_step_kernel<<<blocks, 256, 0, s>>>(key, idx, np2, k, j, needed);
+        bitonic_tile_kernel<<<tiles, 1024, 0, s>>>(key, idx, np2, k, k, needed);
     }
 }
 
@@ -5021,11 +5091,12 @@ struct rt_tree {
     long long run_cap;      // slots allocated (power of two)
     long long* run_key; int32_t* run_ord; int32_t* run_m; int32_t* run_hint; long long* run_pos;
     long long* run_soff; int32_t* run_slen; int32_t* run_ntok;
+    unsigned int* run_unsorted;
     long long* run_pkey; int32_t* run_pinv; int32_t* run_prank;
     unsigned long long* run_partial; RunBcast* run_bc; RunSync* run_sy;
     // scratch of the grouped loop (trees without a budget)
     long long fast_cap;     // slots allocated (power of two)
-    int4* fast_lcp;
+    int4* fast_lcp; unsigned long long* grp_key; int32_t* grp_cnt;
     FDyn* fast_dyn; FStat* fast_stat; unsigned long long* fast_key_arr; int32_t* fast_mem;
     long long* fast_gh; int32_t* fast_gidx; unsigned int* fast_done; unsigned long long* fast_counter;
     long long* fast_lk; int32_t* fast_ls;
@@ -5067,7 +5138,7 @@ void free_tree(rt_tree* t) {
     cudaFree(d.parent); cudaFree(d.depth_start); cudaFree(d.span_len); cudaFree(d.nchild); cudaFree(d.first_tok);
     cudaFree(t->ck_first_tok);
     cudaFree(d.span_off); cudaFree(d.last_access); cudaFree(d.dead); cudaFree(d.clock_owner);
-    cudaFree(d.table); cudaFree(d.pool); cudaFree(d.end_node); cudaFree(d.st); cudaFree(t->match_counter);
+    cudaFree(d.table); cudaFree(d.pool); cudaFree(d.end_node); cudaFree(d.st); cudaFree(t->match_counter); cudaFree(t->run_unsorted);
     cudaFree(t->match_perm); cudaFree(t->match_bucket); cudaFree(t->match_hist); cudaFree(t->own_state);
     cudaFree(t->run_key); cudaFree(t->run_ord); cudaFree(t->run_m); cudaFree(t->run_hint);
     cudaFree(t->run_pos); cudaFree(t->run_soff); cudaFree(t->run_slen); cudaFree(t->run_ntok);
@@ -5075,7 +5146,7 @@ void free_tree(rt_tree* t) {
     cudaFree(t->run_partial); cudaFree(t->run_bc); cudaFree(t->run_sy);
     cudaFree(t->fast_dyn); cudaFree(t->fast_stat); cudaFree(t->fast_key_arr); cudaFree(t->fast_mem);
     cudaFree(t->fast_gh); cudaFree(t->fast_gidx); cudaFree(t->fast_done); cudaFree(t->fast_counter);
-    cudaFree(t->fast_lk); cudaFree(t->fast_ls); cudaFree(t->fast_lcp); cudaFree(t->fast_post); cudaFree(t->fast_bsum);
+    cudaFree(t->fast_lk); cudaFree(t->fast_ls); cudaFree(t->fast_lcp); cudaFree(t->grp_key); cudaFree(t->grp_cnt); cudaFree(t->fast_post); cudaFree(t->fast_bsum);
     cudaFree(t->lru_parked); cudaFree(t->lru_info); cudaFree(t->lru_hintc); cudaFree(t->lru_leaf_run); cudaFree(t->lru_node); cudaFree(t->replay_info);
     cudaFree(t->claim);
     cudaFree(t->bulk_pend_a); cudaFree(t->bulk_pend_b); cudaFree(t->bulk_pm); cudaFree(t->bulk_pnode); cudaFree(t->bulk_poff);
@@ -5120,7 +5191,8 @@ rt_status ensure_fast_scratch(rt_tree* t, long long n) {
     cudaFree(t->fast_dyn); cudaFree(t->fast_stat); cudaFree(t->fast_key_arr); cudaFree(t->fast_mem);
     cudaFree(t->fast_gh); cudaFree(t->fast_gidx); cudaFree(t->fast_done); cudaFree(t->fast_counter);
     cudaFree(t->fast_lk); cudaFree(t->fast_ls); cudaFree(t->fast_lcp);
-    t->fast_lcp = nullptr;
+    cudaFree(t->grp_key); cudaFree(t->grp_cnt);
+    t->fast_lcp = nullptr; t->grp_key = nullptr; t->grp_cnt = nullptr;
     t->fast_lk = nullptr; t->fast_ls = nullptr;
     t->fast_dyn = nullptr; t->fast_stat = nullptr; t->fast_key_arr = nullptr; t->fast_mem = nullptr;
     t->fast_gh = nullptr; t->fast_gidx = nullptr; t->fast_done = nullptr; t->fast_counter = nullptr;
@@ -5137,6 +5209,8 @@ rt_status ensure_fast_scratch(rt_tree* t, long long n) {
     if ((s = dalloc(&t->fast_done, 3 * (np2 / 32 + 32)))) return s;     // processed bitmap, grouped bitmap, passed-over bitmap
     if ((s = dalloc(&t->fast_lk, np2))) return s;
     if ((s = dalloc(&t->fast_lcp, np2))) return s;
+    if ((s = dalloc(&t->grp_key, 2 * np2))) return s;
+    if ((s = dalloc(&t->grp_cnt, 4 * np2 + 1))) return s;
     if ((s = dalloc(&t->fast_ls, np2))) return s;
     if (!t->fast_post && (s = dalloc(&t->fast_post, 1))) return s;
     if (!t->fast_bsum && (s = dalloc(&t->fast_bsum, 1024))) return s;
@@ -5298,7 +5372,7 @@ rt_status rt_create(const rt_config* cfg, rt_tree** out) {
         (s = dalloc(&d.dead, d.max_nodes)) || (s = dalloc(&d.clock_owner, d.max_clock)) ||
         (s = dalloc(&d.table, cap)) || (s = dalloc(&d.pool, d.max_pool)) || (s = dalloc(&d.st, 1)) ||
         (s = dalloc(&d.end_node, d.max_pool)) ||
-        (s = dalloc(&t->match_counter, 1)) || (s = dalloc(&t->run_partial, 1024)) || (s = dalloc(&t->run_bc, 1)) || (s = dalloc(&t->run_sy, 1)) ||
+        (s = dalloc(&t->match_counter, 1)) || (s = dalloc(&t->run_unsorted, 1)) || (s = dalloc(&t->run_partial, 1024)) || (s = dalloc(&t->run_bc, 1)) || (s = dalloc(&t->run_sy, 1)) ||
         (s = dalloc(&t->claim, d.max_nodes))) {
         free_tree(t);
         return s;
@@ -5442,6 +5516,37 @@ rt_status rt_clone(rt_tree* tree, void* stream, rt_tree** out) {
     return RT_OK;
 }
 
+// Everything a later call can modify, from the tree to its checkpoint or back.
+static rt_status copy_checkpoint(rt_tree* t, bool back, cudaStream_t s) {
+    TreeDev& d = t->dev;
+    const size_t cap = (size_t)d.table_mask + 1, nodes = (size_t)d.max_nodes;
+    CopyList L;
+    L.n = 0;
+    long long total = 0;
+    auto add = [&](void* tree_side, void* kept, size_t bytes) {
+        L.dst[L.n] = reinterpret_cast<int4*>(back ? tree_side : kept);
+        L.src[L.n] = reinterpret_cast<const int4*>(back ? kept : tree_side);
+        total += (long long)((bytes + 15) / 16);
+        L.end[L.n++] = total;
+    };
+    add(d.table, t->ck_table, cap * sizeof(Entry));
+    add(d.parent, t->ck_parent, nodes * sizeof(int32_t));
+    add(d.depth_start, t->ck_depth_start, nodes * sizeof(int32_t));
+    add(d.span_len, t->ck_span_len, nodes * sizeof(int32_t));
+    add(d.nchild, t->ck_nchild, nodes * sizeof(int32_t));
+    add(d.first_tok, t->ck_first_tok, nodes * sizeof(int32_t));
+    add(d.span_off, t->ck_span_off, nodes * sizeof(int64_t));
+    add(d.last_access, t->ck_last_access, nodes * sizeof(int64_t));
+    add(d.dead, t->ck_dead, nodes);
+    add(d.clock_owner, t->ck_clock_owner, (size_t)d.max_clock * sizeof(int32_t));
+    add(d.st, t->ck_st, sizeof(TreeState));
+    long long blocks = (total + 512 * 4 - 1) / (512 * 4);
+    if (blocks > (long long)t->num_sms * 4) blocks = (long long)t->num_sms * 4;
+    copy_list_kernel<<<(unsigned)blocks, 512, 0, s>>>(L);
+    CK(cudaGetLastError());
+    return RT_OK;
+}
+
 rt_status rt_checkpoint(rt_tree* tree, void* stream) {
     if (!tree) return RT_ERR_INVALID;
     TreeDev& d = tree->dev;
@@ -5457,18 +5562,7 @@ rt_status rt_checkpoint(rt_tree* tree, void* stream) {
     }
     cudaStream_t st = (cudaStream_t)stream;
     tree->last_stream = st;
-    const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-    CK(cudaMemcpyAsync(tree->ck_parent, d.parent, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_depth_start, d.depth_start, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_span_len, d.span_len, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_nchild, d.nchild, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_first_tok, d.first_tok, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_span_off, d.span_off, d.max_nodes * sizeof(int64_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_last_access, d.last_access, d.max_nodes * sizeof(int64_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_dead, d.dead, d.max_nodes, k, st));
-    CK(cudaMemcpyAsync(tree->ck_clock_owner, d.clock_owner, d.max_clock * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(tree->ck_table, d.table, cap * sizeof(Entry), k, st));
-    CK(cudaMemcpyAsync(tree->ck_st, d.st, sizeof(TreeState), k, st));
+    if ((s = copy_checkpoint(tree, false, st))) return s;
     tree->ck_valid = true;
     return RT_OK;
 }
@@ -5476,23 +5570,9 @@ rt_status rt_checkpoint(rt_tree* tree, void* stream) {
 rt_status rt_rollback(rt_tree* tree, void* stream) {
     if (!tree || !tree->ck_valid) return RT_ERR_INVALID;
     tree->version++;
-    TreeDev& d = tree->dev;
-    const unsigned long long cap = d.table_mask + 1;
     cudaStream_t st = (cudaStream_t)stream;
     tree->last_stream = st;
-    const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-    CK(cudaMemcpyAsync(d.parent, tree->ck_parent, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(d.depth_start, tree->ck_depth_start, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(d.span_len, tree->ck_span_len, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(d.nchild, tree->ck_nchild, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(d.first_tok, tree->ck_first_tok, d.max_nodes * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(d.span_off, tree->ck_span_off, d.max_nodes * sizeof(int64_t), k, st));
-    CK(cudaMemcpyAsync(d.last_access, tree->ck_last_access, d.max_nodes * sizeof(int64_t), k, st));
-    CK(cudaMemcpyAsync(d.dead, tree->ck_dead, d.max_nodes, k, st));
-    CK(cudaMemcpyAsync(d.clock_owner, tree->ck_clock_owner, d.max_clock * sizeof(int32_t), k, st));
-    CK(cudaMemcpyAsync(d.table, tree->ck_table, cap * sizeof(Entry), k, st));
-    CK(cudaMemcpyAsync(d.st, tree->ck_st, sizeof(TreeState), k, st));
-    return RT_OK;
+    return copy_checkpoint(tree, true, st);
 }
 
 rt_status rt_status_detail(rt_tree* tree, int32_t* detail) {
@@ -5681,9 +5761,10 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         CK(cudaGetLastError());
     } else {
         unsigned blocks = (unsigned)((np2 + 255) / 256);
-        rank_init_kernel<<<blocks, 256, 0, s>>>(d_arrival, n, np2, tree->run_key, tree->run_ord);
-        sort_pairs(tree->run_key, tree->run_ord, np2, s);
-        slot_arrays_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tree->run_ord, d_q_offsets, n, tree->run_soff, tree->run_slen);
+        CK(cudaMemsetAsync(tree->run_unsorted, 0, sizeof(unsigned int), s));
+        rank_init_kernel<<<blocks, 256, 0, s>>>(d_arrival, n, np2, tree->run_key, tree->run_ord, tree->run_unsorted);
+        sort_pairs(tree->run_key, tree->run_ord, np2, s, tree->run_unsorted);
+        if (!grouped) slot_arrays_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tree->run_ord, d_q_offsets, n, tree->run_soff, tree->run_slen);
         if (score_mode == 1) hit_rate_guard_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d_q_offsets, n, tree->dev.st);
         if (d_tie_priority) {        // rank of every slot by (priority, slot)
             prio_init_kernel<<<blocks, 256, 0, s>>>(d_tie_priority, tree->run_ord, n, np2, tree->run_pkey, tree->run_pinv);
@@ -5791,8 +5872,14 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         const unsigned nblk = (unsigned)((n + 255) / 256), pblk = (unsigned)((np2 + 255) / 256);
         CK(cudaMemsetAsync(f.done, 0, (size_t)(3 * (np2 / 32 + 32)) * sizeof(unsigned int), s));
         // groups: queries whose match ends at the same position and continues with the same token
-        sort_pairs(f.gh, f.gidx, np2, s);
-        fast_group_kernel<<<nblk, 256, 0, s>>>(f);
+        GroupTable H;
+        H.key = tree->grp_key; H.cnt = tree->grp_cnt; H.off = tree->grp_cnt + 2 * np2; H.used = reinterpret_cast<unsigned int*>(tree->grp_cnt + 4 * np2);
+        H.mask = (unsigned)(2 * np2 - 1); H.ent = tree->run_slen; H.num = tree->run_m;
+        CK(cudaMemsetAsync(H.key, 0, (size_t)(2 * np2) * sizeof(unsigned long long), s));
+        CK(cudaMemsetAsync(tree->grp_cnt, 0, (size_t)(4 * np2 + 1) * sizeof(int32_t), s));
+        group_count_kernel<<<nblk, 256, 0, s>>>(f, H);
+        group_room_kernel<<<nblk, 256, 0, s>>>(f, H);
+        fast_group_kernel<<<nblk, 256, 0, s>>>(f, H);
         {   // one prompt per warp while that keeps every warp resident, up to 32 beyond
             long long per = (long long)n / ((long long)tree->num_sms * 32);
             per = per < 1 ? 1 : per > 32 ? 32 : per;
