@@ -799,15 +799,14 @@ match_wide_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* __
 }
 
 // ------------------------------------------------------------------------------------------------
-// sequential processing of prompts by one CTA: rt_insert and klpm_replay
+// sequential processing of prompts by one CTA: rt_insert, and klpm_replay in its plain form (debug setting run_one_by_one)
 // ------------------------------------------------------------------------------------------------
 struct SeqArgs {
     const int32_t* tok; const int64_t* off; const int64_t* arrival; const int32_t* order;
     int32_t n;                       // prompts to process
     int32_t n_queries;               // prompts in the CSR arrays: entries of `order` must be below this
     long long c_num, c_den, start_tick;
-    int32_t* new_tokens;             // rt_insert: indexed by position
-    int32_t* uncached; int64_t* ttft; int64_t* completion;   // replay: indexed by query
+    int32_t* uncached; int64_t* ttft; int64_t* completion;   // indexed by query
 };
 
 __global__ void __launch_bounds__(1024)
@@ -835,7 +834,6 @@ sequential_kernel(TreeDev T, SeqArgs A) {
                 insert_serial(T, x, len, t.m, t.node, &s_out);
                 if (s_out.ok) {
                     int32_t unc = len - t.m;
-                    if (A.new_tokens) A.new_tokens[k] = unc;
                     if (A.uncached) {
                         long long tj = __ldg(A.arrival + j);
                         long long begin = now > tj ? now : tj;
@@ -854,6 +852,186 @@ sequential_kernel(TreeDev T, SeqArgs A) {
         for (int32_t i = threadIdx.x; i < unc; i += blockDim.x) dst[i] = __ldg(x + m + i);
         __threadfence();
         __syncthreads();
+    }
+}
+
+// rt_insert one prompt after the other (a budget, or per-prompt results asked for).  Every prompt has been matched against
+// the tree as it was before the call (pm, pnode: match length, node), all of them at once; warp 0 then goes through the
+// prompts.  The match as it is now follows from that one without comparing its tokens again: walk up from the node while
+// it has been cut above the match or evicted (an evicted node takes its tokens along), and look for a child only where
+// the match ends on a node boundary.  The insertion is insert_serial with the warp's lanes side by side: the three hash
+// probes at once, 32 clock values per look for the least recently used leaf (kept in registers from prompt to prompt, as
+// in lru_tree_warp).  The other warps copy a prompt's new tokens while warp 0 is at the next one.
+// What bounds it: the chain of L2 round trips per prompt.  16 prompts into a full cache: 57 us (3.5 us a prompt;
+// one thread that walked from the root, probed and scanned the clock one value at a time took 131).
+struct InsertArgs { const int32_t* tok; const int64_t* off; int32_t n; int32_t* new_tokens; const int32_t* pm; const int32_t* pnode; };
+
+__device__ __forceinline__ long long probe_for(const TreeDev& T, unsigned long long key, bool find, Entry* e, long long not_this) {
+    unsigned long long slot = hash_key(key) & T.table_mask;
+    for (unsigned long long probes = 0; probes <= T.table_mask; ++probes) {
+        *e = ld_entry<false>(T.table + slot);
+        if ((long long)slot != not_this) {
+            if (e->key == key) return (long long)slot;
+            if (e->key == 0ULL) return find ? -1 : (long long)slot;
+        }
+        slot = (slot + 1) & T.table_mask;
+    }
+    return -1;
+}
+
+__global__ void __launch_bounds__(512)
+insert_seq_kernel(TreeDev T, InsertArgs A) {
+    __shared__ long long s_dst; __shared__ int32_t s_m, s_unc, s_ok;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    TreeState st = *T.st;
+    long long wbase = st.lru_cursor, wend = wbase;          // the window of clock values (see lru_tree_warp)
+    int32_t wv = 0;
+    bool wok = false;
+    if (threadIdx.x == 0) s_ok = 1;
+    __syncthreads();
+    for (int32_t k = 0; k < A.n; ++k) {
+        const int64_t lo = __ldg(A.off + k), hi = __ldg(A.off + k + 1);
+        if (hi < lo || hi - lo > 0x7fffffffLL) {            // (uniform over the CTA)
+            if (threadIdx.x == 0) set_status(T.st, RT_ERR_INVALID, 108);
+            break;
+        }
+        const int32_t len = (int32_t)(hi - lo);
+        const int32_t* x = A.tok + lo;
+        int32_t m = 0, a = 0;
+        if (warp == 0) {
+            m = __ldcg(A.pm + k); a = __ldcg(A.pnode + k);
+            while (a != 0) {
+                const int32_t ds = T.depth_start[a];
+                if (T.dead[a]) { if (ds < m) m = ds; }
+                else if (m > ds) break;
+                a = T.parent[a];
+            }
+        }
+        __syncthreads();                                    // the tokens of the prompt before are in the pool
+        if (warp == 0) {
+            int32_t ds = T.depth_start[a], sl = T.span_len[a];
+            int32_t o = a == 0 ? 0 : m - ds;
+            if (a == 0 || o == sl) {                        // on a node boundary: another child may continue there now
+                const Term t = walk<false>(T, x, len, a, m);
+                if (t.m > m) { m = t.m; a = t.node; ds = T.depth_start[a]; sl = T.span_len[a]; o = m - ds; }
+            }
+            const int32_t unc = len - m;
+            bool ok = true;
+            long long dst = 0;
+            int32_t copy = 0;
+            if (st.clock + 1 >= T.max_clock || st.n_nodes + 2 > T.max_nodes) { if (lane == 0) set_status(T.st, RT_ERR_CAPACITY); ok = false; }
+            else {
+                const long long clock = ++st.clock;
+                const bool cut = a != 0 && o < sl;
+                const int32_t par = T.parent[a];
+                const long long so = T.span_off[a], la = T.last_access[a];
+                const int32_t u = (int32_t)st.n_nodes;
+                const int32_t end = cut ? u : a;
+                int32_t ft = 0, pt = 0, xm = 0;
+                if (cut) { ft = __ldcg(T.pool + so); pt = __ldcg(T.pool + so + o); }
+                if (unc > 0) xm = __ldg(x + m);
+                // lane 0: the entry of the edge that is cut; lane 1: where its lower part goes; lane 2: where the leaf goes
+                Entry e; e.key = 0; e.child = 0; e.span_len = 0; e.span_off = 0; e.chain_end = 0;
+                const unsigned long long key = lane == 0 ? make_key(par, ft) : lane == 1 ? make_key(u, pt) : make_key(end, xm);
+                long long slot = -1;
+                if ((lane < 2 && cut) || (lane == 2 && unc > 0)) slot = probe_for(T, key, lane == 0, &e, -1);
+                __syncwarp();
+                const long long s1 = __shfl_sync(FULL_MASK, slot, 1), s2 = __shfl_sync(FULL_MASK, slot, 2);
+                if (lane == 2 && cut && unc > 0 && s1 == s2 && s1 >= 0) slot = probe_for(T, key, false, &e, s1);
+                __syncwarp();
+                if (cut) {
+                    ++st.n_nodes; ++st.live_nodes;
+                    const long long ce = __shfl_sync(FULL_MASK, slot >= 0 ? (long long)e.chain_end : (long long)(so + sl), 0);
+                    if (lane == 0) {
+                        if (slot >= 0) { T.table[slot].child = u; T.table[slot].span_len = o; }
+                        else set_status(T.st, RT_ERR_LIMIT, 101);
+                        T.parent[u] = par; T.depth_start[u] = ds; T.span_off[u] = so; T.span_len[u] = o;
+                        T.nchild[u] = 1; T.dead[u] = 0; T.last_access[u] = la; T.first_tok[u] = ft; T.first_tok[a] = pt;
+                        T.span_off[a] = so + o; T.span_len[a] = sl - o; T.depth_start[a] = ds + o; T.parent[a] = u;
+                        T.end_node[so + o - 1] = u;
+                    }
+                    if (lane == 1) {
+                        if (slot >= 0) {
+                            Entry* d = T.table + slot;
+                            d->child = a; d->span_len = sl - o; d->span_off = so + o; d->chain_end = ce; d->key = key;
+                        } else set_status(T.st, RT_ERR_CAPACITY);
+                    }
+                }
+                if (end != 0 && lane == 0) { T.last_access[end] = clock; T.clock_owner[clock] = end; }
+                if (wv == end) wok = false;
+                __syncwarp();
+                while (T.budget > 0 && st.tokens_live + unc > T.budget) {
+                    unsigned okm = __ballot_sync(FULL_MASK, wok);
+                    while (!okm && wend < clock) {          // the next 32 clock values
+                        wbase = wend;
+                        const long long cc = wbase + lane;
+                        wv = cc < clock ? T.clock_owner[cc] : 0;
+                        wend = wbase + 32 < clock ? wbase + 32 : clock;
+                        wok = wv > 0 && wv != end && !T.dead[wv] && T.last_access[wv] == cc && T.nchild[wv] == 0;
+                        okm = __ballot_sync(FULL_MASK, wok);
+                    }
+                    if (!okm) { if (lane == 0) set_status(T.st, RT_ERR_BUDGET); ok = false; break; }
+                    const int src = __ffs(okm) - 1;
+                    const int32_t v = __shfl_sync(FULL_MASK, wv, src);
+                    const long long stamp = wbase + src;
+                    const int32_t P = T.parent[v], vl = T.span_len[v], vt = T.first_tok[v];
+                    Entry ve;
+                    const long long vs = probe_for(T, make_key(P, vt), true, &ve, -1);
+                    const int32_t nc = T.nchild[P] - 1;
+                    long long pl = T.last_access[P];
+                    __syncwarp();
+                    const bool hand = P != 0 && stamp >= pl;
+                    if (hand) pl = stamp;
+                    if (lane == 0) {
+                        T.dead[v] = 1;
+                        if (vs >= 0) T.table[vs].child = -1;
+                        T.nchild[P] = nc;
+                        if (hand) { T.last_access[P] = stamp; T.clock_owner[stamp] = P; }
+                    }
+                    if (lane == src) wok = false;
+                    if (nc == 0 && P != 0 && P != end && pl >= wbase && pl < wend && lane == (int)(pl - wbase)) { wv = P; wok = true; }
+                    st.tokens_live -= vl; --st.live_nodes; ++st.evictions;
+                    __syncwarp();
+                }
+                if (ok && unc > 0) {
+                    const long long ls = __shfl_sync(FULL_MASK, slot, 2);
+                    if (st.pool_used + unc + 6 > T.max_pool || ls < 0) { if (lane == 0) set_status(T.st, RT_ERR_CAPACITY); ok = false; }
+                    else {
+                        const int32_t leaf = (int32_t)st.n_nodes++;
+                        const long long off = ((st.pool_used + 3) & ~3LL) + (m & 3);      // span_off = depth_start (mod 4)
+                        st.pool_used = off + unc;
+                        ++st.live_nodes; st.tokens_live += unc;
+                        if (lane == 2) {
+                            Entry* d = T.table + slot;
+                            d->child = leaf; d->span_len = unc; d->span_off = off; d->chain_end = off + unc; d->key = key;
+                        }
+                        if (lane == 0) {
+                            T.parent[leaf] = end; T.depth_start[leaf] = m; T.span_off[leaf] = off; T.span_len[leaf] = unc;
+                            T.nchild[leaf] = 0; T.dead[leaf] = 0; T.last_access[leaf] = clock; T.first_tok[leaf] = xm;
+                            T.clock_owner[clock] = leaf;
+                            T.nchild[end] = T.nchild[end] + 1;
+                            T.end_node[off + unc - 1] = leaf;
+                        }
+                        dst = off; copy = unc;
+                    }
+                }
+                if (ok && A.new_tokens && lane == 0) A.new_tokens[k] = unc;
+            }
+            __syncwarp();
+            if (lane == 0) { s_dst = dst; s_m = m; s_unc = copy; s_ok = ok ? 1 : 0; }
+        }
+        __syncthreads();
+        if (!s_ok) break;
+        if (warp > 0) {
+            int32_t* d = T.pool + s_dst;
+            const int32_t mm = s_m, cnt = s_unc;
+            for (int32_t i = threadIdx.x - 32; i < cnt; i += blockDim.x - 32) d[i] = __ldg(x + mm + i);
+        }
+    }
+    if (threadIdx.x == 0) {                                 // the counters go back (a status recorded meanwhile stays)
+        TreeState* S = T.st;
+        S->n_nodes = st.n_nodes; S->pool_used = st.pool_used; S->tokens_live = st.tokens_live; S->live_nodes = st.live_nodes;
+        S->clock = st.clock; S->lru_cursor = wbase; S->evictions = st.evictions;
     }
 }
 
@@ -5424,11 +5602,16 @@ rt_status rt_insert(rt_tree* tree, const int32_t* d_tokens, const int64_t* d_off
         tree->last_stream = (cudaStream_t)stream;
         return bulk_insert(tree, d_tokens, d_offsets, n, (cudaStream_t)stream);
     }
-    SeqArgs a;
-    memset(&a, 0, sizeof(a));
-    a.tok = d_tokens; a.off = d_offsets; a.n = n; a.n_queries = n; a.new_tokens = d_new_tokens; a.c_den = 1;
-    tree->last_stream = (cudaStream_t)stream;
-    sequential_kernel<<<1, 1024, 0, (cudaStream_t)stream>>>(tree->dev, a);
+    // one after the other: all matched at once against the tree as it is, then inserted in order
+    cudaStream_t s = (cudaStream_t)stream;
+    tree->last_stream = s;
+    rt_status st = ensure_bulk_scratch(tree, n);
+    if (st) return st;
+    st = launch_match(tree, d_tokens, d_offsets, n, tree->bulk_pm, tree->bulk_pnode, nullptr, nullptr, 0ULL, s);
+    if (st) return st;
+    InsertArgs a;
+    a.tok = d_tokens; a.off = d_offsets; a.n = n; a.new_tokens = d_new_tokens; a.pm = tree->bulk_pm; a.pnode = tree->bulk_pnode;
+    insert_seq_kernel<<<1, 512, 0, s>>>(tree->dev, a);
     CK(cudaGetLastError());
     return RT_OK;
 }

@@ -108,3 +108,46 @@ def test_selection_on_both_sides_of_the_one_cta_kernel(K, n):
         idx = np.nonzero(waiting.numpy())[0]
         best = sorted(idx.tolist(), key=lambda i: (-int(m[i]), int(t[i]), i))[:64]
         assert out.tolist() == best + [-1] * (64 - len(best))
+
+
+@pytest.mark.parametrize("budget", [0, 300, 900])
+@pytest.mark.parametrize("batch", [1, 7, 100])
+def test_insert_in_order_with_results(K, budget, batch):
+    """Prompts stored one after the other in calls of several sizes: prompts of one call that extend, cut and repeat each other, leaves
+    (and then their parents) evicted between a prompt's match and its turn, empty and fully cached prompts."""
+    prompts, _ = W.random_small_queue(77 + batch, 300, vocab=2, max_len=30)
+    more, _ = W.random_small_queue(78, 100, vocab=3, max_len=120)
+    prompts = [p for pair in zip(prompts, more * 3) for p in pair]
+    prompts += prompts[10:60] + [[]] + [p + [1, 1, 0] for p in prompts[20:40]]
+    pt, po = W.to_csr(prompts)
+    n = len(prompts)
+    tree = K.rt_create(max_nodes=2 * n + 16, max_pool_tokens=pt.numel() + 8 * n + 16, budget_tokens=budget, max_clock=n + 16)
+    new = torch.full((n,), -7, dtype=torch.int32, device="cuda")
+    tok, off = pt.cuda(), po.cuda()
+    for a in range(0, n, batch):
+        b = min(n, a + batch)
+        K.rt_insert(tree, tok, off[a:b + 1], new[a:b])
+    assert K.rt_sync_status(tree) == 0
+    ot = oracle.OracleTree(budget)
+    assert np.array_equal(new.cpu().numpy(), ot.insert(pt.numpy(), po.numpy()))
+    st, want = K.rt_stats(tree), ot.stats()
+    for key in ("n_nodes", "tokens", "clock", "evictions"):
+        assert st[key] == want[key], key
+    qs, _ = W.random_small_queue(79, 200, vocab=2, max_len=40)
+    qt, qo = W.to_csr(qs + prompts)
+    m, at = (torch.zeros(len(qs) + n, dtype=torch.int32, device="cuda") for _ in range(2))
+    K.rt_match_batch(tree, qt.cuda(), qo.cuda(), m, None, at)
+    want_m, want_at, _ = ot.match_pos(qt.numpy(), qo.numpy())
+    assert np.array_equal(m.cpu().numpy(), want_m) and np.array_equal(at.cpu().numpy(), want_at)
+    # the loop goes on from the tree that the insertions left
+    if budget:
+        k = 40
+        o = [torch.zeros(k, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64)]
+        q1, q2 = W.to_csr(prompts[:k])
+        tree2 = K.rt_create(max_nodes=2 * (n + k) + 16, max_pool_tokens=pt.numel() + q1.numel() + 8 * (n + k) + 2 * budget + 64, budget_tokens=budget, max_clock=n + k + 16)
+        K.rt_insert(tree2, tok, off, new)
+        K.klpm_run(tree2, q1.cuda(), q2.cuda(), torch.zeros(k, dtype=torch.int64, device="cuda"), K.make_params(K.POLICY_KLPM, 3), *o)
+        assert K.rt_sync_status(tree2) == 0
+        wo, wu, wt, _ = oracle.schedule(q1.numpy(), q2.numpy(), np.zeros(k, dtype=np.int64), oracle.POLICY_KLPM, 3, 0, 1, 0, oracle.CACHE_TREE,
+                                        oracle.TIER_REMATCH, ot)
+        assert np.array_equal(o[0].cpu().numpy(), wo) and np.array_equal(o[1].cpu().numpy(), wu) and np.array_equal(o[2].cpu().numpy(), wt)
