@@ -2402,8 +2402,8 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     {   // as many decisions as those entries allow: the largest x with x - f(x) <= avail, every thread trying four values
         const int32_t hi = n - c < most_ ? n - c : most_;
         int32_t best = 0;
-#pragma unroll 1
-        for (int r = 1; r <= per; ++r) { const int32_t x = tid * per + r; if (x <= hi && x - f(x) <= avail) best = x; }
+#pragma unroll
+        for (int r = 1; r <= 4; ++r) { const int32_t x = tid * per + r; if (r <= per && x <= hi && x - f(x) <= avail) best = x; }
         best = __reduce_max_sync(FULL_MASK, best);
         if ((tid & 31) == 0 && best > 0) atomicMax(&io->B0, best);
     }
@@ -5276,7 +5276,7 @@ struct rt_tree {
     long long fast_cap;     // slots allocated (power of two)
     int4* fast_lcp; unsigned long long* grp_key; int32_t* grp_cnt;
     FDyn* fast_dyn; FStat* fast_stat; unsigned long long* fast_key_arr; int32_t* fast_mem;
-    long long* fast_gh; int32_t* fast_gidx; unsigned int* fast_done; unsigned long long* fast_counter;
+    long long* fast_gh; int32_t* fast_gidx; unsigned int* fast_done;
     long long* fast_lk; int32_t* fast_ls;
     FastPost* fast_post; ChargeFn* fast_bsum;
     long long fast_mem_cap;  // entries of fast_mem
@@ -5285,6 +5285,7 @@ struct rt_tree {
     int2* lru_leaf_run; LNode* lru_node;
     ReplayInfo* replay_info;
     int run_path;           // which loop the last klpm_run took: 0 none yet, 1 one by one, 2 grouped
+    void *run_slab, *fast_slab, *bulk_slab;   // the allocations behind the run_*, fast_* / grp_* and bulk_p* arrays
     int num_sms;
     int32_t* claim;         // bulk insertion: per-node claim words (0x7fffffff when idle)
     long long bulk_cap;     // bulk insertion: prompts its per-prompt scratch holds
@@ -5318,46 +5319,42 @@ void free_tree(rt_tree* t) {
     cudaFree(d.span_off); cudaFree(d.last_access); cudaFree(d.dead); cudaFree(d.clock_owner);
     cudaFree(d.table); cudaFree(d.pool); cudaFree(d.end_node); cudaFree(d.st); cudaFree(t->match_counter); cudaFree(t->run_unsorted);
     cudaFree(t->match_perm); cudaFree(t->match_bucket); cudaFree(t->match_hist); cudaFree(t->own_state);
-    cudaFree(t->run_key); cudaFree(t->run_ord); cudaFree(t->run_m); cudaFree(t->run_hint);
-    cudaFree(t->run_pos); cudaFree(t->run_soff); cudaFree(t->run_slen); cudaFree(t->run_ntok);
-    cudaFree(t->run_pkey); cudaFree(t->run_pinv); cudaFree(t->run_prank);
     cudaFree(t->run_partial); cudaFree(t->run_bc); cudaFree(t->run_sy);
-    cudaFree(t->fast_dyn); cudaFree(t->fast_stat); cudaFree(t->fast_key_arr); cudaFree(t->fast_mem);
-    cudaFree(t->fast_gh); cudaFree(t->fast_gidx); cudaFree(t->fast_done); cudaFree(t->fast_counter);
-    cudaFree(t->fast_lk); cudaFree(t->fast_ls); cudaFree(t->fast_lcp); cudaFree(t->grp_key); cudaFree(t->grp_cnt); cudaFree(t->fast_post); cudaFree(t->fast_bsum);
     cudaFree(t->lru_parked); cudaFree(t->lru_info); cudaFree(t->lru_hintc); cudaFree(t->lru_leaf_run); cudaFree(t->lru_node); cudaFree(t->replay_info);
     cudaFree(t->claim);
-    cudaFree(t->bulk_pend_a); cudaFree(t->bulk_pend_b); cudaFree(t->bulk_pm); cudaFree(t->bulk_pnode); cudaFree(t->bulk_poff);
     cudaFree(t->bulk_sync);
     cudaFree(t->ck_parent); cudaFree(t->ck_depth_start); cudaFree(t->ck_span_len); cudaFree(t->ck_nchild);
     cudaFree(t->ck_clock_owner); cudaFree(t->ck_span_off); cudaFree(t->ck_last_access); cudaFree(t->ck_dead);
     cudaFree(t->ck_table); cudaFree(t->ck_st);
+    cudaFree(t->run_slab); cudaFree(t->fast_slab); cudaFree(t->bulk_slab);
     delete t;
+}
+
+// One allocation for several arrays (an allocation takes 0.1 ms and more on a full device, and a first call needs thirty
+// arrays).  Every part starts on a 256-byte boundary and has 256 bytes to spare.
+struct SlabPart { void** p; size_t bytes; };
+template <typename P> SlabPart slab_part(P** p, long long count) { SlabPart s; s.p = reinterpret_cast<void**>(p); s.bytes = (size_t)count * sizeof(P); return s; }
+rt_status slab_alloc(void** slab, const SlabPart* parts, int n) {
+    cudaFree(*slab);
+    *slab = nullptr;
+    size_t total = 0;
+    for (int i = 0; i < n; ++i) { *parts[i].p = nullptr; total += ((parts[i].bytes + 255) & ~(size_t)255) + 256; }
+    CK(cudaMalloc(slab, total));
+    char* at = (char*)*slab;
+    for (int i = 0; i < n; ++i) { *parts[i].p = at; at += ((parts[i].bytes + 255) & ~(size_t)255) + 256; }
+    return RT_OK;
 }
 
 rt_status ensure_run_scratch(rt_tree* t, long long n) {
     long long np2 = 1;
     while (np2 < n) np2 <<= 1;
     if (np2 <= t->run_cap) return RT_OK;
-    cudaFree(t->run_key); cudaFree(t->run_ord); cudaFree(t->run_m); cudaFree(t->run_hint);
-    cudaFree(t->run_pos); cudaFree(t->run_soff); cudaFree(t->run_slen); cudaFree(t->run_ntok);
-    cudaFree(t->run_pkey); cudaFree(t->run_pinv); cudaFree(t->run_prank);
-    t->run_ntok = nullptr; t->run_pkey = nullptr; t->run_pinv = nullptr; t->run_prank = nullptr;
-    t->run_key = nullptr; t->run_ord = nullptr; t->run_m = nullptr; t->run_hint = nullptr; t->run_pos = nullptr;
-    t->run_soff = nullptr; t->run_slen = nullptr;
     t->run_cap = 0;
-    rt_status s;
-    if ((s = dalloc(&t->run_key, np2))) return s;
-    if ((s = dalloc(&t->run_ord, np2))) return s;
-    if ((s = dalloc(&t->run_m, np2))) return s;
-    if ((s = dalloc(&t->run_hint, np2))) return s;
-    if ((s = dalloc(&t->run_pos, np2))) return s;
-    if ((s = dalloc(&t->run_soff, np2))) return s;
-    if ((s = dalloc(&t->run_slen, np2))) return s;
-    if ((s = dalloc(&t->run_ntok, np2))) return s;
-    if ((s = dalloc(&t->run_pkey, np2))) return s;
-    if ((s = dalloc(&t->run_pinv, np2))) return s;
-    if ((s = dalloc(&t->run_prank, np2))) return s;
+    const SlabPart parts[] = {slab_part(&t->run_key, np2), slab_part(&t->run_ord, np2), slab_part(&t->run_m, np2), slab_part(&t->run_hint, np2),
+                              slab_part(&t->run_pos, np2), slab_part(&t->run_soff, np2), slab_part(&t->run_slen, np2), slab_part(&t->run_ntok, np2),
+                              slab_part(&t->run_pkey, np2), slab_part(&t->run_pinv, np2), slab_part(&t->run_prank, np2)};
+    const rt_status s = slab_alloc(&t->run_slab, parts, (int)(sizeof(parts) / sizeof(parts[0])));
+    if (s) return s;
     t->run_cap = np2;
     return RT_OK;
 }
@@ -5366,32 +5363,16 @@ rt_status ensure_fast_scratch(rt_tree* t, long long n) {
     long long np2 = 1;
     while (np2 < n) np2 <<= 1;
     if (np2 <= t->fast_cap) return RT_OK;
-    cudaFree(t->fast_dyn); cudaFree(t->fast_stat); cudaFree(t->fast_key_arr); cudaFree(t->fast_mem);
-    cudaFree(t->fast_gh); cudaFree(t->fast_gidx); cudaFree(t->fast_done); cudaFree(t->fast_counter);
-    cudaFree(t->fast_lk); cudaFree(t->fast_ls); cudaFree(t->fast_lcp);
-    cudaFree(t->grp_key); cudaFree(t->grp_cnt);
-    t->fast_lcp = nullptr; t->grp_key = nullptr; t->grp_cnt = nullptr;
-    t->fast_lk = nullptr; t->fast_ls = nullptr;
-    t->fast_dyn = nullptr; t->fast_stat = nullptr; t->fast_key_arr = nullptr; t->fast_mem = nullptr;
-    t->fast_gh = nullptr; t->fast_gidx = nullptr; t->fast_done = nullptr; t->fast_counter = nullptr;
     t->fast_cap = 0;
-    rt_status s;
-    if ((s = dalloc(&t->fast_dyn, np2))) return s;
-    if ((s = dalloc(&t->fast_stat, np2))) return s;
-    if ((s = dalloc(&t->fast_key_arr, np2))) return s;
     // trees with a budget: groups formed by evictions are appended behind the first n entries
     t->fast_mem_cap = t->cfg.budget_tokens > 0 ? np2 + (8 * np2 > (1LL << 20) ? 8 * np2 : (1LL << 20)) : np2;
-    if ((s = dalloc(&t->fast_mem, t->fast_mem_cap))) return s;
-    if ((s = dalloc(&t->fast_gh, np2))) return s;
-    if ((s = dalloc(&t->fast_gidx, np2))) return s;
-    if ((s = dalloc(&t->fast_done, 3 * (np2 / 32 + 32)))) return s;     // processed bitmap, grouped bitmap, passed-over bitmap
-    if ((s = dalloc(&t->fast_lk, np2))) return s;
-    if ((s = dalloc(&t->fast_lcp, np2))) return s;
-    if ((s = dalloc(&t->grp_key, 2 * np2))) return s;
-    if ((s = dalloc(&t->grp_cnt, 4 * np2 + 1))) return s;
-    if ((s = dalloc(&t->fast_ls, np2))) return s;
-    if (!t->fast_post && (s = dalloc(&t->fast_post, 1))) return s;
-    if (!t->fast_bsum && (s = dalloc(&t->fast_bsum, 1024))) return s;
+    const SlabPart parts[] = {slab_part(&t->fast_dyn, np2), slab_part(&t->fast_stat, np2), slab_part(&t->fast_key_arr, np2),
+                              slab_part(&t->fast_mem, t->fast_mem_cap), slab_part(&t->fast_gh, np2), slab_part(&t->fast_gidx, np2),
+                              slab_part(&t->fast_done, 3 * (np2 / 32 + 32)),      // processed bitmap, grouped bitmap, passed-over bitmap
+                              slab_part(&t->fast_lk, np2), slab_part(&t->fast_ls, np2), slab_part(&t->fast_lcp, np2), slab_part(&t->grp_key, 2 * np2),
+                              slab_part(&t->grp_cnt, 4 * np2 + 1), slab_part(&t->fast_post, 1), slab_part(&t->fast_bsum, 1024)};
+    const rt_status s = slab_alloc(&t->fast_slab, parts, (int)(sizeof(parts) / sizeof(parts[0])));
+    if (s) return s;
     t->fast_cap = np2;
     return RT_OK;
 }
@@ -5417,11 +5398,10 @@ StaticSelectScratch* g_select_static_addr[64] = {nullptr};   // device address o
 rt_status ensure_bulk_scratch(rt_tree* t, int32_t n) {
     rt_status st = RT_OK;
     if (n > t->bulk_cap) {                     // per-prompt scratch, kept for later calls
-        cudaFree(t->bulk_pend_a); cudaFree(t->bulk_pend_b); cudaFree(t->bulk_pm); cudaFree(t->bulk_pnode); cudaFree(t->bulk_poff);
-        t->bulk_pend_a = t->bulk_pend_b = t->bulk_pm = t->bulk_pnode = t->bulk_poff = nullptr;
         t->bulk_cap = 0;
-        if ((st = dalloc(&t->bulk_pend_a, n)) || (st = dalloc(&t->bulk_pend_b, n)) || (st = dalloc(&t->bulk_pm, n)) ||
-            (st = dalloc(&t->bulk_pnode, n)) || (st = dalloc(&t->bulk_poff, n))) return st;
+        const SlabPart parts[] = {slab_part(&t->bulk_pend_a, n), slab_part(&t->bulk_pend_b, n), slab_part(&t->bulk_pm, n), slab_part(&t->bulk_pnode, n),
+                                  slab_part(&t->bulk_poff, n)};
+        if ((st = slab_alloc(&t->bulk_slab, parts, (int)(sizeof(parts) / sizeof(parts[0]))))) return st;
         t->bulk_cap = n;
     }
     if (!t->bulk_sync && (st = dalloc(&t->bulk_sync, 1))) return st;        // list lengths, work counter, grid barrier
