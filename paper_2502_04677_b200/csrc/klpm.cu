@@ -1770,6 +1770,7 @@ struct FastArgs {
     FDyn* dyn; FStat* stat;
     unsigned long long* key;      // slot -> key it has (or will have once arrived); 0 once processed
     int32_t* mem;                 // member array
+    const long long* sorted_t;    // per slot: arrival, side by side
     int4* lcp;                    // per slot: how far its prompt agrees with a reference prompt (see lcp_kernel)
     const int32_t* pinv;          // rank -> slot, or null
     long long* gh; int32_t* gidx; // group hashes and slots (sorted before the loop; scratch for large groups inside it)
@@ -1792,7 +1793,6 @@ struct FastArgs {
     int32_t mem_cap;              // entries of the member array (groups formed by evictions are appended behind the first n)
     TreeDev T;
     LNode* node;                  // the tree's node arrays, one record per node, while the loop runs
-    const long long* sorted_t;    // per slot: arrival, side by side
     int32_t* parked;              // per node: unprocessed slots whose hint is that node
     int32_t* hintc;               // per slot: the hint once more, side by side (what the scan after an eviction reads)
     int2* leaf_run;               // per node: the member run that holds every slot whose hint is that node (y < 0: no such run is known)
@@ -3133,45 +3133,52 @@ fast_run_kernel(FastArgs A) {
     if (A.list_mode && __ldg(&A.stat[n - 1].t) <= now) { admitted = n; next_t = INF; }
 
     // ================================================================ arrivals pending: one careful step per decision
+    long long tw = INF;                                     // 32 coming arrivals (lane i: slot wb + i)
+    int32_t wb = 0;
+    if (admitted < n) { tw = lane < n ? __ldg(A.sorted_t + lane) : INF; next_t = __shfl_sync(FULL_MASK, tw, 0); }
     while (c < n && !failed && !(A.list_mode && admitted == n)) {
         // ---- time and arrivals: idle until somebody has arrived, then admit everybody who has
         if (head == admitted && next_t > now) now = next_t;
-        if (next_t <= now) {
-            int32_t a1 = admitted;
-            {
-                const long long r = (long long)a1 + lane;
-                const bool in = r < n && __ldg(&A.stat[r].t) <= now;
-                const unsigned bal = __ballot_sync(FULL_MASK, in);
-                const int cnt = bal == FULL_MASK ? 32 : __ffs(~bal) - 1;
-                a1 += cnt;
-                if (cnt == 32 && a1 < n) {                 // a full window: gallop, then bisect (lane 0)
-                    long long lo = a1, hi = n;
-                    if (lane == 0 && __ldg(&A.stat[lo].t) <= now) {
-                        long long step = 1;
-                        ++lo;
-                        while (lo + step <= hi && __ldg(&A.stat[lo + step - 1].t) <= now) { lo += step; step <<= 1; }
-                        if (lo + step < hi) hi = lo + step;
-                        while (lo < hi) { const long long mid = (lo + hi) >> 1; if (__ldg(&A.stat[mid].t) <= now) lo = mid + 1; else hi = mid; }
-                    }
-                    a1 = (int32_t)__shfl_sync(FULL_MASK, lo, 0);
+        while (next_t <= now) {
+            const int off = admitted - wb;
+            const int cnt = __popc(__ballot_sync(FULL_MASK, lane >= off && tw <= now));      // (arrivals are sorted; past the end: INF)
+            const int32_t a1 = admitted + cnt, ra = wb + lane;
+            if (off + cnt == 32 && a1 + 64 < n && __ldg(A.sorted_t + a1 + 64) <= now) {
+                // a crowd: gallop, then bisect (lane 0), and the whole CTA admits them
+                long long lo = a1 + 65, hi = n;
+                if (lane == 0) {
+                    long long step = 1;
+                    while (lo + step <= hi && __ldg(A.sorted_t + lo + step - 1) <= now) { lo += step; step <<= 1; }
+                    if (lo + step < hi) hi = lo + step;
+                    while (lo < hi) { const long long mid = (lo + hi) >> 1; if (__ldg(A.sorted_t + mid) <= now) lo = mid + 1; else hi = mid; }
                 }
-            }
-            if (a1 - admitted <= 32) {
-                const int32_t r = admitted + lane;
-                if (r < a1) atomicMax(R.t1 + (r >> A.lb_shift), __ldcg(A.key + r));
-                __syncwarp();
-                root = tour_update(R, admitted >> A.lb_shift, lane);
-                if (((a1 - 1) >> A.lb_shift) != (admitted >> A.lb_shift)) root = tour_update(R, (a1 - 1) >> A.lb_shift, lane);
-            } else {
-                if (lane == 0) { s_job.type = FAST_JOB_ADMIT; s_job.a0 = admitted; s_job.a1 = a1; }
+                const int32_t all = (int32_t)__shfl_sync(FULL_MASK, lo, 0);
+                if (lane == 0) { s_job.type = FAST_JOB_ADMIT; s_job.a0 = admitted; s_job.a1 = all; }
                 __syncwarp();
                 named_bar(1, KLPM_FAST_THREADS);
                 const FastJob J = s_job;
                 fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
                 root = tour_top(R, lane);
+                admitted = all;
+            } else {
+                // keys only come in: every level above takes the larger of what it holds and the newcomers (one or two leaf blocks)
+                const unsigned long long ak = ra >= admitted && ra < a1 ? __ldcg(A.key + ra) : 0ULL;
+                const int32_t b0 = admitted >> A.lb_shift, b1 = (a1 - 1) >> A.lb_shift;
+                for (int32_t bb = b0; bb <= b1; ++bb) {
+                    const unsigned long long km = warp_max64r((ra >> A.lb_shift) == bb ? ak : 0ULL);
+                    const unsigned long long p1 = R.t1[bb], p2 = R.t2[bb >> 5], p3 = R.t3[bb >> 10];
+                    __syncwarp();
+                    R.t1[bb] = km > p1 ? km : p1; R.t2[bb >> 5] = km > p2 ? km : p2; R.t3[bb >> 10] = km > p3 ? km : p3;
+                    root = km > root ? km : root;
+                    __syncwarp();
+                }
+                admitted = a1;
             }
-            admitted = a1;
-            next_t = admitted < n ? __ldg(&A.stat[admitted].t) : INF;
+            if (admitted >= wb + 32) {
+                wb = admitted;
+                tw = wb + lane < n ? __ldg(A.sorted_t + wb + lane) : INF;
+            }
+            next_t = __shfl_sync(FULL_MASK, tw, admitted - wb);
         }
         // ---- pick
         const bool fcfs_turn = A.policy == KLPM_POLICY_FCFS || (A.policy == KLPM_POLICY_KLPM && cyc == 0);
@@ -3182,16 +3189,28 @@ fast_run_kernel(FastArgs A) {
             slot = A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
         }
         if (slot < 0 || slot >= admitted || slot_done(R, A, slot)) { if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 105); failed = true; break; }   // cannot happen
-        // ---- the pick leaves its leaf block (its two records are asked for first: they travel with the block's keys)
+        // ---- the pick leaves its leaf block: its records and the block's keys travel together, the levels above are read meanwhile
+        const int32_t b = slot >> A.lb_shift, i2 = b >> 5, i3 = i2 >> 5;
+        const long long r = ((long long)b << A.lb_shift) + lane;
+        const unsigned long long kk = r < n ? __ldcg(A.key + r) : 0ULL;
         const FDyn pd = ld_dyn(A.dyn + slot);
         const FStat ps = ld_stat(A.stat + slot);
-        const int32_t b = slot >> A.lb_shift;
+        const unsigned long long x1 = lane == (b & 31) ? 0ULL : R.t1[(i2 << 5) + lane];
+        const unsigned long long x2 = lane == (i2 & 31) ? 0ULL : R.t2[(i3 << 5) + lane];
+        const unsigned long long x3 = lane == i3 ? 0ULL : R.t3[lane];
+        const unsigned long long o1 = warp_max64r(x1), o2 = warp_max64r(x2), o3 = warp_max64r(x3);
         unsigned long long bm = 0;
-        for (int32_t u = lane; u < (1 << A.lb_shift); u += 32) {
-            const long long r = ((long long)b << A.lb_shift) + u;
-            if (r < admitted && r != slot && !slot_done(R, A, r)) { const unsigned long long kk = __ldcg(A.key + r); if (kk > bm) bm = kk; }
+        if (r < admitted && r != slot && lane < (1 << A.lb_shift) && !slot_done(R, A, r)) bm = kk;
+        for (int32_t u = lane + 32; u < (1 << A.lb_shift); u += 32) {
+            const long long r2 = ((long long)b << A.lb_shift) + u;
+            if (r2 < admitted && r2 != slot && !slot_done(R, A, r2)) { const unsigned long long k2 = __ldcg(A.key + r2); if (k2 > bm) bm = k2; }
         }
-        root = tour_set(R, b, warp_max64r(bm), lane);
+        bm = warp_max64r(bm);
+        {
+            const unsigned long long v2 = bm > o1 ? bm : o1, v3 = v2 > o2 ? v2 : o2;
+            R.t1[b] = bm; R.t2[i2] = v2; R.t3[i3] = v3;     // (every lane stores the same)
+            root = v3 > o3 ? v3 : o3;
+        }
         mark_done(slot);
         careful(slot, true, pd, ps);
         if (slot == head) advance_head();
@@ -3512,7 +3531,9 @@ fast_run_kernel(FastArgs A) {
 // prepares the decision afresh.  A pick whose group has other members waits for its new leaf's id before the group is
 // dissolved.  The other warps join for work that is worth sharing; so does warp 1, which is idle then.
 // The two hand over through named barriers 2 (a job for warp 1) and 3 (its answer), helpers wait at barrier 1.
-// What bounds it: @@LRU@@
+// What bounds it: the instruction streams of the two warps (4 to 7 cycles an instruction, most of it fixed-latency
+// dependencies), no longer the L2 round trips.  120,000 queries on a cold cache with 93,000 evictions: 232 ms = 1.9 us a
+// decision (3,800 cycles); one warp doing everything took 441 ms.  12,007 on a warm cache: 32 ms (48.6).
 struct LruJob { int32_t type; int32_t hint, m, len, gstart, gcount; int32_t moved; long long vleaf; };   // moved: queries have been parked elsewhere since the last job
 struct LruAnswer { int32_t failed, scan, n_small, leaf; int32_t small_v[8]; };
 enum { LRU_JOB_EXIT = 0, LRU_JOB_STEP = 1, LRU_JOB_JOIN = 2 };
@@ -5966,7 +5987,7 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             if (!tree->lru_leaf_run && (st = dalloc(&tree->lru_leaf_run, tree->dev.max_nodes))) return st;
             f.leaf_run = tree->lru_leaf_run;
             if (!tree->lru_node && (st = dalloc(&tree->lru_node, tree->dev.max_nodes))) return st;
-            f.node = tree->lru_node; f.sorted_t = tree->run_key;
+            f.node = tree->lru_node;
             f.pk = tree->fast_lk; f.pi = tree->fast_ls;      // (the key list of list mode is not used on these trees)
             CK(cudaMemsetAsync(tree->lru_leaf_run, 0xff, (size_t)tree->dev.max_nodes * sizeof(int2), s));
             f.lru = 1; f.T = tree->dev; f.parked = tree->lru_parked; f.skip = &tree->lru_info->skip;
@@ -5984,7 +6005,7 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         f.c_num = params->c_num; f.c_den = params->c_den; f.start_tick = params->start_tick;
         f.order = d_order; f.uncached = d_uncached; f.ttft = d_ttft; f.completion = d_completion;
         f.dyn = tree->fast_dyn; f.stat = tree->fast_stat; f.key = tree->fast_key_arr; f.mem = tree->fast_mem;
-        f.lcp = tree->fast_lcp;
+        f.lcp = tree->fast_lcp; f.sorted_t = tree->run_key;
         f.pinv = d_tie_priority ? tree->run_pinv : nullptr;
         f.gh = tree->fast_gh; f.gidx = tree->fast_gidx; f.done = tree->fast_done;
         f.arrival = d_arrival; f.post = tree->fast_post;
