@@ -799,7 +799,7 @@ match_wide_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* __
 }
 
 // ------------------------------------------------------------------------------------------------
-// sequential processing of prompts by one CTA: rt_insert, and klpm_replay in its plain form (debug setting run_one_by_one)
+// sequential processing of prompts by one CTA: rt_insert and klpm_replay (its plain form, debug setting run_one_by_one)
 // ------------------------------------------------------------------------------------------------
 struct SeqArgs {
     const int32_t* tok; const int64_t* off; const int64_t* arrival; const int32_t* order;
