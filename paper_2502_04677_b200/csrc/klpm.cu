@@ -3740,9 +3740,25 @@ __device__ __forceinline__ void lru_touch_warp(const FastArgs& A, const LruTouch
     }
 }
 
+// Trees with a budget: a match of m tokens that ended in node *a or above it, as it is now: up from *a past every node
+// that has been evicted (it takes its tokens along) or cut above the match.  *a and *w: the node it ends in and its record.
+__device__ __forceinline__ int32_t lru_match_now(const FastArgs& A, int32_t m, int32_t* a, LNode* w) {
+    *w = ld_node(A.node + *a);
+    while (*a != 0) {
+        if (w->nchild < 0) { if (w->depth < m) m = w->depth; }
+        else if (m > w->depth) break;
+        *a = w->parent;
+        *w = ld_node(A.node + *a);
+    }
+    return m;
+}
+
 // Warp 0: the queries parked in leaves that the last decision evicted, when known member runs hold them all.  All leaves
 // are taken together: two of them, one above the other, send their queries to one group.  Returns false, nothing changed,
 // if more than 32 slots lose matched tokens (the caller has the CTA scan for them); *failed if there is no room.
+// Which slots lose tokens is found by the walk that moves them.  The depth of the evicted leaf alone does not tell: hints
+// stay with the lower part of an edge that is cut, so a match can end above the leaf its slot is parked in, in a node
+// that the same decision has evicted too.
 __device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTour& R, const int32_t* small_v, int n_small, int32_t admitted,
                                                  int32_t* s_memcur, unsigned long long* root, bool* failed, int lane) {
     int32_t n_fall = 0, listed = 0;
@@ -3750,11 +3766,15 @@ __device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTo
     for (int sv = 0; sv < n_small && listed > 32; ++sv) {   // (up to 32 slots in the runs: no need to count first)
         const int32_t v = small_v[sv];
         const int2 lr = __ldcg(A.leaf_run + v);
-        const int32_t ds_v = A.node[v].depth;
         for (int32_t base = 0; base < lr.y; base += 32) {
             const int32_t r = base + lane < lr.y ? __ldcg(A.mem + lr.x + base + lane) : -1;
             bool hit = r >= 0 && !slot_done(R, A, r) && __ldcg(A.hintc + r) == v;
-            if (hit) hit = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2) > ds_v;
+            if (hit) {
+                const int32_t m0 = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2);
+                int32_t a = v;
+                LNode w;
+                hit = lru_match_now(A, m0, &a, &w) != m0;
+            }
             const unsigned same = __match_any_sync(FULL_MASK, hit ? r : -1 - lane);       // a slot can be listed twice in a run
             if (hit && (int)(__ffs(same) - 1) != lane) hit = false;
             n_fall += __popc(__ballot_sync(FULL_MASK, hit));
@@ -3777,14 +3797,9 @@ __device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTo
             unsigned long long h = KLPM_FAST_NOGROUP;
             if (hit) {
                 const int32_t m0 = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2);
-                int32_t mm = m0, a = v;
-                LNode w = ld_node(A.node + a);
-                while (a != 0) {
-                    if (w.nchild < 0) { if (w.depth < mm) mm = w.depth; }
-                    else if (mm > w.depth) break;
-                    a = w.parent;
-                    w = ld_node(A.node + a);
-                }
+                int32_t a = v;
+                LNode w;
+                const int32_t mm = lru_match_now(A, m0, &a, &w);
                 st_dyn_hint(A.dyn + r, a);
                 __stcg(A.hintc + r, a);
                 atomicAdd(A.parked + a, 1);
