@@ -2226,6 +2226,7 @@ struct FastBatchIO {
     int32_t colPhi[32], colRk[32], remH[32], remE[32];
     int32_t hard;                     // out: the batch stopped before a decision that needs the one-at-a-time path
     int32_t Braw;                     // out: decisions the batch could have made (it makes none below KLPM_FAST_CTA_MIN)
+    int32_t play_max;                 // in: 0: no batch is played through; else: after how many decisions one that is dear ends
     int32_t wide;                     // in: look at as many slots and entries as the scratch holds (the last batch had many meetings)
     int32_t played;                   // out: the batch was played through decision by decision (more than 32 meetings)
     int32_t played_t, played_u;       // scratch: ranks of the last slot and the last entry taken, -1 if none
@@ -2236,6 +2237,7 @@ struct FastBatchIO {
 #define KLPM_FAST_CTA_MIN 32         // smaller batches are left to the warp-wide step (an attempt costs about 10,000 cycles)
 #endif
 #define KLPM_FAST_PLAY 48
+#define KLPM_FAST_DEAR 160            // cycles per decision above which a played batch is dear (where the orders agree it takes 45 to 100)
 #ifndef KLPM_FAST_CB_MAX
 #define KLPM_FAST_CB_MAX 32           // longest back-off (loop iterations) after CTA-wide attempts that failed
 #endif
@@ -2542,10 +2544,10 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
     }
     // More meetings than that (two orders that run side by side): the batch is played through decision by decision.  Warp 0
     // holds one bit per rank of either side (word w in lane w; the word a side is at also in a uniform register): the next
-    // rank whose bit is clear is the pick, and its slot's bit on the other side is set: about 250 cycles a decision, and
-    // far less where the two orders agree, where the one-at-a-time path takes 1,000.  A batch that gets KLPM_FAST_PLAY decisions far without it costs less that way
-    // (9,000 cycles in all).
-    const bool play = both_kinds && ncol > 32 && io->limB < KLPM_FAST_PLAY;
+    // rank whose bit is clear is the pick, and its slot's bit on the other side is set: 540 cycles a decision where every turn
+    // changes sides, 45 where the two orders agree; the one-at-a-time path takes 1,000 to 1,500.  A batch that gets KLPM_FAST_PLAY
+    // decisions far without it costs less that way (9,000 cycles in all).
+    const bool play = both_kinds && io->play_max > 0 && ncol > 32 && io->limB < KLPM_FAST_PLAY;
     if (play) {
         for (int32_t x = tid; x < nFa; x += KLPM_FAST_THREADS) sBack[x] = -1;
         __syncthreads();
@@ -2555,11 +2557,17 @@ __device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchI
             const int lane = tid;
             const int32_t capF = io->limF < nFa ? io->limF : nFa, capL = io->limL < nEa ? io->limL : nEa;
             const int32_t most = n - c < KLPM_FAST_CTA_BATCH ? n - c : KLPM_FAST_CTA_BATCH;      // (wide: both sides in sight beyond the list window)
+            const unsigned t_play = (unsigned)clock();
+            int32_t look = io->play_max;                    // where the cost so far is looked at
             unsigned mh = 0, me = 0;                        // ranks that are taken, of this lane's word
             unsigned ch = 0, ce = 0;                        // the words the two sides are at
             int32_t t = 0, u = 0, lt = -1, lu = -1, x = 0, turn = cyc;
             bool stop_f = false, stop_l = false;            // ran into the end of what is in sight, or into a limit, on which side
             for (; x < most; ++x) {
+                if (x >= look) {
+                    if ((unsigned)clock() - t_play > KLPM_FAST_DEAR * (unsigned)x) break;
+                    look = x + 64;
+                }
                 // Where both sides are at the same slot, that slot is the next pick whichever turn it is, and so on for as
                 // long as the two orders agree: up to 32 decisions at once.
                 {
@@ -3385,24 +3393,44 @@ fast_run_kernel(FastArgs A) {
         // a batch that was cut short stopped before a decision only the one-at-a-time path can take: that one comes
         // next, without another attempt that would find it again
         bool one_next = false;
+        // Is playing batches through better than what happens between CTA-wide attempts?  Where the two orders block each
+        // other that is one decision at a time, where they merely meet often it is full warp-wide steps (110 cycles a decision), and
+        // then playing can cost five times as much (1,000 queries on 64 long prefixes: 408 us, now 255).
+        // What the stretches between attempts have cost is kept (the older half fades), and what the last played batch
+        // has, its 9,000 fixed cycles spread over 128 decisions.  A dear batch ends after 128 decisions, the first one after 64,
+        // and a warp-wide step is tried after it, unless that is known to cost more than twice as much.
+        long long alt_cy = 0, alt_dec = 0, play_cpd = 0, t_out = clock64();
+        int32_t c_out = c, probe = 0, play_max = 64;
         long long iters = 0;                                // every iteration makes a decision or gives up an attempt for a while
         while (c < n && !failed) {
             if (++iters > 64LL * n + 4096) { if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 118); failed = true; break; }      // cannot happen
             // first choice: the whole CTA makes up to 1,024 decisions (the sort scratch is free between dissolves)
-            if (!one_next && cb_wait <= 0 && (calm >= KLPM_FAST_CALM || c >= calm_until) && c >= cb_until && n - c >= KLPM_FAST_CTA_MIN) {
+            if (!one_next && probe <= 0 && cb_wait <= 0 && (calm >= KLPM_FAST_CALM || c >= calm_until) && c >= cb_until && n - c >= KLPM_FAST_CTA_MIN) {
+                const long long t_cta = clock64();
+                if (c > c_out) { alt_cy += t_cta - t_out; alt_dec += c - c_out; if (alt_dec > 512) { alt_cy >>= 1; alt_dec >>= 1; } }
                 if (lane == 0) {
+                    const bool may_play = alt_dec == 0 || alt_cy > (play_cpd > 130 ? play_cpd : 130) * alt_dec;
+                    s_bio.play_max = may_play ? play_max : 0;
+                    if (!may_play) s_bio.wide = 0;
                     s_bio.per = per_now; s_bio.cur = cur; s_bio.head = head; s_bio.c = c; s_bio.cyc = cyc; s_bio.root = root; s_bio.B = 0;
                     s_job.type = FAST_JOB_BATCH;
                 }
                 __syncwarp();
-                const long long t_cta = clock64();
                 ++n_cta_try;
                 named_bar(1, KLPM_FAST_THREADS);
                 fast_batch_job<G>(A, R, &s_bio, sr, sr + 1024, sr + 2048, reinterpret_cast<int32_t*>(sh), s_scan, nwords);
                 const int32_t Bc = s_bio.B;
-                const long long cy_this = clock64() - t_cta;
+                t_out = clock64();
+                const long long cy_this = t_out - t_cta;
                 cy_cta += cy_this;
+                c_out = c + Bc;
                 if (Bc > 0) {
+                    if (s_bio.played) {
+                        play_cpd = (cy_this > 9000 ? (cy_this - 9000) / Bc : 0) + 70;
+                        const bool ahead = alt_dec >= 16 && alt_cy > 2 * play_cpd * alt_dec;      // (still the better half)
+                        play_max = ahead ? KLPM_FAST_CTA_BATCH : 128;
+                        if (play_cpd > KLPM_FAST_DEAR + 70 && !ahead) probe = 1;
+                    }
                     ++n_cta_ok; dec_cta += Bc;
                     per_now = s_bio.wide || Bc >= (per_now == 1 ? 224 : 160) ? 4 : 1;
                     const int32_t consumed = s_bio.consumed, hmax = s_bio.hmax;
@@ -3414,7 +3442,7 @@ fast_run_kernel(FastArgs A) {
                     else if (head < n && ((bm_ld(s_done, head >> 5, gdone) >> (head & 31)) & 1u)) advance_head();
                     // did it pay?  its cycles per decision against what the warp-wide steps have cost per decision so far
                     const long long warp_cpd = dec_warp >= 256 ? cy_warp / dec_warp : 100;
-                    if (s_bio.played /* the alternative is one at a time */ || cy_this <= (long long)Bc * warp_cpd) { cb_back = 8; cb_fail = 0; continue; }
+                    if (s_bio.played /* judged above */ || cy_this <= (long long)Bc * warp_cpd) { cb_back = 8; cb_fail = 0; continue; }
                     // committed, but too short to have paid for the attempt: warp-wide steps for a while, as after a failure
                     cb_wait = cb_back;
                     cb_back = cb_back < KLPM_FAST_CB_MAX ? cb_back * 2 : KLPM_FAST_CB_MAX;
@@ -3428,14 +3456,18 @@ fast_run_kernel(FastArgs A) {
                 if (cb_fail < KLPM_FAST_FAIL_CAP) ++cb_fail;
             }
             --cb_wait;
+            const bool probing = !one_next && probe > 0;
+            if (probing) --probe;
             if (!one_next && vb_wait <= 0) {
                 const int32_t c_was = c;
                 const long long t_w = clock64();
                 const bool took = try_batch();
                 cy_warp += clock64() - t_w;
-                if (took) { ++n_warp_ok; dec_warp += c - c_was; vb_back = 1; if (c - c_was == 32) ++calm; else { if (calm > 0) calm_until = c + 64; calm = 0; } one_next = tb_cut; continue; }
-                if (calm > 0) calm_until = c + 64;          // (where warp-wide steps keep failing the whole CTA may do better)
-                calm = 0;
+                if (took) { ++n_warp_ok; dec_warp += c - c_was; vb_back = 1; if (c - c_was == 32) ++calm; else if (!probing) { if (calm > 0) calm_until = c + 64; calm = 0; } one_next = tb_cut; continue; }
+                if (!probing) {
+                    if (calm > 0) calm_until = c + 64;      // (where warp-wide steps keep failing the whole CTA may do better)
+                    calm = 0;
+                }
                 vb_wait = vb_back;
                 vb_back = vb_back < 64 ? vb_back * 2 : 64;
             }

@@ -350,3 +350,26 @@ def test_long_batches_where_the_two_pick_orders_meet(K, k):
     got = run_gpu(K, prefill, prompts, arr, 2, k)
     want = run_oracle(prefill, prompts, arr, 2, k)
     same(got, want)
+
+
+@pytest.mark.parametrize("k", [4, 8])
+def test_played_batches_give_way_to_warp_wide_steps(K, k):
+    """1,000 waiting queries on long shared prefixes: the two orders meet often but rarely block each other, so warp-wide steps get to make
+    many of the decisions (a batch played through decision by decision costs five times as much here; played through, all but 84 and
+    all were).  Same results, whoever makes them."""
+    w = W.medium(seed=2, scale=1 / 8)
+    pt, po = w.prefill.materialize()
+    n = 1000
+    qt, qo = w.queries.select(torch.arange(n)).materialize()
+    arr = np.zeros(n, dtype=np.int64)
+    tree = K.rt_build(pt.cuda(), po.cuda(), max_nodes=2 * (n + w.prefill.n) + 16, max_pool_tokens=pt.numel() + qt.numel() + 8 * (n + w.prefill.n) + 16)
+    out = [torch.full((n,), -1, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64, torch.int64)]
+    K.klpm_run(tree, qt.cuda(), qo.cuda(), torch.from_numpy(arr).cuda(), K.make_params(K.POLICY_KLPM, k), *out)
+    assert K.rt_sync_status(tree) == 0
+    c = K.rt_debug_counters(tree)
+    assert c["warp_step_decisions"] >= 200, c
+    ot = oracle.OracleTree()
+    ot.insert(pt.numpy(), po.numpy())
+    want = oracle.schedule(qt.numpy(), qo.numpy(), arr, oracle.POLICY_KLPM, k, 0, 1, 0, oracle.CACHE_TREE, oracle.TIER_UPDATE, ot)
+    for g, x in zip(out, want):
+        assert np.array_equal(g.cpu().numpy(), x)
