@@ -140,9 +140,11 @@ rt_status rt_rollback(rt_tree* tree, void* stream);
 rt_status rt_sync_status(rt_tree* tree, void* stream);
 
 /* A number that says which device-side check recorded the status word (0 if none did): 101/104 a child entry
- * that should exist was not found, 102/112 a bounded wait of the scheduling loop / of the concurrent insertion ran out, 103/105/107 an internal
- * prediction did not hold, 106 a child lookup probed the whole table, 108 an order entry that is not a query
- * (or a prompt with a negative length), 109 a prompt too long for the hit-rate score.  A debugging aid;
+ * that should exist was not found, 102/112 a bounded wait of the scheduling loop / of the concurrent insertion ran out,
+ * 103/105/107/111/118 an internal prediction did not hold, 106 a child lookup probed the whole table, 108 an order entry that
+ * is not a query (or a prompt with a negative length), 109 a prompt too long for the hit-rate score, 110 a match record that is
+ * not the one expected, 113 no room for the groups of queries that fell back, 114 to 117 no room in the tree (check before the
+ * loop, tokens and child table after it), 119 an entry of a group that is not a query.  A debugging aid;
  * synchronises like rt_stats. */
 rt_status rt_status_detail(rt_tree* tree, int32_t* detail);
 

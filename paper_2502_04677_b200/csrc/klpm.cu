@@ -2179,6 +2179,14 @@ __device__ __forceinline__ void set_grouped(const FastTour& R, int32_t r, bool g
     else atomicAnd(R.gb + (r >> 5), ~(1u << (r & 31)));
 }
 
+// An entry of the member array: a slot, always.  Anything else is recorded and passed over (-1) instead of being used as an index.
+__device__ __forceinline__ int32_t ld_member(const FastArgs& A, int32_t i) {
+    const int32_t r = __ldcg(A.mem + i);
+    if ((unsigned)r < (unsigned)A.n) return r;
+    set_status(A.st, RT_ERR_LIMIT, 119);
+    return -1;
+}
+
 struct FastPick {             // the prompt being processed, as its group's members need it
     int32_t slot, m, len, ntok;
     const int32_t* x;         // its tokens
@@ -2310,7 +2318,7 @@ __device__ __forceinline__ bool dissolve_is_small(const FastPick& P) { return P.
 
 // The sequencer warp dissolves a group of at most 32 members and regroups it inside its run; returns the tournament's root.
 __device__ __forceinline__ unsigned long long dissolve_small(const FastArgs& A, const FastPick& P, const FastTour& R, unsigned long long root, int lane) {
-    const int32_t r = lane < P.gcount ? __ldcg(A.mem + P.gstart + lane) : -1;
+    const int32_t r = lane < P.gcount ? ld_member(A, P.gstart + lane) : -1;
     bool touched;
     const unsigned long long h = fast_member(A, P, R, r, lane, &touched);
     int32_t rank = 0, start = 0, cnt = 0;
@@ -2914,7 +2922,7 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
             __syncthreads();
             for (int32_t base = warp * 32; base < gc; base += nwarps * 32) {
                 const int32_t i = base + lane;
-                const int32_t r = i < gc ? __ldcg(A.mem + gs + i) : -1;
+                const int32_t r = i < gc ? ld_member(A, gs + i) : -1;
                 const bool act = r >= 0 && r != P.slot;
                 unsigned long long h = KLPM_FAST_NOGROUP;
                 if (act && !slot_done(R, A, r)) {
@@ -2968,7 +2976,7 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
         } else {
             for (int32_t base = warp * 32; base < gc; base += nwarps * 32) {
                 const int32_t i = base + lane;
-                const int32_t r = i < gc ? __ldcg(A.mem + gs + i) : -1;
+                const int32_t r = i < gc ? ld_member(A, gs + i) : -1;
                 bool touched;
                 const unsigned long long h = fast_member(A, P, R, r, lane, &touched);
                 if (i < gc) { __stcg(A.gh + i, (long long)h); __stcg(A.gidx + i, r); }
@@ -3799,7 +3807,7 @@ __device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTo
         const int32_t v = small_v[sv];
         const int2 lr = __ldcg(A.leaf_run + v);
         for (int32_t base = 0; base < lr.y; base += 32) {
-            const int32_t r = base + lane < lr.y ? __ldcg(A.mem + lr.x + base + lane) : -1;
+            const int32_t r = base + lane < lr.y ? ld_member(A, lr.x + base + lane) : -1;
             bool hit = r >= 0 && !slot_done(R, A, r) && __ldcg(A.hintc + r) == v;
             if (hit) {
                 const int32_t m0 = __ldcg(reinterpret_cast<const int32_t*>(A.dyn + r) + 2);
@@ -3821,7 +3829,7 @@ __device__ __noinline__ bool lru_fall_back_small(const FastArgs& A, const FastTo
         const int32_t v = small_v[sv];
         const int2 lr = __ldcg(A.leaf_run + v);
         for (int32_t base = 0; base < lr.y; base += 32) {
-            const int32_t r = base + lane < lr.y ? __ldcg(A.mem + lr.x + base + lane) : -1;
+            const int32_t r = base + lane < lr.y ? ld_member(A, lr.x + base + lane) : -1;
             bool hit = r >= 0 && !slot_done(R, A, r) && __ldcg(A.hintc + r) == v;
             const unsigned same = __match_any_sync(FULL_MASK, hit ? r : -1 - lane);
             if (hit && (int)(__ffs(same) - 1) != lane) hit = false;
