@@ -3155,9 +3155,9 @@ fast_run_kernel(FastArgs A) {
     while (c < n && !failed && !(A.list_mode && admitted == n)) {
         // ---- time and arrivals: idle until somebody has arrived, then admit everybody who has
         if (head == admitted && next_t > now) now = next_t;
-        while (next_t <= now) {
+        while (admitted < n && next_t <= now) {             // (an arrival can be the largest time there is, like the padding)
             const int off = admitted - wb;
-            const int cnt = __popc(__ballot_sync(FULL_MASK, lane >= off && tw <= now));      // (arrivals are sorted; past the end: INF)
+            const int cnt = __popc(__ballot_sync(FULL_MASK, lane >= off && wb + lane < n && tw <= now));      // (arrivals are sorted)
             const int32_t a1 = admitted + cnt, ra = wb + lane;
             if (off + cnt == 32 && a1 + 64 < n && __ldg(A.sorted_t + a1 + 64) <= now) {
                 // a crowd: gallop, then bisect (lane 0), and the whole CTA admits them
@@ -4047,9 +4047,9 @@ lru_run_kernel(const __grid_constant__ FastArgs A) {
         } else {
             // ---- time and arrivals: idle until somebody has arrived, then admit everybody who has
             if (head == admitted && next_t > now) now = next_t;
-            while (next_t <= now && !failed) {
+            while (admitted < n && next_t <= now && !failed) {      // (an arrival can be the largest time there is, like the padding)
                 const int off = admitted - wb;
-                const int cnt = __popc(__ballot_sync(FULL_MASK, lane >= off && tw <= now));      // (arrivals are sorted; past the end: INF)
+                const int cnt = __popc(__ballot_sync(FULL_MASK, lane >= off && wb + lane < n && tw <= now));      // (arrivals are sorted)
                 const int32_t a1 = admitted + cnt, ra = wb + lane;
                 if (off + cnt == 32 && a1 + 64 < n && __ldg(A.sorted_t + a1 + 64) <= now) {
                     // a crowd: gallop, then bisect (lane 0), and the whole CTA admits them
