@@ -864,7 +864,10 @@ sequential_kernel(TreeDev T, SeqArgs A) {
 // in lru_tree_warp).  The other warps copy a prompt's new tokens while warp 0 is at the next one.
 // What bounds it: the chain of L2 round trips per prompt.  16 prompts into a full cache: 57 us (3.5 us a prompt;
 // one thread that walked from the root, probed and scanned the clock one value at a time took 131).
-struct InsertArgs { const int32_t* tok; const int64_t* off; int32_t n; int32_t* new_tokens; const int32_t* pm; const int32_t* pnode; };
+// A long call is cut into parts of KLPM_INSERT_PART prompts, so that the matches fit memory the tree has had from the start and
+// the call allocates nothing; a part that ends early says so to the ones behind it (*stop).
+#define KLPM_INSERT_PART 1024
+struct InsertArgs { const int32_t* tok; const int64_t* off; int32_t n; int32_t* new_tokens; const int32_t* pm; const int32_t* pnode; int32_t* stop; int32_t first; };
 
 __device__ __forceinline__ long long probe_for(const TreeDev& T, unsigned long long key, bool find, Entry* e, long long not_this) {
     unsigned long long slot = hash_key(key) & T.table_mask;
@@ -883,8 +886,10 @@ __global__ void __launch_bounds__(512)
 insert_seq_kernel(TreeDev T, InsertArgs A) {
     __shared__ long long s_dst; __shared__ int32_t s_m, s_unc, s_ok;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (!A.first && __ldcg(A.stop)) return;                 // (uniform over the CTA)
     TreeState st = *T.st;
     long long wbase = st.lru_cursor, wend = wbase;          // the window of clock values (see lru_tree_warp)
+    bool bad = false;
     int32_t wv = 0;
     bool wok = false;
     if (threadIdx.x == 0) s_ok = 1;
@@ -893,6 +898,7 @@ insert_seq_kernel(TreeDev T, InsertArgs A) {
         const int64_t lo = __ldg(A.off + k), hi = __ldg(A.off + k + 1);
         if (hi < lo || hi - lo > 0x7fffffffLL) {            // (uniform over the CTA)
             if (threadIdx.x == 0) set_status(T.st, RT_ERR_INVALID, 108);
+            bad = true;
             break;
         }
         const int32_t len = (int32_t)(hi - lo);
@@ -1032,6 +1038,7 @@ insert_seq_kernel(TreeDev T, InsertArgs A) {
         TreeState* S = T.st;
         S->n_nodes = st.n_nodes; S->pool_used = st.pool_used; S->tokens_live = st.tokens_live; S->live_nodes = st.live_nodes;
         S->clock = st.clock; S->lru_cursor = wbase; S->evictions = st.evictions;
+        *A.stop = bad || !s_ok;
     }
 }
 
@@ -5363,6 +5370,7 @@ struct rt_tree {
     int run_path;           // which loop the last klpm_run took: 0 none yet, 1 one by one, 2 grouped
     void *run_slab, *fast_slab, *bulk_slab;   // the allocations behind the run_*, fast_* / grp_* and bulk_p* arrays
     int num_sms;
+    int32_t *ins_pm, *ins_pnode, *ins_stop;   // insertion in order: matches of a part (one allocation), and whether a part ended early
     int32_t* claim;         // bulk insertion: per-node claim words (0x7fffffff when idle)
     long long bulk_cap;     // bulk insertion: prompts its per-prompt scratch holds
     int32_t *bulk_pend_a, *bulk_pend_b, *bulk_pm, *bulk_pnode, *bulk_poff;
@@ -5397,7 +5405,7 @@ void free_tree(rt_tree* t) {
     cudaFree(t->match_perm); cudaFree(t->match_bucket); cudaFree(t->match_hist); cudaFree(t->own_state);
     cudaFree(t->run_partial); cudaFree(t->run_bc); cudaFree(t->run_sy);
     cudaFree(t->lru_parked); cudaFree(t->lru_info); cudaFree(t->lru_hintc); cudaFree(t->lru_leaf_run); cudaFree(t->lru_node); cudaFree(t->replay_info);
-    cudaFree(t->claim);
+    cudaFree(t->claim); cudaFree(t->ins_pm);
     cudaFree(t->bulk_sync);
     cudaFree(t->ck_parent); cudaFree(t->ck_depth_start); cudaFree(t->ck_span_len); cudaFree(t->ck_nchild);
     cudaFree(t->ck_clock_owner); cudaFree(t->ck_span_off); cudaFree(t->ck_last_access); cudaFree(t->ck_dead);
@@ -5607,10 +5615,11 @@ rt_status rt_create(const rt_config* cfg, rt_tree** out) {
         (s = dalloc(&d.table, cap)) || (s = dalloc(&d.pool, d.max_pool)) || (s = dalloc(&d.st, 1)) ||
         (s = dalloc(&d.end_node, d.max_pool)) ||
         (s = dalloc(&t->match_counter, 1)) || (s = dalloc(&t->run_unsorted, 1)) || (s = dalloc(&t->run_partial, 1024)) || (s = dalloc(&t->run_bc, 1)) || (s = dalloc(&t->run_sy, 1)) ||
-        (s = dalloc(&t->claim, d.max_nodes))) {
+        (s = dalloc(&t->ins_pm, 2 * KLPM_INSERT_PART + 1)) || (s = dalloc(&t->claim, d.max_nodes))) {
         free_tree(t);
         return s;
     }
+    t->ins_pnode = t->ins_pm + KLPM_INSERT_PART; t->ins_stop = t->ins_pnode + KLPM_INSERT_PART;
     // root: node 0, empty edge
     cudaError_t e = cudaMemset(d.table, 0, cap * sizeof(Entry));
     if (e == cudaSuccess) e = cudaMemset(d.end_node, 0xff, d.max_pool * sizeof(int32_t) + 256);
@@ -5658,17 +5667,20 @@ rt_status rt_insert(rt_tree* tree, const int32_t* d_tokens, const int64_t* d_off
         tree->last_stream = (cudaStream_t)stream;
         return bulk_insert(tree, d_tokens, d_offsets, n, (cudaStream_t)stream);
     }
-    // one after the other: all matched at once against the tree as it is, then inserted in order
+    // one after the other, a part at a time: all matched at once against the tree as it is, then inserted in order
     cudaStream_t s = (cudaStream_t)stream;
     tree->last_stream = s;
-    rt_status st = ensure_bulk_scratch(tree, n);
-    if (st) return st;
-    st = launch_match(tree, d_tokens, d_offsets, n, tree->bulk_pm, tree->bulk_pnode, nullptr, nullptr, 0ULL, s);
-    if (st) return st;
-    InsertArgs a;
-    a.tok = d_tokens; a.off = d_offsets; a.n = n; a.new_tokens = d_new_tokens; a.pm = tree->bulk_pm; a.pnode = tree->bulk_pnode;
-    insert_seq_kernel<<<1, 512, 0, s>>>(tree->dev, a);
-    CK(cudaGetLastError());
+    for (int32_t at = 0; at < n;) {
+        const int32_t part = n - at < KLPM_INSERT_PART ? n - at : KLPM_INSERT_PART;
+        const rt_status st = launch_match(tree, d_tokens, d_offsets + at, part, tree->ins_pm, tree->ins_pnode, nullptr, nullptr, 0ULL, s);
+        if (st) return st;
+        InsertArgs a;
+        a.tok = d_tokens; a.off = d_offsets + at; a.n = part; a.new_tokens = d_new_tokens ? d_new_tokens + at : nullptr;
+        a.pm = tree->ins_pm; a.pnode = tree->ins_pnode; a.stop = tree->ins_stop; a.first = at == 0;
+        insert_seq_kernel<<<1, 512, 0, s>>>(tree->dev, a);
+        CK(cudaGetLastError());
+        at += part;
+    }
     return RT_OK;
 }
 
