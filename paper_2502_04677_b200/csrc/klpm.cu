@@ -709,6 +709,9 @@ match_batch_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* _
 // contiguous pool runs (trees without a budget), otherwise hop by hop.
 // 32 queries of 1,024 to 8,192 tokens, caches cold: 10 us (match_batch_kernel 21), on a tree without a budget 12 us
 // (match_chain_kernel 33).
+// With `in_order` (1: the first part of a call, 2: a later one) the batch is about to be inserted one prompt after the other, which ends at
+// the first prompt that is not one (a negative length, or more tokens than an int32 counts): nothing from there on is
+// looked at, here either.  The insertion itself reports it.
 __device__ __forceinline__ int32_t wide_mismatch(const int32_t* __restrict__ a, const int32_t* __restrict__ b, int32_t n,
                                                  int32_t* s_min, unsigned& phase) {
     const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -733,12 +736,21 @@ __device__ __forceinline__ int32_t wide_mismatch(const int32_t* __restrict__ a, 
 template <bool CHAIN>
 __global__ void __launch_bounds__(256, 4)
 match_wide_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* __restrict__ qoff, int32_t* __restrict__ mlen,
-                  int32_t* __restrict__ tnode, int32_t* __restrict__ toff, MatchState* __restrict__ state, unsigned long long tag) {
+                  int32_t* __restrict__ tnode, int32_t* __restrict__ toff, MatchState* __restrict__ state, unsigned long long tag,
+                  int32_t in_order, const int32_t* stop) {
     __shared__ int32_t s_min[3];
     if (threadIdx.x < 3) s_min[threadIdx.x] = 0x7fffffff;
-    __syncthreads();
-    unsigned phase = 0;
     const int64_t i = blockIdx.x;
+    bool bad = false;
+    if (in_order) {
+        bad = in_order == 2 && *stop != 0;
+        for (int64_t j = threadIdx.x; j <= i; j += blockDim.x) {
+            const int64_t l = __ldg(qoff + j + 1) - __ldg(qoff + j);
+            bad = bad || l < 0 || l > 0x7fffffffLL;
+        }
+    }
+    if (__syncthreads_or(bad)) return;
+    unsigned phase = 0;
     const int64_t lo = __ldg(qoff + i);
     int64_t len64 = __ldg(qoff + i + 1) - lo;
     if (len64 < 0 || len64 > 0x7fffffffLL) { if (threadIdx.x == 0) set_status(T.st, RT_ERR_INVALID); len64 = 0; }
@@ -5534,21 +5546,23 @@ rt_status bulk_insert(rt_tree* t, const int32_t* d_tokens, const int64_t* d_offs
 //   reads the trunk from HBM again unless they are taken together.
 #define KLPM_WIDE_MAX_CHAIN 16384
 #define KLPM_WIDE_MAX_HOPS 65536
+static_assert(KLPM_INSERT_PART <= KLPM_WIDE_MAX_CHAIN && KLPM_INSERT_PART <= KLPM_WIDE_MAX_HOPS, "the parts of an insertion in order are matched by match_wide_kernel");
 std::atomic<unsigned long long> g_match_tag{0};
 
 // The batched match: the order in which the queries are taken, then the kernel.  `state` (nullable) receives the
 // per-query records, stamped with `tag`.
 rt_status launch_match(rt_tree* t, const int32_t* d_q_tokens, const int64_t* d_q_offsets, int32_t nq, int32_t* d_match_len,
-                       int32_t* d_term_node, int32_t* d_term_off, MatchState* state, unsigned long long tag, cudaStream_t s) {
+                       int32_t* d_term_node, int32_t* d_term_off, MatchState* state, unsigned long long tag, cudaStream_t s,
+                       int32_t in_order = 0) {
     if (nq <= (t->cfg.budget_tokens == 0 ? KLPM_WIDE_MAX_CHAIN : KLPM_WIDE_MAX_HOPS)) {
         // as many warps per query (a power of two, 8 at most) as leave every query of the batch resident at once
         const long long resident = (long long)t->num_sms * 32;
         int warps = 8;
         while (warps > 1 && (long long)nq * warps > resident) warps >>= 1;
         if (t->cfg.budget_tokens == 0) match_wide_kernel<true><<<(unsigned)nq, warps * 32, 0, s>>>(t->dev, d_q_tokens, d_q_offsets, d_match_len,
-                                                                                                  d_term_node, d_term_off, state, tag);
+                                                                                                  d_term_node, d_term_off, state, tag, in_order, t->ins_stop);
         else match_wide_kernel<false><<<(unsigned)nq, warps * 32, 0, s>>>(t->dev, d_q_tokens, d_q_offsets, d_match_len, d_term_node,
-                                                                          d_term_off, state, tag);
+                                                                          d_term_off, state, tag, in_order, t->ins_stop);
         CK(cudaGetLastError());
         return RT_OK;
     }
@@ -5672,7 +5686,8 @@ rt_status rt_insert(rt_tree* tree, const int32_t* d_tokens, const int64_t* d_off
     tree->last_stream = s;
     for (int32_t at = 0; at < n;) {
         const int32_t part = n - at < KLPM_INSERT_PART ? n - at : KLPM_INSERT_PART;
-        const rt_status st = launch_match(tree, d_tokens, d_offsets + at, part, tree->ins_pm, tree->ins_pnode, nullptr, nullptr, 0ULL, s);
+        const rt_status st = launch_match(tree, d_tokens, d_offsets + at, part, tree->ins_pm, tree->ins_pnode, nullptr, nullptr, 0ULL, s,
+                                          at == 0 ? 1 : 2);
         if (st) return st;
         InsertArgs a;
         a.tok = d_tokens; a.off = d_offsets + at; a.n = part; a.new_tokens = d_new_tokens ? d_new_tokens + at : nullptr;

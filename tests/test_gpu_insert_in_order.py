@@ -82,3 +82,25 @@ def test_no_room_left_in_one_of_the_parts(K, room):
     got = new.cpu().numpy()
     assert np.array_equal(got[:stored], want) and (got[stored:] == -7).all()
     same_tree(K, tree, ot, prompts)
+
+
+@pytest.mark.parametrize("budget", [0, 2000])
+@pytest.mark.parametrize("n,at", [(5, 0), (40, 17), (1500, 1023), (2600, 1030)])
+def test_offsets_that_are_not_prompts(K, budget, n, at):
+    """A prompt of negative length ends the call there: what is before it is stored, nothing behind it is looked at (its offsets may be
+    anything), and the status says which check it was."""
+    prompts = some_prompts(n)
+    pt, po = W.to_csr(prompts)
+    bad = po.clone()
+    bad[at + 1] = bad[at] - 1
+    bad[at + 2:] = torch.tensor([-5, 1 << 40, 7, -(1 << 40)], dtype=torch.int64).repeat(n)[:n - at - 1]
+    tree = K.rt_create(max_nodes=2 * n + 16, max_pool_tokens=pt.numel() + 8 * n + 16, budget_tokens=budget, max_clock=n + 16)
+    new = torch.full((n,), -7, dtype=torch.int32, device="cuda")
+    K.rt_insert(tree, pt.cuda(), bad.cuda(), new)
+    assert K.rt_sync_status(tree) == -1
+    assert K.rt_status_detail(tree) == 108
+    ot = oracle.OracleTree(budget)
+    want = ot.insert(*[x.numpy() for x in W.to_csr(prompts[:at])]) if at else np.zeros(0, dtype=np.int32)
+    got = new.cpu().numpy()
+    assert np.array_equal(got[:at], want) and (got[at:] == -7).all()
+    same_tree(K, tree, ot, prompts)

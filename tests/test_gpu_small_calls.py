@@ -151,3 +151,34 @@ def test_insert_in_order_with_results(K, budget, batch):
         wo, wu, wt, _ = oracle.schedule(q1.numpy(), q2.numpy(), np.zeros(k, dtype=np.int64), oracle.POLICY_KLPM, 3, 0, 1, 0, oracle.CACHE_TREE,
                                         oracle.TIER_REMATCH, ot)
         assert np.array_equal(o[0].cpu().numpy(), wo) and np.array_equal(o[1].cpu().numpy(), wu) and np.array_equal(o[2].cpu().numpy(), wt)
+
+
+@pytest.mark.parametrize("n,budget", [(16_385, 0), (65_537, 60_000)])
+def test_ordered_match_kernels_on_long_edges(K, n, budget):
+    """The smallest batches of the ordered kernels, one without and one with a budget: the long queries at full length at every 16-byte
+    phase between short ones, match length and where the match ended."""
+    cached, queries = long_edges()
+    ct, co = W.to_csr(cached)
+    tree = K.rt_create(max_nodes=4 * len(cached) + 16, max_pool_tokens=ct.numel() + 8 * len(cached) + 16, budget_tokens=budget,
+                       max_clock=len(cached) + 16)
+    K.rt_insert(tree, ct.cuda(), co.cuda())
+    ot = oracle.OracleTree(budget)
+    ot.insert(ct.numpy(), co.numpy())
+    short = [q[:9 + i % 7] for i, q in enumerate(queries)]
+    both = queries + short
+    which = len(queries) + np.arange(n) % len(short)
+    at_long = np.random.RandomState(4).permutation(n)[:8 * len(queries)]
+    which[at_long] = np.arange(8 * len(queries)) % len(queries)
+    flat = [torch.tensor(q, dtype=torch.int32) for q in both]
+    off = np.concatenate([[0], np.cumsum([len(both[w]) for w in which])]).astype(np.int64)
+    tok = torch.cat([flat[w] for w in which]).cuda()
+    m, node, at = (torch.full((n,), -7, dtype=torch.int32, device="cuda") for _ in range(3))
+    K.rt_match_batch(tree, tok, torch.from_numpy(off).cuda(), m, node, at)
+    assert K.rt_sync_status(tree) == 0
+    qt, qo = W.to_csr(both)
+    want_m, want_at, want_depth = (np.asarray(x)[which] for x in ot.match_pos(qt.numpy(), qo.numpy()))
+    assert np.array_equal(m.cpu().numpy(), want_m)
+    assert np.array_equal(at.cpu().numpy(), want_at)
+    assert np.array_equal((m - at).cpu().numpy(), want_depth)
+    assert np.array_equal((node == 0).cpu().numpy(), want_m == 0)
+    assert len({int(off[i]) % 4 for i in at_long}) == 4
