@@ -2027,10 +2027,12 @@ __global__ void fast_group_kernel(FastArgs A, GroupTable H) {
 // overlap in the smaller e; with equal e and different next tokens, or one of them at its end, in exactly e; otherwise
 // they agree beyond e and are compared from there (overlap_known).  That holds for any two prompts whatever happens to
 // their groups later.  A warp takes `per` consecutive entries of the member array.
+// `wanted` (null: all): per first entry of a group, whether it is looked at.  A given order (klpm_replay) that is short against the
+// queue touches few groups, and the others are never dissolved.
 // 120,000 prompts of 256 shared prefixes: 296 us, bound by the 0.9 GB of prefix tokens it compares; eight warps of the loop's
 // CTA, which did the comparing before, took 73 ms for the same (220,000 cycles per group of a shared prefix, now 44,000).
 __global__ void __launch_bounds__(256)
-lcp_kernel(FastArgs A, int32_t per) {
+lcp_kernel(FastArgs A, int32_t per, const int32_t* __restrict__ wanted) {
     const int lane = threadIdx.x & 31;
     const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long i0 = w * per;
@@ -2041,7 +2043,7 @@ lcp_kernel(FastArgs A, int32_t per) {
     if (lane < per && i < A.n) {
         r = A.mem[i];
         const FDyn d = ld_dyn(A.dyn + r);
-        if (d.gcount > 1) {
+        if (d.gcount > 1 && (!wanted || wanted[d.gstart])) {
             ref = A.mem[d.gstart];
             const FStat s = ld_stat(A.stat + r);
             m = d.m; len = s.len; soff = s.soff;
@@ -2063,6 +2065,13 @@ lcp_kernel(FastArgs A, int32_t per) {
         if (lane == src) e = x;
     }
     if (r >= 0) A.lcp[r] = make_int4(ref, e, e < len ? __ldg(A.tok + soff + e) : 0, 0);
+}
+// The groups that a given order touches (see lcp_kernel).
+__global__ void lcp_wanted_kernel(FastArgs A, int32_t* wanted) {
+    const int32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= *A.n_fixed) return;
+    const FDyn d = ld_dyn(A.dyn + A.fixed[p]);
+    if (d.gcount > 1) wanted[d.gstart] = 1;
 }
 // The overlap of two prompts as far as their records tell it: true if *e is it, false if they agree at least up to *e.
 __device__ __forceinline__ bool overlap_known(const int4& a, int32_t len_a, const int4& b, int32_t len_b, int32_t m, int32_t* e) {
@@ -6150,7 +6159,15 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             long long per = (long long)n / ((long long)tree->num_sms * 32);
             per = per < 1 ? 1 : per > 32 ? 32 : per;
             const long long warps = ((long long)n + per - 1) / per;
-            lcp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(f, (int32_t)per);
+            // An order of less than an eighth of the queue marks its groups first.  16 entries that share nothing out of 120,000
+            // queries with shared prefixes: 475 us with the marks, 785 without; from an eighth on the order's own steps cost more.
+            int32_t* wanted = nullptr;
+            if (d_fixed && n_fixed < n / 8) {
+                wanted = tree->run_hint;
+                CK(cudaMemsetAsync(wanted, 0, (size_t)n * sizeof(int32_t), s));
+                lcp_wanted_kernel<<<(unsigned)((n_fixed + 255) / 256), 256, 0, s>>>(f, wanted);
+            }
+            lcp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(f, (int32_t)per, wanted);
         }
         if (lru) {                   // per node of the tree: the slots parked in it as the loop starts
             sort_pairs(f.pk, f.pi, np2, s);
