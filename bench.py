@@ -374,11 +374,12 @@ def run_ours(args):
     # launch, a single one where their number is odd) and one tile launch
     big = max(0, lg - 12)
     sort_launches = 1 + sum((st + 1) // 2 + 1 for st in range(1, big + 1))
+    group_launches = 1 if nq <= 1024 else 3
     if run_path == K.RUN_PATH_GROUPED and w.budget_tokens > 0:
-        # bucketing + match; slot keys, arrival sort; capacity check (2), node records; slot records, slot states, groups (3),
-        # overlaps, sort by node, parked slots, the loop; node arrays, tokens of the surviving nodes, table clear, table
+        # bucketing + match; slot keys, arrival sort; capacity check (2), node records; slot records, slot states, groups,
+        # overlaps, sort by node, parked slots, the loop; node arrays (and an empty table), tokens of the surviving nodes, table
         order_launches = 3 if nq > 65536 else 0
-        launches_per_step = (order_launches + 1) + (1 + sort_launches) + 3 + (2 + 3 + 1 + sort_launches + 1 + 1) + 4
+        launches_per_step = (order_launches + 1) + (1 + sort_launches) + 3 + (2 + group_launches + 1 + sort_launches + 1 + 1) + 3
         loop_kernel = "lru_run_kernel"
         loop_note = ("all decisions in one CTA, one at a time (arrivals are pending throughout): admit, pick from a 32-ary "
                      "tournament or the oldest slot, charge, bring the tree's node arrays up to date (cut, stamp, evict the "
@@ -387,12 +388,12 @@ def run_ours(args):
                      "that are still alive are written after the loop; one warp decides while another keeps the tree")
     elif run_path == K.RUN_PATH_GROUPED:
         # match (bucketing by first token: three kernels; the match itself); slot keys, arrival sort (it ends at once where
-        # the arrivals are in order); slot records, slot states from the match records, groups (3), overlaps, key list and
+        # the arrivals are in order); slot records, slot states from the match records, groups, overlaps, key list and
         # its sort, the loop, the three charge kernels; bulk insertion of the processed prompts: claim words, pending list,
         # the first round of two kernels, the later rounds
         list_launches = 1 + sort_launches + 3                               # key list, its sort, the three charge kernels
         order_launches = 3 if nq > 16384 else 0
-        launches_per_step = (order_launches + 1) + (1 + sort_launches) + (2 + 3 + 1 + list_launches + 1) + (1 + 1 + 2 + 1)
+        launches_per_step = (order_launches + 1) + (1 + sort_launches) + (2 + group_launches + 1 + list_launches + 1) + (1 + 1 + 2 + 1)
         loop_kernel = "fast_run_kernel"
         loop_note = ("all decisions in one CTA: once everybody has arrived, longest-match picks come from a presorted list "
                      "of keys and oldest-first picks from a bitmap cursor, up to 1,024 decisions per CTA-wide batch (32 per "
@@ -401,7 +402,7 @@ def run_ours(args):
                      "from the records rt_match_batch_ex kept (no query is walked twice); the time includes the sort of the keys "
                      "and the bulk insertion of the processed prompts")
     else:
-        launches_per_step = (3 if nq >= 2048 else 0) + 1 + 1 + sort_launches + 1 + 1      # bucketing, match, slot keys, bitonic steps, slot arrays, scheduling loop
+        launches_per_step = (3 if nq > (65536 if w.budget_tokens > 0 else 16384) else 0) + 1 + 1 + sort_launches + 1 + 1      # bucketing, match, slot keys, bitonic steps, slot arrays, scheduling loop
         loop_kernel = "run_kernel"
         loop_note = "sequential chain: every pick depends on the tree after the previous one"
     ttft_cpu = ttft.cpu()

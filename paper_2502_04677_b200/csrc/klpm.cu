@@ -1976,8 +1976,7 @@ __global__ void lru_parklist_kernel(FastArgs A) {
 // every slot finds its entry and its number there, one slot per entry takes room in the member array, and every slot
 // writes itself down.
 struct GroupTable { unsigned long long* key; int32_t* cnt; int32_t* off; unsigned mask; int32_t* ent; int32_t* num; unsigned int* used; };
-__global__ void group_count_kernel(FastArgs A, GroupTable H) {
-    const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void group_count(const FastArgs& A, const GroupTable& H, int32_t r) {
     const bool in = r < A.n;
     unsigned e = 0;
     if (in) {
@@ -1998,11 +1997,10 @@ __global__ void group_count_kernel(FastArgs A, GroupTable H) {
     at = __shfl_sync(FULL_MASK, at, lead) + __popc(same & ((1u << lane) - 1u));
     if (in) { H.ent[r] = (int32_t)e; H.num[r] = at; }
 }
-__global__ void group_room_kernel(FastArgs A, GroupTable H) {
-    const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void group_room(const FastArgs& A, const GroupTable& H, int32_t r) {
     const int lane = threadIdx.x & 31;
     const bool first = r < A.n && H.num[r] == 0;
-    const int32_t e = first ? H.ent[r] : 0, cnt = first ? H.cnt[e] : 0;
+    const int32_t e = first ? H.ent[r] : 0, cnt = first ? __ldcg(H.cnt + e) : 0;
     int32_t inc = cnt;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) { const int32_t o = __shfl_up_sync(FULL_MASK, inc, d); if (lane >= d) inc += o; }
@@ -2011,13 +2009,28 @@ __global__ void group_room_kernel(FastArgs A, GroupTable H) {
     base = __shfl_sync(FULL_MASK, base, 31);
     if (first) H.off[e] = (int32_t)base + inc - cnt;
 }
-__global__ void fast_group_kernel(FastArgs A, GroupTable H) {
-    const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void group_place(const FastArgs& A, const GroupTable& H, int32_t r) {
     if (r >= A.n) return;
-    const int32_t e = H.ent[r], first = H.off[e], cnt = H.cnt[e];
+    const int32_t e = H.ent[r], first = H.off[e], cnt = __ldcg(H.cnt + e);
     A.mem[first + H.num[r]] = r;
     st_dyn_group(A.dyn + r, first, cnt);
     if (cnt > 1) atomicOr(A.gbits + (r >> 5), 1u << (r & 31));
+}
+__global__ void group_count_kernel(FastArgs A, GroupTable H) { group_count(A, H, blockIdx.x * blockDim.x + threadIdx.x); }
+__global__ void group_room_kernel(FastArgs A, GroupTable H) { group_room(A, H, blockIdx.x * blockDim.x + threadIdx.x); }
+__global__ void fast_group_kernel(FastArgs A, GroupTable H) { group_place(A, H, blockIdx.x * blockDim.x + threadIdx.x); }
+// The three, and the clearing of the table, in one launch for queues of up to a thread per slot of one CTA (four launches cost a
+// queue of one prompt on a full cache 10 of 87 us, 1,000 prompts 5 of 102).
+__global__ void __launch_bounds__(1024)
+group_small_kernel(FastArgs A, GroupTable H) {
+    for (unsigned i = threadIdx.x; i <= H.mask; i += 1024) { H.key[i] = 0ULL; H.cnt[i] = 0; }
+    if (threadIdx.x == 0) *H.used = 0u;
+    __syncthreads();
+    group_count(A, H, threadIdx.x);
+    __syncthreads();
+    group_room(A, H, threadIdx.x);
+    __syncthreads();
+    group_place(A, H, threadIdx.x);
 }
 
 // Overlaps inside the groups the loop starts from, worked out by the whole chip before the one CTA of the loop needs them.
@@ -5133,11 +5146,14 @@ lru_tokens_kernel(TreeDev T, const int32_t* __restrict__ order, const int32_t* _
     }
 }
 
-// The node arrays as records for the loop, and back.
-__global__ void lru_pack_kernel(TreeDev T, LNode* node, const LruInfo* info) {
+// Before the loop: the node arrays as records, no query parked anywhere, no member run known.  After it: the arrays from the
+// records, and the child table empty.  (One launch each: a queue of one prompt pays for every launch: 101 us on a full cache with separate clears, now 87.)
+__global__ void lru_pack_kernel(TreeDev T, LNode* node, int32_t* parked, int2* leaf_run, const LruInfo* info) {
+    const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    for (long long v = first; v < T.max_nodes; v += step) { parked[v] = 0; leaf_run[v] = make_int2(-1, -1); }
     if (info->skip) return;
-    const long long n = T.st->n_nodes, step = (long long)gridDim.x * blockDim.x;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += step) {
+    const long long n = T.st->n_nodes;
+    for (long long v = first; v < n; v += step) {
         LNode r;
         r.parent = T.parent[v]; r.depth = T.depth_start[v]; r.len = T.span_len[v]; r.nchild = T.dead[v] ? -1 : T.nchild[v];
         r.last = T.last_access[v]; r.off = T.span_off[v];
@@ -5146,24 +5162,16 @@ __global__ void lru_pack_kernel(TreeDev T, LNode* node, const LruInfo* info) {
 }
 __global__ void lru_unpack_kernel(TreeDev T, const LNode* __restrict__ node, const LruInfo* info) {
     if (info->skip) return;
-    const long long n = T.st->n_nodes, step = (long long)gridDim.x * blockDim.x;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += step) {
+    const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    const long long n = T.st->n_nodes, n16 = (long long)(T.table_mask + 1) * 2;      // (an entry is two 16-byte units)
+    for (long long v = first; v < n; v += step) {
         const LNode r = ld_node(node + v);
         T.parent[v] = r.parent; T.depth_start[v] = r.depth; T.span_len[v] = r.len; T.nchild[v] = r.nchild < 0 ? 0 : r.nchild;
         T.dead[v] = r.nchild < 0; T.last_access[v] = r.last; T.span_off[v] = r.off;
     }
-}
-
-__global__ void table_clear_kernel(TreeDev T, const LruInfo* info) {
-    if (info->skip) return;
     int4* p = reinterpret_cast<int4*>(T.table);
-    const unsigned long long n16 = (T.table_mask + 1) * 2;              // an entry is two 16-byte units
-    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (unsigned long long)gridDim.x * blockDim.x)
-        p[i] = make_int4(0, 0, 0, 0);
+    for (long long i = first; i < n16; i += step) p[i] = make_int4(0, 0, 0, 0);
 }
-
-// One thread per node: every live node's first token, the mark at the end of its edge, and its entry in the (cleared)
-// child table.
 __global__ void lru_table_kernel(TreeDev T, long long vbase, const LruInfo* info) {
     if (info->skip) return;
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -5378,7 +5386,7 @@ struct rt_tree {
     unsigned long long* run_partial; RunBcast* run_bc; RunSync* run_sy;
     // scratch of the grouped loop (trees without a budget)
     long long fast_cap;     // slots allocated (power of two)
-    int4* fast_lcp; unsigned long long* grp_key; int32_t* grp_cnt;
+    int4* fast_lcp; unsigned long long* grp_key;
     FDyn* fast_dyn; FStat* fast_stat; unsigned long long* fast_key_arr; int32_t* fast_mem;
     long long* fast_gh; int32_t* fast_gidx; unsigned int* fast_done;
     long long* fast_lk; int32_t* fast_ls;
@@ -5474,8 +5482,9 @@ rt_status ensure_fast_scratch(rt_tree* t, long long n) {
     const SlabPart parts[] = {slab_part(&t->fast_dyn, np2), slab_part(&t->fast_stat, np2), slab_part(&t->fast_key_arr, np2),
                               slab_part(&t->fast_mem, t->fast_mem_cap), slab_part(&t->fast_gh, np2), slab_part(&t->fast_gidx, np2),
                               slab_part(&t->fast_done, 3 * (np2 / 32 + 32)),      // processed bitmap, grouped bitmap, passed-over bitmap
-                              slab_part(&t->fast_lk, np2), slab_part(&t->fast_ls, np2), slab_part(&t->fast_lcp, np2), slab_part(&t->grp_key, 2 * np2),
-                              slab_part(&t->grp_cnt, 4 * np2 + 1), slab_part(&t->fast_post, 1), slab_part(&t->fast_bsum, 1024)};
+                              slab_part(&t->fast_lk, np2), slab_part(&t->fast_ls, np2), slab_part(&t->fast_lcp, np2), 
+                              slab_part(&t->grp_key, 4 * np2 + 1),                // keys, and as many counts and offsets (see run_impl)
+                              slab_part(&t->fast_post, 1), slab_part(&t->fast_bsum, 1024)};
     const rt_status s = slab_alloc(&t->fast_slab, parts, (int)(sizeof(parts) / sizeof(parts[0])));
     if (s) return s;
     t->fast_cap = np2;
@@ -6080,16 +6089,14 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             if (!tree->lru_node && (st = dalloc(&tree->lru_node, tree->dev.max_nodes))) return st;
             f.node = tree->lru_node;
             f.pk = tree->fast_lk; f.pi = tree->fast_ls;      // (the key list of list mode is not used on these trees)
-            CK(cudaMemsetAsync(tree->lru_leaf_run, 0xff, (size_t)tree->dev.max_nodes * sizeof(int2), s));
             f.lru = 1; f.T = tree->dev; f.parked = tree->lru_parked; f.skip = &tree->lru_info->skip;
             f.mem_cap = (int32_t)(tree->fast_mem_cap < 0x7fffffffLL ? tree->fast_mem_cap : 0x7fffffffLL);
             // all or nothing: is there room for whatever the loop can leave behind?
             CK(cudaMemsetAsync(tree->lru_info, 0, sizeof(LruInfo), s));
-            CK(cudaMemsetAsync(tree->lru_parked, 0, (size_t)tree->dev.max_nodes * sizeof(int32_t), s));
             if (d_fixed) lru_sum_order_kernel<<<(unsigned)((n_fixed + 255) / 256), 256, 0, s>>>(d_q_offsets, d_fixed, n_fixed, n, tree->lru_info);
             else lru_sum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d_q_offsets, n, tree->lru_info);
             lru_check_kernel<<<1, 1, 0, s>>>(tree->dev, d_fixed ? n_fixed : n, tree->lru_info);
-            lru_pack_kernel<<<(unsigned)tree->num_sms * 4, 256, 0, s>>>(tree->dev, tree->lru_node, tree->lru_info);
+            lru_pack_kernel<<<(unsigned)tree->num_sms * 8, 256, 0, s>>>(tree->dev, tree->lru_node, tree->lru_parked, tree->lru_leaf_run, tree->lru_info);
         }
         f.tok = d_q_tokens; f.n = n; f.policy = params->policy; f.k = params->k; f.score_mode = score_mode;
         f.recip_k1 = params->k > 2 && params->k <= 4096 ? (unsigned)(((1ULL << 32) + (unsigned long long)(params->k - 2)) / (unsigned long long)(params->k - 1)) : 0u;
@@ -6148,14 +6155,16 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         CK(cudaMemsetAsync(f.done, 0, (size_t)(3 * (np2 / 32 + 32)) * sizeof(unsigned int), s));
         // groups: queries whose match ends at the same position and continues with the same token
         GroupTable H;
-        H.key = tree->grp_key; H.cnt = tree->grp_cnt; H.off = tree->grp_cnt + 2 * np2; H.used = reinterpret_cast<unsigned int*>(tree->grp_cnt + 4 * np2);
+        H.key = tree->grp_key; H.cnt = reinterpret_cast<int32_t*>(H.key + 2 * np2); H.off = H.cnt + 2 * np2; H.used = reinterpret_cast<unsigned int*>(H.off + 2 * np2);
         H.mask = (unsigned)(2 * np2 - 1); H.ent = tree->run_slen; H.num = tree->run_m;
-        CK(cudaMemsetAsync(H.key, 0, (size_t)(2 * np2) * sizeof(unsigned long long), s));
-        CK(cudaMemsetAsync(tree->grp_cnt, 0, (size_t)(4 * np2 + 1) * sizeof(int32_t), s));
-        group_count_kernel<<<nblk, 256, 0, s>>>(f, H);
-        group_room_kernel<<<nblk, 256, 0, s>>>(f, H);
-        fast_group_kernel<<<nblk, 256, 0, s>>>(f, H);
-        {   // one prompt per warp while that keeps every warp resident, up to 32 beyond
+        if (n <= 1024) group_small_kernel<<<1, 1024, 0, s>>>(f, H);
+        else {
+            CK(cudaMemsetAsync(H.key, 0, (size_t)(4 * np2 + 1) * sizeof(unsigned long long), s));
+            group_count_kernel<<<nblk, 256, 0, s>>>(f, H);
+            group_room_kernel<<<nblk, 256, 0, s>>>(f, H);
+            fast_group_kernel<<<nblk, 256, 0, s>>>(f, H);
+        }
+        if (n > 1) {   // (a queue of one has no overlaps); one prompt per warp while that keeps every warp resident, up to 32 beyond
             long long per = (long long)n / ((long long)tree->num_sms * 32);
             per = per < 1 ? 1 : per > 32 ? 32 : per;
             const long long warps = ((long long)n + per - 1) / per;
@@ -6206,9 +6215,8 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         if (lru) {
             // the nodes that are alive after the loop get their tokens, and the child table is written afresh
             const TreeDev& d = tree->dev;
-            lru_unpack_kernel<<<(unsigned)tree->num_sms * 4, 256, 0, s>>>(d, tree->lru_node, tree->lru_info);
+            lru_unpack_kernel<<<(unsigned)tree->num_sms * 8, 256, 0, s>>>(d, tree->lru_node, tree->lru_info);
             lru_tokens_kernel<<<(unsigned)tree->num_sms * 8, 256, 0, s>>>(d, d_fixed ? d_fixed : d_order, d_q_tokens, d_q_offsets, f.vbase, tree->lru_info);
-            table_clear_kernel<<<(unsigned)tree->num_sms * 8, 256, 0, s>>>(d, tree->lru_info);
             lru_table_kernel<<<(unsigned)((d.max_nodes + 255) / 256), 256, 0, s>>>(d, f.vbase, tree->lru_info);
             CK(cudaGetLastError());
             return RT_OK;

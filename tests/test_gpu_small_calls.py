@@ -182,3 +182,31 @@ def test_ordered_match_kernels_on_long_edges(K, n, budget):
     assert np.array_equal((m - at).cpu().numpy(), want_depth)
     assert np.array_equal((node == 0).cpu().numpy(), want_m == 0)
     assert len({int(off[i]) % 4 for i in at_long}) == 4
+
+
+@pytest.mark.parametrize("budget", [0, 1200])
+@pytest.mark.parametrize("n", [1, 2, 33, 1023, 1024, 1025])
+def test_schedule_around_the_one_cta_set_up_of_groups(K, n, budget):
+    """Queues with groups of all sizes on both sides of the longest that one CTA groups, on a cache that holds some of them, twice."""
+    rng = np.random.RandomState(n)
+    stems = [rng.randint(0, 9, size=80).tolist() for _ in range(5)]
+    tails, _ = W.random_small_queue(n, n, vocab=2, max_len=10)
+    prompts = [(stems[i % 6][:int(rng.randint(1, 81))] if i % 6 < 5 else []) + t for i, t in enumerate(tails)]
+    prompts[0] = prompts[0] + [1]
+    qt, qo = W.to_csr(prompts)
+    arr = np.zeros(n, dtype=np.int64)
+    tree = K.rt_create(max_nodes=8 * n + 64, max_pool_tokens=4 * qt.numel() + 64 * n + 2 * budget + 64, budget_tokens=budget, max_clock=4 * n + 64)
+    ct, co = W.to_csr([s[:40] for s in stems])
+    K.rt_insert(tree, ct.cuda(), co.cuda())
+    ot = oracle.OracleTree(budget)
+    ot.insert(ct.numpy(), co.numpy())
+    for policy, k in ((K.POLICY_KLPM, 3), (K.POLICY_LPM, 1)):
+        out = [torch.full((n,), -1, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64, torch.int64)]
+        K.klpm_run(tree, qt.cuda(), qo.cuda(), torch.from_numpy(arr).cuda(), K.make_params(policy, k, 1, 3, 2), *out)
+        assert K.rt_sync_status(tree) == 0
+        want = oracle.schedule(qt.numpy(), qo.numpy(), arr, policy, k, 1, 3, 2, oracle.CACHE_TREE, oracle.TIER_REMATCH, ot)
+        for g, w in zip(out, want):
+            assert np.array_equal(g.cpu().numpy(), w)
+    st, ost = K.rt_stats(tree), ot.stats()
+    for key in ("n_nodes", "tokens", "clock", "evictions"):
+        assert st[key] == ost[key], key
