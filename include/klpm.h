@@ -82,11 +82,13 @@ rt_status rt_build(const int32_t* d_tokens, const int64_t* d_offsets, int32_t n_
  * logical clock advances by one, and (with a budget) least-recently-used leaves are evicted first to
  * make room.  d_new_tokens (nullable, int32[n]) receives |x_i| - match length at its own insertion.
  * If the device runs out of capacity the prompts before the failing one stay inserted and the tree
- * stays valid; the condition is reported by rt_sync_status.
+ * stays valid; the condition is reported by rt_sync_status.  A prompt of negative length ends the call in the same way
+ * (RT_ERR_INVALID, detail 108): nothing behind it is looked at.  This form allocates nothing.
  * When d_new_tokens is NULL, the tree has no budget and n >= 64, the prompts are inserted concurrently
  * in rounds instead (same resulting set of cached prefixes and node boundaries; node numbering may
  * differ from run to run).  The rounds run on the device (the later ones inside one cooperative kernel
- * whose grid-wide waits are bounded like every other wait); the call does not wait for them. */
+ * whose grid-wide waits are bounded like every other wait); the call does not wait for them.  The first such call for a
+ * number of prompts allocates scratch (synchronously). */
 rt_status rt_insert(rt_tree* tree, const int32_t* d_tokens, const int64_t* d_offsets, int32_t n,
                     int32_t* d_new_tokens, void* stream);
 
@@ -109,9 +111,8 @@ typedef struct { int64_t w[4]; } klpm_match_state;
  * queries.  The records are good for that one purpose while (a) the tree has not been changed by any call since
  * (rt_insert, klpm_replay, klpm_run*, rt_rollback), (b) d_q_tokens / d_q_offsets / nq are the ones passed here
  * and their contents have not changed, and (c) no later rt_match_batch_ex with a state buffer was made on this
- * tree.  On a tree with a budget the records are written but klpm_run_ex does not use them (the tree changes
- * under the loop).  Large batches (more than 16,384 queries) are taken in an order bucketed by first token, for which
- * the first such call allocates scratch (synchronously); results do not depend on the order. */
+ * tree.  Large batches (more than 16,384 queries; 65,536 on a tree with a budget) are taken in an order bucketed by first
+ * token, for which the first such call allocates scratch (synchronously); results do not depend on the order. */
 rt_status rt_match_batch_ex(rt_tree* tree, const int32_t* d_q_tokens, const int64_t* d_q_offsets, int32_t nq,
                             int32_t* d_match_len, int32_t* d_term_node, int32_t* d_term_off,
                             klpm_match_state* d_state, void* stream);
@@ -235,8 +236,8 @@ rt_status klpm_run(rt_tree* tree, const int32_t* d_q_tokens, const int64_t* d_q_
                    int32_t* d_uncached, int64_t* d_ttft, int64_t* d_completion, void* stream);
 
 /* Which loop the last klpm_run / klpm_run_ex on this tree took: 0 = none yet, 1 = one decision at a time on the
- * tree itself (trees with a budget), 2 = the grouped loop (trees without a budget; see klpm_run).  Both give the
- * same outputs.  The debug setting "run_one_by_one" makes trees without a budget take loop 1 too. */
+ * tree itself (the debug setting "run_one_by_one" only), 2 = the grouped loop (see klpm_run).  Both give the same
+ * outputs. */
 int32_t klpm_run_path(const rt_tree* tree);
 
 /* What the grouped loop of the last klpm_run / klpm_run_ex on this tree did (zeros if it has not run): out16[0] decisions

@@ -1103,7 +1103,8 @@ template <bool LPM> __device__ Cand block_best(Cand c, Cand* smem /*32*/) {
 // other.  A pick is four hardware reductions per warp (match, the two halves of the arrival, index), one barrier, and
 // the same over the warps' winners, which every warp does for itself.  No scratch in global memory, no ticket.
 // 4,001 queries (warm): the 3 best 7.3 us (select_topk_kernel 17.4, one pass over the queue per pick), one pick 7 (8.2);
-// 32 queries, one pick 2.4 us (4.4).  Longer queues are spread over CTAs.
+// 32 queries, one pick 2.4 us (4.4).  At the line, 8,192 queries, calls back to back: one pick 6.2 us (10.6), the 3 best 8.6 (18.9),
+// the 64 best 99 (255).  Longer queues do not fit the registers of one CTA; they are spread over CTAs.
 #define KLPM_SELECT_SMALL 8192
 struct PickKey { unsigned m, th, tl, idx; };      // match and arrival in a form that orders as unsigned; idx = 0xffffffff: none
 __device__ __forceinline__ PickKey warp_pick(const PickKey k) {
@@ -4837,7 +4838,7 @@ __device__ __forceinline__ int32_t first_mismatch_short(const int32_t* __restric
 //     one; with equal e and different next tokens in exactly e.  Only members that leave the pivot at the same place
 //     with the same token (`twin`, rare) still have to be compared with each other, from e on.
 // What bounds it: the issue rate (about 50 warp instructions per decision, 32 comparisons of 128 tokens); the tokens are
-// read from HBM once.  65,536 queues of 32 prompts of 128 tokens: 395 us (2.97 TB/s, 5.3 G decisions/s); two passes over
+// read from HBM once.  65,536 queues of 32 prompts of 128 tokens: 376 us (3.1 TB/s, 5.6 G decisions/s); two passes over
 // the queue and two token comparisons per decision, as longer queues still do it, took 1,482 us.
 // Every warp-wide operation below is executed by all 32 lanes: lanes beyond the queue's length take part with values
 // that never win.
