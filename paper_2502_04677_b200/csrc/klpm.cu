@@ -741,6 +741,7 @@ match_wide_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* __
     __shared__ int32_t s_min[3];
     if (threadIdx.x < 3) s_min[threadIdx.x] = 0x7fffffff;
     const int64_t i = blockIdx.x;
+    const int64_t lo = __ldg(qoff + i), hi = __ldg(qoff + i + 1);
     bool bad = false;
     if (in_order) {
         bad = in_order == 2 && *stop != 0;
@@ -751,8 +752,7 @@ match_wide_kernel(TreeDev T, const int32_t* __restrict__ qtok, const int64_t* __
     }
     if (__syncthreads_or(bad)) return;
     unsigned phase = 0;
-    const int64_t lo = __ldg(qoff + i);
-    int64_t len64 = __ldg(qoff + i + 1) - lo;
+    int64_t len64 = hi - lo;
     if (len64 < 0 || len64 > 0x7fffffffLL) { if (threadIdx.x == 0) set_status(T.st, RT_ERR_INVALID); len64 = 0; }
     const int32_t len = (int32_t)len64;
     const int32_t* q = qtok + lo;
@@ -896,21 +896,19 @@ __device__ __forceinline__ long long probe_for(const TreeDev& T, unsigned long l
 
 __global__ void __launch_bounds__(512)
 insert_seq_kernel(TreeDev T, InsertArgs A) {
-    __shared__ long long s_dst; __shared__ int32_t s_m, s_unc, s_ok;
+    __shared__ long long s_dst; __shared__ int32_t s_m, s_unc, s_ok, s_bad;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (!A.first && __ldcg(A.stop)) return;                 // (uniform over the CTA)
     TreeState st = *T.st;
     long long wbase = st.lru_cursor, wend = wbase;          // the window of clock values (see lru_tree_warp)
-    bool bad = false;
     int32_t wv = 0;
     bool wok = false;
-    if (threadIdx.x == 0) s_ok = 1;
+    if (threadIdx.x == 0) { s_ok = 1; s_bad = 0; }
     __syncthreads();
     for (int32_t k = 0; k < A.n; ++k) {
         const int64_t lo = __ldg(A.off + k), hi = __ldg(A.off + k + 1);
         if (hi < lo || hi - lo > 0x7fffffffLL) {            // (uniform over the CTA)
-            if (threadIdx.x == 0) set_status(T.st, RT_ERR_INVALID, 108);
-            bad = true;
+            if (threadIdx.x == 0) { set_status(T.st, RT_ERR_INVALID, 108); s_bad = 1; }
             break;
         }
         const int32_t len = (int32_t)(hi - lo);
@@ -1050,7 +1048,7 @@ insert_seq_kernel(TreeDev T, InsertArgs A) {
         TreeState* S = T.st;
         S->n_nodes = st.n_nodes; S->pool_used = st.pool_used; S->tokens_live = st.tokens_live; S->live_nodes = st.live_nodes;
         S->clock = st.clock; S->lru_cursor = wbase; S->evictions = st.evictions;
-        *A.stop = bad || !s_ok;
+        *A.stop = s_bad || !s_ok;
     }
 }
 
@@ -2277,6 +2275,10 @@ struct FastBatchIO {
     int32_t hard;                     // out: the batch stopped before a decision that needs the one-at-a-time path
     int32_t Braw;                     // out: decisions the batch could have made (it makes none below KLPM_FAST_CTA_MIN)
     int32_t play_max;                 // in: 0: no batch is played through; else: after how many decisions one that is dear ends
+    // kept between attempts by the sequencer's lane 0: cost and number of the decisions made between attempts, cycles per
+    // decision of the last played batch, when and at which decision the last attempt ended, the next play_max, whether to try a warp-wide step first
+    unsigned alt_cy, alt_dec, play_cpd, t_out;
+    int32_t c_out, play_next, probe;
     int32_t wide;                     // in: look at as many slots and entries as the scratch holds (the last batch had many meetings)
     int32_t played;                   // out: the batch was played through decision by decision (more than 32 meetings)
     int32_t played_t, played_u;       // scratch: ranks of the last slot and the last entry taken, -1 if none
@@ -3449,37 +3451,49 @@ fast_run_kernel(FastArgs A) {
         // What the stretches between attempts have cost is kept (the older half fades), and what the last played batch
         // has, its 9,000 fixed cycles spread over 128 decisions.  A dear batch ends after 128 decisions, the first one after 64,
         // and a warp-wide step is tried after it, unless that is known to cost more than twice as much.
-        long long alt_cy = 0, alt_dec = 0, play_cpd = 0, t_out = clock64();
-        int32_t c_out = c, probe = 0, play_max = 64;
+        int32_t probe = 0;
+        if (lane == 0) {
+            s_bio.alt_cy = 0; s_bio.alt_dec = 0; s_bio.play_cpd = 0; s_bio.t_out = (unsigned)clock();
+            s_bio.c_out = c; s_bio.play_next = 64; s_bio.probe = 0;
+        }
         long long iters = 0;                                // every iteration makes a decision or gives up an attempt for a while
         while (c < n && !failed) {
             if (++iters > 64LL * n + 4096) { if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 118); failed = true; break; }      // cannot happen
             // first choice: the whole CTA makes up to 1,024 decisions (the sort scratch is free between dissolves)
             if (!one_next && probe <= 0 && cb_wait <= 0 && (calm >= KLPM_FAST_CALM || c >= calm_until) && c >= cb_until && n - c >= KLPM_FAST_CTA_MIN) {
-                const long long t_cta = clock64();
-                if (c > c_out) { alt_cy += t_cta - t_out; alt_dec += c - c_out; if (alt_dec > 512) { alt_cy >>= 1; alt_dec >>= 1; } }
                 if (lane == 0) {
-                    const bool may_play = alt_dec == 0 || alt_cy > (play_cpd > 130 ? play_cpd : 130) * alt_dec;
-                    s_bio.play_max = may_play ? play_max : 0;
+                    unsigned acy = s_bio.alt_cy, adec = s_bio.alt_dec;
+                    if (c > s_bio.c_out) {
+                        acy += (unsigned)clock() - s_bio.t_out; adec += (unsigned)(c - s_bio.c_out);
+                        if (adec > 512u) { acy >>= 1; adec >>= 1; }
+                        s_bio.alt_cy = acy; s_bio.alt_dec = adec;
+                    }
+                    const unsigned cpd = s_bio.play_cpd > 130u ? s_bio.play_cpd : 130u;
+                    const bool may_play = adec == 0 || acy / adec >= cpd;
+                    s_bio.play_max = may_play ? s_bio.play_next : 0;
                     if (!may_play) s_bio.wide = 0;
                     s_bio.per = per_now; s_bio.cur = cur; s_bio.head = head; s_bio.c = c; s_bio.cyc = cyc; s_bio.root = root; s_bio.B = 0;
                     s_job.type = FAST_JOB_BATCH;
                 }
                 __syncwarp();
+                const long long t_cta = clock64();
                 ++n_cta_try;
                 named_bar(1, KLPM_FAST_THREADS);
                 fast_batch_job<G>(A, R, &s_bio, sr, sr + 1024, sr + 2048, reinterpret_cast<int32_t*>(sh), s_scan, nwords);
                 const int32_t Bc = s_bio.B;
-                t_out = clock64();
-                const long long cy_this = t_out - t_cta;
+                const long long cy_this = clock64() - t_cta;
                 cy_cta += cy_this;
-                c_out = c + Bc;
+                if (lane == 0) { s_bio.t_out = (unsigned)clock(); s_bio.c_out = c + Bc; }
                 if (Bc > 0) {
                     if (s_bio.played) {
-                        play_cpd = (cy_this > 9000 ? (cy_this - 9000) / Bc : 0) + 70;
-                        const bool ahead = alt_dec >= 16 && alt_cy > 2 * play_cpd * alt_dec;      // (still the better half)
-                        play_max = ahead ? KLPM_FAST_CTA_BATCH : 128;
-                        if (play_cpd > KLPM_FAST_DEAR + 70 && !ahead) probe = 1;
+                        if (lane == 0) {
+                            const unsigned cpd = (cy_this > 9000 ? (unsigned)(cy_this - 9000) / (unsigned)Bc : 0u) + 70u;
+                            const bool ahead = s_bio.alt_dec >= 16u && s_bio.alt_cy / s_bio.alt_dec >= 2u * cpd;      // (still the better half)
+                            s_bio.play_cpd = cpd; s_bio.play_next = ahead ? KLPM_FAST_CTA_BATCH : 128;
+                            s_bio.probe = cpd > KLPM_FAST_DEAR + 70 && !ahead ? 1 : 0;
+                        }
+                        __syncwarp();
+                        probe = s_bio.probe;
                     }
                     ++n_cta_ok; dec_cta += Bc;
                     per_now = s_bio.wide || Bc >= (per_now == 1 ? 224 : 160) ? 4 : 1;
