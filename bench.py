@@ -393,12 +393,12 @@ def run_ours(args):
         # the first round of two kernels, the later rounds
         list_launches = 1 + sort_launches + 3                               # key list, its sort, the three charge kernels
         order_launches = 3 if nq > 16384 else 0
-        launches_per_step = (order_launches + 1) + (1 + sort_launches) + (2 + group_launches + 1 + list_launches + 1) + (1 + 1 + 2 + 1)
-        loop_kernel = "fast_run_kernel"
+        launches_per_step = (order_launches + 1) + (1 + sort_launches) + (2 + group_launches + 1 + list_launches + 2) + (1 + 1 + 2 + 1)
+        loop_kernel = "list_run_kernel"
         loop_note = ("all decisions in one CTA: once everybody has arrived, longest-match picks come from a presorted list "
-                     "of keys and oldest-first picks from a bitmap cursor, up to 1,024 decisions per CTA-wide batch (32 per "
-                     "warp-wide step) when they cannot interfere; picks whose group has other members take a careful step; those decisions are "
-                     "charged by a parallel pass after the loop; bound by the instruction issue of one warp; the loop starts "
+                     "of keys and oldest-first picks from a bitmap; windows of 2,048 entries of either order, who takes what is worked out by "
+                     "iteration over prefix sums; picks whose group has other members, and those whose key has changed, are made one at a time; the "
+                     "decisions are charged by a parallel pass after the loop; bound by the barriers of one CTA; the loop starts "
                      "from the records rt_match_batch_ex kept (no query is walked twice); the time includes the sort of the keys "
                      "and the bulk insertion of the processed prompts")
     else:

@@ -334,7 +334,8 @@ def klpm_run_last_only_batch(tokens: torch.Tensor, offsets: torch.Tensor, arriva
 
 
 def rt_debug_counters(tree: Tree) -> dict:
-    """What the grouped loop of the last klpm_run on this tree did (see include/klpm.h)."""
+    """What the grouped loop of the last klpm_run on this tree did (see include/klpm.h).  Once everybody has arrived: cta_batches_tried
+    counts the windows, cta_batches the batches in which both pick orders agree, warp_steps those worked out by iteration."""
     v = (_i64 * 16)()
     _check(_lib.rt_debug_counters(tree.handle, ctypes.byref(v)), "rt_debug_counters")
     names = ("careful_steps", "cta_dissolves", "fallback_scans", "fallen_back", "evictions", "cycles_tree", "cycles_scans",

@@ -1770,11 +1770,12 @@ struct alignas(32) FStat {    // constant during the loop; the first 16 bytes ar
 struct alignas(32) LNode { int32_t parent, depth, len, nchild; long long last, off; };
 
 struct FastPost {
-    int32_t c0; int32_t pad; long long now0;    // first decision made in list mode; the time it was made at
+    int32_t c0; int32_t list_c;                 // decisions the charge pass after the loop starts from; decisions made before everybody had arrived
+    long long now0; int32_t head, cyc;          // the time then, the oldest unprocessed slot, decisions made mod k
     // what the loop did (rt_debug_counters): careful steps, dissolves by the whole CTA, fallback scans, slots that fell
-    // back, evictions; cycles spent in tree updates, fallback scans, dissolves; list mode: CTA-wide batches tried and
-    // committed, decisions they made, warp-wide steps, decisions they made, decisions made one at a time; cycles in
-    // CTA-wide attempts and in warp-wide attempts
+    // back, evictions; cycles spent in tree updates, fallback scans, dissolves; list mode: windows, batches in which the two
+    // orders agree and the decisions they made, batches worked out by iteration and the decisions they made, decisions
+    // made one at a time; cycles spent on new windows and on decisions made one at a time
     long long counters[16];
 };
 
@@ -1790,6 +1791,7 @@ struct FastArgs {
     int32_t* mem;                 // member array
     const long long* sorted_t;    // per slot: arrival, side by side
     int4* lcp;                    // per slot: how far its prompt agrees with a reference prompt (see lcp_kernel)
+    int4* pair;                   // list mode, per slot that starts in a group: of two, the other slot, its match length and key once this one is processed; else -2
     const int32_t* pinv;          // rank -> slot, or null
     long long* gh; int32_t* gidx; // group hashes and slots (sorted before the loop; scratch for large groups inside it)
     unsigned int* done;           // bitmap of processed slots (used when it does not fit in shared memory)
@@ -2049,14 +2051,16 @@ lcp_kernel(FastArgs A, int32_t per, const int32_t* __restrict__ wanted) {
     const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long i0 = w * per;
     const long long i = i0 + lane;
-    int32_t r = -1, ref = -1, m = 0, len = 0;
+    int32_t r = -1, ref = -1, m = 0, len = 0, count = 0, other = -1;
     long long soff = 0;
     bool cmp = false;
     if (lane < per && i < A.n) {
         r = A.mem[i];
         const FDyn d = ld_dyn(A.dyn + r);
         if (d.gcount > 1 && (!wanted || wanted[d.gstart])) {
+            count = d.gcount;
             ref = A.mem[d.gstart];
+            other = ref;
             const FStat s = ld_stat(A.stat + r);
             m = d.m; len = s.len; soff = s.soff;
             if (ref != r) {
@@ -2077,6 +2081,20 @@ lcp_kernel(FastArgs A, int32_t per, const int32_t* __restrict__ wanted) {
         if (lane == src) e = x;
     }
     if (r >= 0) A.lcp[r] = make_int4(ref, e, e < len ? __ldg(A.tok + soff + e) : 0, 0);
+    // A group of two is known completely: whoever is processed first, the other one matches e tokens from then on.  (Two slots that share
+    // a run by a hash collision are no group.)
+    if (!A.list_mode || count < 2) return;
+    if (count > 2) { A.pair[r] = make_int4(-2, 0, 0, 0); return; }
+    if (other == r) return;                                 // (the other slot's lane writes both)
+    if (!cmp) {
+        atomicAnd(A.gbits + (r >> 5), ~(1u << (r & 31)));
+        atomicAnd(A.gbits + (other >> 5), ~(1u << (other & 31)));
+        return;
+    }
+    const FStat s = ld_stat(A.stat + r), f = ld_stat(A.stat + other);
+    const unsigned long long kr = fast_key(e, s.len, s.rank, A.score_mode), kf = fast_key(e, f.len, f.rank, A.score_mode);
+    A.pair[r] = make_int4(other, e, (int)(unsigned)kf, (int)(unsigned)(kf >> 32));
+    A.pair[other] = make_int4(r, e, (int)(unsigned)kr, (int)(unsigned)(kr >> 32));
 }
 // The groups that a given order touches (see lcp_kernel).
 __global__ void lcp_wanted_kernel(FastArgs A, int32_t* wanted) {
@@ -2094,12 +2112,13 @@ __device__ __forceinline__ bool overlap_known(const int4& a, int32_t len_a, cons
     return false;
 }
 
-// list mode: every slot's key in a form that sorts largest first (padding last)
-__global__ void fast_list_kernel(const unsigned long long* __restrict__ key, int32_t n, long long np2, long long* lk, int32_t* ls) {
+// list mode: every slot's key in a form that sorts largest first (processed slots last, then the padding)
+__global__ void fast_list_kernel(FastArgs A, long long np2) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= np2) return;
-    lk[i] = i < n ? (long long)(~key[i] ^ 0x8000000000000000ULL) : 0x7fffffffffffffffLL;
-    ls[i] = i < n ? (int32_t)i : 0x7fffffff;
+    const bool in = i < A.n, live = in && !(A.post->list_c > 0 && ((__ldcg(A.done + (i >> 5)) >> (i & 31)) & 1u));
+    const_cast<long long*>(A.lk)[i] = live ? (long long)(~A.key[i] ^ 0x8000000000000000ULL) : 0x7fffffffffffffffLL;
+    const_cast<int32_t*>(A.ls)[i] = in ? (int32_t)i : 0x7fffffff;
 }
 
 // Largest of the warp's 64-bit values with two hardware reductions: the high halves, then the low halves of
@@ -2203,16 +2222,6 @@ __device__ __forceinline__ bool slot_done(const FastTour& R, const FastArgs& A, 
     const unsigned w = bm_ld(R.done, r >> 5, R.g_done);
     return (w >> (r & 31)) & 1u;
 }
-// position of the k-th set bit of w (k >= 1, at most the number of set bits)
-__device__ __forceinline__ int kth_set_bit(unsigned w, int k) {
-    int pos = 0;
-    int cnt = __popc(w & 0xffffu); if (k > cnt) { k -= cnt; pos += 16; w >>= 16; }
-    cnt = __popc(w & 0xffu);       if (k > cnt) { k -= cnt; pos += 8; w >>= 8; }
-    cnt = __popc(w & 0xfu);        if (k > cnt) { k -= cnt; pos += 4; w >>= 4; }
-    cnt = __popc(w & 0x3u);        if (k > cnt) { k -= cnt; pos += 2; w >>= 2; }
-    if (k > (int)(w & 1u)) pos += 1;
-    return pos;
-}
 __device__ __forceinline__ void set_grouped(const FastTour& R, int32_t r, bool grouped) {
     if (!R.gb) return;
     if (grouped) atomicOr(R.gb + (r >> 5), 1u << (r & 31));
@@ -2238,7 +2247,7 @@ struct FastPick {             // the prompt being processed, as its group's memb
     int32_t leaf;             // trees with a budget: id of its new leaf (the tied members are parked in it from now on)
 };
 struct FastJob { int32_t type; int32_t a0, a1; FastPick pick; };
-enum { FAST_JOB_EXIT = 0, FAST_JOB_ADMIT = 1, FAST_JOB_DISSOLVE = 2, FAST_JOB_REBUILD = 3, FAST_JOB_BATCH = 4, FAST_JOB_FALLBACK = 5 };
+enum { FAST_JOB_EXIT = 0, FAST_JOB_ADMIT = 1, FAST_JOB_DISSOLVE = 2, FAST_JOB_FALLBACK = 3 };
 
 // trees with a budget: slot r's match now ends inside node `to` (it was counted for node `from`)
 __device__ __forceinline__ void lru_move(const FastArgs& A, int32_t r, int32_t from, int32_t to) {
@@ -2259,61 +2268,6 @@ __device__ __forceinline__ unsigned long long changed_block_max(const FastArgs& 
         }
     }
     return warp_max64r(v);
-}
-
-// What the sequencer hands to a CTA-wide batch of decisions, and what it gets back.
-struct FastBatchIO {
-    int32_t per;                      // in: list entries per thread, 4 (1,024 decisions at most) or 1 (256: cheaper where batches end early)
-    int32_t cur, head, c, cyc;        // in: list cursor, oldest unprocessed slot, decisions made, c mod k
-    unsigned long long root;          // in: largest key in the tournament
-    int32_t B, consumed, hmax;        // out: decisions made (0: none), list entries passed, last slot taken by an oldest-first turn
-    int32_t B0, Bmax, limF, limL;     // scratch
-    // scratch: the slots both kinds of turn reach inside the batch (rank among the oldest-first picks, rank among the
-    // list entries), and after they are resolved the ranks each side passes over, ascending
-    int32_t ncol, nRH, nRE;
-    int32_t colPhi[32], colRk[32], remH[32], remE[32];
-    int32_t hard;                     // out: the batch stopped before a decision that needs the one-at-a-time path
-    int32_t Braw;                     // out: decisions the batch could have made (it makes none below KLPM_FAST_CTA_MIN)
-    int32_t play_max;                 // in: 0: no batch is played through; else: after how many decisions one that is dear ends
-    // kept between attempts by the sequencer's lane 0: cost and number of the decisions made between attempts, cycles per
-    // decision of the last played batch, when and at which decision the last attempt ended, the next play_max, whether to try a warp-wide step first
-    unsigned alt_cy, alt_dec, play_cpd, t_out;
-    int32_t c_out, play_next, probe;
-    int32_t wide;                     // in: look at as many slots and entries as the scratch holds (the last batch had many meetings)
-    int32_t played;                   // out: the batch was played through decision by decision (more than 32 meetings)
-    int32_t played_t, played_u;       // scratch: ranks of the last slot and the last entry taken, -1 if none
-    int32_t limB;                     // scratch: the batch must end before this decision (list entries that an oldest-first pick would meet)
-};
-#define KLPM_FAST_CTA_BATCH 1024      // decisions per CTA-wide batch at most (4 list entries per thread)
-#ifndef KLPM_FAST_CTA_MIN
-#define KLPM_FAST_CTA_MIN 32         // smaller batches are left to the warp-wide step (an attempt costs about 10,000 cycles)
-#endif
-#define KLPM_FAST_PLAY 48
-#define KLPM_FAST_DEAR 160            // cycles per decision above which a played batch is dear (where the orders agree it takes 45 to 100)
-#ifndef KLPM_FAST_CB_MAX
-#define KLPM_FAST_CB_MAX 32           // longest back-off (loop iterations) after CTA-wide attempts that failed
-#endif
-#ifndef KLPM_FAST_FAIL_CAP
-#define KLPM_FAST_FAIL_CAP 6          // failed CTA-wide attempts in a row that still lengthen the wait (8 << that many decisions)
-#endif
-#ifndef KLPM_FAST_CALM
-#define KLPM_FAST_CALM 1              // full warp-wide steps in a row before a CTA-wide batch is tried again
-#endif
-
-// Exclusive prefix sum of v over the CTA's 256 threads; *total receives the sum.  s_w: 8 ints of shared scratch.
-__device__ __forceinline__ int32_t block_excl_scan(int32_t v, int32_t* s_w, int32_t* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int32_t inc = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) { const int32_t o = __shfl_up_sync(FULL_MASK, inc, d); if (lane >= d) inc += o; }
-    __syncthreads();                   // s_w may still be read from an earlier scan
-    if (lane == 31) s_w[warp] = inc;
-    __syncthreads();
-    int32_t before = 0, all = 0;
-#pragma unroll
-    for (int w = 0; w < KLPM_FAST_THREADS / 32; ++w) { const int32_t x = s_w[w]; if (w < warp) before += x; all += x; }
-    *total = all;
-    return before + inc - v;
 }
 
 // One member of the dissolving group per lane (r < 0: none).  Members tied with the processed prompt are
@@ -2384,345 +2338,6 @@ __device__ __forceinline__ unsigned long long dissolve_small(const FastArgs& A, 
         root = tour_update(R, bb, lane);
     }
     return root;
-}
-
-// The warp-wide step of list mode (see fast_run_kernel) with the whole CTA: 1,024 list entries and 8,192 bitmap slots
-// are examined at once, the same checks cut the batch short, block-wide prefix sums replace the warp's ballots.
-// Every thread calls it.  Nothing is changed unless at least KLPM_FAST_CTA_MIN decisions can be made.
-template <bool G>
-__device__ void fast_batch_job(const FastArgs& A, const FastTour& R0, FastBatchIO* io, int32_t* sH, int32_t* sE, int32_t* sEpos,
-                               int32_t* sF, int32_t* s_w, int32_t nwords) {
-    FastTour R = R0;                                        // with the bitmaps in shared memory the flags fold away
-    if (!G) { R.g_done = 0; R.g_bits = 0; }
-    const int tid = threadIdx.x;
-    const int32_t n = A.n, cur = io->cur, head = io->head, c = io->c, cyc = io->cyc;
-    const unsigned long long root = io->root;
-    const int32_t per = io->per, most_ = KLPM_FAST_THREADS * per;      // list entries per thread; decisions the batch can make
-    // the list entries cur + 4 tid .. + 3 (asked for first: the table below is filled while they travel)
-    long long kk[4]; int32_t es[4]; bool ok[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const long long idx = (long long)cur + tid * per + r;
-        kk[r] = 0; es[r] = 0;
-        if (r < per && idx < n) { kk[r] = __ldg(A.lk + idx); es[r] = __ldg(A.ls + idx); }
-    }
-    // sF[x] = oldest-first turns among the next x decisions, x = 0 .. 1,024.  Under k-LPM the first such turn is
-    // decision (k - cyc) mod k and then every k-th, which is floor((x + s) / k) with s = (cyc + k - 1) mod k; one
-    // division per thread, the later entries follow by adding 256 = Q k + Rm.
-    {
-        const int32_t sft = cyc == 0 ? A.k - 1 : cyc - 1;
-        int32_t q = 0, rem = 0, Q = 0, Rm = 0;
-        if (A.policy == KLPM_POLICY_KLPM) { q = (tid + sft) / A.k; rem = (tid + sft) - q * A.k; Q = KLPM_FAST_THREADS / A.k; Rm = KLPM_FAST_THREADS - Q * A.k; }
-        for (int32_t x = tid; x <= KLPM_FAST_CTA_BATCH; x += KLPM_FAST_THREADS) {
-            sF[x] = A.policy == KLPM_POLICY_FCFS ? x : A.policy == KLPM_POLICY_LPM ? 0 : q;
-            q += Q; rem += Rm;
-            if (rem >= A.k) { rem -= A.k; ++q; }
-        }
-    }
-    // the limits start open; every thread reads them capped by what the batch can hold
-    if (tid == 0) { io->B0 = 0; io->Bmax = 0; io->limF = 0x7fffffff; io->limL = 0x7fffffff; io->limB = 0x7fffffff; io->ncol = 0; io->nRH = 0; io->nRE = 0; }
-    auto f = [&](int32_t x) -> int32_t { return sF[x]; };
-    // those of the entries that still count
-    int32_t cnt = 0;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const long long idx = (long long)cur + tid * per + r;
-        ok[r] = r < per && idx < n && !((bm_ld(R.skip, es[r] >> 5, R.g_bits) >> (es[r] & 31)) & 1u);
-        cnt += ok[r];
-    }
-    // the unprocessed slots from `head` on, one bitmap word per thread
-    const int32_t w0 = head >> 5;
-    unsigned fr;
-    {
-        const int32_t wi = w0 + tid;
-        unsigned w = wi < nwords ? bm_ld(R.done, wi, R.g_done) : 0xffffffffu;
-        if (wi == nwords - 1 && (n & 31)) w |= ~((1u << (n & 31)) - 1u);
-        if (wi == w0) w |= (1u << (head & 31)) - 1u;
-        fr = ~w;
-    }
-    // both prefix sums with one scan: usable entries (at most 1,024) in the low half, free slots (at most 8,192) above
-    int32_t both;
-    const int32_t base2 = block_excl_scan(cnt + (__popc(fr) << 16), s_w, &both);    // (its barriers also publish sF and the limits)
-    const int32_t base = base2 & 0xffff, qk = base2 >> 16;
-    const int32_t avail = both & 0xffff, nfree = both >> 16;
-    int32_t* sP = sF + KLPM_FAST_CTA_BATCH + 8;             // per word: free slots before it
-    unsigned* sFr = reinterpret_cast<unsigned*>(sP + KLPM_FAST_THREADS);
-    sP[tid] = qk; sFr[tid] = fr;
-    int32_t* sMet = reinterpret_cast<int32_t*>(sFr + KLPM_FAST_THREADS);      // per entry rank: rank of its slot among the oldest-first picks, or -1
-    int32_t* sBack = sMet + KLPM_FAST_CTA_BATCH;            // and the other way round
-    int32_t* sSel = sBack + KLPM_FAST_CTA_BATCH;            // a batch that is played through: the slot of every decision
-    // u / (k - 1) for u up to 2,048: a multiplication by the reciprocal rounded up
-    auto per_k1 = [&](int32_t u) -> int32_t { return A.k == 2 ? u : (int32_t)__umulhi((unsigned)u, A.recip_k1); };
-    {   // as many decisions as those entries allow: the largest x with x - f(x) <= avail, every thread trying four values
-        const int32_t hi = n - c < most_ ? n - c : most_;
-        int32_t best = 0;
-#pragma unroll
-        for (int r = 1; r <= 4; ++r) { const int32_t x = tid * per + r; if (r <= per && x <= hi && x - f(x) <= avail) best = x; }
-        best = __reduce_max_sync(FULL_MASK, best);
-        if ((tid & 31) == 0 && best > 0) atomicMax(&io->B0, best);
-    }
-    __syncthreads();
-    const int32_t B0 = io->B0, nF0 = f(B0), nL0 = B0 - nF0;
-    // One slot and one entry more than a full batch takes are looked at: where the two pick orders meet once inside the
-    // batch (a slot that is both among the oldest unprocessed and among the next list entries), the side that comes
-    // later passes over it and takes one more of its own.
-    const bool both_kinds = A.policy == KLPM_POLICY_KLPM && A.k >= 2;       // (k = 1: every turn is an oldest-first turn)
-    const bool wide = both_kinds && io->wide != 0;
-    const int32_t nFw = wide ? KLPM_FAST_CTA_BATCH : both_kinds ? (nF0 + 32 < KLPM_FAST_CTA_BATCH ? nF0 + 32 : KLPM_FAST_CTA_BATCH) : nF0;
-    const int32_t nLw = wide ? KLPM_FAST_CTA_BATCH : both_kinds ? (nL0 + 32 < KLPM_FAST_CTA_BATCH ? nL0 + 32 : KLPM_FAST_CTA_BATCH) : nL0;
-    const int32_t nFa = nfree < nFw ? nfree : nFw;          // oldest-first picks there are slots for
-    const int32_t nEa = avail < nLw ? avail : nLw;          // longest-match picks there are entries for
-    // the next nFa unprocessed slots in order: a thread per slot, eight words at a time; the slot's rank among the free
-    // ones is where it goes; one whose key sits in the tournament or that is grouped needs the careful step
-    {
-        const int bit = tid & 31;
-        for (int32_t wl = tid >> 5; wl < KLPM_FAST_THREADS && sP[wl] < nFa; wl += KLPM_FAST_THREADS / 32) {
-            const unsigned fw = sFr[wl];
-            if ((fw >> bit) & 1u) {
-                const int32_t rank = sP[wl] + __popc(fw & ((1u << bit) - 1u));
-                if (rank < nFa) {
-                    const int32_t hs = (w0 + wl) * 32 + bit;
-                    sH[rank] = hs;
-                    if (((bm_ld(R.skip, hs >> 5, R.g_bits) | bm_ld(R.gb, hs >> 5, R.g_bits)) >> (hs & 31)) & 1u) atomicMin(&io->limF, rank);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    const int32_t hmax0 = nFa > 0 ? sH[nFa - 1] : -1;
-    // The usable entries by rank.  One that is grouped or lies below the tournament's root stops the batch before its
-    // turn.  One whose slot is among the slots the oldest-first picks would take (rank phi there) is taken by whichever
-    // side reaches it first.  The first such meeting (the one whose earlier decision comes first) is resolved inside
-    // the batch: the other side passes over the slot, its later picks move up by one.  The batch ends well before any
-    // further meeting: k + 1 decisions before the earlier of its two decisions as computed without the shift, which
-    // moves a decision forward by at most k -- or before the later of its two decisions where those are far enough
-    // apart for the shift not to change their order (the earlier one is an ordinary pick then).
-    {
-        int32_t rk = base;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            if (ok[r]) {
-                if (rk < nEa) {
-                    sE[rk] = es[r]; sEpos[rk] = tid * per + r;
-                    const unsigned long long ek = ~((unsigned long long)kk[r] ^ 0x8000000000000000ULL);
-                    int32_t met = -1;
-                    if ((((bm_ld(R.gb, es[r] >> 5, R.g_bits) >> (es[r] & 31)) & 1u)) || root > ek) {
-                        atomicMin(&io->limL, rk);
-                    } else if (es[r] >= head && es[r] <= hmax0) {
-                        // phi: slots of sH before this one (its word is one of those looked at: it lies between head and hmax0)
-                        const int32_t wl = (es[r] >> 5) - w0;
-                        const int32_t phi = sP[wl] + __popc(sFr[wl] & ((1u << (es[r] & 31)) - 1u));
-                        met = phi;
-                        // decision of the oldest-first turn of rank phi, and of the longest-match turn of rank rk
-                        int32_t xF, xL;
-                        if (A.policy == KLPM_POLICY_FCFS) { xF = phi; xL = B0; }
-                        else if (A.policy == KLPM_POLICY_LPM) { xF = B0; xL = rk; }
-                        else {
-                            const int32_t i0 = cyc == 0 ? 0 : A.k - cyc;
-                            const long long xF64 = i0 + (long long)phi * A.k;
-                            xF = xF64 < 0x3ffffff ? (int32_t)xF64 : 0x3ffffff;
-                            xL = rk;                                       // before the first oldest-first turn; after it k - 1 of every k decisions
-                            if (rk >= i0 && A.k >= 2) { const int32_t u1 = rk - i0; xL = rk + 1 + per_k1(u1); }
-                        }
-                        // without resolving: the batch would have to end before the later of the two decisions (used
-                        // where there are more such slots than are resolved)
-                        atomicMin(&io->limB, xF > xL ? xF : xL);
-                        if (both_kinds) {
-                            const int32_t ci = atomicAdd(&io->ncol, 1);
-                            if (ci < 32) { io->colPhi[ci] = phi; io->colRk[ci] = rk; }
-                        }
-                    }
-                    if (both_kinds) sMet[rk] = met;
-                }
-                ++rk;
-            }
-        }
-    }
-    __syncthreads();
-    // Where the two orders meet, sequential processing gives the slot to whichever turn comes first, and the other side
-    // passes over it: its later picks move up by one.  Warp 0 plays the meetings through in the order of their first
-    // decision (lane i holds meeting i; the time at which a side reaches a slot is its rank minus the ranks below it
-    // that this side has passed over so far, turned into a decision number; the earliest pending decision is final,
-    // because whatever happens later moves later picks only).  Result: the ranks each side passes over, ascending.
-    const int32_t ncol = io->ncol;                          // (block-uniform)
-    const bool resolve = both_kinds && ncol > 0 && ncol <= 32;
-    if (resolve) {
-        if (tid < 32) {
-            const int lane = tid;
-            const bool mine = lane < ncol;
-            const int32_t phi = mine ? io->colPhi[lane] : 0x7fffffff, rk = mine ? io->colRk[lane] : 0x7fffffff;
-            unsigned belowPhi = 0, belowRk = 0;             // meetings with a smaller rank on either side
-            for (int j = 0; j < ncol; ++j) {
-                const int32_t pj = __shfl_sync(FULL_MASK, phi, j), rj = __shfl_sync(FULL_MASK, rk, j);
-                if (pj < phi) belowPhi |= 1u << j;
-                if (rj < rk) belowRk |= 1u << j;
-            }
-            const int32_t i0 = cyc == 0 ? 0 : A.k - cyc;    // decisions before the first oldest-first turn
-            const int32_t FAR = 0x3ffffff;
-            // decision of the longest-match turn of rank u, of the oldest-first turn of rank t (capped)
-            auto l_turn = [&](int32_t u) -> int32_t { return u < i0 ? u : u + 1 + per_k1(u - i0); };
-            auto f_turn = [&](int32_t t) -> int32_t { const long long x = i0 + (long long)t * A.k; return x < FAR ? (int32_t)x : FAR; };
-            // no batch gets past the first slot or entry that needs the careful step, whoever passes over what
-            const int32_t capF = io->limF < nFa ? io->limF : nFa, capL = io->limL < nEa ? io->limL : nEa;
-            int32_t bcap = B0;
-            { const int32_t a1 = f_turn(capF), a2 = l_turn(capL); if (a1 < bcap) bcap = a1; if (a2 < bcap) bcap = a2; }
-            int32_t xF = FAR, xL = FAR;
-            // oldest-first turns before a longest-match turn of rank u are 1 + u1 / (k - 1): whether u1 is the first of its k - 1
-            int32_t cur_rk = rk;                            // the entry's rank less those this side has passed over below it
-            if (mine) { xF = f_turn(phi); xL = l_turn(rk); }
-            unsigned remH = 0, remE = 0, open_ = ncol == 32 ? 0xffffffffu : ((1u << ncol) - 1u);
-            while (open_) {
-                unsigned key = 0xffffffffu;
-                const bool l_first = xL < xF;
-                if (mine && ((open_ >> lane) & 1u)) key = ((unsigned)(l_first ? xL : xF) << 5) | (unsigned)lane;
-                const unsigned win = __reduce_min_sync(FULL_MASK, key);
-                if ((int32_t)(win >> 5) >= bcap) break;   // beyond what the batch can reach: nothing more to settle
-                const int wl = (int)(win & 31u);
-                const bool wl_first = __shfl_sync(FULL_MASK, (int)l_first, wl) != 0;
-                open_ &= ~(1u << wl);
-                if (wl_first) {                             // a longest-match turn took that slot: later oldest-first picks come one turn earlier
-                    remH |= 1u << wl;
-                    if (((belowPhi >> wl) & 1u) && xF < FAR) xF -= A.k;
-                } else {                                    // an oldest-first turn took that entry's slot: later list picks come one turn earlier
-                    remE |= 1u << wl;
-                    if ((belowRk >> wl) & 1u) { --cur_rk; xL = l_turn(cur_rk); }
-                }
-            }
-            if (mine && ((remH >> lane) & 1u)) io->remH[__popc(remH & belowPhi)] = phi;
-            if (mine && ((remE >> lane) & 1u)) io->remE[__popc(remE & belowRk)] = rk;
-            if (lane == 0) { io->nRH = __popc(remH); io->nRE = __popc(remE); }
-        }
-        __syncthreads();
-    }
-    // More meetings than that (two orders that run side by side): the batch is played through decision by decision.  Warp 0
-    // holds one bit per rank of either side (word w in lane w; the word a side is at also in a uniform register): the next
-    // rank whose bit is clear is the pick, and its slot's bit on the other side is set: 540 cycles a decision where every turn
-    // changes sides, 45 where the two orders agree; the one-at-a-time path takes 1,000 to 1,500.  A batch that gets KLPM_FAST_PLAY
-    // decisions far without it costs less that way (9,000 cycles in all).
-    const bool play = both_kinds && io->play_max > 0 && ncol > 32 && io->limB < KLPM_FAST_PLAY;
-    if (play) {
-        for (int32_t x = tid; x < nFa; x += KLPM_FAST_THREADS) sBack[x] = -1;
-        __syncthreads();
-        for (int32_t x = tid; x < nEa; x += KLPM_FAST_THREADS) if (sMet[x] >= 0) sBack[sMet[x]] = x;
-        __syncthreads();
-        if (tid < 32) {
-            const int lane = tid;
-            const int32_t capF = io->limF < nFa ? io->limF : nFa, capL = io->limL < nEa ? io->limL : nEa;
-            const int32_t most = n - c < KLPM_FAST_CTA_BATCH ? n - c : KLPM_FAST_CTA_BATCH;      // (wide: both sides in sight beyond the list window)
-            const unsigned t_play = (unsigned)clock();
-            int32_t look = io->play_max;                    // where the cost so far is looked at
-            unsigned mh = 0, me = 0;                        // ranks that are taken, of this lane's word
-            unsigned ch = 0, ce = 0;                        // the words the two sides are at
-            int32_t t = 0, u = 0, lt = -1, lu = -1, x = 0, turn = cyc;
-            bool stop_f = false, stop_l = false;            // ran into the end of what is in sight, or into a limit, on which side
-            for (; x < most; ++x) {
-                if (x >= look) {
-                    if ((unsigned)clock() - t_play > KLPM_FAST_DEAR * (unsigned)x) break;
-                    look = x + 64;
-                }
-                // Where both sides are at the same slot, that slot is the next pick whichever turn it is, and so on for as
-                // long as the two orders agree: up to 32 decisions at once.
-                {
-                    const unsigned fh = ~ch & (0xffffffffu << (t & 31)), fe = ~ce & (0xffffffffu << (u & 31));
-                    if (fh && fe) {
-                        t = (t & ~31) + __ffs(fh) - 1;
-                        u = (u & ~31) + __ffs(fe) - 1;
-                        const int32_t tt = t + lane, uu = u + lane;
-                        const bool same = tt < capF && uu < capL && x + lane < most && (tt >> 5) == (t >> 5) && !((ch >> (tt & 31)) & 1u) && sMet[uu] == tt;
-                        const unsigned no = ~__ballot_sync(FULL_MASK, same);
-                        const int r = no ? __ffs(no) - 1 : 32;
-                        if (r >= 2) {
-                            if (lane < r) sSel[x + lane] = sH[tt];
-                            const unsigned run = r == 32 ? 0xffffffffu : (1u << r) - 1u;
-                            const unsigned long long runE = (unsigned long long)run << (u & 31);
-                            ch |= run << (t & 31);
-                            if (lane == (t >> 5)) mh |= run << (t & 31);
-                            if (lane == (u >> 5)) me |= (unsigned)runE;
-                            if (lane == (u >> 5) + 1) me |= (unsigned)(runE >> 32);
-                            ce |= (unsigned)runE;
-                            lt = t + r - 1; lu = u + r - 1;
-                            x += r - 1;
-                            turn = (turn + r) % A.k;
-                            continue;
-                        }
-                    }
-                }
-                const bool fcfs_turn = turn == 0;
-                if (++turn == A.k) turn = 0;
-                int32_t other, slot;
-                if (fcfs_turn) {
-                    unsigned free_ = ~ch & (0xffffffffu << (t & 31));
-                    while (!free_ && (t | 31) + 1 < capF) { t = (t | 31) + 1; ch = __shfl_sync(FULL_MASK, mh, t >> 5); free_ = ~ch; }
-                    stop_f = !free_;
-                    if (!stop_f) { t = (t & ~31) + __ffs(free_) - 1; stop_f = t >= capF; }
-                    if (stop_f) break;
-                    slot = sH[t]; other = sBack[t]; lt = t;
-                    ch |= 1u << (t & 31);
-                    if (lane == (t >> 5)) mh |= 1u << (t & 31);
-                    if (other >= 0) { const unsigned bit = 1u << (other & 31); if ((other >> 5) == (u >> 5)) ce |= bit; if (lane == (other >> 5)) me |= bit; }
-                } else {
-                    unsigned free_ = ~ce & (0xffffffffu << (u & 31));
-                    while (!free_ && (u | 31) + 1 < capL) { u = (u | 31) + 1; ce = __shfl_sync(FULL_MASK, me, u >> 5); free_ = ~ce; }
-                    stop_l = !free_;
-                    if (!stop_l) { u = (u & ~31) + __ffs(free_) - 1; stop_l = u >= capL; }
-                    if (stop_l) break;
-                    slot = sE[u]; other = sMet[u]; lu = u;
-                    ce |= 1u << (u & 31);
-                    if (lane == (u >> 5)) me |= 1u << (u & 31);
-                    if (other >= 0) { const unsigned bit = 1u << (other & 31); if ((other >> 5) == (t >> 5)) ch |= bit; if (lane == (other >> 5)) mh |= bit; }
-                }
-                if (lane == 0) sSel[x] = slot;
-            }
-            if (lane == 0) {
-                io->played_t = lt; io->played_u = lu; io->Bmax = x;
-                // stopped by a decision only the one-at-a-time path can take, not by the end of what is in sight?
-                io->hard = (stop_f && io->limF < nFa) || (stop_l && io->limL < nEa) ? 1 : 0;
-            }
-        }
-        __syncthreads();
-    }
-    // the limits, capped by what is in sight
-    const int32_t limF = io->limF < nFa ? io->limF : nFa, limL = io->limL < nEa ? io->limL : nEa;
-    const int32_t limB = resolve || io->limB > B0 ? B0 : io->limB;
-    const int32_t nRH = io->nRH, nRE = io->nRE;
-    // rank t among the oldest-first picks -> index of its slot in sH; rank u among the longest-match picks -> index in sE
-    auto hI = [&](int32_t t) -> int32_t { for (int32_t j = 0; j < nRH; ++j) { if (io->remH[j] <= t) ++t; else break; } return t; };
-    auto eI = [&](int32_t u) -> int32_t { for (int32_t j = 0; j < nRE; ++j) { if (io->remE[j] <= u) ++u; else break; } return u; };
-    if (!play) {   // the largest x that respects the limits, every thread trying four values
-        int32_t best = 0;
-#pragma unroll 1
-        for (int r = 1; r <= per; ++r) {
-            const int32_t x = tid * per + r, nf = f(x), nl = x - nf;
-            if (x <= limB && (nf == 0 || hI(nf - 1) < limF) && (nl == 0 || eI(nl - 1) < limL)) best = x;
-        }
-        best = __reduce_max_sync(FULL_MASK, best);
-        if ((tid & 31) == 0 && best > 0) atomicMax(&io->Bmax, best);
-    }
-    __syncthreads();
-    const int32_t Braw = io->Bmax;
-    const int32_t B = Braw >= KLPM_FAST_CTA_MIN ? Braw : 0;     // nothing is changed by a batch too short to pay
-    if (tid == 0) { io->B = B; io->Braw = Braw; io->played = play ? 1 : 0; io->wide = play ? 1 : 0; }
-    if (tid == 0 && play) {
-        io->consumed = io->played_u >= 0 ? sEpos[io->played_u] + 1 : 0;
-        io->hmax = io->played_t >= 0 ? sH[io->played_t] : -1;
-        if (B == 0) io->hard = 0;
-    } else if (tid == 0) {
-        const int32_t nF = f(B), nL = B - nF;
-        io->consumed = nL > 0 ? sEpos[eI(nL - 1)] + 1 : 0;
-        io->hmax = nF > 0 ? sH[hI(nF - 1)] : -1;
-        // stopped by a decision only the one-at-a-time path can take (not by the end of what is in sight, nor by a
-        // further slot both kinds of turn reach: the next batch sorts that out)
-        const int32_t nf1 = f(B + 1), nl1 = B + 1 - nf1;
-        io->hard = B > 0 && B < B0 && ((nf1 > 0 && hI(nf1 - 1) >= io->limF) || (nl1 > 0 && eI(nl1 - 1) >= io->limL)) ? 1 : 0;
-    }
-    for (int32_t x = tid; x < B; x += KLPM_FAST_THREADS) {   // thread makes decisions c + x
-        const int32_t f0 = f(x);
-        const int32_t slot = play ? sSel[x] : f(x + 1) > f0 ? sH[hI(f0)] : sE[eI(x - f0)];
-        atomicOr(R.done + (slot >> 5), 1u << (slot & 31));
-        atomicOr(R.skip + (slot >> 5), 1u << (slot & 31));
-        A.order[c + x] = slot;
-    }
-    __syncthreads();
 }
 
 // sh[0..p2) / sr[0..p2) hold the group hash and the slot of cnt members (padded with KLPM_FAST_NOGROUP / -1 up to the
@@ -2947,12 +2562,6 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
             }
         }
       }
-    } else if (J.type == FAST_JOB_REBUILD) {
-        // entering list mode (32-slot leaf blocks): the tournament keeps only the unprocessed slots whose key has changed
-        for (int32_t b = warp; b < A.nb; b += nwarps) {
-            const unsigned long long v = changed_block_max(A, R, b, lane);
-            if (lane == 0) R.t1[b] = v;
-        }
     } else {
         // dissolve a group of more than 32 members, or a smaller one whose members have long compares ahead
         const FastPick& P = J.pick;
@@ -3041,15 +2650,9 @@ __device__ void fast_job(const FastArgs& A, const FastTour& R, const FastJob& J,
     __syncthreads();
 }
 
-// The loop.  While arrivals are pending every decision is one careful step: admit who has arrived, pick from the
-// tournament over all arrived slots (or the oldest slot), take the pick out of its leaf block, charge it and
-// dissolve its group.  Once everybody has arrived the time of a pick no longer decides who can be picked, and the
-// loop changes to list mode: all keys were sorted before the loop, so the longest-match pick is the next entry of
-// that list that is still unprocessed and whose key has not changed since; the tournament is cut down to the slots
-// whose key has changed (members of dissolved groups) and the pick is the larger of the two candidates.  A pick
-// from the list touches no tournament at all, up to 32 decisions are made by one warp-wide step (up to 1,024 by a
-// CTA-wide one, fast_batch_job), and the loop only records which slot each decision takes: the charge pass after the
-// loop computes their outputs.
+// The loop while arrivals are pending: every decision is one careful step: admit who has arrived, pick from the
+// tournament over all arrived slots (or the oldest slot), take the pick out of its leaf block, charge it and dissolve its
+// group.  Once everybody has arrived the time of a pick no longer decides who can be picked, and list_run_kernel goes on.
 // G: some of the loop's bitmaps live in global memory (queues too long for shared memory).  The instance without them
 // reads its bitmaps as plain shared-memory words.
 template <bool G>
@@ -3058,12 +2661,16 @@ fast_run_kernel(FastArgs A) {
     extern __shared__ __align__(16) unsigned char fast_smem[];
     __shared__ FastJob s_job;
     __shared__ int s_cnt;
-    __shared__ int32_t s_H[32], s_E[32];      // a batch's oldest-first and longest-match picks, by rank
-    __shared__ FastBatchIO s_bio;             // a CTA-wide batch: what the sequencer hands over and gets back
-    __shared__ int32_t s_scan[KLPM_FAST_THREADS / 32];
     __shared__ int32_t s_memcur;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t n = A.n;
+    if (A.list_mode && __ldg(&A.stat[n - 1].t) <= A.start_tick) {      // everybody is waiting as the loop starts: nothing to do here
+        if (threadIdx.x == 0) {
+            A.post->c0 = 0; A.post->list_c = 0; A.post->now0 = A.start_tick; A.post->head = 0; A.post->cyc = 0;
+            for (int i = 0; i < 16; ++i) A.post->counters[i] = 0;
+        }
+        return;
+    }
     const int32_t nb1p = (A.nb + 31) & ~31, n2 = nb1p >> 5, n2p = (n2 + 31) & ~31, n3 = n2p >> 5;
     const int32_t nwords = (n + 31) >> 5;
     FastTour R;
@@ -3078,24 +2685,31 @@ fast_run_kernel(FastArgs A) {
     R.g_done = A.done_in_smem ? 0 : 1;
     R.g_bits = A.bits_in_smem ? 0 : 1;
     R.done = A.done_in_smem ? s_bits : A.done;
-    R.skip = !A.list_mode ? nullptr : A.bits_in_smem ? s_bits + nwords : A.gskip;
+    R.skip = nullptr;
     R.gb = !A.list_mode ? nullptr : A.bits_in_smem ? s_bits + 2 * nwords : A.gbits;
     R.dirty = nullptr;
     unsigned int* const s_done = R.done;
     if (!G) { R.g_done = 0; R.g_bits = 0; }
-    const int gdone = G ? R.g_done : 0, gbits = G ? R.g_bits : 0;
+    const int gdone = G ? R.g_done : 0;
     for (int32_t i = threadIdx.x; i < nb1p + n2p + 32; i += blockDim.x) R.t1[i] = 0ULL;
     if (threadIdx.x == 0) s_memcur = n;
     if (A.done_in_smem) for (int32_t i = threadIdx.x; i < nwords; i += blockDim.x) s_bits[i] = 0u;
-    if (A.list_mode && A.bits_in_smem) for (int32_t i = threadIdx.x; i < nwords; i += blockDim.x) { R.skip[i] = 0u; R.gb[i] = __ldcg(A.gbits + i); }
+    if (A.list_mode && A.bits_in_smem) for (int32_t i = threadIdx.x; i < nwords; i += blockDim.x) R.gb[i] = __ldcg(A.gbits + i);
     __syncthreads();
 
     if (warp != 0) {
         for (;;) {
             named_bar(1, KLPM_FAST_THREADS);
             const FastJob J = s_job;
-            if (J.type == FAST_JOB_EXIT) return;
-            if (J.type == FAST_JOB_BATCH) { fast_batch_job<G>(A, R, &s_bio, sr, sr + 1024, sr + 2048, reinterpret_cast<int32_t*>(sh), s_scan, nwords); continue; }
+            if (J.type == FAST_JOB_EXIT) {
+                if (J.a0) {                                 // list_run_kernel takes over: it needs the bitmaps
+                    for (int32_t i = threadIdx.x - 32; i < nwords; i += KLPM_FAST_THREADS - 32) {
+                        if (A.done_in_smem) __stcg(A.done + i, R.done[i]);
+                        if (A.bits_in_smem) __stcg(A.gbits + i, R.gb[i]);
+                    }
+                }
+                return;
+            }
             fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
         }
     }
@@ -3116,13 +2730,9 @@ fast_run_kernel(FastArgs A) {
     auto mark_done = [&](int32_t j) {
         if (!gdone) s_done[j >> 5] |= 1u << (j & 31);
         else if (lane == 0) __stcg(s_done + (j >> 5), __ldcg(s_done + (j >> 5)) | (1u << (j & 31)));
-        if (R.skip) {
-            if (!gbits) R.skip[j >> 5] |= 1u << (j & 31);
-            else if (lane == 0) __stcg(R.skip + (j >> 5), __ldcg(R.skip + (j >> 5)) | (1u << (j & 31)));
-        }
         __syncwarp();
     };
-    // Charge pick `slot` (Definition 2), write its outputs, and let the queries tied with it match into its new
+    // Charge pick `slot` (Definition 2; not in a given order, whose charging is the pass after the loop), write its outputs, and let the queries tied with it match into its new
     // leaf.  The caller has taken the slot out of the tournament or the list and marked it processed.
     auto careful = [&](int32_t slot, bool charge, const FDyn& d, const FStat& s) {
         const int32_t m = d.m, len = s.len, unc = len - m;
@@ -3135,8 +2745,6 @@ fast_run_kernel(FastArgs A) {
                 A.uncached[s.ord] = unc; A.ttft[s.ord] = Rj - s.t;
                 if (A.completion) A.completion[s.ord] = Rj;
             }
-        } else if (lane == 0) {
-            if (A.order) A.order[c] = slot;                 // list mode: the charge pass after the loop does the rest
         }
         // the new leaf's positions: unique per decision, above every real pool index
         const long long vleaf = A.vbase + ((long long)c << 32);
@@ -3188,9 +2796,6 @@ fast_run_kernel(FastArgs A) {
         }
         c = n;                                               // nothing is left for the policy loops below
     }
-
-    // everybody is waiting as the loop starts: no arrival will ever have to be admitted
-    if (A.list_mode && __ldg(&A.stat[n - 1].t) <= now) { admitted = n; next_t = INF; }
 
     // ================================================================ arrivals pending: one careful step per decision
     long long tw = INF;                                     // 32 coming arrivals (lane i: slot wb + i)
@@ -3277,331 +2882,11 @@ fast_run_kernel(FastArgs A) {
         __syncwarp();
     }
 
-    // ================================================================ list mode
-    if (c < n && !failed) {
-        if (lane == 0) s_job.type = FAST_JOB_REBUILD;
-        __syncwarp();
-        named_bar(1, KLPM_FAST_THREADS);
-        {
-            const FastJob J = s_job;
-            fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
-        }
-        root = tour_top(R, lane);
-        // the sorted list, 32 entries at a time: lane l holds entry (cur & ~31) + l, the next 32 are on their way
-        int32_t cur = 0;
-        auto window = [&](int32_t base, long long* wk_, int32_t* ws_) {
-            const long long i = (long long)base + lane;
-            *wk_ = i < n ? __ldg(A.lk + i) : INF;
-            *ws_ = i < n ? __ldg(A.ls + i) : -1;
-        };
-        long long wk, nk; int32_t ws, ns;
-        window(0, &wk, &ws);
-        window(32, &nk, &ns);
-        auto advance_cur = [&]() {
-            ++cur;
-            if ((cur & 31) == 0) { wk = nk; ws = ns; window(cur + 32, &nk, &ns); }
-        };
-        // From here on the time of a decision influences no decision, so the loop only records which slot each
-        // decision takes (in `order`); the charge pass after the loop turns that into query indices, uncached tokens,
-        // completion times and TTFTs (Definition 2 with R_prev >= t_j is a running sum of the costs).
-        if (lane == 0) { A.post->c0 = c; A.post->now0 = now; }
-        int32_t myj = 0;
-        // Up to 32 decisions at once.  As long as nothing interferes, the coming longest-match picks are the next
-        // entries of the list that still count and the coming oldest-first picks are the next unprocessed slots,
-        // interleaved as the policy says.  The warp gathers both sets side by side and checks that they cannot
-        // have influenced each other: no slot in both (a list entry inside the range of slots the oldest-first
-        // picks consume), none whose group has other members, none whose key sits in the tournament, and the
-        // tournament's root below the smallest key taken from the list.  The batch is cut before the first decision
-        // that fails a check; then lane i makes decision c + i.  If fewer than two decisions are left that way,
-        // nothing has been changed and the next decisions are made one at a time below.
-        const int32_t lane_div_k = lane / A.k;              // y / k for y = 0..31, looked up by shuffle
-        bool tb_cut = false;                                // the last warp-wide step stopped before a decision it could not take
-        auto try_batch = [&]() -> bool {
-            // oldest-first turns among the next x decisions, for x = lane (f_lo) and x = lane + 1 (f_hi): under k-LPM
-            // the first such turn is decision i0 = (k - cyc) mod k, then every k-th
-            int32_t f_lo, f_hi;
-            if (A.policy == KLPM_POLICY_FCFS) { f_lo = lane; f_hi = lane + 1; }
-            else if (A.policy == KLPM_POLICY_LPM) { f_lo = 0; f_hi = 0; }
-            else {
-                const int32_t i0 = cyc == 0 ? 0 : A.k - cyc;
-                const int32_t y_lo = lane - i0 - 1, y_hi = lane - i0;
-                const int32_t q_lo = __shfl_sync(FULL_MASK, lane_div_k, y_lo > 0 ? y_lo : 0);
-                const int32_t q_hi = __shfl_sync(FULL_MASK, lane_div_k, y_hi > 0 ? y_hi : 0);
-                f_lo = y_lo >= 0 ? q_lo + 1 : 0;
-                f_hi = y_hi >= 0 ? q_hi + 1 : 0;
-            }
-            // the list entries cur .. cur + 31 (in this window or the next) that still count
-            long long kk; int32_t es; unsigned mask;
-            {
-                const int32_t off = (cur & 31) + lane;
-                const long long k0 = __shfl_sync(FULL_MASK, wk, off & 31), k1 = __shfl_sync(FULL_MASK, nk, off & 31);
-                const int32_t s0 = __shfl_sync(FULL_MASK, ws, off & 31), s1 = __shfl_sync(FULL_MASK, ns, off & 31);
-                kk = off < 32 ? k0 : k1;
-                es = off < 32 ? s0 : s1;
-                const bool valid = (long long)cur + lane < n;
-                mask = __ballot_sync(FULL_MASK, valid && !((bm_ld(R.skip, es >> 5, gbits) >> (es & 31)) & 1u));
-            }
-            // as many decisions as those entries allow: lane x asks whether x + 1 decisions need no more of them
-            const int32_t avail = __popc(mask);
-            const int32_t B0 = __popc(__ballot_sync(FULL_MASK, c + lane < n && (lane + 1) - f_hi <= avail));
-            if (B0 < 2) return false;
-            const int32_t nF0 = __shfl_sync(FULL_MASK, f_hi, B0 - 1), nL0 = B0 - nF0;
-            // the next nF0 unprocessed slots; limF = how many of them can be taken before one needs the careful step
-            int32_t hs = -1, hmax0 = -1, limF = nF0;
-            if (nF0 > 0) {
-                const int32_t w0 = head >> 5;
-                const int32_t qk = lane < nF0 ? lane : nF0 - 1;       // lane q looks for the q-th unprocessed slot
-                auto free_word = [&](int32_t wi) -> unsigned {        // unprocessed slots of bitmap word wi, from head on
-                    unsigned w = wi < nwords ? bm_ld(s_done, wi, gdone) : 0xffffffffu;
-                    if (wi == nwords - 1 && (n & 31)) w |= ~((1u << (n & 31)) - 1u);
-                    if (wi == w0) w |= (1u << (head & 31)) - 1u;
-                    return ~w;
-                };
-                const unsigned f0 = free_word(w0), f1 = free_word(w0 + 1);
-                const int32_t c0 = __popc(f0);
-                if (c0 + __popc(f1) >= nF0) {                         // the usual case: they are all in the first two words
-                    hs = qk < c0 ? w0 * 32 + kth_set_bit(f0, qk + 1) : (w0 + 1) * 32 + kth_set_bit(f1, qk - c0 + 1);
-                } else {                                              // up to 32 words: running counts, then a search per lane
-                    const unsigned fr = free_word(w0 + lane);
-                    const int32_t cnt = __popc(fr);
-                    int32_t inc = cnt;
-#pragma unroll
-                    for (int dlt = 1; dlt < 32; dlt <<= 1) { const int32_t o = __shfl_up_sync(FULL_MASK, inc, dlt); if (lane >= dlt) inc += o; }
-                    if (__shfl_sync(FULL_MASK, inc, 31) < nF0) return false;
-                    int L = 0;
-#pragma unroll
-                    for (int step = 16; step > 0; step >>= 1) if (__shfl_sync(FULL_MASK, inc, L + step - 1) <= qk) L += step;
-                    const unsigned frL = __shfl_sync(FULL_MASK, fr, L);
-                    const int32_t preL = __shfl_sync(FULL_MASK, inc - cnt, L);
-                    hs = (w0 + L) * 32 + kth_set_bit(frL, qk - preL + 1);
-                }
-                hmax0 = __shfl_sync(FULL_MASK, hs, nF0 - 1);
-                // its key sits in the tournament, or its group has other members
-                const unsigned badH = __ballot_sync(FULL_MASK, lane < nF0 && ((((bm_ld(R.skip, hs >> 5, gbits) | bm_ld(R.gb, hs >> 5, gbits)) >> (hs & 31)) & 1u)));
-                if (badH) limF = __ffs(badH) - 1;
-            }
-            // limL = how many list entries can be taken before one is grouped, could also be an oldest-first pick of
-            // this batch, or has a key below the tournament's root
-            const bool ok = (mask >> lane) & 1u;
-            const int32_t rank = __popc(mask & ((1u << lane) - 1u));
-            int32_t limL = nL0;
-            int32_t soft = -1;                              // slot of the entry that stops the batch, if it is only suspected of being an oldest-first pick too
-            {
-                const unsigned long long ek = ~((unsigned long long)kk ^ 0x8000000000000000ULL);
-                const bool hard = (((bm_ld(R.gb, es >> 5, gbits) >> (es & 31)) & 1u)) || root > ek;
-                const unsigned badE = __ballot_sync(FULL_MASK, ok && rank < nL0 && (hard || (es >= head && es <= hmax0)));
-                if (badE) {
-                    const int src = __ffs(badE) - 1;
-                    limL = __popc(mask & ((1u << src) - 1u));
-                    if (!__shfl_sync(FULL_MASK, (int)hard, src)) soft = __shfl_sync(FULL_MASK, es, src);
-                }
-            }
-            int32_t B = __popc(__ballot_sync(FULL_MASK, lane < B0 && f_hi <= limF && (lane + 1) - f_hi <= limL));
-            if (soft >= 0 && B < B0 && B < 32) {
-                // the decision after the batch (lane B's): if it is the longest-match turn that takes that entry and the
-                // oldest-first picks made until then all lie before its slot, it becomes the batch's last decision
-                const int32_t fl = __shfl_sync(FULL_MASK, f_lo, B), fh = __shfl_sync(FULL_MASK, f_hi, B);
-                const int32_t last_h = __shfl_sync(FULL_MASK, hs, fl > 0 ? fl - 1 : 0);
-                if (fh == fl && B - fl == limL && fl <= limF && (fl == 0 || last_h < soft)) { ++B; ++limL; }
-            }
-            if (B < 2) return false;
-            tb_cut = B < B0 && soft < 0;
-            const int32_t nF = __shfl_sync(FULL_MASK, f_hi, B - 1), nL = B - nF;
-            const int32_t hmax = nF > 0 ? __shfl_sync(FULL_MASK, hs, nF - 1) : -1;
-            if (lane < nF) s_H[lane] = hs;
-            int32_t consumed = 0;
-            if (nL > 0) {
-                consumed = kth_set_bit(mask, nL) + 1;
-                if (ok && rank < nL) s_E[rank] = es;
-            }
-            __syncwarp();
-            // commit: lane i makes decision c + i
-            if (lane < B) {
-                myj = f_hi > f_lo ? s_H[f_lo] : s_E[lane - f_lo];
-                atomicOr(s_done + (myj >> 5), 1u << (myj & 31));
-                atomicOr(R.skip + (myj >> 5), 1u << (myj & 31));
-            }
-            __syncwarp();
-            if (lane < B) A.order[c + lane] = myj;
-            c += B;
-            if (A.policy == KLPM_POLICY_KLPM) cyc = (cyc + B) % A.k;
-            if (consumed) {
-                const int32_t ncur = cur + consumed;
-                if ((ncur >> 5) != (cur >> 5)) { wk = nk; ws = ns; window((ncur & ~31) + 32, &nk, &ns); }
-                cur = ncur;
-            }
-            if (nF > 0) { head = hmax; advance_head(); }
-            else if (head < n && ((bm_ld(s_done, head >> 5, gdone) >> (head & 31)) & 1u)) advance_head();
-            return true;
-        };
-        int32_t vb_wait = 0, vb_back = 1;                   // decisions until the next attempt; doubles while attempts fail
-        int32_t cb_wait = 0, cb_back = 8;                   // the same for the CTA-wide batch (loop iterations; 8 .. 1,024)
-        int32_t cb_until = 0, cb_fail = 0;                  // after an attempt that made no decision: not before decision cb_until; attempts failed in a row
-        if (lane == 0) s_bio.wide = 0;
-        int32_t per_now = 4;
-        int32_t calm_until = 0;
-        int32_t calm = KLPM_FAST_CALM;                      // consecutive full warp-wide steps: the CTA-wide batch is tried in calm water only
-        long long n_cta_try = 0, n_cta_ok = 0, dec_cta = 0, n_warp_ok = 0, dec_warp = 0, dec_one = 0, cy_cta = 0, cy_warp = 0;
-        // a batch that was cut short stopped before a decision only the one-at-a-time path can take: that one comes
-        // next, without another attempt that would find it again
-        bool one_next = false;
-        // Is playing batches through better than what happens between CTA-wide attempts?  Where the two orders block each
-        // other that is one decision at a time, where they merely meet often it is full warp-wide steps (110 cycles a decision), and
-        // then playing can cost five times as much (1,000 queries on 64 long prefixes: 408 us, now 255).
-        // What the stretches between attempts have cost is kept (the older half fades), and what the last played batch
-        // has, its 9,000 fixed cycles spread over 128 decisions.  A dear batch ends after 128 decisions, the first one after 64,
-        // and a warp-wide step is tried after it, unless that is known to cost more than twice as much.
-        int32_t probe = 0;
-        if (lane == 0) {
-            s_bio.alt_cy = 0; s_bio.alt_dec = 0; s_bio.play_cpd = 0; s_bio.t_out = (unsigned)clock();
-            s_bio.c_out = c; s_bio.play_next = 64; s_bio.probe = 0;
-        }
-        long long iters = 0;                                // every iteration makes a decision or gives up an attempt for a while
-        while (c < n && !failed) {
-            if (++iters > 64LL * n + 4096) { if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 118); failed = true; break; }      // cannot happen
-            // first choice: the whole CTA makes up to 1,024 decisions (the sort scratch is free between dissolves)
-            if (!one_next && probe <= 0 && cb_wait <= 0 && (calm >= KLPM_FAST_CALM || c >= calm_until) && c >= cb_until && n - c >= KLPM_FAST_CTA_MIN) {
-                if (lane == 0) {
-                    unsigned acy = s_bio.alt_cy, adec = s_bio.alt_dec;
-                    if (c > s_bio.c_out) {
-                        acy += (unsigned)clock() - s_bio.t_out; adec += (unsigned)(c - s_bio.c_out);
-                        if (adec > 512u) { acy >>= 1; adec >>= 1; }
-                        s_bio.alt_cy = acy; s_bio.alt_dec = adec;
-                    }
-                    const unsigned cpd = s_bio.play_cpd > 130u ? s_bio.play_cpd : 130u;
-                    const bool may_play = adec == 0 || acy / adec >= cpd;
-                    s_bio.play_max = may_play ? s_bio.play_next : 0;
-                    if (!may_play) s_bio.wide = 0;
-                    s_bio.per = per_now; s_bio.cur = cur; s_bio.head = head; s_bio.c = c; s_bio.cyc = cyc; s_bio.root = root; s_bio.B = 0;
-                    s_job.type = FAST_JOB_BATCH;
-                }
-                __syncwarp();
-                const long long t_cta = clock64();
-                ++n_cta_try;
-                named_bar(1, KLPM_FAST_THREADS);
-                fast_batch_job<G>(A, R, &s_bio, sr, sr + 1024, sr + 2048, reinterpret_cast<int32_t*>(sh), s_scan, nwords);
-                const int32_t Bc = s_bio.B;
-                const long long cy_this = clock64() - t_cta;
-                cy_cta += cy_this;
-                if (lane == 0) { s_bio.t_out = (unsigned)clock(); s_bio.c_out = c + Bc; }
-                if (Bc > 0) {
-                    if (s_bio.played) {
-                        if (lane == 0) {
-                            const unsigned cpd = (cy_this > 9000 ? (unsigned)(cy_this - 9000) / (unsigned)Bc : 0u) + 70u;
-                            const bool ahead = s_bio.alt_dec >= 16u && s_bio.alt_cy / s_bio.alt_dec >= 2u * cpd;      // (still the better half)
-                            s_bio.play_cpd = cpd; s_bio.play_next = ahead ? KLPM_FAST_CTA_BATCH : 128;
-                            s_bio.probe = cpd > KLPM_FAST_DEAR + 70 && !ahead ? 1 : 0;
-                        }
-                        __syncwarp();
-                        probe = s_bio.probe;
-                    }
-                    ++n_cta_ok; dec_cta += Bc;
-                    per_now = s_bio.wide || Bc >= (per_now == 1 ? 224 : 160) ? 4 : 1;
-                    const int32_t consumed = s_bio.consumed, hmax = s_bio.hmax;
-                    c += Bc;
-                    one_next = s_bio.hard != 0;
-                    if (A.policy == KLPM_POLICY_KLPM) cyc = (cyc + Bc) % A.k;
-                    if (consumed) { cur += consumed; window(cur & ~31, &wk, &ws); window((cur & ~31) + 32, &nk, &ns); }
-                    if (hmax >= 0) { head = hmax; advance_head(); }
-                    else if (head < n && ((bm_ld(s_done, head >> 5, gdone) >> (head & 31)) & 1u)) advance_head();
-                    // did it pay?  its cycles per decision against what the warp-wide steps have cost per decision so far
-                    const long long warp_cpd = dec_warp >= 256 ? cy_warp / dec_warp : 100;
-                    if (s_bio.played /* judged above */ || cy_this <= (long long)Bc * warp_cpd) { cb_back = 8; cb_fail = 0; continue; }
-                    // committed, but too short to have paid for the attempt: warp-wide steps for a while, as after a failure
-                    cb_wait = cb_back;
-                    cb_back = cb_back < KLPM_FAST_CB_MAX ? cb_back * 2 : KLPM_FAST_CB_MAX;
-                    calm = 0; calm_until = c + 64;
-                    continue;
-                }
-                per_now = 1; calm_until = c + 64;
-                // too few decisions before one that needs the one-at-a-time path: the next attempt waits until that one has
-                // been made (and longer when attempts keep failing: such decisions come in runs)
-                cb_until = c + s_bio.Braw + 1 + (cb_fail > 0 ? (8 << cb_fail) : 0);
-                if (cb_fail < KLPM_FAST_FAIL_CAP) ++cb_fail;
-            }
-            --cb_wait;
-            const bool probing = !one_next && probe > 0;
-            if (probing) --probe;
-            if (!one_next && vb_wait <= 0) {
-                const int32_t c_was = c;
-                const long long t_w = clock64();
-                const bool took = try_batch();
-                cy_warp += clock64() - t_w;
-                if (took) { ++n_warp_ok; dec_warp += c - c_was; vb_back = 1; if (c - c_was == 32) ++calm; else if (!probing) { if (calm > 0) calm_until = c + 64; calm = 0; } one_next = tb_cut; continue; }
-                if (!probing) {
-                    if (calm > 0) calm_until = c + 64;      // (where warp-wide steps keep failing the whole CTA may do better)
-                    calm = 0;
-                }
-                vb_wait = vb_back;
-                vb_back = vb_back < 64 ? vb_back * 2 : 64;
-            }
-            if (!one_next) --vb_wait;
-            one_next = false;
-            ++dec_one;
-            const bool fcfs_turn = A.policy == KLPM_POLICY_FCFS || (A.policy == KLPM_POLICY_KLPM && cyc == 0);
-            if (++cyc == A.k) cyc = 0;
-            int32_t j;
-            bool in_tour;                                   // the pick's key is in the tournament (it changed after the sort)
-            if (fcfs_turn) {
-                j = head;
-                in_tour = (bm_ld(R.skip, j >> 5, gbits) >> (j & 31)) & 1u;
-            } else {
-                unsigned long long ek = 0;                  // next entry of the list that still counts
-                int32_t es = -1;
-                while (cur < n) {                           // (a window's 32 entries are examined at once: stale entries come in runs)
-                    const int32_t wbase = cur & ~31;
-                    const bool usable = lane >= (cur & 31) && (long long)wbase + lane < n && !((bm_ld(R.skip, ws >> 5, gbits) >> (ws & 31)) & 1u);
-                    const unsigned bal = __ballot_sync(FULL_MASK, usable);
-                    if (bal) {
-                        const int src = __ffs(bal) - 1;
-                        cur = wbase + src;
-                        const long long kk = __shfl_sync(FULL_MASK, wk, src);
-                        es = __shfl_sync(FULL_MASK, ws, src);
-                        ek = ~((unsigned long long)kk ^ 0x8000000000000000ULL);
-                        break;
-                    }
-                    cur = wbase + 32; wk = nk; ws = ns; window(cur + 32, &nk, &ns);
-                }
-                if (cur > n) cur = n;
-                if (root > ek) {
-                    const unsigned rk = 0xffffffffu - (unsigned)(root & 0xffffffffULL);
-                    j = A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
-                    in_tour = true;
-                } else {
-                    j = es;
-                    in_tour = false;
-                    advance_cur();
-                }
-            }
-            if (j < 0 || j >= n || ((bm_ld(s_done, j >> 5, gdone) >> (j & 31)) & 1u)) { if (lane == 0) set_status(A.st, RT_ERR_LIMIT, 107); failed = true; break; }   // cannot happen
-            mark_done(j);
-            if (in_tour) {                                  // its leaf block's largest changed key, without it
-                const int32_t b = j >> A.lb_shift;
-                unsigned long long kk;
-                if (!G && A.lb_shift == 5) {                // 32-slot blocks, bitmaps in shared memory: one word of each
-                    const unsigned w = R.skip[b] & ~s_done[b];
-                    kk = warp_max64r(((w >> lane) & 1u) ? __ldcg(A.key + ((long long)b << 5) + lane) : 0ULL);
-                } else {
-                    kk = changed_block_max(A, R, b, lane);
-                }
-                root = tour_set(R, b, kk, lane);
-            }
-            if (j == head) advance_head();
-            if ((bm_ld(R.gb, j >> 5, gbits) >> (j & 31)) & 1u) {
-                careful(j, false, ld_dyn(A.dyn + j), ld_stat(A.stat + j));
-            } else {
-                if (lane == 0) A.order[c] = j;
-                ++c;
-            }
-        }
-        if (lane == 0) {
-            long long* cn = A.post->counters;
-            cn[8] = n_cta_try; cn[9] = n_cta_ok; cn[10] = dec_cta; cn[11] = n_warp_ok; cn[12] = dec_warp; cn[13] = dec_one;
-            cn[14] = cy_cta; cn[15] = cy_warp;
-        }
-    } else if (lane == 0) {
-        A.post->c0 = A.fixed ? 0 : n;                       // list mode never began: nothing is left to charge (a given order: everything)
-        A.post->now0 = now;
+    // ---- everybody has arrived: list_run_kernel goes on from here
+    if (lane == 0) {
+        A.post->c0 = A.fixed ? 0 : failed ? n : c;          // (a given order: everything is charged after the loop)
+        A.post->list_c = A.fixed || failed ? n : c;
+        A.post->now0 = now; A.post->head = head; A.post->cyc = cyc;
         for (int i = 8; i < 16; ++i) A.post->counters[i] = 0;
     }
     __syncwarp();
@@ -3609,9 +2894,707 @@ fast_run_kernel(FastArgs A) {
         long long* cn = A.post->counters;
         cn[0] = n_careful; cn[1] = n_cta_dissolve; cn[2] = 0; cn[3] = 0; cn[4] = 0; cn[5] = 0; cn[6] = 0; cn[7] = cy_dissolve;
     }
-    if (lane == 0) s_job.type = FAST_JOB_EXIT;
+    if (lane == 0) { s_job.type = FAST_JOB_EXIT; s_job.a0 = A.list_mode && !failed && c < n; }
     __syncwarp();
     named_bar(1, KLPM_FAST_THREADS);
+}
+
+// ------------------------------------------------------------------------------------------------
+// List mode: everybody has arrived.  The time of a pick no longer decides who can be picked, so the decisions are a merge
+// of two orders that are known: the oldest-first turns take the next unprocessed slot, the longest-match turns the next entry
+// of the sorted key list that is unprocessed and whose key has not changed since the sort -- or the root of the
+// tournament, which holds the slots whose key has changed, where that is larger.  Which turn is which is fixed by the
+// policy.  One CTA goes through the two orders a window at a time (2,048 unprocessed slots, 2,048 list positions) and
+// works out who takes what by iteration:
+//   * a slot that only one of the two sides has in its window is taken by that side, at the turn that its rank among
+//     the side's picks gives it;
+//   * a slot that both sides have (a meeting) is taken by whichever reaches it first.  Given for every meeting a guess of
+//     who takes it, prefix sums over one bit per slot and side give both its ranks, those both its turns, and those a new
+//     guess.  Let T be the earliest turn at which a meeting whose guess has changed would be taken.  Then every decision
+//     before T is final: by induction over the turns, the ranks of whoever is taken at t depend only on the guesses of
+//     slots that are taken before t.  So every round settles at least one turn more, and a few settle a window;
+//   * only where the two orders agree for a stretch (one match length left, ties by arrival) does a round settle just one
+//     or two turns: every guess there hangs on the one before.  But then the next decisions are that common order, whoever
+//     makes them: R decisions, if the unprocessed slots and the live list entries have their first R elements in common.
+// A decision is made outside this scheme only where it changes a key or follows from one (a step): the pick's group has
+// other members, its key sits in the tournament, or the tournament's root beats the list.  The window goes on after it;
+// only a group dissolved by the whole CTA takes its memory.
+// Decisions are recorded as slots in `order`; the charge pass after the loop computes their outputs.
+// What bounds it: the barriers and shared-memory round trips of one CTA: about 1,500 cycles per round, 6,000 per step with the
+// batch before it, 8,000 per window.  klpm_run of 32,768 / 65,536 / 262,144 waiting queries (medium, hierarchical, adversarial): 0.64 / 2.6 /
+// 3.0 ms in this kernel; batches of up to 1,024 decisions cut at every decision that touches a group, whose meetings one
+// warp resolved one after the other (or played through decision by decision), took 1.39 / 4.1 / 3.9.
+// G: some of the loop's bitmaps live in global memory (queues too long for shared memory).
+#define KLPM_LIST_THREADS 512
+#define KLPM_LIST_WIN 2048            // (4 per thread, 64 words of one bit each: two per lane of a warp)
+#define KLPM_LIST_ROUNDS 16           // rounds on one state of the window before what is settled is committed
+#define KLPM_LIST_AGREE 24            // stretches shorter than this are left to the rounds
+#define KLPM_LIST_FAR 0x3ffffff
+struct ListWin {                      // the window, in the scratch of the sorts
+    int32_t* fs;                      // unprocessed slots, oldest first
+    int32_t* ls; long long* lk;       // list positions from `cur` on: slot, key as the list holds it
+    unsigned* col;                    // meetings: index in fs | position << 16
+    int32_t* fp; unsigned* fw;        // per bitmap word from head on: free slots before it, free slots
+    uint2 *F, *L;                     // per 32 indices / positions: one bit each, taken by this side (as guessed, for a meeting); such bits before
+    unsigned *LF, *LL;                // still there
+    unsigned *EF, *EL;                // needs a step of its own
+    unsigned* eq;                     // agreement, one bit per rank
+};
+struct ListShared {
+    int4 pre[2][4];                              // records of lcp_kernel's pairs for the last four steps found on either side, on their way since then
+    int32_t pre_n[2], pre_slot[2][4];
+    int32_t head, cur, job, made, failed;
+    int32_t ncol;
+    int32_t tot_f, tot_l, ev_f, ev_l, ev_r;      // picks of either side in the window; ranks of the first that needs a step, of the first list entry below the root
+    int32_t ix_f, ix_l;                          // index / position of those two
+    int32_t tstar[2];
+    int32_t step_f, step_l, mate_f, mate;        // what a step took (index, position) and changed (index, slot); -1: nothing
+    unsigned long long root;
+    int32_t w[KLPM_LIST_THREADS / 32];
+};
+static_assert(KLPM_LIST_WIN * (4 + 4 + 8 + 4) + KLPM_LIST_THREADS * 8 + 9 * (KLPM_LIST_WIN / 32) * 4 <= KLPM_FAST_SORT_CAP * 12, "a window fits the sort scratch");
+
+// first set bit of a bitmap of 64 words, or -1.  One warp.
+__device__ __forceinline__ int32_t list_first(const unsigned* w, int lane) {
+    const unsigned a = w[2 * lane], b = w[2 * lane + 1];
+    const unsigned m = __ballot_sync(FULL_MASK, (a | b) != 0u);
+    if (!m) return -1;
+    const int src = __ffs(m) - 1;
+    const unsigned x = __shfl_sync(FULL_MASK, a, src), y = __shfl_sync(FULL_MASK, b, src);
+    return src * 64 + (x ? __ffs(x) - 1 : 31 + __ffs(y));
+}
+// Bits before each word of a bitmap of 64 words; returns the number of set bits.  One warp.
+__device__ __forceinline__ int32_t list_prefix(uint2* w, int lane, unsigned* a, unsigned* b, int32_t* before) {
+    const uint4 v = reinterpret_cast<uint4*>(w)[lane];
+    const int32_t ca = __popc(v.x), both = ca + __popc(v.z);
+    int32_t inc = both;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const int32_t o = __shfl_up_sync(FULL_MASK, inc, d); if (lane >= d) inc += o; }
+    *a = v.x; *b = v.z; *before = inc - both;
+    reinterpret_cast<uint4*>(w)[lane] = make_uint4(v.x, (unsigned)(inc - both), v.z, (unsigned)(inc - both + ca));
+    return __shfl_sync(FULL_MASK, inc, 31);
+}
+// The first of the flagged bits (fa, fb: this lane's two words of the flags, already masked by a, b): its position, and its rank among the
+// bits of (a, b).  One warp; position -1: none.
+__device__ __forceinline__ int32_t list_event(unsigned fa, unsigned fb, unsigned a, unsigned b, int32_t before, int lane, int32_t* at) {
+    const unsigned m = __ballot_sync(FULL_MASK, (fa | fb) != 0u);
+    if (!m) { *at = -1; return KLPM_LIST_FAR; }
+    int32_t pos, rank;
+    if (fa) { const int f = __ffs(fa) - 1; pos = 64 * lane + f; rank = before + __popc(a & ((1u << f) - 1u)); }
+    else { const int f = fb ? __ffs(fb) - 1 : 0; pos = 64 * lane + 32 + f; rank = before + __popc(a) + __popc(b & ((1u << f) - 1u)); }
+    const int src = __ffs(m) - 1;
+    *at = __shfl_sync(FULL_MASK, pos, src);
+    return __shfl_sync(FULL_MASK, rank, src);
+}
+// 16 bytes from global to shared memory without waiting for them
+__device__ __forceinline__ void list_fetch16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void list_fetch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+template <bool G>
+__global__ void __launch_bounds__(KLPM_LIST_THREADS, 1)
+list_run_kernel(FastArgs A) {
+    extern __shared__ __align__(16) unsigned char fast_smem[];
+    __shared__ FastJob s_job;
+    __shared__ int s_cnt;
+    __shared__ int32_t s_memcur;
+    __shared__ ListShared S;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int NW = KLPM_LIST_THREADS / 32, WORDS = KLPM_LIST_WIN / 32, PER = KLPM_LIST_WIN / KLPM_LIST_THREADS;
+    const int32_t n = A.n;
+    int32_t c = A.post->list_c, cyc = A.post->cyc;
+    if (c >= n) return;
+    // ---- shared memory as in fast_run_kernel: tournament, sort scratch (here also the window), bitmaps
+    const int32_t nb1p = (A.nb + 31) & ~31, n2 = nb1p >> 5, n2p = (n2 + 31) & ~31, n3 = n2p >> 5;
+    const int32_t nwords = (n + 31) >> 5;
+    FastTour R;
+    R.t1 = reinterpret_cast<unsigned long long*>(fast_smem);
+    R.t2 = R.t1 + nb1p;
+    R.t3 = R.t2 + n2p;
+    R.n2 = n2; R.n3 = n3;
+    unsigned long long* sh = R.t3 + 32;
+    int32_t* sr = reinterpret_cast<int32_t*>(sh + KLPM_FAST_SORT_CAP);
+    unsigned int* s_bits = reinterpret_cast<unsigned int*>(sr + KLPM_FAST_SORT_CAP);
+    R.g_done = !G || A.done_in_smem ? 0 : 1;
+    R.g_bits = !G || A.bits_in_smem ? 0 : 1;
+    R.done = A.done_in_smem ? s_bits : A.done;
+    R.skip = A.bits_in_smem ? s_bits + nwords : A.gskip;
+    R.gb = A.bits_in_smem ? s_bits + 2 * nwords : A.gbits;
+    R.dirty = nullptr;
+    const int gdone = G ? R.g_done : 0, gbits = G ? R.g_bits : 0;
+    ListWin W;
+    W.lk = reinterpret_cast<long long*>(sh);
+    W.fs = reinterpret_cast<int32_t*>(W.lk + KLPM_LIST_WIN);
+    W.ls = W.fs + KLPM_LIST_WIN;
+    W.col = reinterpret_cast<unsigned*>(W.ls + KLPM_LIST_WIN);
+    W.fp = reinterpret_cast<int32_t*>(W.col + KLPM_LIST_WIN);
+    W.fw = reinterpret_cast<unsigned*>(W.fp + KLPM_LIST_THREADS);
+    W.F = reinterpret_cast<uint2*>(W.fw + KLPM_LIST_THREADS); W.L = W.F + WORDS;
+    W.LF = reinterpret_cast<unsigned*>(W.L + WORDS); W.LL = W.LF + WORDS; W.EF = W.LL + WORDS; W.EL = W.EF + WORDS; W.eq = W.EL + WORDS;
+    for (int32_t i = tid; i < nb1p + n2p + 32; i += KLPM_LIST_THREADS) R.t1[i] = 0ULL;
+    if (tid == 0) {
+        s_memcur = n;
+        S.head = A.post->head; S.cur = 0; S.root = 0ULL; S.failed = 0; S.job = 0; S.pre_n[0] = 0; S.pre_n[1] = 0;
+    }
+    if (A.done_in_smem) for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) R.done[i] = c > 0 ? __ldcg(A.done + i) : 0u;
+    for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {      // (the list passes over processed slots, so far)
+        R.skip[i] = c > 0 ? __ldcg(A.done + i) : 0u;
+        if (A.bits_in_smem) R.gb[i] = __ldcg(A.gbits + i);
+    }
+    __syncthreads();
+    auto bit_of = [&](const unsigned* bm, int32_t slot, int g) -> unsigned { return (bm_ld(bm, slot >> 5, g) >> (slot & 31)) & 1u; };
+    // ---- turns, counted from the next decision: the t-th oldest-first turn, the u-th longest-match turn, oldest-first turns among x decisions.
+    // (a k beyond what a window holds is as good as any such k)
+    const bool use_f = A.policy != KLPM_POLICY_LPM;
+    const bool use_l = A.policy == KLPM_POLICY_LPM || (A.policy == KLPM_POLICY_KLPM && A.k >= 2);
+    const int32_t kk = A.policy == KLPM_POLICY_KLPM ? (A.k < 8192 ? A.k : 8192) : 1;
+    int32_t i0 = 0;                                         // the first oldest-first turn
+    auto set_i0 = [&]() {
+        if (!use_f) i0 = KLPM_LIST_FAR;
+        else if (A.policy == KLPM_POLICY_FCFS || cyc == 0) i0 = 0;
+        else i0 = A.k - cyc < KLPM_LIST_FAR / 2 ? A.k - cyc : KLPM_LIST_FAR / 2;
+    };
+    auto per_k1 = [&](int32_t u) -> int32_t { return A.k == 2 ? u : (int32_t)__umulhi((unsigned)u, A.recip_k1); };
+    auto f_turn = [&](int32_t t) -> int32_t { return use_f ? i0 + t * kk : KLPM_LIST_FAR; };
+    auto l_turn = [&](int32_t u) -> int32_t { return !use_l ? KLPM_LIST_FAR : u < i0 ? u : u + 1 + per_k1(u - i0); };
+    auto f_count = [&](int32_t x) -> int32_t { return !use_f || x <= i0 ? 0 : (x - i0 - 1) / kk + 1; };
+
+    // the oldest-first slots worth looking at: twice the turns that 2,048 list entries leave for them
+    const int32_t most_f = use_l && A.k > 2 && 2 * KLPM_LIST_WIN / (A.k - 1) + 128 < KLPM_LIST_WIN ? 2 * KLPM_LIST_WIN / (A.k - 1) + 128 : KLPM_LIST_WIN;
+    int32_t n_f = 0, n_l = 0;                               // the window: slots, list positions
+    bool list_end = false;                                  // it reaches the end of the list
+    int32_t w0 = 0, head0 = 0;                              // its first bitmap word and slot
+    unsigned cv[PER], alive = 0;                            // this thread's meetings; one bit each while both sides still have the slot
+#pragma unroll
+    for (int r = 0; r < PER; ++r) cv[r] = 0u;
+    // index of a slot among the window's oldest-first slots, or -1
+    auto index_of = [&](int32_t s) -> int32_t {
+        if (!use_f || n_f == 0 || s < head0 || s > W.fs[n_f - 1]) return -1;
+        const int32_t wl = (s >> 5) - w0;
+        const unsigned f = W.fw[wl];
+        const int32_t phi = W.fp[wl] + __popc(f & ((1u << (s & 31)) - 1u));
+        return ((f >> (s & 31)) & 1u) && phi < n_f ? phi : -1;
+    };
+    // Everything about the window's slots again, after a group has been dissolved.
+    auto refresh = [&]() {
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int w = warp + NW * r, i = w * 32 + lane;
+            const bool hf = (W.LF[w] >> lane) & 1u, hl = (W.LL[w] >> lane) & 1u;
+            const int32_t sf = hf ? W.fs[i] : 0, sl = hl ? W.ls[i] : 0;
+            const bool in_f = hf && !bit_of(R.done, sf, gdone), in_l = hl && !bit_of(R.skip, sl, gbits);
+            const unsigned lf = __ballot_sync(FULL_MASK, in_f), ll = __ballot_sync(FULL_MASK, in_l);
+            const unsigned ef = __ballot_sync(FULL_MASK, in_f && ((use_l ? bit_of(R.skip, sf, gbits) : 0u) | bit_of(R.gb, sf, gbits)));
+            const unsigned el = __ballot_sync(FULL_MASK, in_l && bit_of(R.gb, sl, gbits));
+            if (lane == 0) { W.LF[w] = lf; W.F[w].x &= lf; W.EF[w] = ef; W.LL[w] = ll; W.L[w].x &= ll; W.EL[w] = el; }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            if (!((alive >> r) & 1u)) continue;
+            const int32_t i = (int32_t)(cv[r] & 0xffffu), p = (int32_t)(cv[r] >> 16);
+            const bool lf = (W.LF[i >> 5] >> (i & 31)) & 1u, ll = (W.LL[p >> 5] >> (p & 31)) & 1u;
+            if (lf && ll) continue;
+            alive &= ~(1u << r);
+            if (lf) atomicOr(&W.F[i >> 5].x, 1u << (i & 31));      // its list entry has gone stale: the oldest-first side has it alone
+        }
+        __syncthreads();
+    };
+    auto build = [&]() {
+        int32_t cur = S.cur;
+        const int32_t head = S.head;
+        long long key_in[PER];
+        int32_t slot_in[PER];
+        w0 = head >> 5; head0 = head;
+        n_f = 0;
+        if (use_l) {
+            for (;;) {                                      // (a stretch of the list without a live entry is passed over)
+                int any = 0;
+#pragma unroll
+                for (int r = 0; r < PER; ++r) {
+                    const long long idx = (long long)cur + tid + KLPM_LIST_THREADS * r;
+                    slot_in[r] = idx < n ? __ldg(A.ls + idx) : -1;
+                    key_in[r] = idx < n ? __ldg(A.lk + idx) : 0LL;
+                }
+#pragma unroll
+                for (int r = 0; r < PER; ++r) {
+                    const int w = warp + NW * r;
+                    const bool in = slot_in[r] >= 0 && !bit_of(R.skip, slot_in[r], gbits);
+                    const unsigned live = __ballot_sync(FULL_MASK, in), ev = __ballot_sync(FULL_MASK, in && bit_of(R.gb, slot_in[r], gbits));
+                    if (lane == 0) { W.LL[w] = live; W.L[w].x = live; W.EL[w] = ev; }
+                    any |= live != 0u;
+                }
+                if (__syncthreads_or(any) || (long long)cur + KLPM_LIST_WIN >= n) break;
+                cur += KLPM_LIST_WIN;
+            }
+            n_l = n - cur < KLPM_LIST_WIN ? n - cur : KLPM_LIST_WIN;
+            list_end = (long long)cur + KLPM_LIST_WIN >= n;
+#pragma unroll
+            for (int r = 0; r < PER; ++r) { W.ls[tid + KLPM_LIST_THREADS * r] = slot_in[r]; W.lk[tid + KLPM_LIST_THREADS * r] = key_in[r]; }
+        } else {
+            if (tid < WORDS) { W.LL[tid] = 0u; W.L[tid].x = 0u; W.EL[tid] = 0u; }
+            n_l = 0; list_end = true;
+        }
+        if (use_f) {
+            const int32_t wi = w0 + tid;
+            unsigned w = wi < nwords ? bm_ld(R.done, wi, gdone) : 0xffffffffu;
+            if (wi == nwords - 1 && (n & 31)) w |= ~((1u << (n & 31)) - 1u);
+            if (wi == w0) w |= (1u << (head & 31)) - 1u;
+            const unsigned fr = ~w;
+            const int32_t cnt = __popc(fr);
+            int32_t inc = cnt;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) { const int32_t o = __shfl_up_sync(FULL_MASK, inc, d); if (lane >= d) inc += o; }
+            if (lane == 31) S.w[warp] = inc;
+            __syncthreads();
+            int32_t before = 0, all = 0;
+#pragma unroll
+            for (int v = 0; v < NW; ++v) { const int32_t x = S.w[v]; if (v < warp) before += x; all += x; }
+            W.fp[tid] = before + inc - cnt; W.fw[tid] = fr;
+            n_f = all < most_f ? all : most_f;
+            __syncthreads();
+            for (int32_t wl = warp; wl < KLPM_LIST_THREADS && W.fp[wl] < n_f; wl += NW) {
+                const unsigned f = W.fw[wl];
+                if ((f >> lane) & 1u) {
+                    const int32_t rank = W.fp[wl] + __popc(f & ((1u << lane) - 1u));
+                    if (rank < n_f) W.fs[rank] = (w0 + wl) * 32 + lane;
+                }
+            }
+        } else if (tid < WORDS) { W.LF[tid] = 0u; W.F[tid].x = 0u; W.EF[tid] = 0u; }
+        if (tid == 0) { S.ncol = 0; S.cur = cur; }
+        __syncthreads();
+        if (use_f) {
+#pragma unroll
+            for (int r = 0; r < PER; ++r) {
+                const int w = warp + NW * r, i = w * 32 + lane;
+                const bool in = i < n_f;
+                const int32_t s = in ? W.fs[i] : 0;
+                const unsigned live = __ballot_sync(FULL_MASK, in);
+                const unsigned ev = __ballot_sync(FULL_MASK, in && ((use_l ? bit_of(R.skip, s, gbits) : 0u) | bit_of(R.gb, s, gbits)));
+                if (lane == 0) { W.LF[w] = live; W.F[w].x = live; W.EF[w] = ev; }
+            }
+        }
+        if (use_f && use_l && n_f > 0) {                    // the meetings
+            const int32_t hmax = W.fs[n_f - 1];
+#pragma unroll
+            for (int r = 0; r < PER; ++r) {
+                const int32_t s = slot_in[r];
+                bool met = s >= head && s <= hmax && !bit_of(R.skip, s, gbits);
+                int32_t phi = 0;
+                if (met) {
+                    const int32_t wl = (s >> 5) - w0;       // (below KLPM_LIST_THREADS: hmax is)
+                    const unsigned f = W.fw[wl];
+                    phi = W.fp[wl] + __popc(f & ((1u << (s & 31)) - 1u));
+                    met = ((f >> (s & 31)) & 1u) && phi < n_f;
+                }
+                const unsigned bal = __ballot_sync(FULL_MASK, met);
+                if (bal) {
+                    int32_t base = 0;
+                    if (lane == __ffs(bal) - 1) base = atomicAdd(&S.ncol, __popc(bal));
+                    base = __shfl_sync(FULL_MASK, base, __ffs(bal) - 1);
+                    if (met) W.col[base + __popc(bal & ((1u << lane) - 1u))] = (unsigned)phi | (unsigned)(tid + KLPM_LIST_THREADS * r) << 16;
+                }
+            }
+        }
+        if (use_l) {                                        // the list behind this window, into L1 for the next one
+            const long long at = (long long)cur + KLPM_LIST_WIN;
+            if (tid < 128) { const long long e = at + tid * 16; if (e < n) asm volatile("prefetch.global.L1 [%0];" ::"l"(A.lk + e)); }
+            else if (tid < 192) { const long long e = at + (tid - 128) * 32; if (e < n) asm volatile("prefetch.global.L1 [%0];" ::"l"(A.ls + e)); }
+        }
+        __syncthreads();
+        const int32_t ncol = S.ncol;
+        alive = 0;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int32_t x = tid + KLPM_LIST_THREADS * r;
+            cv[r] = x < ncol ? W.col[x] : 0u;
+            if (x < ncol) alive |= 1u << r;
+        }
+    };
+    // Prefix sums of the guesses, and what ends a batch: the rank of the first pick of either side that needs a step, and of the first
+    // list entry that the tournament's root beats.  The caller synchronises.
+    auto ranks = [&]() {
+        if (warp < 2) {
+            unsigned a, b;
+            int32_t before, at;
+            uint2* const V = warp == 0 ? W.F : W.L;
+            const unsigned* const E = warp == 0 ? W.EF : W.EL;
+            const int32_t tot = list_prefix(V, lane, &a, &b, &before);
+            const int32_t ev = list_event(E[2 * lane] & a, E[2 * lane + 1] & b, a, b, before, lane, &at);
+            if (lane == 0) {
+                if (warp == 0) { S.tot_f = tot; S.ev_f = ev; S.ix_f = at; }
+                else { S.tot_l = tot; S.ev_l = ev; S.ix_l = at; }
+                if (at >= 0) {
+                    const int32_t slot = warp == 0 ? W.fs[at] : W.ls[at];
+                    const int32_t k = S.pre_n[warp];
+                    if (k == 0 || S.pre_slot[warp][(k - 1) & 3] != slot) {
+                        if ((k & 3) == 0) list_fetch_wait();
+                        S.pre_slot[warp][k & 3] = slot; S.pre_n[warp] = k + 1;
+                        list_fetch16(&S.pre[warp][k & 3], A.pair + slot);
+                    }
+                }
+            }
+        } else if (warp == 2) {
+            // the list holds ~key with the top bit flipped, ascending: the first position with a larger value than the root's
+            int32_t jr = n_l;
+            const unsigned long long root = S.root;
+            if (root != 0ULL && n_l > 0) {
+                const long long rk = (long long)(~root ^ 0x8000000000000000ULL);
+                const int32_t p = 64 * lane + 63 < n_l ? 64 * lane + 63 : n_l - 1;
+                const unsigned m = __ballot_sync(FULL_MASK, W.lk[p] > rk);
+                if (m) {
+                    const int32_t b0 = 64 * (__ffs(m) - 1), q = b0 + lane;
+                    const unsigned m0 = __ballot_sync(FULL_MASK, q < n_l && W.lk[q] > rk), m1 = __ballot_sync(FULL_MASK, q + 32 < n_l && W.lk[q + 32] > rk);
+                    jr = m0 ? b0 + __ffs(m0) - 1 : m1 ? b0 + 31 + __ffs(m1) : n_l;
+                }
+            }
+            // its picks before jr (the prefix sums are another warp's, at the same time)
+            int32_t cnt = 0;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int32_t w = 2 * lane + u, left = jr - 32 * w;
+                if (left > 0) cnt += __popc(left >= 32 ? W.L[w].x : W.L[w].x & ((1u << left) - 1u));
+            }
+            cnt = (int32_t)__reduce_add_sync(FULL_MASK, (unsigned)cnt);
+            if (lane == 0) S.ev_r = root != 0ULL && (jr < n_l || list_end) ? cnt : KLPM_LIST_FAR;
+        }
+    };
+    auto take = [&](int32_t slot, int32_t at) {
+        atomicOr(R.done + (slot >> 5), 1u << (slot & 31));
+        atomicOr(R.skip + (slot >> 5), 1u << (slot & 31));
+        A.order[c + at] = slot;
+    };
+    // Warp 0: one decision that needs a step -- the oldest slot (kind 0), the next list entry (1) or the tournament's root (2).
+    long long n_one = 0, n_dis = 0, cy_step = 0;
+    // `at`: its number.  Other warps commit the batch before it at the same time: what both change is changed by atomics.
+    auto one_step = [&](int kind, int32_t at, int32_t turn) {
+        const long long t0 = clock64();
+        unsigned long long root = S.root;
+        int32_t j;
+        if (kind == 2) {
+            const unsigned rk = 0xffffffffu - (unsigned)(root & 0xffffffffULL);
+            j = A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
+        } else j = kind == 0 ? W.fs[S.ix_f] : W.ls[S.ix_l];
+        if (j < 0 || j >= n || bit_of(R.done, j, gdone)) { if (lane == 0) { set_status(A.st, RT_ERR_LIMIT, 107); S.failed = 1; } return; }   // cannot happen
+        const bool in_tour = kind == 2 || (kind == 0 && use_l && bit_of(R.skip, j, gbits) != 0u);      // its key changed after the sort
+        const bool grouped = bit_of(R.gb, j, gbits) != 0u;
+        const int32_t step_f = kind == 0 ? S.ix_f : index_of(j);
+        int32_t mate_f = -1, mate_s = -1, job = 0;
+        bool both = false;                                  // the other one of a pair was taken right after it
+        __syncwarp();
+        if (lane == 0) {
+            atomicOr(R.done + (j >> 5), 1u << (j & 31));
+            if (!in_tour) atomicOr(R.skip + (j >> 5), 1u << (j & 31));
+            A.order[at] = j;
+        }
+        __syncwarp();
+        if (in_tour) {                                      // its leaf block's largest changed key, without it
+            const int32_t b = j >> A.lb_shift;
+            const bool alone = A.lb_shift == 5 && !(bm_ld(R.skip, b, gbits) & ~bm_ld(R.done, b, gdone));
+            root = tour_set(R, b, alone ? 0ULL : changed_block_max(A, R, b, lane), lane);
+            __syncwarp();
+        }
+        ++n_one;
+        if (grouped) {
+            ++n_dis;
+            int4 rec;
+            const int last = kind < 2 ? (S.pre_n[kind] - 1) & 3 : 0;      // (found by the round before this step)
+            if (kind < 2 && S.pre_slot[kind][last] == j) rec = S.pre[kind][last];
+            else rec = __ldcg(A.pair + j);
+            if (rec.x >= 0) {                               // one other prompt, and what becomes of it is known
+                mate_s = rec.x;
+                const unsigned long long key = (unsigned long long)(unsigned)rec.w << 32 | (unsigned)rec.z;
+                if (lane == 0) {
+                    __stcg(reinterpret_cast<int32_t*>(A.dyn + mate_s) + 2, rec.y);
+                    __stcg(A.key + mate_s, key);
+                    atomicOr(R.skip + (mate_s >> 5), 1u << (mate_s & 31));
+                    atomicAnd(R.gb + (mate_s >> 5), ~(1u << (mate_s & 31)));
+                    atomicAnd(R.gb + (j >> 5), ~(1u << (j & 31)));
+                }
+                mate_f = index_of(mate_s);
+                // Mostly the other one is the next longest-match pick: its key beats the entry just taken, and with it the rest of the list.
+                both = kind == 1 && at + 1 < n && key > root && key > ~((unsigned long long)W.lk[S.ix_l] ^ 0x8000000000000000ULL) &&
+                       (A.policy == KLPM_POLICY_LPM || (turn + 1) % A.k != 0);
+                if (both) {
+                    if (lane == 0) { atomicOr(R.done + (mate_s >> 5), 1u << (mate_s & 31)); A.order[at + 1] = mate_s; }
+                    ++n_one;
+                } else {
+                    const int32_t b = mate_s >> A.lb_shift;
+                    const unsigned long long p1 = R.t1[b], p2 = R.t2[b >> 5], p3 = R.t3[b >> 10];
+                    __syncwarp();
+                    R.t1[b] = key > p1 ? key : p1; R.t2[b >> 5] = key > p2 ? key : p2; R.t3[b >> 10] = key > p3 ? key : p3;      // (every lane stores the same)
+                    root = key > root ? key : root;
+                }
+                __syncwarp();
+            } else {
+                const FDyn d = ld_dyn(A.dyn + j);
+                const FStat s = ld_stat(A.stat + j);
+                if (s.len > d.m && d.gcount > 1) {
+                    FastPick P;
+                    P.slot = j; P.m = d.m; P.len = s.len; P.ntok = d.ntok; P.x = A.tok + s.soff; P.pos = d.pos; P.vleaf = A.vbase + ((long long)at << 32);
+                    P.admitted = n; P.gstart = d.gstart; P.gcount = d.gcount; P.leaf = -1;
+                    P.lcp = __ldcg(A.lcp + j);
+                    if (dissolve_is_small(P)) { root = dissolve_small(A, P, R, root, lane); job = 1; }      // (anything about the window's slots may have changed)
+                    else { job = 2; if (lane == 0) { s_job.type = FAST_JOB_DISSOLVE; s_job.pick = P; } }
+                    __syncwarp();
+                }
+            }
+        }
+        if (lane == 0) {
+            S.made = both ? 2 : 1;
+            S.root = root; S.job = job; S.step_f = step_f; S.step_l = kind == 1 ? S.ix_l : -1; S.mate_f = mate_f; S.mate = mate_s;
+            if (step_f >= 0) { atomicAnd(&W.LF[step_f >> 5], ~(1u << (step_f & 31))); atomicAnd(&W.F[step_f >> 5].x, ~(1u << (step_f & 31))); }
+            if (mate_f >= 0 && both) { atomicAnd(&W.LF[mate_f >> 5], ~(1u << (mate_f & 31))); atomicAnd(&W.F[mate_f >> 5].x, ~(1u << (mate_f & 31))); }
+            else if (mate_f >= 0) {
+                atomicOr(&W.F[mate_f >> 5].x, 1u << (mate_f & 31));
+                if (use_l) atomicOr(&W.EF[mate_f >> 5], 1u << (mate_f & 31));
+                else atomicAnd(&W.EF[mate_f >> 5], ~(1u << (mate_f & 31)));
+            }
+        }
+        cy_step += clock64() - t0;
+    };
+    // What the step leaves to do for the window, every thread: the list entries of the two slots, and their meetings.
+    auto after_step = [&]() {
+        const int32_t sf = S.step_f, mf = S.mate_f, ms = S.mate;
+        int32_t js = -2;
+        if (sf >= 0) js = W.fs[sf];
+        else if (S.step_l >= 0) js = W.ls[S.step_l];
+        if (use_l) {
+#pragma unroll
+            for (int r = 0; r < PER; ++r) {
+                const int32_t i = tid + KLPM_LIST_THREADS * r, s = W.ls[i];
+                if (s >= 0 && (s == js || s == ms)) { atomicAnd(&W.LL[i >> 5], ~(1u << (i & 31))); atomicAnd(&W.L[i >> 5].x, ~(1u << (i & 31))); }
+            }
+#pragma unroll
+            for (int r = 0; r < PER; ++r) {
+                const int32_t i = (int32_t)(cv[r] & 0xffffu);
+                if (i == sf || i == mf) alive &= ~(1u << r);
+            }
+        }
+        __syncthreads();
+    };
+    // Where the two orders stand, for the next window.
+    auto leave = [&]() {
+        if (warp == 0) {
+            int32_t head = S.head, cur = S.cur;
+            if (use_f && n_f > 0) {
+                const int32_t i = list_first(W.LF, lane);
+                head = i >= 0 ? W.fs[i] : next_head(R.done, gdone, nwords, n, W.fs[n_f - 1], lane);
+            }
+            if (use_l && n_l > 0) {
+                const int32_t j = list_first(W.LL, lane);
+                cur += j >= 0 ? j : n_l;
+            }
+            if (lane == 0) { S.head = head; S.cur = cur; }
+        }
+        __syncthreads();
+    };
+
+    bool fresh = true, agree = false;
+    int32_t agree_wait = 0, agree_back = 1;                 // batches until agreement is tried again; doubles while it fails
+    long long n_win = 0, n_run = 0, dec_run = 0, n_iter = 0, dec_iter = 0, cy_build = 0, n_cta_dissolve = 0, cy_dissolve = 0;
+    long long iters = 0;                                    // (every pass makes a decision, or a new window)
+    while (c < n) {
+        if (++iters > 64LL * n + 4096) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen
+        if (fresh) {
+            const long long t0 = clock64();
+            leave();
+            build();
+            ++n_win;
+            cy_build += clock64() - t0;
+            fresh = false;
+        }
+        set_i0();
+        const int32_t left = n - c;
+        int32_t B = 0, kind = -1;                           // decisions of this batch; the step that comes next (-1: none)
+        bool spent = false;                                 // the window holds no more
+        if (agree) {
+            // ---- the stretch on which both orders agree
+            if (tid < WORDS) { W.F[tid].x = W.LF[tid]; W.L[tid].x = W.LL[tid]; W.eq[tid] = 0u; }
+            __syncthreads();
+            ranks();
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < PER; ++r) {
+                if (!((alive >> r) & 1u)) continue;
+                const int32_t i = (int32_t)(cv[r] & 0xffffu), p = (int32_t)(cv[r] >> 16);
+                const uint2 f = W.F[i >> 5], l = W.L[p >> 5];
+                const int32_t rf = (int32_t)f.y + __popc(f.x & ((1u << (i & 31)) - 1u));
+                if (rf == (int32_t)l.y + __popc(l.x & ((1u << (p & 31)) - 1u))) atomicOr(W.eq + (rf >> 5), 1u << (rf & 31));
+            }
+            list_fetch_wait();
+            __syncthreads();
+            int32_t run;
+            {
+                const unsigned a = ~W.eq[2 * lane], b = ~W.eq[2 * lane + 1];
+                const unsigned m = __ballot_sync(FULL_MASK, (a | b) != 0u);
+                const int src = m ? __ffs(m) - 1 : 0;
+                const unsigned x = __shfl_sync(FULL_MASK, a, src), y = __shfl_sync(FULL_MASK, b, src);
+                run = !m ? KLPM_LIST_WIN : src * 64 + (x ? __ffs(x) - 1 : 31 + __ffs(y));
+            }
+            if (run < KLPM_LIST_AGREE) { agree = false; agree_wait = agree_back; agree_back = agree_back < 16 ? 2 * agree_back : 16; }
+            else agree_back = 1;
+            const int32_t e1 = S.ev_f, e2 = S.ev_l, e3 = S.ev_r;
+            B = run < left ? run : left;
+            if (e1 < B) B = e1;
+            if (e2 < B) B = e2;
+            if (e3 < B) B = e3;
+            if (B > 0) {
+                const bool f_next = use_f && B >= i0 && (B - i0) % kk == 0;
+                if (B < left) kind = f_next ? (B == e1 ? 0 : -1) : B == e3 ? 2 : B == e2 ? 1 : -1;
+                spent = kind < 0 && B == run && (run == S.tot_f || run == S.tot_l);
+                if (kind >= 0 && warp == 0) one_step(kind, c + B, cyc + B);
+                else {
+                    for (int w = kind >= 0 ? warp - 1 : warp; w < WORDS; w += kind >= 0 ? NW - 1 : NW) {
+                        const uint2 f = W.F[w], l = W.L[w];      // (the same slots on both sides)
+                        if (f.x && (int32_t)f.y < B) {
+                            const int32_t rank = (int32_t)f.y + __popc(f.x & ((1u << lane) - 1u));
+                            const bool mine = ((f.x >> lane) & 1u) && rank < B;
+                            if (mine) take(W.fs[w * 32 + lane], rank);
+                            const unsigned m = __ballot_sync(FULL_MASK, mine);
+                            if (lane == 0) { atomicAnd(&W.F[w].x, ~m); atomicAnd(&W.LF[w], ~m); }
+                        }
+                        if (l.x && (int32_t)l.y < B) {
+                            const int32_t rank = (int32_t)l.y + __popc(l.x & ((1u << lane) - 1u));
+                            const unsigned m = __ballot_sync(FULL_MASK, ((l.x >> lane) & 1u) && rank < B);
+                            if (lane == 0) { atomicAnd(&W.L[w].x, ~m); atomicAnd(&W.LL[w], ~m); }
+                        }
+                    }
+                }
+                ++n_run; dec_run += B;
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < PER; ++r) {
+                    const int32_t i = (int32_t)(cv[r] & 0xffffu);
+                    if (((alive >> r) & 1u) && !((W.LF[i >> 5] >> (i & 31)) & 1u)) alive &= ~(1u << r);
+                }
+            }
+        }
+        if (B == 0) {
+            // ---- rounds: ranks from the guesses, new guesses from the ranks
+            int32_t T = 0, win = 0, ev = 0, e2 = 0, e3 = 0;
+            int32_t tf[PER], tl[PER];
+            unsigned own = 0;                               // bits 0-3: guessed to go to the oldest-first side, 4-7: to the list
+            if (tid == 0) { S.tstar[0] = KLPM_LIST_FAR; S.tstar[1] = KLPM_LIST_FAR; }
+            for (int it = 0;; ++it) {
+                ranks();
+                __syncthreads();
+                int32_t best = KLPM_LIST_FAR;
+                unsigned flip = 0;
+                own = 0;
+#pragma unroll
+                for (int r = 0; r < PER; ++r) {
+                    tf[r] = KLPM_LIST_FAR; tl[r] = KLPM_LIST_FAR;
+                    if ((alive >> r) & 1u) {
+                        const int32_t i = (int32_t)(cv[r] & 0xffffu), p = (int32_t)(cv[r] >> 16);
+                        const unsigned bi = 1u << (i & 31), bp = 1u << (p & 31);
+                        const uint2 f = W.F[i >> 5], l = W.L[p >> 5];
+                        tf[r] = f_turn((int32_t)f.y + __popc(f.x & (bi - 1u)));
+                        tl[r] = l_turn((int32_t)l.y + __popc(l.x & (bp - 1u)));
+                        const bool is_f = (f.x & bi) != 0u, is_l = (l.x & bp) != 0u, to_f = tf[r] < tl[r];
+                        if (is_f) own |= 1u << r;
+                        if (is_l) own |= 16u << r;
+                        if (is_f != to_f) flip |= 1u << r;
+                        if (is_l == to_f) flip |= 16u << r;
+                        if ((flip >> r) & 0x11u) { const int32_t t = to_f ? tf[r] : tl[r]; if (t < best) best = t; }
+                    }
+                }
+                best = (int32_t)__reduce_min_sync(FULL_MASK, (unsigned)best);
+                if (lane == 0 && best < KLPM_LIST_FAR) atomicMin(&S.tstar[it & 1], best);
+                list_fetch_wait();
+                __syncthreads();
+                T = S.tstar[it & 1];
+                const int32_t e1 = S.ev_f < KLPM_LIST_FAR ? f_turn(S.ev_f) : KLPM_LIST_FAR;
+                e2 = S.ev_l < KLPM_LIST_FAR ? l_turn(S.ev_l) : KLPM_LIST_FAR;
+                e3 = S.ev_r < KLPM_LIST_FAR ? l_turn(S.ev_r) : KLPM_LIST_FAR;
+                ev = e1 < e2 ? e1 : e2;
+                if (e3 < ev) ev = e3;
+                const int32_t wf = f_turn(S.tot_f), wl = l_turn(S.tot_l);
+                win = wf < wl ? wf : wl;
+                // (what needs a step, and what the window cannot answer any more, is only known once everything before has been settled)
+                if (T > ev || T >= left || T > win || it >= KLPM_LIST_ROUNDS || (it >= 3 && T > 0 && T < 12 * it)) break;
+                if (tid == 0) S.tstar[(it + 1) & 1] = KLPM_LIST_FAR;
+#pragma unroll
+                for (int r = 0; r < PER; ++r) {
+                    const int32_t i = (int32_t)(cv[r] & 0xffffu), p = (int32_t)(cv[r] >> 16);
+                    if ((flip >> r) & 1u) atomicXor(&W.F[i >> 5].x, 1u << (i & 31));
+                    if ((flip >> r) & 16u) atomicXor(&W.L[p >> 5].x, 1u << (p & 31));
+                }
+                __syncthreads();
+            }
+            if (T <= win) win = KLPM_LIST_FAR;
+            B = T < ev ? T : ev;
+            if (left < B) B = left;
+            if (win < B) B = win;
+            if (B < left && B == ev && T > ev) kind = e3 == ev ? 2 : e2 == ev ? 1 : 0;
+            spent = kind < 0 && B == win;
+            if (B == 0 && kind < 0 && !spent) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen: a second round settles the first turn
+            if (agree_wait > 0) --agree_wait;
+            else if (use_f && use_l && T <= ev && T < left && T < 64) agree = true;      // next to nothing settled: do the orders agree?
+            if (kind >= 0 && warp == 0) one_step(kind, c + B, cyc + B);
+            else if (B > 0) {
+                const int32_t nfb = f_count(B), nlb = B - nfb;
+                for (int w = kind >= 0 ? warp - 1 : warp; w < WORDS; w += kind >= 0 ? NW - 1 : NW) {
+                    const uint2 f = W.F[w], l = W.L[w];
+                    if (f.x && (int32_t)f.y < nfb) {
+                        const int32_t rank = (int32_t)f.y + __popc(f.x & ((1u << lane) - 1u));
+                        const bool mine = ((f.x >> lane) & 1u) && rank < nfb;
+                        if (mine) take(W.fs[w * 32 + lane], f_turn(rank));
+                        const unsigned m = __ballot_sync(FULL_MASK, mine);
+                        if (lane == 0) { atomicAnd(&W.F[w].x, ~m); atomicAnd(&W.LF[w], ~m); }
+                    }
+                    if (l.x && (int32_t)l.y < nlb) {
+                        const int32_t rank = (int32_t)l.y + __popc(l.x & ((1u << lane) - 1u));
+                        const bool mine = ((l.x >> lane) & 1u) && rank < nlb;
+                        if (mine) take(W.ls[w * 32 + lane], l_turn(rank));
+                        const unsigned m = __ballot_sync(FULL_MASK, mine);
+                        if (lane == 0) { atomicAnd(&W.L[w].x, ~m); atomicAnd(&W.LL[w], ~m); }
+                    }
+                }
+            }
+            if (B > 0) {
+#pragma unroll
+                for (int r = 0; r < PER; ++r) {             // the other side of a meeting that is over
+                    const int32_t i = (int32_t)(cv[r] & 0xffffu), p = (int32_t)(cv[r] >> 16);
+                    if (((own >> r) & 1u) && tf[r] < B) { atomicAnd(&W.LL[p >> 5], ~(1u << (p & 31))); alive &= ~(1u << r); }
+                    if (((own >> r) & 16u) && tl[r] < B) { atomicAnd(&W.LF[i >> 5], ~(1u << (i & 31))); alive &= ~(1u << r); }
+                }
+                ++n_iter; dec_iter += B;
+            }
+        }
+        c += B;
+        if (A.policy == KLPM_POLICY_KLPM) cyc = (int32_t)(((long long)cyc + B) % A.k);
+        if (c >= n) break;
+        __syncthreads();
+        if (kind >= 0) {
+            if (S.failed) break;
+            const int32_t made = S.made;
+            c += made;
+            if (A.policy == KLPM_POLICY_KLPM) cyc = (cyc + made) % A.k;
+            if (S.job == 2) {                               // a group that the whole CTA dissolves: its sorts use the window's memory
+                const long long t1 = clock64();
+                refresh();
+                leave();
+                const FastJob J = s_job;
+                fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
+                if (warp == 0) { const unsigned long long r = tour_top(R, lane); if (lane == 0) S.root = r; }
+                __syncthreads();
+                if (c < n) build();
+                ++n_win; ++n_cta_dissolve;
+                cy_dissolve += clock64() - t1;
+            } else if (S.job == 1) refresh();
+            else after_step();
+        }
+        if (spent) fresh = true;
+    }
+    list_fetch_wait();
+    __syncthreads();
+    if (tid == 0) {
+        long long* cn = A.post->counters;
+        cn[0] += n_dis; cn[1] += n_cta_dissolve; cn[7] += cy_dissolve;
+        cn[8] = n_win; cn[9] = n_run; cn[10] = dec_run; cn[11] = n_iter; cn[12] = dec_iter; cn[13] = n_one; cn[14] = cy_build; cn[15] = cy_step;
+    }
 }
 
 // The loop on a tree with a budget (and klpm_replay on one).  Every decision is a careful step, and a step has two
@@ -5401,7 +5384,7 @@ struct rt_tree {
     unsigned long long* run_partial; RunBcast* run_bc; RunSync* run_sy;
     // scratch of the grouped loop (trees without a budget)
     long long fast_cap;     // slots allocated (power of two)
-    int4* fast_lcp; unsigned long long* grp_key;
+    int4 *fast_lcp, *fast_pair; unsigned long long* grp_key;
     FDyn* fast_dyn; FStat* fast_stat; unsigned long long* fast_key_arr; int32_t* fast_mem;
     long long* fast_gh; int32_t* fast_gidx; unsigned int* fast_done;
     long long* fast_lk; int32_t* fast_ls;
@@ -5497,7 +5480,7 @@ rt_status ensure_fast_scratch(rt_tree* t, long long n) {
     const SlabPart parts[] = {slab_part(&t->fast_dyn, np2), slab_part(&t->fast_stat, np2), slab_part(&t->fast_key_arr, np2),
                               slab_part(&t->fast_mem, t->fast_mem_cap), slab_part(&t->fast_gh, np2), slab_part(&t->fast_gidx, np2),
                               slab_part(&t->fast_done, 3 * (np2 / 32 + 32)),      // processed bitmap, grouped bitmap, passed-over bitmap
-                              slab_part(&t->fast_lk, np2), slab_part(&t->fast_ls, np2), slab_part(&t->fast_lcp, np2), 
+                              slab_part(&t->fast_lk, np2), slab_part(&t->fast_ls, np2), slab_part(&t->fast_lcp, np2), slab_part(&t->fast_pair, np2),
                               slab_part(&t->grp_key, 4 * np2 + 1),                // keys, and as many counts and offsets (see run_impl)
                               slab_part(&t->fast_post, 1), slab_part(&t->fast_bsum, 1024)};
     const rt_status s = slab_alloc(&t->fast_slab, parts, (int)(sizeof(parts) / sizeof(parts[0])));
@@ -6118,7 +6101,7 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         f.c_num = params->c_num; f.c_den = params->c_den; f.start_tick = params->start_tick;
         f.order = d_order; f.uncached = d_uncached; f.ttft = d_ttft; f.completion = d_completion;
         f.dyn = tree->fast_dyn; f.stat = tree->fast_stat; f.key = tree->fast_key_arr; f.mem = tree->fast_mem;
-        f.lcp = tree->fast_lcp; f.sorted_t = tree->run_key;
+        f.lcp = tree->fast_lcp; f.pair = tree->fast_pair; f.sorted_t = tree->run_key;
         f.pinv = d_tie_priority ? tree->run_pinv : nullptr;
         f.gh = tree->fast_gh; f.gidx = tree->fast_gidx; f.done = tree->fast_done;
         f.arrival = d_arrival; f.post = tree->fast_post;
@@ -6197,11 +6180,12 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
             sort_pairs(f.pk, f.pi, np2, s);
             lru_parklist_kernel<<<nblk, 256, 0, s>>>(f);
         }
-        if (f.list_mode) {           // all keys, largest first
-            f.lk = tree->fast_lk; f.ls = tree->fast_ls;
-            fast_list_kernel<<<pblk, 256, 0, s>>>(f.key, n, np2, tree->fast_lk, tree->fast_ls);
+        f.lk = tree->fast_lk; f.ls = tree->fast_ls;
+        // list mode: all keys as they are once everybody has arrived, largest first
+        auto sort_keys = [&]() {
+            fast_list_kernel<<<pblk, 256, 0, s>>>(f, np2);
             sort_pairs(tree->fast_lk, tree->fast_ls, np2, s);
-        }
+        };
         CK(cudaGetLastError());
         if (lru && f.done_in_smem) {
             CK(cudaFuncSetAttribute(lru_run_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -6212,9 +6196,19 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         } else if (f.done_in_smem && (f.bits_in_smem || !f.list_mode)) {
             CK(cudaFuncSetAttribute(fast_run_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             fast_run_kernel<false><<<1, KLPM_FAST_THREADS, smem, s>>>(f);
+            if (f.list_mode) {
+                sort_keys();
+                CK(cudaFuncSetAttribute(list_run_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                list_run_kernel<false><<<1, KLPM_LIST_THREADS, smem, s>>>(f);
+            }
         } else {
             CK(cudaFuncSetAttribute(fast_run_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             fast_run_kernel<true><<<1, KLPM_FAST_THREADS, smem, s>>>(f);
+            if (f.list_mode) {
+                sort_keys();
+                CK(cudaFuncSetAttribute(list_run_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                list_run_kernel<true><<<1, KLPM_LIST_THREADS, smem, s>>>(f);
+            }
         }
         if (!lru) {                  // the decisions made in list mode are charged here (none if list mode never began), or a given order
             const long long nc = d_fixed ? n_fixed : n;
