@@ -1791,7 +1791,7 @@ struct FastArgs {
     int32_t* mem;                 // member array
     const long long* sorted_t;    // per slot: arrival, side by side
     int4* lcp;                    // per slot: how far its prompt agrees with a reference prompt (see lcp_kernel)
-    int4* pair;                   // list mode, per slot that starts in a group: of two, the other slot, its match length and key once this one is processed; else -2
+    int4* pair;                   // list mode, two per slot that starts in a group: of two, the other slot, its match length and key once this one is processed, then the same of this slot; else -2
     const int32_t* pinv;          // rank -> slot, or null
     long long* gh; int32_t* gidx; // group hashes and slots (sorted before the loop; scratch for large groups inside it)
     unsigned int* done;           // bitmap of processed slots (used when it does not fit in shared memory)
@@ -1801,7 +1801,7 @@ struct FastArgs {
     int32_t done_in_smem;
     int32_t list_mode;            // the list mode of the loop can be used (trees without a budget)
     unsigned int* gbits;          // bitmap of slots whose group has more than one member, as the loop starts (and throughout, if the bitmaps stay in global memory)
-    unsigned int* gskip;          // list mode with the bitmaps in global memory: slots the sorted list must pass over
+    unsigned int* gskip;          // list mode with the bitmaps in global memory: slots whose key has changed since the sort
     int32_t bits_in_smem;         // list mode: those two bitmaps are in shared memory
     const long long* lk;          // list mode: every slot's key, largest first, stored as ~key with the top bit flipped
     const int32_t* ls;            //            and the slot it belongs to
@@ -2084,7 +2084,7 @@ lcp_kernel(FastArgs A, int32_t per, const int32_t* __restrict__ wanted) {
     // A group of two is known completely: whoever is processed first, the other one matches e tokens from then on.  (Two slots that share
     // a run by a hash collision are no group.)
     if (!A.list_mode || count < 2) return;
-    if (count > 2) { A.pair[r] = make_int4(-2, 0, 0, 0); return; }
+    if (count > 2) { A.pair[2LL * r] = make_int4(-2, 0, 0, 0); return; }
     if (other == r) return;                                 // (the other slot's lane writes both)
     if (!cmp) {
         atomicAnd(A.gbits + (r >> 5), ~(1u << (r & 31)));
@@ -2093,8 +2093,9 @@ lcp_kernel(FastArgs A, int32_t per, const int32_t* __restrict__ wanted) {
     }
     const FStat s = ld_stat(A.stat + r), f = ld_stat(A.stat + other);
     const unsigned long long kr = fast_key(e, s.len, s.rank, A.score_mode), kf = fast_key(e, f.len, f.rank, A.score_mode);
-    A.pair[r] = make_int4(other, e, (int)(unsigned)kf, (int)(unsigned)(kf >> 32));
-    A.pair[other] = make_int4(r, e, (int)(unsigned)kr, (int)(unsigned)(kr >> 32));
+    const int4 mine = make_int4(other, e, (int)(unsigned)kf, (int)(unsigned)(kf >> 32)), its = make_int4(r, e, (int)(unsigned)kr, (int)(unsigned)(kr >> 32));
+    A.pair[2LL * r] = mine; A.pair[2LL * r + 1] = its;
+    A.pair[2LL * other] = its; A.pair[2LL * other + 1] = mine;
 }
 // The groups that a given order touches (see lcp_kernel).
 __global__ void lcp_wanted_kernel(FastArgs A, int32_t* wanted) {
@@ -2139,7 +2140,7 @@ struct FastTour {
     unsigned long long* t2;   // per 32 leaf blocks (padded likewise)
     unsigned long long* t3;   // 32 entries
     unsigned int* done;       // bitmap of processed slots (shared memory), or null
-    unsigned int* skip;       // bitmap of slots the sorted list must pass over: processed, or key changed (shared memory), or null
+    unsigned int* skip;       // bitmap of slots whose key has changed since the sort (the list passes over them), or null
     unsigned int* gb;         // bitmap of slots whose group has more than one member (shared memory), or null
     unsigned int* dirty;      // trees with a budget: bitmap of leaf blocks to recompute after a fallback (256 words, shared memory)
     int g_done, g_bits;       // the processed bitmap / the other two bitmaps live in global memory (queues too long for shared memory)
@@ -2255,19 +2256,6 @@ __device__ __forceinline__ void lru_move(const FastArgs& A, int32_t r, int32_t f
     __stcg(A.hintc + r, to);
     atomicSub(A.parked + from, 1);
     atomicAdd(A.parked + to, 1);
-}
-
-// List mode: the largest key among the unprocessed slots of leaf block b whose key has changed since the sort.  One warp.
-__device__ __forceinline__ unsigned long long changed_block_max(const FastArgs& A, const FastTour& R, int32_t b, int lane) {
-    unsigned long long v = 0;
-    for (int32_t u = lane; u < (1 << A.lb_shift); u += 32) {
-        const long long r = ((long long)b << A.lb_shift) + u;
-        if (r < A.n) {
-            const unsigned w = bm_ld(R.skip, r >> 5, R.g_bits) & ~bm_ld(R.done, r >> 5, R.g_done);
-            if ((w >> (r & 31)) & 1u) { const unsigned long long kk = __ldcg(A.key + r); if (kk > v) v = kk; }
-        }
-    }
-    return warp_max64r(v);
 }
 
 // One member of the dissolving group per lane (r < 0: none).  Members tied with the processed prompt are
@@ -2930,6 +2918,8 @@ fast_run_kernel(FastArgs A) {
 #define KLPM_LIST_ROUNDS 16           // rounds on one state of the window before what is settled is committed
 #define KLPM_LIST_AGREE 24            // stretches shorter than this are left to the rounds
 #define KLPM_LIST_FAR 0x3ffffff
+struct ListLane;
+struct ListTaken;
 struct ListWin {                      // the window, in the scratch of the sorts
     int32_t* fs;                      // unprocessed slots, oldest first
     int32_t* ls; long long* lk;       // list positions from `cur` on: slot, key as the list holds it
@@ -2939,20 +2929,39 @@ struct ListWin {                      // the window, in the scratch of the sorts
     unsigned *LF, *LL;                // still there
     unsigned *EF, *EL;                // needs a step of its own
     unsigned* eq;                     // agreement, one bit per rank
+    int32_t* cand; short* cand_p;     // slots in groups found in the window, and their list positions
+    ListLane* lane; ListTaken *taken, *unsorted;       // in the place of `col` once every thread has its meetings
 };
+// The prompts of a group of two, and prompts whose key has grown because the other one was processed, are worked out by the same
+// rounds, each by a thread of its own (see `lane_round`).
+struct alignas(16) ListLane {
+    unsigned long long key;           // the key it has, or will have once the other one is processed
+    int32_t slot, m2;                 // m2: its match length then
+    short fi, lp, jr;                 // index among the oldest-first slots, list position, first list position that its key beats (-1: not in the window)
+    unsigned char kind, taken;        // kind 0: none, 1: its key has grown, 2: one of a group of two; taken: guessed to be taken with that key,
+    int32_t o, A;                     // at this longest-match turn; longest-match turns that are over when the key grows
+};
+struct ListTaken { unsigned long long key; int32_t A, o, jr, lane; };
+#define KLPM_LIST_LANES 128           // the first half for grown keys, the second for groups of two
+#define KLPM_LIST_LANE_MIN 8192        // shorter queues make those decisions one at a time: they are few, and lanes lengthen every round (1,000 queries: 65 us, with lanes 121)
+#define KLPM_LIST_CAND 288
+#define KLPM_LIST_CAND_MIN 8           // so do windows with fewer: their lanes would cost what some two steps cost
+#define KLPM_LIST_TAKEN 80             // guessed to be taken with a grown key at a time, at most (more are not guessed)
 struct ListShared {
+    int32_t n_cand, n_pair, n_grown, n_taken, lane_lim;
     int4 pre[2][4];                              // records of lcp_kernel's pairs for the last four steps found on either side, on their way since then
     int32_t pre_n[2], pre_slot[2][4];
-    int32_t head, cur, job, made, failed;
+    int32_t head, cur, job, failed;
     int32_t ncol;
     int32_t tot_f, tot_l, ev_f, ev_l, ev_r;      // picks of either side in the window; ranks of the first that needs a step, of the first list entry below the root
-    int32_t ix_f, ix_l;                          // index / position of those two
+    int32_t ix_f, ix_l, ix_r;                    // index / positions of those three
     int32_t tstar[2];
     int32_t step_f, step_l, mate_f, mate;        // what a step took (index, position) and changed (index, slot); -1: nothing
     unsigned long long root;
     int32_t w[KLPM_LIST_THREADS / 32];
 };
-static_assert(KLPM_LIST_WIN * (4 + 4 + 8 + 4) + KLPM_LIST_THREADS * 8 + 9 * (KLPM_LIST_WIN / 32) * 4 <= KLPM_FAST_SORT_CAP * 12, "a window fits the sort scratch");
+static_assert(KLPM_LIST_WIN * (4 + 4 + 8 + 4) + KLPM_LIST_THREADS * 8 + 9 * (KLPM_LIST_WIN / 32) * 4 + KLPM_LIST_CAND * 6 <= KLPM_FAST_SORT_CAP * 12, "a window fits the sort scratch");
+static_assert(KLPM_LIST_LANES * sizeof(ListLane) + 2 * KLPM_LIST_TAKEN * sizeof(ListTaken) <= KLPM_LIST_WIN * 4, "the lanes fit the place of the meetings");
 
 // first set bit of a bitmap of 64 words, or -1.  One warp.
 __device__ __forceinline__ int32_t list_first(const unsigned* w, int lane) {
@@ -2994,7 +3003,7 @@ __device__ __forceinline__ void list_fetch_wait() { asm volatile("cp.async.wait_
 
 template <bool G>
 __global__ void __launch_bounds__(KLPM_LIST_THREADS, 1)
-list_run_kernel(FastArgs A) {
+list_run_kernel(const __grid_constant__ FastArgs A) {
     extern __shared__ __align__(16) unsigned char fast_smem[];
     __shared__ FastJob s_job;
     __shared__ int s_cnt;
@@ -3032,18 +3041,21 @@ list_run_kernel(FastArgs A) {
     W.fw = reinterpret_cast<unsigned*>(W.fp + KLPM_LIST_THREADS);
     W.F = reinterpret_cast<uint2*>(W.fw + KLPM_LIST_THREADS); W.L = W.F + WORDS;
     W.LF = reinterpret_cast<unsigned*>(W.L + WORDS); W.LL = W.LF + WORDS; W.EF = W.LL + WORDS; W.EL = W.EF + WORDS; W.eq = W.EL + WORDS;
+    W.cand = reinterpret_cast<int32_t*>(W.eq + WORDS); W.cand_p = reinterpret_cast<short*>(W.cand + KLPM_LIST_CAND);
+    W.lane = reinterpret_cast<ListLane*>(W.col); W.taken = reinterpret_cast<ListTaken*>(W.lane + KLPM_LIST_LANES); W.unsorted = W.taken + KLPM_LIST_TAKEN;
     for (int32_t i = tid; i < nb1p + n2p + 32; i += KLPM_LIST_THREADS) R.t1[i] = 0ULL;
     if (tid == 0) {
         s_memcur = n;
-        S.head = A.post->head; S.cur = 0; S.root = 0ULL; S.failed = 0; S.job = 0; S.pre_n[0] = 0; S.pre_n[1] = 0;
+        S.head = A.post->head; S.cur = 0; S.root = 0ULL; S.failed = 0; S.job = 0; S.pre_n[0] = 0; S.pre_n[1] = 0; S.n_taken = 0;
     }
     if (A.done_in_smem) for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) R.done[i] = c > 0 ? __ldcg(A.done + i) : 0u;
-    for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {      // (the list passes over processed slots, so far)
-        R.skip[i] = c > 0 ? __ldcg(A.done + i) : 0u;
+    for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {
+        R.skip[i] = 0u;                                     // (slots whose key has changed since the sort)
         if (A.bits_in_smem) R.gb[i] = __ldcg(A.gbits + i);
     }
     __syncthreads();
     auto bit_of = [&](const unsigned* bm, int32_t slot, int g) -> unsigned { return (bm_ld(bm, slot >> 5, g) >> (slot & 31)) & 1u; };
+    auto stale = [&](int32_t s) -> bool { return (((bm_ld(R.done, s >> 5, gdone) | bm_ld(R.skip, s >> 5, gbits)) >> (s & 31)) & 1u) != 0u; };      // the list passes over it
     // ---- turns, counted from the next decision: the t-th oldest-first turn, the u-th longest-match turn, oldest-first turns among x decisions.
     // (a k beyond what a window holds is as good as any such k)
     const bool use_f = A.policy != KLPM_POLICY_LPM;
@@ -3065,6 +3077,10 @@ list_run_kernel(FastArgs A) {
     int32_t n_f = 0, n_l = 0;                               // the window: slots, list positions
     bool list_end = false;                                  // it reaches the end of the list
     int32_t w0 = 0, head0 = 0;                              // its first bitmap word and slot
+    const int x = tid - 96;                                 // this thread's lane, if 0 <= x < KLPM_LIST_LANES (whole warps)
+    const bool laner = x >= 0 && x < KLPM_LIST_LANES;
+    int32_t sv_slot = -1, sv_m2 = 0;                        // a grown key, from one window to the next
+    unsigned long long sv_key = 0;
     unsigned cv[PER], alive = 0;                            // this thread's meetings; one bit each while both sides still have the slot
 #pragma unroll
     for (int r = 0; r < PER; ++r) cv[r] = 0u;
@@ -3076,6 +3092,11 @@ list_run_kernel(FastArgs A) {
         const int32_t phi = W.fp[wl] + __popc(f & ((1u << (s & 31)) - 1u));
         return ((f >> (s & 31)) & 1u) && phi < n_f ? phi : -1;
     };
+    auto no_event = [&](int32_t fi, int32_t lp) {
+        if (fi >= 0) atomicAnd(&W.EF[fi >> 5], ~(1u << (fi & 31)));
+        if (lp >= 0) atomicAnd(&W.EL[lp >> 5], ~(1u << (lp & 31)));
+    };
+    auto lane_bar = [&]() { named_bar(2, KLPM_LIST_LANES); };
     // Everything about the window's slots again, after a group has been dissolved.
     auto refresh = [&]() {
 #pragma unroll
@@ -3083,7 +3104,7 @@ list_run_kernel(FastArgs A) {
             const int w = warp + NW * r, i = w * 32 + lane;
             const bool hf = (W.LF[w] >> lane) & 1u, hl = (W.LL[w] >> lane) & 1u;
             const int32_t sf = hf ? W.fs[i] : 0, sl = hl ? W.ls[i] : 0;
-            const bool in_f = hf && !bit_of(R.done, sf, gdone), in_l = hl && !bit_of(R.skip, sl, gbits);
+            const bool in_f = hf && !bit_of(R.done, sf, gdone), in_l = hl && !stale(sl);
             const unsigned lf = __ballot_sync(FULL_MASK, in_f), ll = __ballot_sync(FULL_MASK, in_l);
             const unsigned ef = __ballot_sync(FULL_MASK, in_f && ((use_l ? bit_of(R.skip, sf, gbits) : 0u) | bit_of(R.gb, sf, gbits)));
             const unsigned el = __ballot_sync(FULL_MASK, in_l && bit_of(R.gb, sl, gbits));
@@ -3099,6 +3120,80 @@ list_run_kernel(FastArgs A) {
             alive &= ~(1u << r);
             if (lf) atomicOr(&W.F[i >> 5].x, 1u << (i & 31));      // its list entry has gone stale: the oldest-first side has it alone
         }
+        if (laner && W.lane[x].kind) no_event(W.lane[x].fi, W.lane[x].lp);
+        __syncthreads();
+    };
+    auto to_tournament = [&]() {                            // a grown key that is not a lane's any more
+        const int32_t b = sv_slot >> A.lb_shift;
+        atomicMax(R.t1 + b, sv_key); atomicMax(R.t2 + (b >> 5), sv_key); atomicMax(R.t3 + (b >> 10), sv_key); atomicMax(&S.root, sv_key);
+        const int32_t f = index_of(sv_slot);
+        if (f >= 0 && use_l) atomicOr(&W.EF[f >> 5], 1u << (f & 31));
+    };
+    // The lanes of a new window: the grown keys kept from the last one, and both prompts of the groups of two that have one in the window.
+    // What finds no lane goes on as before: a grown key to the tournament, a group as an event.
+    auto lanes = [&]() {
+        const int32_t n_cand = S.n_cand >= KLPM_LIST_CAND_MIN && S.n_cand <= KLPM_LIST_CAND && n >= KLPM_LIST_LANE_MIN ? S.n_cand : 0;      // (too many to know all positions: none)
+        if (n_cand == 0) {
+            if (laner) W.lane[x].kind = 0;
+            if (sv_slot >= 0 && !bit_of(R.done, sv_slot, gdone)) to_tournament();
+            __syncthreads();
+            return;
+        }
+        int32_t* const low = reinterpret_cast<int32_t*>(W.taken);              // per candidate: the smaller slot of its pair (no key is guessed to be taken yet)
+        if (laner) W.lane[x].kind = 0;
+        if (tid < WORDS) W.eq[tid] = 0u;
+        short* const place = reinterpret_cast<short*>(low + KLPM_LIST_CAND);    // and, of the first of them, the pair's number
+        int32_t mine = -1, mate = -1, lead = 0;
+        int4 rec = make_int4(-2, 0, 0, 0), back = rec;
+        if (tid < n_cand) {
+            mine = W.cand[tid];
+            rec = __ldg(A.pair + 2LL * mine); back = __ldg(A.pair + 2LL * mine + 1);
+            mate = rec.x;
+            low[tid] = mate < 0 ? -1 : mine < mate ? mine : mate;
+        }
+        __syncthreads();
+        if (sv_slot >= 0 && !bit_of(R.done, sv_slot, gdone)) {
+            const int32_t at = atomicAdd(&S.n_grown, 1);
+            if (at < KLPM_LIST_LANES / 2) {
+                ListLane l;
+                l.key = sv_key; l.slot = sv_slot; l.m2 = sv_m2; l.fi = (short)index_of(sv_slot); l.lp = -1; l.jr = -1; l.o = 0; l.A = 0; l.kind = 1; l.taken = 0;
+                W.lane[at] = l;
+            } else to_tournament();
+        }
+        if (mate >= 0) {
+            const int32_t lo = low[tid];
+            while (low[lead] != lo) ++lead;                 // (at the latest its own)
+            if (lead == tid) {
+                const int32_t at = atomicAdd(&S.n_pair, 1);
+                place[tid] = (short)at;
+                if (at < KLPM_LIST_LANES / 4) {
+                    ListLane l;
+                    l.lp = -1; l.jr = -1; l.o = 0; l.A = 0; l.kind = 2; l.taken = 0; l.m2 = rec.y;
+                    l.slot = mine; l.fi = (short)index_of(mine); l.key = (unsigned long long)(unsigned)back.w << 32 | (unsigned)back.z;
+                    W.lane[KLPM_LIST_LANES / 2 + 2 * at] = l;
+                    l.slot = mate; l.fi = (short)index_of(mate); l.key = (unsigned long long)(unsigned)rec.w << 32 | (unsigned)rec.z;
+                    W.lane[KLPM_LIST_LANES / 2 + 2 * at + 1] = l;
+                }
+            }
+        }
+        __syncthreads();
+        if (mate >= 0 && W.cand_p[tid] >= 0 && place[lead] < KLPM_LIST_LANES / 4) {
+            ListLane* const l = W.lane + KLPM_LIST_LANES / 2 + 2 * place[lead];
+            l[l[0].slot == mine ? 0 : 1].lp = W.cand_p[tid];
+        }
+        __syncthreads();
+        if (laner && W.lane[x].kind) {
+            ListLane& l = W.lane[x];
+            const long long rk = (long long)(~l.key ^ 0x8000000000000000ULL);      // (the list holds ~key with the top bit flipped, ascending)
+            int32_t lo = 0, hi = n_l;
+            while (lo < hi) { const int32_t mid = (lo + hi) >> 1; if (W.lk[mid] > rk) hi = mid; else lo = mid + 1; }
+            l.jr = (short)lo;
+            no_event(l.fi, l.lp);
+            if (l.fi >= 0) atomicOr(&W.eq[l.fi >> 5], 1u << (l.fi & 31));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < PER; ++r) { const int32_t i = (int32_t)(cv[r] & 0xffffu); if (((alive >> r) & 1u) && ((W.eq[i >> 5] >> (i & 31)) & 1u)) alive &= ~(1u << r); }
         __syncthreads();
     };
     auto build = [&]() {
@@ -3120,7 +3215,7 @@ list_run_kernel(FastArgs A) {
 #pragma unroll
                 for (int r = 0; r < PER; ++r) {
                     const int w = warp + NW * r;
-                    const bool in = slot_in[r] >= 0 && !bit_of(R.skip, slot_in[r], gbits);
+                    const bool in = slot_in[r] >= 0 && !stale(slot_in[r]);
                     const unsigned live = __ballot_sync(FULL_MASK, in), ev = __ballot_sync(FULL_MASK, in && bit_of(R.gb, slot_in[r], gbits));
                     if (lane == 0) { W.LL[w] = live; W.L[w].x = live; W.EL[w] = ev; }
                     any |= live != 0u;
@@ -3162,8 +3257,12 @@ list_run_kernel(FastArgs A) {
                 }
             }
         } else if (tid < WORDS) { W.LF[tid] = 0u; W.F[tid].x = 0u; W.EF[tid] = 0u; }
-        if (tid == 0) { S.ncol = 0; S.cur = cur; }
+        if (tid == 0) { S.ncol = 0; S.cur = cur; S.n_cand = 0; S.n_pair = 0; S.n_grown = 0; S.n_taken = 0; }
         __syncthreads();
+        auto candidate = [&](int32_t s, int32_t pos) {
+            const int32_t at = atomicAdd(&S.n_cand, 1);
+            if (at < KLPM_LIST_CAND) { W.cand[at] = s; W.cand_p[at] = (short)pos; asm volatile("prefetch.global.L1 [%0];" ::"l"(A.pair + 2LL * s)); }
+        };
         if (use_f) {
 #pragma unroll
             for (int r = 0; r < PER; ++r) {
@@ -3173,14 +3272,20 @@ list_run_kernel(FastArgs A) {
                 const unsigned live = __ballot_sync(FULL_MASK, in);
                 const unsigned ev = __ballot_sync(FULL_MASK, in && ((use_l ? bit_of(R.skip, s, gbits) : 0u) | bit_of(R.gb, s, gbits)));
                 if (lane == 0) { W.LF[w] = live; W.F[w].x = live; W.EF[w] = ev; }
+                if (in && bit_of(R.gb, s, gbits)) candidate(s, -1);
             }
+        }
+        if (use_l) {
+#pragma unroll
+            for (int r = 0; r < PER; ++r)
+                if (slot_in[r] >= 0 && !stale(slot_in[r]) && bit_of(R.gb, slot_in[r], gbits)) candidate(slot_in[r], tid + KLPM_LIST_THREADS * r);
         }
         if (use_f && use_l && n_f > 0) {                    // the meetings
             const int32_t hmax = W.fs[n_f - 1];
 #pragma unroll
             for (int r = 0; r < PER; ++r) {
                 const int32_t s = slot_in[r];
-                bool met = s >= head && s <= hmax && !bit_of(R.skip, s, gbits);
+                bool met = s >= head && s <= hmax && !stale(s);
                 int32_t phi = 0;
                 if (met) {
                     const int32_t wl = (s >> 5) - w0;       // (below KLPM_LIST_THREADS: hmax is)
@@ -3207,10 +3312,12 @@ list_run_kernel(FastArgs A) {
         alive = 0;
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
-            const int32_t x = tid + KLPM_LIST_THREADS * r;
-            cv[r] = x < ncol ? W.col[x] : 0u;
-            if (x < ncol) alive |= 1u << r;
+            const int32_t at = tid + KLPM_LIST_THREADS * r;
+            cv[r] = at < ncol ? W.col[at] : 0u;
+            if (at < ncol) alive |= 1u << r;
         }
+        __syncthreads();
+        lanes();
     };
     // Prefix sums of the guesses, and what ends a batch: the rank of the first pick of either side that needs a step, and of the first
     // list entry that the tournament's root beats.  The caller synchronises.
@@ -3231,7 +3338,7 @@ list_run_kernel(FastArgs A) {
                     if (k == 0 || S.pre_slot[warp][(k - 1) & 3] != slot) {
                         if ((k & 3) == 0) list_fetch_wait();
                         S.pre_slot[warp][k & 3] = slot; S.pre_n[warp] = k + 1;
-                        list_fetch16(&S.pre[warp][k & 3], A.pair + slot);
+                        list_fetch16(&S.pre[warp][k & 3], A.pair + 2LL * slot);
                     }
                 }
             }
@@ -3257,42 +3364,140 @@ list_run_kernel(FastArgs A) {
                 if (left > 0) cnt += __popc(left >= 32 ? W.L[w].x : W.L[w].x & ((1u << left) - 1u));
             }
             cnt = (int32_t)__reduce_add_sync(FULL_MASK, (unsigned)cnt);
+            if (lane == 0) S.ix_r = jr;
             if (lane == 0) S.ev_r = root != 0ULL && (jr < n_l || list_end) ? cnt : KLPM_LIST_FAR;
         }
     };
+    // The longest-match turn at which the list entry at position p, of rank r, is reached: a grown key that beats it goes first if it has
+    // grown by then.  (They are sorted by when they grow.)
+    auto ord = [&](int32_t r, int32_t p) -> int32_t {
+        const int32_t nt = S.n_taken;
+        for (int32_t u = 0; u < nt && W.taken[u].A <= r; ++u) r += W.taken[u].jr <= p;
+        return r;
+    };
+    auto list_rank = [&](int32_t p) -> int32_t { const uint2 l = W.L[p >> 5]; return (int32_t)l.y + __popc(l.x & ((1u << (p & 31)) - 1u)); };
+    auto l_count = [&](int32_t t) -> int32_t { return use_l ? t - f_count(t) : 0; };
+    // Before the threads look at their meetings: the slots that are guessed to be taken with a grown key, by when it grows.
+    auto lane_turns = [&]() {
+        ListLane& l = W.lane[x];
+        if (x == 0) S.n_taken = 0;
+        lane_bar();
+        int32_t at = -1;
+        if (l.kind && l.taken) {
+            at = atomicAdd(&S.n_taken, 1);
+            if (at < KLPM_LIST_TAKEN) { ListTaken t; t.key = l.key; t.A = l.A; t.o = l.o; t.jr = l.jr; t.lane = x; W.unsorted[at] = t; }
+            else { l.taken = 0; at = -1; }
+        }
+        lane_bar();
+        const int32_t nt = S.n_taken < KLPM_LIST_TAKEN ? S.n_taken : KLPM_LIST_TAKEN;
+        if (at >= 0) {
+            int32_t rank = 0;
+            for (int32_t u = 0; u < nt; ++u) { const int32_t a = W.unsorted[u].A; rank += a < l.A || (a == l.A && u < at); }
+            W.taken[rank] = W.unsorted[at];
+        }
+        lane_bar();
+        if (x == 0) S.n_taken = nt;
+    };
+    // A lane's turns from the guesses, and its new guess.  Of a group of two, whoever is reached first is an ordinary pick of either side.
+    // The other one's key grows at that moment: A longest-match turns are over by then.  It is taken before the first list entry
+    // that it beats, but not before it has grown, and after the grown keys that are larger and have grown by its turn.
+    // (The proof of the rounds holds for it too: its turn depends on slots that are taken before it only, and where its guess changes T is
+    // no later than any turn, old or new, from which on it matters to others.)
+    int32_t lane_tf = KLPM_LIST_FAR, lane_tl = KLPM_LIST_FAR, lane_o = 0, lane_A = 0;
+    unsigned lane_now = 0, lane_new = 0;                    // guesses: 1 oldest-first, 2 list entry, 4 grown key
+    auto lane_round = [&]() -> int32_t {
+        const ListLane l = W.lane[x];
+        int32_t tf = KLPM_LIST_FAR, tl = KLPM_LIST_FAR, tr = KLPM_LIST_FAR, at = 0, o = 0;
+        unsigned now_ = 0;
+        if (l.kind) {
+            if (l.fi >= 0) { const uint2 f = W.F[l.fi >> 5]; tf = f_turn((int32_t)f.y + __popc(f.x & ((1u << (l.fi & 31)) - 1u))); if ((f.x >> (l.fi & 31)) & 1u) now_ |= 1u; }
+            if (l.lp >= 0) { tl = l_turn(ord(list_rank(l.lp), l.lp)); if ((W.L[l.lp >> 5].x >> (l.lp & 31)) & 1u) now_ |= 2u; }
+            if (l.taken) now_ |= 4u;
+        }
+        const int32_t t1 = tf < tl ? tf : tl, tm = __shfl_xor_sync(FULL_MASK, t1, 1);
+        const bool grown = l.kind == 1 || (l.kind == 2 && tm < t1);
+        const int32_t r0 = !l.kind || !use_l ? 0 : l.jr < n_l ? list_rank(l.jr) : S.tot_l;      // list picks before the first entry that its key beats
+        if (grown && use_l && (l.jr < n_l || list_end)) {
+            if (l.kind == 2) at = l_count(tm + 1);
+            o = r0;
+            int32_t o2 = at;
+            const int32_t nt = S.n_taken;
+            for (int32_t u = 0; u < nt; ++u) {
+                const ListTaken t = W.taken[u];
+                if (t.A > o && t.A > o2) break;
+                if (t.lane == x || t.key < l.key) continue;
+                if (t.A <= o) ++o;
+                if (t.A <= o2 && t.o >= at) ++o2;
+            }
+            if (o2 > o) o = o2;
+            tr = l_turn(o);
+        }
+        unsigned new_ = 0;
+        if (l.kind) {
+            const int32_t other = grown ? tr : tl;
+            if (l.fi >= 0 && (tf < other || other >= KLPM_LIST_FAR)) new_ = 1u;
+            else if (other < KLPM_LIST_FAR) new_ = grown ? 4u : 2u;
+        }
+        int32_t best = KLPM_LIST_FAR;
+        if (new_ != now_ || ((new_ & 4u) && (o != l.o || at != l.A))) {
+            // (with its grown key it matters to turns after it has grown, of entries that it beats)
+            best = t1 < tr ? t1 : tr;
+            if (new_ & 4u) { const int32_t w = l_turn(r0 > at ? r0 : at); if (w < best) best = w; }
+            if (now_ & 4u) { const int32_t e = r0 > l.A ? r0 : l.A, w = l_turn(l.o < e ? l.o : e); if (w < best) best = w; }
+        }
+        lane_tf = tf; lane_tl = tl; lane_o = o; lane_A = at; lane_now = now_; lane_new = new_;
+        return best;
+    };
     auto take = [&](int32_t slot, int32_t at) {
         atomicOr(R.done + (slot >> 5), 1u << (slot & 31));
-        atomicOr(R.skip + (slot >> 5), 1u << (slot & 31));
         A.order[c + at] = slot;
     };
     // Warp 0: one decision that needs a step -- the oldest slot (kind 0), the next list entry (1) or the tournament's root (2).
     long long n_one = 0, n_dis = 0, cy_step = 0;
     // `at`: its number.  Other warps commit the batch before it at the same time: what both change is changed by atomics.
-    auto one_step = [&](int kind, int32_t at, int32_t turn) {
+    auto one_step = [&](int kind, int32_t at) {
         const long long t0 = clock64();
         unsigned long long root = S.root;
         int32_t j;
+        bool from_lane = false;
         if (kind == 2) {
             const unsigned rk = 0xffffffffu - (unsigned)(root & 0xffffffffULL);
-            j = A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
+            unsigned long long best = 0;                    // a grown key may be larger still
+            int32_t at_lane = -1;
+#pragma unroll
+            for (int u = 0; u < KLPM_LIST_LANES / 32; ++u) { const ListLane& l = W.lane[32 * u + lane]; if (l.kind == 1 && l.key > best) { best = l.key; at_lane = 32 * u + lane; } }
+            const unsigned long long top = warp_max64r(best);
+            const bool other = top > root;
+            if (other) {
+                const int src = __ffs(__ballot_sync(FULL_MASK, best == top)) - 1;
+                at_lane = __shfl_sync(FULL_MASK, at_lane, src);
+                j = W.lane[at_lane].slot;
+                __syncwarp();
+                if (lane == 0) W.lane[at_lane].kind = 0;
+                from_lane = true;
+            } else j = A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
         } else j = kind == 0 ? W.fs[S.ix_f] : W.ls[S.ix_l];
         if (j < 0 || j >= n || bit_of(R.done, j, gdone)) { if (lane == 0) { set_status(A.st, RT_ERR_LIMIT, 107); S.failed = 1; } return; }   // cannot happen
-        const bool in_tour = kind == 2 || (kind == 0 && use_l && bit_of(R.skip, j, gbits) != 0u);      // its key changed after the sort
+        const bool in_tour = (kind == 2 && !from_lane) || (kind == 0 && use_l && bit_of(R.skip, j, gbits) != 0u);      // its key changed after the sort
         const bool grouped = bit_of(R.gb, j, gbits) != 0u;
         const int32_t step_f = kind == 0 ? S.ix_f : index_of(j);
         int32_t mate_f = -1, mate_s = -1, job = 0;
-        bool both = false;                                  // the other one of a pair was taken right after it
         __syncwarp();
         if (lane == 0) {
             atomicOr(R.done + (j >> 5), 1u << (j & 31));
-            if (!in_tour) atomicOr(R.skip + (j >> 5), 1u << (j & 31));
             A.order[at] = j;
         }
         __syncwarp();
         if (in_tour) {                                      // its leaf block's largest changed key, without it
             const int32_t b = j >> A.lb_shift;
-            const bool alone = A.lb_shift == 5 && !(bm_ld(R.skip, b, gbits) & ~bm_ld(R.done, b, gdone));
-            root = tour_set(R, b, alone ? 0ULL : changed_block_max(A, R, b, lane), lane);
+            unsigned long long v = 0;
+            for (int32_t u = 0; u < (1 << A.lb_shift); u += 32) {
+                const long long r = ((long long)b << A.lb_shift) + u + lane;
+                bool in = r < n && bit_of(R.skip, (int32_t)r, gbits) && !bit_of(R.done, (int32_t)r, gdone);
+                for (int32_t l = 0; l < KLPM_LIST_LANES && __any_sync(FULL_MASK, in); ++l) in = in && !(W.lane[l].kind == 1 && W.lane[l].slot == (int32_t)r);      // (a lane's key is not in the tournament)
+                if (in) { const unsigned long long key = __ldcg(A.key + r); if (key > v) v = key; }
+            }
+            root = tour_set(R, b, warp_max64r(v), lane);
             __syncwarp();
         }
         ++n_one;
@@ -3301,7 +3506,7 @@ list_run_kernel(FastArgs A) {
             int4 rec;
             const int last = kind < 2 ? (S.pre_n[kind] - 1) & 3 : 0;      // (found by the round before this step)
             if (kind < 2 && S.pre_slot[kind][last] == j) rec = S.pre[kind][last];
-            else rec = __ldcg(A.pair + j);
+            else rec = __ldg(A.pair + 2LL * j);
             if (rec.x >= 0) {                               // one other prompt, and what becomes of it is known
                 mate_s = rec.x;
                 const unsigned long long key = (unsigned long long)(unsigned)rec.w << 32 | (unsigned)rec.z;
@@ -3313,19 +3518,11 @@ list_run_kernel(FastArgs A) {
                     atomicAnd(R.gb + (j >> 5), ~(1u << (j & 31)));
                 }
                 mate_f = index_of(mate_s);
-                // Mostly the other one is the next longest-match pick: its key beats the entry just taken, and with it the rest of the list.
-                both = kind == 1 && at + 1 < n && key > root && key > ~((unsigned long long)W.lk[S.ix_l] ^ 0x8000000000000000ULL) &&
-                       (A.policy == KLPM_POLICY_LPM || (turn + 1) % A.k != 0);
-                if (both) {
-                    if (lane == 0) { atomicOr(R.done + (mate_s >> 5), 1u << (mate_s & 31)); A.order[at + 1] = mate_s; }
-                    ++n_one;
-                } else {
-                    const int32_t b = mate_s >> A.lb_shift;
-                    const unsigned long long p1 = R.t1[b], p2 = R.t2[b >> 5], p3 = R.t3[b >> 10];
-                    __syncwarp();
-                    R.t1[b] = key > p1 ? key : p1; R.t2[b >> 5] = key > p2 ? key : p2; R.t3[b >> 10] = key > p3 ? key : p3;      // (every lane stores the same)
-                    root = key > root ? key : root;
-                }
+                const int32_t b = mate_s >> A.lb_shift;
+                const unsigned long long p1 = R.t1[b], p2 = R.t2[b >> 5], p3 = R.t3[b >> 10];
+                __syncwarp();
+                R.t1[b] = key > p1 ? key : p1; R.t2[b >> 5] = key > p2 ? key : p2; R.t3[b >> 10] = key > p3 ? key : p3;      // (every lane stores the same)
+                root = key > root ? key : root;
                 __syncwarp();
             } else {
                 const FDyn d = ld_dyn(A.dyn + j);
@@ -3342,11 +3539,9 @@ list_run_kernel(FastArgs A) {
             }
         }
         if (lane == 0) {
-            S.made = both ? 2 : 1;
             S.root = root; S.job = job; S.step_f = step_f; S.step_l = kind == 1 ? S.ix_l : -1; S.mate_f = mate_f; S.mate = mate_s;
             if (step_f >= 0) { atomicAnd(&W.LF[step_f >> 5], ~(1u << (step_f & 31))); atomicAnd(&W.F[step_f >> 5].x, ~(1u << (step_f & 31))); }
-            if (mate_f >= 0 && both) { atomicAnd(&W.LF[mate_f >> 5], ~(1u << (mate_f & 31))); atomicAnd(&W.F[mate_f >> 5].x, ~(1u << (mate_f & 31))); }
-            else if (mate_f >= 0) {
+            if (mate_f >= 0) {
                 atomicOr(&W.F[mate_f >> 5].x, 1u << (mate_f & 31));
                 if (use_l) atomicOr(&W.EF[mate_f >> 5], 1u << (mate_f & 31));
                 else atomicAnd(&W.EF[mate_f >> 5], ~(1u << (mate_f & 31)));
@@ -3375,6 +3570,7 @@ list_run_kernel(FastArgs A) {
         __syncthreads();
     };
     // Where the two orders stand, for the next window.
+    bool built = false;
     auto leave = [&]() {
         if (warp == 0) {
             int32_t head = S.head, cur = S.cur;
@@ -3388,15 +3584,18 @@ list_run_kernel(FastArgs A) {
             }
             if (lane == 0) { S.head = head; S.cur = cur; }
         }
+        sv_slot = -1;
+        if (laner && built && W.lane[x].kind == 1) { sv_slot = W.lane[x].slot; sv_key = W.lane[x].key; sv_m2 = W.lane[x].m2; }
+        built = true;
         __syncthreads();
     };
 
     bool fresh = true, agree = false;
     int32_t agree_wait = 0, agree_back = 1;                 // batches until agreement is tried again; doubles while it fails
     long long n_win = 0, n_run = 0, dec_run = 0, n_iter = 0, dec_iter = 0, cy_build = 0, n_cta_dissolve = 0, cy_dissolve = 0;
-    long long iters = 0;                                    // (every pass makes a decision, or a new window)
+    int32_t idle = 0;                                       // passes in a row without a decision (a new window, and then one must follow)
     while (c < n) {
-        if (++iters > 64LL * n + 4096) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen
+        if (++idle > 8) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen
         if (fresh) {
             const long long t0 = clock64();
             leave();
@@ -3408,13 +3607,20 @@ list_run_kernel(FastArgs A) {
         set_i0();
         const int32_t left = n - c;
         int32_t B = 0, kind = -1;                           // decisions of this batch; the step that comes next (-1: none)
-        bool spent = false;                                 // the window holds no more
+        bool lanes_on = false;                              // the commit has changed lanes
+        int32_t gone_f = -1, gone_l = -1;
+        bool spent = false, late = false;                   // the window holds no more; the step comes after the commit
         if (agree) {
             // ---- the stretch on which both orders agree
             if (tid < WORDS) { W.F[tid].x = W.LF[tid]; W.L[tid].x = W.LL[tid]; W.eq[tid] = 0u; }
+            if (tid == 0) S.lane_lim = KLPM_LIST_FAR;
             __syncthreads();
             ranks();
             __syncthreads();
+            if (laner) {
+                W.lane[x].taken = 0;
+                if (W.lane[x].kind == 1) { const int32_t jr = W.lane[x].jr; if (jr < n_l || list_end) atomicMin(&S.lane_lim, jr < n_l ? list_rank(jr) : S.tot_l); }
+            }
 #pragma unroll
             for (int r = 0; r < PER; ++r) {
                 if (!((alive >> r) & 1u)) continue;
@@ -3440,11 +3646,12 @@ list_run_kernel(FastArgs A) {
             if (e1 < B) B = e1;
             if (e2 < B) B = e2;
             if (e3 < B) B = e3;
+            if (S.lane_lim < B) B = S.lane_lim;
             if (B > 0) {
                 const bool f_next = use_f && B >= i0 && (B - i0) % kk == 0;
-                if (B < left) kind = f_next ? (B == e1 ? 0 : -1) : B == e3 ? 2 : B == e2 ? 1 : -1;
+                if (B < left) kind = f_next ? (B == e1 ? 0 : -1) : B == e3 ? 2 : B == S.lane_lim ? -1 : B == e2 ? 1 : -1;
                 spent = kind < 0 && B == run && (run == S.tot_f || run == S.tot_l);
-                if (kind >= 0 && warp == 0) one_step(kind, c + B, cyc + B);
+                if (kind >= 0 && warp == 0) one_step(kind, c + B);
                 else {
                     for (int w = kind >= 0 ? warp - 1 : warp; w < WORDS; w += kind >= 0 ? NW - 1 : NW) {
                         const uint2 f = W.F[w], l = W.L[w];      // (the same slots on both sides)
@@ -3477,10 +3684,16 @@ list_run_kernel(FastArgs A) {
             int32_t tf[PER], tl[PER];
             unsigned own = 0;                               // bits 0-3: guessed to go to the oldest-first side, 4-7: to the list
             if (tid == 0) { S.tstar[0] = KLPM_LIST_FAR; S.tstar[1] = KLPM_LIST_FAR; }
+            const bool with_lanes = S.n_pair > 0 || S.n_grown > 0;
             for (int it = 0;; ++it) {
                 ranks();
                 __syncthreads();
                 int32_t best = KLPM_LIST_FAR;
+                if (with_lanes) {
+                    if (laner) lane_turns();
+                    __syncthreads();
+                    if (laner) best = lane_round();
+                }
                 unsigned flip = 0;
                 own = 0;
 #pragma unroll
@@ -3491,7 +3704,7 @@ list_run_kernel(FastArgs A) {
                         const unsigned bi = 1u << (i & 31), bp = 1u << (p & 31);
                         const uint2 f = W.F[i >> 5], l = W.L[p >> 5];
                         tf[r] = f_turn((int32_t)f.y + __popc(f.x & (bi - 1u)));
-                        tl[r] = l_turn((int32_t)l.y + __popc(l.x & (bp - 1u)));
+                        tl[r] = l_turn(ord((int32_t)l.y + __popc(l.x & (bp - 1u)), p));
                         const bool is_f = (f.x & bi) != 0u, is_l = (l.x & bp) != 0u, to_f = tf[r] < tl[r];
                         if (is_f) own |= 1u << r;
                         if (is_l) own |= 16u << r;
@@ -3506,11 +3719,11 @@ list_run_kernel(FastArgs A) {
                 __syncthreads();
                 T = S.tstar[it & 1];
                 const int32_t e1 = S.ev_f < KLPM_LIST_FAR ? f_turn(S.ev_f) : KLPM_LIST_FAR;
-                e2 = S.ev_l < KLPM_LIST_FAR ? l_turn(S.ev_l) : KLPM_LIST_FAR;
-                e3 = S.ev_r < KLPM_LIST_FAR ? l_turn(S.ev_r) : KLPM_LIST_FAR;
+                e2 = S.ev_l < KLPM_LIST_FAR ? l_turn(ord(S.ev_l, S.ix_l)) : KLPM_LIST_FAR;
+                e3 = S.ev_r < KLPM_LIST_FAR ? l_turn(ord(S.ev_r, S.ix_r - 1)) : KLPM_LIST_FAR;      // (at the earliest)
                 ev = e1 < e2 ? e1 : e2;
                 if (e3 < ev) ev = e3;
-                const int32_t wf = f_turn(S.tot_f), wl = l_turn(S.tot_l);
+                const int32_t wf = f_turn(S.tot_f), wl = l_turn(ord(S.tot_l, KLPM_LIST_WIN));
                 win = wf < wl ? wf : wl;
                 // (what needs a step, and what the window cannot answer any more, is only known once everything before has been settled)
                 if (T > ev || T >= left || T > win || it >= KLPM_LIST_ROUNDS || (it >= 3 && T > 0 && T < 12 * it)) break;
@@ -3520,6 +3733,13 @@ list_run_kernel(FastArgs A) {
                     const int32_t i = (int32_t)(cv[r] & 0xffffu), p = (int32_t)(cv[r] >> 16);
                     if ((flip >> r) & 1u) atomicXor(&W.F[i >> 5].x, 1u << (i & 31));
                     if ((flip >> r) & 16u) atomicXor(&W.L[p >> 5].x, 1u << (p & 31));
+                }
+                if (with_lanes && laner && W.lane[x].kind) {
+                    ListLane& l = W.lane[x];
+                    const unsigned d = lane_now ^ lane_new;
+                    if (d & 1u) atomicXor(&W.F[l.fi >> 5].x, 1u << (l.fi & 31));
+                    if (d & 2u) atomicXor(&W.L[l.lp >> 5].x, 1u << (l.lp & 31));
+                    l.taken = lane_new >> 2; l.o = lane_o; l.A = lane_A;
                 }
                 __syncthreads();
             }
@@ -3532,10 +3752,13 @@ list_run_kernel(FastArgs A) {
             if (B == 0 && kind < 0 && !spent) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen: a second round settles the first turn
             if (agree_wait > 0) --agree_wait;
             else if (use_f && use_l && T <= ev && T < left && T < 64) agree = true;      // next to nothing settled: do the orders agree?
-            if (kind >= 0 && warp == 0) one_step(kind, c + B, cyc + B);
+            const bool beside = kind >= 0 && !(kind != 1 && with_lanes);      // (where a changed key is involved the step looks at the grown keys, and the commit changes those)
+            late = kind >= 0 && !beside;
+            lanes_on = with_lanes && B > 0;
+            if (beside && warp == 0) one_step(kind, c + B);
             else if (B > 0) {
                 const int32_t nfb = f_count(B), nlb = B - nfb;
-                for (int w = kind >= 0 ? warp - 1 : warp; w < WORDS; w += kind >= 0 ? NW - 1 : NW) {
+                for (int w = beside ? warp - 1 : warp; w < WORDS; w += beside ? NW - 1 : NW) {
                     const uint2 f = W.F[w], l = W.L[w];
                     if (f.x && (int32_t)f.y < nfb) {
                         const int32_t rank = (int32_t)f.y + __popc(f.x & ((1u << lane) - 1u));
@@ -3545,7 +3768,7 @@ list_run_kernel(FastArgs A) {
                         if (lane == 0) { atomicAnd(&W.F[w].x, ~m); atomicAnd(&W.LF[w], ~m); }
                     }
                     if (l.x && (int32_t)l.y < nlb) {
-                        const int32_t rank = (int32_t)l.y + __popc(l.x & ((1u << lane) - 1u));
+                        const int32_t rank = ord((int32_t)l.y + __popc(l.x & ((1u << lane) - 1u)), w * 32 + lane);
                         const bool mine = ((l.x >> lane) & 1u) && rank < nlb;
                         if (mine) take(W.ls[w * 32 + lane], l_turn(rank));
                         const unsigned m = __ballot_sync(FULL_MASK, mine);
@@ -3560,18 +3783,51 @@ list_run_kernel(FastArgs A) {
                     if (((own >> r) & 1u) && tf[r] < B) { atomicAnd(&W.LL[p >> 5], ~(1u << (p & 31))); alive &= ~(1u << r); }
                     if (((own >> r) & 16u) && tl[r] < B) { atomicAnd(&W.LF[i >> 5], ~(1u << (i & 31))); alive &= ~(1u << r); }
                 }
+                if (with_lanes && laner) {
+                    // this lane's turn, if the batch holds it: by the guesses that the rounds ended with
+                    ListLane& l = W.lane[x];
+                    const int32_t nlb = l_count(B);
+                    unsigned by = 0;                        // which side took it
+                    if (l.kind) by = (lane_now & 1u) && lane_tf < B ? 1u : (lane_now & 2u) && lane_tl < B ? 2u : (lane_now & 4u) && l.o < nlb ? 4u : 0u;
+                    const int32_t t = by == 1u ? lane_tf : by == 2u ? lane_tl : by == 4u ? l_turn(l.o) : KLPM_LIST_FAR;
+                    const int32_t tm = __shfl_xor_sync(FULL_MASK, t, 1);
+                    if (by) {                               // its marks on the other sides go (the guesses only once everybody has read them)
+                        if (by == 4u) take(l.slot, t);
+                        if (by != 1u && l.fi >= 0) { atomicAnd(&W.LF[l.fi >> 5], ~(1u << (l.fi & 31))); gone_f = l.fi; }
+                        if (l.lp >= 0) { atomicAnd(&W.LL[l.lp >> 5], ~(1u << (l.lp & 31))); gone_l = l.lp; }
+                    }
+                    if (l.kind == 2 && (by || tm < KLPM_LIST_FAR)) {      // the group is dissolved
+                        atomicAnd(R.gb + (l.slot >> 5), ~(1u << (l.slot & 31)));
+                        if (tm < t) {                       // the other one came first: its key has grown
+                            __stcg(reinterpret_cast<int32_t*>(A.dyn + l.slot) + 2, l.m2);
+                            __stcg(A.key + l.slot, l.key);
+                            atomicOr(R.skip + (l.slot >> 5), 1u << (l.slot & 31));
+                            if (l.lp >= 0) { atomicAnd(&W.LL[l.lp >> 5], ~(1u << (l.lp & 31))); gone_l = l.lp; }
+                            l.lp = -1;
+                        }
+                        l.kind = by ? 0 : 1;
+                    } else if (by) l.kind = 0;
+                    l.o -= nlb; l.A = l.A > nlb && l.kind == 2 ? l.A - nlb : 0;
+                    if (l.o < 0) l.taken = 0;
+                }
                 ++n_iter; dec_iter += B;
             }
         }
+        if (B > 0 || kind >= 0) idle = 0;
         c += B;
         if (A.policy == KLPM_POLICY_KLPM) cyc = (int32_t)(((long long)cyc + B) % A.k);
         if (c >= n) break;
         __syncthreads();
+        if (lanes_on) {
+            if (gone_f >= 0) atomicAnd(&W.F[gone_f >> 5].x, ~(1u << (gone_f & 31)));
+            if (gone_l >= 0) atomicAnd(&W.L[gone_l >> 5].x, ~(1u << (gone_l & 31)));
+            __syncthreads();
+        }
+        if (late) { if (warp == 0) one_step(kind, c); __syncthreads(); }
         if (kind >= 0) {
             if (S.failed) break;
-            const int32_t made = S.made;
-            c += made;
-            if (A.policy == KLPM_POLICY_KLPM) cyc = (cyc + made) % A.k;
+            ++c;
+            if (A.policy == KLPM_POLICY_KLPM && ++cyc == A.k) cyc = 0;
             if (S.job == 2) {                               // a group that the whole CTA dissolves: its sorts use the window's memory
                 const long long t1 = clock64();
                 refresh();
@@ -5480,7 +5736,7 @@ rt_status ensure_fast_scratch(rt_tree* t, long long n) {
     const SlabPart parts[] = {slab_part(&t->fast_dyn, np2), slab_part(&t->fast_stat, np2), slab_part(&t->fast_key_arr, np2),
                               slab_part(&t->fast_mem, t->fast_mem_cap), slab_part(&t->fast_gh, np2), slab_part(&t->fast_gidx, np2),
                               slab_part(&t->fast_done, 3 * (np2 / 32 + 32)),      // processed bitmap, grouped bitmap, passed-over bitmap
-                              slab_part(&t->fast_lk, np2), slab_part(&t->fast_ls, np2), slab_part(&t->fast_lcp, np2), slab_part(&t->fast_pair, np2),
+                              slab_part(&t->fast_lk, np2), slab_part(&t->fast_ls, np2), slab_part(&t->fast_lcp, np2), slab_part(&t->fast_pair, 2 * np2),
                               slab_part(&t->grp_key, 4 * np2 + 1),                // keys, and as many counts and offsets (see run_impl)
                               slab_part(&t->fast_post, 1), slab_part(&t->fast_bsum, 1024)};
     const rt_status s = slab_alloc(&t->fast_slab, parts, (int)(sizeof(parts) / sizeof(parts[0])));

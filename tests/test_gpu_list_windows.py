@@ -1,0 +1,46 @@
+"""Queues that take several windows of the list-mode loop (2,048 entries of either pick order each), with prompts that share their
+continuation in twos and threes: compared with the one-decision-at-a-time loop, which the oracle checks at smaller sizes."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2502_04677_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def K():
+    from paper_2502_04677_b200 import binding
+    return binding
+
+
+@pytest.mark.parametrize("n", [2047, 2049, 8191, 8193, 12288])
+@pytest.mark.parametrize("own", [900, 40_000])
+def test_windows_against_the_one_by_one_loop(K, n, own):
+    """`own` different continuations of 12 prefixes (two of one length): about 40 prompts of a prefix share theirs at 900, few at 40,000.
+    Queues of 8,192 and more work groups of two out inside the rounds."""
+    rng = np.random.RandomState(n + own)
+    prefixes = [rng.randint(0, 1000, size=ln).tolist() for ln in (3, 9, 17, 17, 25, 33, 40, 41, 50, 64, 80, 90)]
+    prompts = [prefixes[rng.randint(12)] + [2000 + int(rng.randint(own))] + rng.randint(0, 9, size=rng.randint(0, 4)).tolist() for _ in range(n)]
+    ct, co = W.to_csr([p + [1001] for p in prefixes])
+    qt, qo = W.to_csr(prompts)
+    arr = torch.from_numpy(np.sort(rng.randint(0, 50, size=n)).astype(np.int64)).cuda()
+    prio = torch.from_numpy(rng.randint(0, 20, size=n).astype(np.int64)).cuda()
+    d_qt, d_qo = qt.cuda(), qo.cuda()
+    tree = K.rt_build(ct.cuda(), co.cuda(), max_nodes=2 * n + 64, max_pool_tokens=ct.numel() + qt.numel() + 8 * n + 64, max_clock=n + 64)
+    K.rt_checkpoint(tree)
+    for policy, k, ties, mode in ((2, 2, False, 0), (2, 4, False, 0), (2, 5, True, 1), (2, 300, False, 0), (1, 1, True, 0), (0, 1, False, 0)):
+        got = []
+        for one_by_one in (0, 1):
+            K.rt_rollback(tree)
+            out = [torch.full((n,), -1, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64, torch.int64)]
+            K.klpm_debug_set("run_one_by_one", one_by_one)
+            try:
+                K.klpm_run_ex(tree, d_qt, d_qo, arr, K.make_params(policy, k, 1, 3, 50), prio if ties else None, mode, *out)
+                assert K.rt_sync_status(tree) == 0
+            finally:
+                K.klpm_debug_set("run_one_by_one", -1)
+            got.append(out)
+        for a, b in zip(*got):
+            assert torch.equal(a, b), (policy, k, ties, mode)
