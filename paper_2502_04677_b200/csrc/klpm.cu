@@ -1801,7 +1801,7 @@ struct FastArgs {
     int32_t done_in_smem;
     int32_t list_mode;            // the list mode of the loop can be used (trees without a budget)
     unsigned int* gbits;          // bitmap of slots whose group has more than one member, as the loop starts (and throughout, if the bitmaps stay in global memory)
-    unsigned int* gskip;          // list mode with the bitmaps in global memory: slots whose key has changed since the sort
+    unsigned int* gskip;          // list mode with the bitmaps in global memory: slots the sorted list must pass over
     int32_t bits_in_smem;         // list mode: those two bitmaps are in shared memory
     const long long* lk;          // list mode: every slot's key, largest first, stored as ~key with the top bit flipped
     const int32_t* ls;            //            and the slot it belongs to
@@ -2140,7 +2140,7 @@ struct FastTour {
     unsigned long long* t2;   // per 32 leaf blocks (padded likewise)
     unsigned long long* t3;   // 32 entries
     unsigned int* done;       // bitmap of processed slots (shared memory), or null
-    unsigned int* skip;       // bitmap of slots whose key has changed since the sort (the list passes over them), or null
+    unsigned int* skip;       // bitmap of slots the sorted list must pass over: processed, or key changed (shared memory), or null
     unsigned int* gb;         // bitmap of slots whose group has more than one member (shared memory), or null
     unsigned int* dirty;      // trees with a budget: bitmap of leaf blocks to recompute after a fallback (256 words, shared memory)
     int g_done, g_bits;       // the processed bitmap / the other two bitmaps live in global memory (queues too long for shared memory)
@@ -2945,7 +2945,6 @@ struct ListTaken { unsigned long long key; int32_t A, o, jr, lane; };
 #define KLPM_LIST_LANES 128           // the first half for grown keys, the second for groups of two
 #define KLPM_LIST_LANE_MIN 8192        // shorter queues make those decisions one at a time: they are few, and lanes lengthen every round (1,000 queries: 65 us, with lanes 121)
 #define KLPM_LIST_CAND 288
-#define KLPM_LIST_CAND_MIN 8           // so do windows with fewer: their lanes would cost what some two steps cost
 #define KLPM_LIST_TAKEN 80             // guessed to be taken with a grown key at a time, at most (more are not guessed)
 struct ListShared {
     int32_t n_cand, n_pair, n_grown, n_taken, lane_lim;
@@ -3049,13 +3048,12 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         S.head = A.post->head; S.cur = 0; S.root = 0ULL; S.failed = 0; S.job = 0; S.pre_n[0] = 0; S.pre_n[1] = 0; S.n_taken = 0;
     }
     if (A.done_in_smem) for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) R.done[i] = c > 0 ? __ldcg(A.done + i) : 0u;
-    for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {
-        R.skip[i] = 0u;                                     // (slots whose key has changed since the sort)
+    for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {      // (the list passes over processed slots, so far)
+        R.skip[i] = c > 0 ? __ldcg(A.done + i) : 0u;
         if (A.bits_in_smem) R.gb[i] = __ldcg(A.gbits + i);
     }
     __syncthreads();
     auto bit_of = [&](const unsigned* bm, int32_t slot, int g) -> unsigned { return (bm_ld(bm, slot >> 5, g) >> (slot & 31)) & 1u; };
-    auto stale = [&](int32_t s) -> bool { return (((bm_ld(R.done, s >> 5, gdone) | bm_ld(R.skip, s >> 5, gbits)) >> (s & 31)) & 1u) != 0u; };      // the list passes over it
     // ---- turns, counted from the next decision: the t-th oldest-first turn, the u-th longest-match turn, oldest-first turns among x decisions.
     // (a k beyond what a window holds is as good as any such k)
     const bool use_f = A.policy != KLPM_POLICY_LPM;
@@ -3104,7 +3102,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             const int w = warp + NW * r, i = w * 32 + lane;
             const bool hf = (W.LF[w] >> lane) & 1u, hl = (W.LL[w] >> lane) & 1u;
             const int32_t sf = hf ? W.fs[i] : 0, sl = hl ? W.ls[i] : 0;
-            const bool in_f = hf && !bit_of(R.done, sf, gdone), in_l = hl && !stale(sl);
+            const bool in_f = hf && !bit_of(R.done, sf, gdone), in_l = hl && !bit_of(R.skip, sl, gbits);
             const unsigned lf = __ballot_sync(FULL_MASK, in_f), ll = __ballot_sync(FULL_MASK, in_l);
             const unsigned ef = __ballot_sync(FULL_MASK, in_f && ((use_l ? bit_of(R.skip, sf, gbits) : 0u) | bit_of(R.gb, sf, gbits)));
             const unsigned el = __ballot_sync(FULL_MASK, in_l && bit_of(R.gb, sl, gbits));
@@ -3123,22 +3121,11 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         if (laner && W.lane[x].kind) no_event(W.lane[x].fi, W.lane[x].lp);
         __syncthreads();
     };
-    auto to_tournament = [&]() {                            // a grown key that is not a lane's any more
-        const int32_t b = sv_slot >> A.lb_shift;
-        atomicMax(R.t1 + b, sv_key); atomicMax(R.t2 + (b >> 5), sv_key); atomicMax(R.t3 + (b >> 10), sv_key); atomicMax(&S.root, sv_key);
-        const int32_t f = index_of(sv_slot);
-        if (f >= 0 && use_l) atomicOr(&W.EF[f >> 5], 1u << (f & 31));
-    };
     // The lanes of a new window: the grown keys kept from the last one, and both prompts of the groups of two that have one in the window.
     // What finds no lane goes on as before: a grown key to the tournament, a group as an event.
     auto lanes = [&]() {
-        const int32_t n_cand = S.n_cand >= KLPM_LIST_CAND_MIN && S.n_cand <= KLPM_LIST_CAND && n >= KLPM_LIST_LANE_MIN ? S.n_cand : 0;      // (too many to know all positions: none)
-        if (n_cand == 0) {
-            if (laner) W.lane[x].kind = 0;
-            if (sv_slot >= 0 && !bit_of(R.done, sv_slot, gdone)) to_tournament();
-            __syncthreads();
-            return;
-        }
+        const int32_t n_cand = S.n_cand <= KLPM_LIST_CAND && n >= KLPM_LIST_LANE_MIN ? S.n_cand : 0;      // (too many to know all positions: none)
+        if (n_cand == 0 && !__syncthreads_or(sv_slot >= 0)) { if (laner) W.lane[x].kind = 0; __syncthreads(); return; }
         int32_t* const low = reinterpret_cast<int32_t*>(W.taken);              // per candidate: the smaller slot of its pair (no key is guessed to be taken yet)
         if (laner) W.lane[x].kind = 0;
         if (tid < WORDS) W.eq[tid] = 0u;
@@ -3158,7 +3145,10 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                 ListLane l;
                 l.key = sv_key; l.slot = sv_slot; l.m2 = sv_m2; l.fi = (short)index_of(sv_slot); l.lp = -1; l.jr = -1; l.o = 0; l.A = 0; l.kind = 1; l.taken = 0;
                 W.lane[at] = l;
-            } else to_tournament();
+            } else {
+                const int32_t b = sv_slot >> A.lb_shift;
+                atomicMax(R.t1 + b, sv_key); atomicMax(R.t2 + (b >> 5), sv_key); atomicMax(R.t3 + (b >> 10), sv_key); atomicMax(&S.root, sv_key);
+            }
         }
         if (mate >= 0) {
             const int32_t lo = low[tid];
@@ -3215,7 +3205,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
 #pragma unroll
                 for (int r = 0; r < PER; ++r) {
                     const int w = warp + NW * r;
-                    const bool in = slot_in[r] >= 0 && !stale(slot_in[r]);
+                    const bool in = slot_in[r] >= 0 && !bit_of(R.skip, slot_in[r], gbits);
                     const unsigned live = __ballot_sync(FULL_MASK, in), ev = __ballot_sync(FULL_MASK, in && bit_of(R.gb, slot_in[r], gbits));
                     if (lane == 0) { W.LL[w] = live; W.L[w].x = live; W.EL[w] = ev; }
                     any |= live != 0u;
@@ -3278,14 +3268,14 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         if (use_l) {
 #pragma unroll
             for (int r = 0; r < PER; ++r)
-                if (slot_in[r] >= 0 && !stale(slot_in[r]) && bit_of(R.gb, slot_in[r], gbits)) candidate(slot_in[r], tid + KLPM_LIST_THREADS * r);
+                if (slot_in[r] >= 0 && !bit_of(R.skip, slot_in[r], gbits) && bit_of(R.gb, slot_in[r], gbits)) candidate(slot_in[r], tid + KLPM_LIST_THREADS * r);
         }
         if (use_f && use_l && n_f > 0) {                    // the meetings
             const int32_t hmax = W.fs[n_f - 1];
 #pragma unroll
             for (int r = 0; r < PER; ++r) {
                 const int32_t s = slot_in[r];
-                bool met = s >= head && s <= hmax && !stale(s);
+                bool met = s >= head && s <= hmax && !bit_of(R.skip, s, gbits);
                 int32_t phi = 0;
                 if (met) {
                     const int32_t wl = (s >> 5) - w0;       // (below KLPM_LIST_THREADS: hmax is)
@@ -3450,6 +3440,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     };
     auto take = [&](int32_t slot, int32_t at) {
         atomicOr(R.done + (slot >> 5), 1u << (slot & 31));
+        atomicOr(R.skip + (slot >> 5), 1u << (slot & 31));
         A.order[c + at] = slot;
     };
     // Warp 0: one decision that needs a step -- the oldest slot (kind 0), the next list entry (1) or the tournament's root (2).
@@ -3485,6 +3476,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         __syncwarp();
         if (lane == 0) {
             atomicOr(R.done + (j >> 5), 1u << (j & 31));
+            if (!in_tour) atomicOr(R.skip + (j >> 5), 1u << (j & 31));
             A.order[at] = j;
         }
         __syncwarp();
