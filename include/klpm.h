@@ -255,6 +255,8 @@ rt_status rt_debug_counters(rt_tree* tree, int64_t* out16);
  *   "fast_smem_kb"     grouped loop: the shared memory it may use, in KiB (default 0 = 224)
  *   "wait_limit_ns"    one-by-one loop: how long a CTA waits for another before it gives up, records
  *                      RT_ERR_LIMIT (detail 102) and lets every CTA return (default 5e9; 0 = give up at once)
+ *   "list_max_windows" grouped loop, once everybody has arrived: it gives up before the window after this many, records
+ *                      RT_ERR_LIMIT (detail 118) and charges none of the decisions made since then (default 2^31 - 1)
  * RT_ERR_INVALID for an unknown name. */
 rt_status klpm_debug_set(const char* name, int64_t value);
 

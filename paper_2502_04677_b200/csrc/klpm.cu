@@ -1770,7 +1770,7 @@ struct alignas(32) FStat {    // constant during the loop; the first 16 bytes ar
 struct alignas(32) LNode { int32_t parent, depth, len, nchild; long long last, off; };
 
 struct FastPost {
-    int32_t c0; int32_t list_c;                 // decisions the charge pass after the loop starts from; decisions made before everybody had arrived
+    int32_t c0; int32_t list_c;                 // first decision the charge pass after the loop charges (n: none, as after a loop that gave up); decisions made before everybody had arrived
     long long now0; int32_t head, cyc;          // the time then, the oldest unprocessed slot, decisions made mod k
     // what the loop did (rt_debug_counters): careful steps, dissolves by the whole CTA, fallback scans, slots that fell
     // back, evictions; cycles spent in tree updates, fallback scans, dissolves; list mode: windows, batches in which the two
@@ -1805,6 +1805,7 @@ struct FastArgs {
     int32_t bits_in_smem;         // list mode: those two bitmaps are in shared memory
     const long long* lk;          // list mode: every slot's key, largest first, stored as ~key with the top bit flipped
     const int32_t* ls;            //            and the slot it belongs to
+    int32_t max_windows;          // list mode: windows after which the loop gives up (debug setting)
     const int64_t* arrival;       // per query: arrival (for the charge pass after the loop)
     struct FastPost* post;        // where list mode began, for the charge pass after the loop
     TreeState* st;
@@ -2958,6 +2959,7 @@ struct ListShared {
     int32_t step_f, step_l, mate_f, mate;        // what a step took (index, position) and changed (index, slot); -1: nothing
     unsigned long long root;
     int32_t w[KLPM_LIST_THREADS / 32];
+    long long cn[16];                            // what the loop did (FastPost::counters), kept by thread 0: registers are short here
 };
 static_assert(KLPM_LIST_WIN * (4 + 4 + 8 + 4) + KLPM_LIST_THREADS * 8 + 9 * (KLPM_LIST_WIN / 32) * 4 + KLPM_LIST_CAND * 6 <= KLPM_FAST_SORT_CAP * 12, "a window fits the sort scratch");
 static_assert(KLPM_LIST_LANES * sizeof(ListLane) + 2 * KLPM_LIST_TAKEN * sizeof(ListTaken) <= KLPM_LIST_WIN * 4, "the lanes fit the place of the meetings");
@@ -3046,7 +3048,9 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     if (tid == 0) {
         s_memcur = n;
         S.head = A.post->head; S.cur = 0; S.root = 0ULL; S.failed = 0; S.job = 0; S.pre_n[0] = 0; S.pre_n[1] = 0; S.n_taken = 0;
+        for (int i = 0; i < 16; ++i) S.cn[i] = 0;
     }
+    auto count = [&](int i, long long v) { if (tid == 0) S.cn[i] += v; };
     if (A.done_in_smem) for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) R.done[i] = c > 0 ? __ldcg(A.done + i) : 0u;
     for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {      // (the list passes over processed slots, so far)
         R.skip[i] = c > 0 ? __ldcg(A.done + i) : 0u;
@@ -3444,10 +3448,9 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         A.order[c + at] = slot;
     };
     // Warp 0: one decision that needs a step -- the oldest slot (kind 0), the next list entry (1) or the tournament's root (2).
-    long long n_one = 0, n_dis = 0, cy_step = 0;
     // `at`: its number.  Other warps commit the batch before it at the same time: what both change is changed by atomics.
     auto one_step = [&](int kind, int32_t at) {
-        const long long t0 = clock64();
+        const unsigned t0 = (unsigned)clock();
         unsigned long long root = S.root;
         int32_t j;
         bool from_lane = false;
@@ -3492,9 +3495,9 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             root = tour_set(R, b, warp_max64r(v), lane);
             __syncwarp();
         }
-        ++n_one;
+        count(13, 1);
         if (grouped) {
-            ++n_dis;
+            count(0, 1);
             int4 rec;
             const int last = kind < 2 ? (S.pre_n[kind] - 1) & 3 : 0;      // (found by the round before this step)
             if (kind < 2 && S.pre_slot[kind][last] == j) rec = S.pre[kind][last];
@@ -3539,7 +3542,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                 else atomicAnd(&W.EF[mate_f >> 5], ~(1u << (mate_f & 31)));
             }
         }
-        cy_step += clock64() - t0;
+        count(15, (unsigned)clock() - t0);
     };
     // What the step leaves to do for the window, every thread: the list entries of the two slots, and their meetings.
     auto after_step = [&]() {
@@ -3584,16 +3587,14 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
 
     bool fresh = true, agree = false;
     int32_t agree_wait = 0, agree_back = 1;                 // batches until agreement is tried again; doubles while it fails
-    long long n_win = 0, n_run = 0, dec_run = 0, n_iter = 0, dec_iter = 0, cy_build = 0, n_cta_dissolve = 0, cy_dissolve = 0;
     int32_t idle = 0;                                       // passes in a row without a decision (a new window, and then one must follow)
     while (c < n) {
-        if (++idle > 8) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen
+        if (++idle > 8 || (fresh && S.cn[8] >= A.max_windows)) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen (without the debug setting)
         if (fresh) {
-            const long long t0 = clock64();
+            const unsigned t0 = (unsigned)clock();
             leave();
             build();
-            ++n_win;
-            cy_build += clock64() - t0;
+            count(8, 1); count(14, (unsigned)clock() - t0);
             fresh = false;
         }
         set_i0();
@@ -3661,7 +3662,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                         }
                     }
                 }
-                ++n_run; dec_run += B;
+                count(9, 1); count(10, B);
                 __syncthreads();
 #pragma unroll
                 for (int r = 0; r < PER; ++r) {
@@ -3802,7 +3803,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                     l.o -= nlb; l.A = l.A > nlb && l.kind == 2 ? l.A - nlb : 0;
                     if (l.o < 0) l.taken = 0;
                 }
-                ++n_iter; dec_iter += B;
+                count(11, 1); count(12, B);
             }
         }
         if (B > 0 || kind >= 0) idle = 0;
@@ -3821,7 +3822,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             ++c;
             if (A.policy == KLPM_POLICY_KLPM && ++cyc == A.k) cyc = 0;
             if (S.job == 2) {                               // a group that the whole CTA dissolves: its sorts use the window's memory
-                const long long t1 = clock64();
+                const unsigned t1 = (unsigned)clock();
                 refresh();
                 leave();
                 const FastJob J = s_job;
@@ -3829,8 +3830,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                 if (warp == 0) { const unsigned long long r = tour_top(R, lane); if (lane == 0) S.root = r; }
                 __syncthreads();
                 if (c < n) build();
-                ++n_win; ++n_cta_dissolve;
-                cy_dissolve += clock64() - t1;
+                count(8, 1); count(1, 1); count(7, (unsigned)clock() - t1);
             } else if (S.job == 1) refresh();
             else after_step();
         }
@@ -3839,9 +3839,9 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     list_fetch_wait();
     __syncthreads();
     if (tid == 0) {
+        if (c < n) A.post->c0 = n;                          // gave up: the entries of `order` that were never written are no slots, and nothing is charged
         long long* cn = A.post->counters;
-        cn[0] += n_dis; cn[1] += n_cta_dissolve; cn[7] += cy_dissolve;
-        cn[8] = n_win; cn[9] = n_run; cn[10] = dec_run; cn[11] = n_iter; cn[12] = dec_iter; cn[13] = n_one; cn[14] = cy_build; cn[15] = cy_step;
+        for (int i = 0; i < 16; ++i) cn[i] += S.cn[i];      // (the last eight are list mode's alone)
     }
 }
 
@@ -5747,8 +5747,9 @@ struct DebugKnobs {
     long long fast_max_blocks;    // grouped loop: most tournament leaf blocks (0 = the built-in 8,192)
     long long fast_smem_kb;       // grouped loop: shared memory it may use (0 = the built-in 224 KB)
     long long wait_limit_ns;      // one-by-one loop: limit of a hand-over wait
+    long long list_max_windows;   // grouped loop, everybody waiting: windows after which it gives up
 };
-DebugKnobs g_knobs = {0, 0, 0, KLPM_WAIT_LIMIT_NS};
+DebugKnobs g_knobs = {0, 0, 0, KLPM_WAIT_LIMIT_NS, 0x7fffffffLL};
 
 SelectScratch* g_select_scratch[64] = {nullptr};
 TopkScratch* g_topk_scratch[64] = {nullptr};
@@ -6393,6 +6394,7 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
         if (f.done_in_smem) smem += (size_t)nwords * 4;
         // list mode (trees without a budget) needs two more bitmaps: in shared memory while they fit, in global memory beyond
         f.list_mode = (lru || d_fixed) ? 0 : 1;
+        f.max_windows = (int32_t)g_knobs.list_max_windows;
         f.bits_in_smem = (f.list_mode && f.done_in_smem && smem + (size_t)nwords * 8 <= smem_max) ? 1 : 0;
         if (f.bits_in_smem) smem += (size_t)nwords * 8;
         f.gbits = tree->fast_done + (np2 / 32 + 32);
@@ -6562,11 +6564,12 @@ rt_status rt_debug_counters(rt_tree* tree, int64_t* out16) {
 
 rt_status klpm_debug_set(const char* name, int64_t value) {
     if (!name) return RT_ERR_INVALID;
-    const DebugKnobs defaults = {0, 0, 0, KLPM_WAIT_LIMIT_NS};
+    const DebugKnobs defaults = {0, 0, 0, KLPM_WAIT_LIMIT_NS, 0x7fffffffLL};
     if (!strcmp(name, "run_one_by_one")) g_knobs.run_one_by_one = value < 0 ? defaults.run_one_by_one : (value != 0);
     else if (!strcmp(name, "fast_max_blocks")) g_knobs.fast_max_blocks = value < 0 ? defaults.fast_max_blocks : value;
     else if (!strcmp(name, "fast_smem_kb")) g_knobs.fast_smem_kb = value < 0 ? defaults.fast_smem_kb : value;
     else if (!strcmp(name, "wait_limit_ns")) g_knobs.wait_limit_ns = value < 0 ? defaults.wait_limit_ns : value;
+    else if (!strcmp(name, "list_max_windows")) g_knobs.list_max_windows = value < 0 || value > defaults.list_max_windows ? defaults.list_max_windows : value;
     else return RT_ERR_INVALID;
     return RT_OK;
 }

@@ -44,3 +44,39 @@ def test_windows_against_the_one_by_one_loop(K, n, own):
             got.append(out)
         for a, b in zip(*got):
             assert torch.equal(a, b), (policy, k, ties, mode)
+
+
+@pytest.mark.parametrize("windows", [0, 1, 2])
+@pytest.mark.parametrize("start", [50, 0])
+def test_a_loop_that_gives_up_charges_nothing(K, windows, start):
+    """The loop stops after that many windows of list mode: the status word says so, and the charge pass leaves the outputs of the
+    decisions made there alone (the entries of `order` behind them were never written and name no prompt).  With start 0 some
+    decisions come before everybody has arrived, and those stand.  A tree that is asked again gives what it always gives."""
+    n = 9000
+    rng = np.random.RandomState(windows)
+    prompts = [[int(rng.randint(40)), 100 + int(rng.randint(3)), 1000 + i] for i in range(n)]
+    qt, qo = W.to_csr(prompts)
+    d_qt, d_qo = qt.cuda(), qo.cuda()
+    arr = torch.from_numpy(np.sort(rng.randint(0, 50, size=n)).astype(np.int64)).cuda()
+    params = K.make_params(K.POLICY_KLPM, 3, 0, 1, start)
+    got = []
+    for limit in (windows, -1):
+        tree = K.rt_create(max_nodes=2 * n + 64, max_pool_tokens=qt.numel() + 8 * n + 64, max_clock=n + 64)
+        out = [torch.full((n,), -1, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64, torch.int64)]
+        K.klpm_debug_set("list_max_windows", limit)
+        try:
+            K.klpm_run(tree, d_qt, d_qo, arr, params, *out)
+            status, detail = K.rt_sync_status(tree), K.rt_status_detail(tree)
+        finally:
+            K.klpm_debug_set("list_max_windows", -1)
+        got.append((status, detail, [o.cpu().numpy() for o in out]))
+        K.rt_destroy(tree)
+    (status, detail, cut), (ok, _, full) = got
+    assert status == K.RT_ERR_LIMIT and detail == 118 and ok == 0
+    charged = cut[1] >= 0
+    before = int(charged.sum())                             # decisions made while arrivals were pending
+    assert (before == 0) == (start == 50) and before < n
+    assert np.array_equal(np.sort(full[0][:before]), np.flatnonzero(charged))
+    assert np.array_equal(cut[0][:before], full[0][:before])
+    for c, f in zip(cut[1:], full[1:]):
+        assert np.array_equal(c[charged], f[charged]) and (c[~charged] == -1).all()
