@@ -55,13 +55,14 @@ def test_a_loop_that_gives_up_charges_nothing(K, windows, start):
     n = 9000
     rng = np.random.RandomState(windows)
     prompts = [[int(rng.randint(40)), 100 + int(rng.randint(3)), 1000 + i] for i in range(n)]
+    ct, co = W.to_csr([[a, 100 + b, 999] for a in range(40) for b in range(3)])      # what they share is cached: no groups, every decision is a window's
     qt, qo = W.to_csr(prompts)
     d_qt, d_qo = qt.cuda(), qo.cuda()
     arr = torch.from_numpy(np.sort(rng.randint(0, 50, size=n)).astype(np.int64)).cuda()
     params = K.make_params(K.POLICY_KLPM, 3, 0, 1, start)
     got = []
     for limit in (windows, -1):
-        tree = K.rt_create(max_nodes=2 * n + 64, max_pool_tokens=qt.numel() + 8 * n + 64, max_clock=n + 64)
+        tree = K.rt_build(ct.cuda(), co.cuda(), max_nodes=2 * n + 512, max_pool_tokens=ct.numel() + qt.numel() + 8 * n + 1024, max_clock=n + 256)
         out = [torch.full((n,), -1, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64, torch.int64)]
         K.klpm_debug_set("list_max_windows", limit)
         try:
