@@ -3495,9 +3495,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             root = tour_set(R, b, warp_max64r(v), lane);
             __syncwarp();
         }
-        count(13, 1);
         if (grouped) {
-            count(0, 1);
             int4 rec;
             const int last = kind < 2 ? (S.pre_n[kind] - 1) & 3 : 0;      // (found by the round before this step)
             if (kind < 2 && S.pre_slot[kind][last] == j) rec = S.pre[kind][last];
@@ -3534,6 +3532,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             }
         }
         if (lane == 0) {
+            S.cn[13] += 1; S.cn[0] += grouped; S.cn[15] += (unsigned)clock() - t0;      // (here and not where they happen: a branch of one lane before the dissolve has it run for lane 0 and the others in turn)
             S.root = root; S.job = job; S.step_f = step_f; S.step_l = kind == 1 ? S.ix_l : -1; S.mate_f = mate_f; S.mate = mate_s;
             if (step_f >= 0) { atomicAnd(&W.LF[step_f >> 5], ~(1u << (step_f & 31))); atomicAnd(&W.F[step_f >> 5].x, ~(1u << (step_f & 31))); }
             if (mate_f >= 0) {
@@ -3542,7 +3541,6 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                 else atomicAnd(&W.EF[mate_f >> 5], ~(1u << (mate_f & 31)));
             }
         }
-        count(15, (unsigned)clock() - t0);
     };
     // What the step leaves to do for the window, every thread: the list entries of the two slots, and their meetings.
     auto after_step = [&]() {
