@@ -1801,7 +1801,7 @@ struct FastArgs {
     int32_t done_in_smem;
     int32_t list_mode;            // the list mode of the loop can be used (trees without a budget)
     unsigned int* gbits;          // bitmap of slots whose group has more than one member, as the loop starts (and throughout, if the bitmaps stay in global memory)
-    unsigned int* gskip;          // list mode with the bitmaps in global memory: slots the sorted list must pass over
+    unsigned int* gskip;          // list mode with the bitmaps in global memory: slots whose key has changed since the sort
     int32_t bits_in_smem;         // list mode: those two bitmaps are in shared memory
     const long long* lk;          // list mode: every slot's key, largest first, stored as ~key with the top bit flipped
     const int32_t* ls;            //            and the slot it belongs to
@@ -2141,7 +2141,7 @@ struct FastTour {
     unsigned long long* t2;   // per 32 leaf blocks (padded likewise)
     unsigned long long* t3;   // 32 entries
     unsigned int* done;       // bitmap of processed slots (shared memory), or null
-    unsigned int* skip;       // bitmap of slots the sorted list must pass over: processed, or key changed (shared memory), or null
+    unsigned int* skip;       // bitmap of slots whose key has changed since the sort (the list passes over them), or null
     unsigned int* gb;         // bitmap of slots whose group has more than one member (shared memory), or null
     unsigned int* dirty;      // trees with a budget: bitmap of leaf blocks to recompute after a fallback (256 words, shared memory)
     int g_done, g_bits;       // the processed bitmap / the other two bitmaps live in global memory (queues too long for shared memory)
@@ -3052,12 +3052,13 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     }
     auto count = [&](int i, long long v) { if (tid == 0) S.cn[i] += v; };
     if (A.done_in_smem) for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) R.done[i] = c > 0 ? __ldcg(A.done + i) : 0u;
-    for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {      // (the list passes over processed slots, so far)
-        R.skip[i] = c > 0 ? __ldcg(A.done + i) : 0u;
+    for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {
+        R.skip[i] = 0u;                                     // (slots whose key has changed since the sort)
         if (A.bits_in_smem) R.gb[i] = __ldcg(A.gbits + i);
     }
     __syncthreads();
     auto bit_of = [&](const unsigned* bm, int32_t slot, int g) -> unsigned { return (bm_ld(bm, slot >> 5, g) >> (slot & 31)) & 1u; };
+    auto stale = [&](int32_t s) -> bool { return (((bm_ld(R.done, s >> 5, gdone) | bm_ld(R.skip, s >> 5, gbits)) >> (s & 31)) & 1u) != 0u; };      // the list passes over it
     // ---- turns, counted from the next decision: the t-th oldest-first turn, the u-th longest-match turn, oldest-first turns among x decisions.
     // (a k beyond what a window holds is as good as any such k)
     const bool use_f = A.policy != KLPM_POLICY_LPM;
@@ -3106,7 +3107,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             const int w = warp + NW * r, i = w * 32 + lane;
             const bool hf = (W.LF[w] >> lane) & 1u, hl = (W.LL[w] >> lane) & 1u;
             const int32_t sf = hf ? W.fs[i] : 0, sl = hl ? W.ls[i] : 0;
-            const bool in_f = hf && !bit_of(R.done, sf, gdone), in_l = hl && !bit_of(R.skip, sl, gbits);
+            const bool in_f = hf && !bit_of(R.done, sf, gdone), in_l = hl && !stale(sl);
             const unsigned lf = __ballot_sync(FULL_MASK, in_f), ll = __ballot_sync(FULL_MASK, in_l);
             const unsigned ef = __ballot_sync(FULL_MASK, in_f && ((use_l ? bit_of(R.skip, sf, gbits) : 0u) | bit_of(R.gb, sf, gbits)));
             const unsigned el = __ballot_sync(FULL_MASK, in_l && bit_of(R.gb, sl, gbits));
@@ -3195,11 +3196,13 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         const int32_t head = S.head;
         long long key_in[PER];
         int32_t slot_in[PER];
+        unsigned live_l = 0;                                // which of them still count
         w0 = head >> 5; head0 = head;
         n_f = 0;
         if (use_l) {
             for (;;) {                                      // (a stretch of the list without a live entry is passed over)
                 int any = 0;
+                live_l = 0;
 #pragma unroll
                 for (int r = 0; r < PER; ++r) {
                     const long long idx = (long long)cur + tid + KLPM_LIST_THREADS * r;
@@ -3209,7 +3212,8 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
 #pragma unroll
                 for (int r = 0; r < PER; ++r) {
                     const int w = warp + NW * r;
-                    const bool in = slot_in[r] >= 0 && !bit_of(R.skip, slot_in[r], gbits);
+                    const bool in = slot_in[r] >= 0 && !stale(slot_in[r]);
+                    if (in) live_l |= 1u << r;
                     const unsigned live = __ballot_sync(FULL_MASK, in), ev = __ballot_sync(FULL_MASK, in && bit_of(R.gb, slot_in[r], gbits));
                     if (lane == 0) { W.LL[w] = live; W.L[w].x = live; W.EL[w] = ev; }
                     any |= live != 0u;
@@ -3272,14 +3276,14 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         if (use_l) {
 #pragma unroll
             for (int r = 0; r < PER; ++r)
-                if (slot_in[r] >= 0 && !bit_of(R.skip, slot_in[r], gbits) && bit_of(R.gb, slot_in[r], gbits)) candidate(slot_in[r], tid + KLPM_LIST_THREADS * r);
+                if (((live_l >> r) & 1u) && bit_of(R.gb, slot_in[r], gbits)) candidate(slot_in[r], tid + KLPM_LIST_THREADS * r);
         }
         if (use_f && use_l && n_f > 0) {                    // the meetings
             const int32_t hmax = W.fs[n_f - 1];
 #pragma unroll
             for (int r = 0; r < PER; ++r) {
                 const int32_t s = slot_in[r];
-                bool met = s >= head && s <= hmax && !bit_of(R.skip, s, gbits);
+                bool met = ((live_l >> r) & 1u) && s >= head && s <= hmax;
                 int32_t phi = 0;
                 if (met) {
                     const int32_t wl = (s >> 5) - w0;       // (below KLPM_LIST_THREADS: hmax is)
@@ -3444,11 +3448,13 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     };
     auto take = [&](int32_t slot, int32_t at) {
         atomicOr(R.done + (slot >> 5), 1u << (slot & 31));
-        atomicOr(R.skip + (slot >> 5), 1u << (slot & 31));
         A.order[c + at] = slot;
     };
     // Warp 0: one decision that needs a step -- the oldest slot (kind 0), the next list entry (1) or the tournament's root (2).
-    // `at`: its number.  Other warps commit the batch before it at the same time: what both change is changed by atomics.
+    // `at`: its number.  Other warps commit the batch before it at the same time.  What both change is changed by atomics.  What a step
+    // reads of the bitmaps does not depend on how far the commit is: it looks at the pick and the members of its group, which are events
+    // and so not in the batch, and in the pick's leaf block at slots whose key has changed.  No commit beside such a look takes or marks
+    // one (a changed key is an event too, and where lanes hold some the step comes after the commit): none of the bits in motion is asked for.
     auto one_step = [&](int kind, int32_t at) {
         const unsigned t0 = (unsigned)clock();
         unsigned long long root = S.root;
@@ -3479,7 +3485,6 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         __syncwarp();
         if (lane == 0) {
             atomicOr(R.done + (j >> 5), 1u << (j & 31));
-            if (!in_tour) atomicOr(R.skip + (j >> 5), 1u << (j & 31));
             A.order[at] = j;
         }
         __syncwarp();

@@ -81,3 +81,44 @@ def test_a_loop_that_gives_up_charges_nothing(K, windows, start):
     assert np.array_equal(cut[0][:before], full[0][:before])
     for c, f in zip(cut[1:], full[1:]):
         assert np.array_equal(c[charged], f[charged]) and (c[~charged] == -1).all()
+
+
+@pytest.mark.parametrize("smem_kb", [0, 51, 50])
+@pytest.mark.parametrize("k", [2, 3, 8])
+def test_changed_keys_are_looked_for_beside_a_commit(K, smem_kb, k):
+    """A third of the prompts come in pairs, so a key grows every few decisions and waits in the tournament.  A step that takes such a key
+    looks through its block of 32 slots while the others commit the batch before it, of which the oldest slots lie in that very block.
+    In 51 KiB the bitmap of processed slots is in shared memory and that of changed keys is not, in 50 neither is."""
+    n = 6000
+    rng = np.random.RandomState(k)
+    trunk = rng.randint(0, 30000, size=300).tolist()
+    prompts = []
+    while len(prompts) < n:
+        m, own = rng.randint(1, 300), 100_000 + len(prompts)
+        more = rng.randint(0, 30000, size=rng.randint(0, 8)).tolist()
+        prompts += [trunk[:m] + [own] + more + [90_000 + i] for i in range(2 if rng.rand() < 0.2 else 1)]
+    prompts = [prompts[i] for i in rng.permutation(len(prompts))[:n]]
+    ct, co = W.to_csr([trunk + [7]])
+    qt, qo = W.to_csr(prompts)
+    d_qt, d_qo = qt.cuda(), qo.cuda()
+    arr = torch.arange(n, dtype=torch.int64).cuda()
+    tree = K.rt_build(ct.cuda(), co.cuda(), max_nodes=2 * n + 64, max_pool_tokens=ct.numel() + qt.numel() + 8 * n + 64, max_clock=n + 64)
+    K.rt_checkpoint(tree)
+    got = []
+    for one_by_one in (1, 0, 0, 0):                         # (one order of the threads may go well)
+        K.rt_rollback(tree)
+        out = [torch.full((n,), -1, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64, torch.int64)]
+        K.klpm_debug_set("run_one_by_one", one_by_one)
+        K.klpm_debug_set("fast_smem_kb", smem_kb)
+        try:
+            K.klpm_run(tree, d_qt, d_qo, arr, K.make_params(K.POLICY_KLPM, k, 0, 1, n), *out)
+            assert K.rt_sync_status(tree) == 0
+        finally:
+            K.klpm_debug_set("run_one_by_one", -1)
+            K.klpm_debug_set("fast_smem_kb", -1)
+        got.append(out)
+    assert K.rt_debug_counters(tree)["single_decisions"] > n // 10
+    for out in got[1:]:
+        for a, b in zip(got[0], out):
+            assert torch.equal(a, b)
+    K.rt_destroy(tree)
