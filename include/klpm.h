@@ -243,7 +243,8 @@ int32_t klpm_run_path(const rt_tree* tree);
 /* What the grouped loop of the last klpm_run / klpm_run_ex on this tree did (zeros if it has not run): out16[0] decisions
  * taken by a careful step, [1] groups dissolved by the whole CTA, [2] scans after an eviction of a leaf with queries
  * parked in it, [3] queries that fell back out of evicted leaves, [4] evictions, [5..7] clock cycles spent waiting for
- * tree updates, in those scans, in dissolves by the whole CTA; once everybody had arrived: [8] windows looked at,
+ * tree updates, in those scans, in dissolves by the whole CTA (on a tree without a budget instead: [3] decisions taken by the
+ * threads of groups of two and of grown keys, [4] the most of those that were guessed to take one at a time); once everybody had arrived: [8] windows looked at,
  * [9] batches in which both pick orders agree, [10] decisions they made, [11] batches worked out by iteration, [12] decisions
  * they made, [13] decisions made one at a time, [14..15] clock cycles spent on new windows and on single decisions.  A debugging aid; synchronises
  * like rt_stats. */

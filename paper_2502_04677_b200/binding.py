@@ -134,8 +134,9 @@ def make_params(policy: int, k: int = 1, c_num: int = 0, c_den: int = 1, start_t
 class Tree:
     """Handle of a device radix tree (rt_tree*)."""
 
-    def __init__(self, handle: ctypes.c_void_p):
+    def __init__(self, handle: ctypes.c_void_p, budget_tokens: int = 0):
         self._h = handle
+        self.budget_tokens = int(budget_tokens)
 
     @property
     def handle(self) -> ctypes.c_void_p:
@@ -159,7 +160,7 @@ def rt_create(max_nodes: int, max_pool_tokens: int, budget_tokens: int = 0, voca
     cfg = rt_config(int(vocab), int(max_nodes), int(max_pool_tokens), int(budget_tokens), int(max_clock))
     h = ctypes.c_void_p()
     _check(_lib.rt_create(ctypes.byref(cfg), ctypes.byref(h)), "rt_create")
-    return Tree(h)
+    return Tree(h, budget_tokens)
 
 
 def rt_build(tokens: torch.Tensor, offsets: torch.Tensor, max_nodes: int, max_pool_tokens: int,
@@ -169,7 +170,7 @@ def rt_build(tokens: torch.Tensor, offsets: torch.Tensor, max_nodes: int, max_po
     n = offsets.numel() - 1
     _check(_lib.rt_build(_dev(tokens, torch.int32, "tokens", n == 0), _dev(offsets, torch.int64, "offsets"), n,
                          ctypes.byref(cfg), _stream(), ctypes.byref(h)), "rt_build")
-    return Tree(h)
+    return Tree(h, budget_tokens)
 
 
 def rt_insert(tree: Tree, tokens: torch.Tensor, offsets: torch.Tensor, new_tokens: Optional[torch.Tensor] = None) -> None:
@@ -212,7 +213,7 @@ def rt_stats(tree: Tree) -> dict:
 def rt_clone(tree: Tree) -> Tree:
     h = ctypes.c_void_p()
     _check(_lib.rt_clone(tree.handle, _stream(), ctypes.byref(h)), "rt_clone")
-    return Tree(h)
+    return Tree(h, tree.budget_tokens)
 
 
 def rt_checkpoint(tree: Tree) -> None:
@@ -334,14 +335,22 @@ def klpm_run_last_only_batch(tokens: torch.Tensor, offsets: torch.Tensor, arriva
 
 
 def rt_debug_counters(tree: Tree) -> dict:
-    """What the grouped loop of the last klpm_run on this tree did (see include/klpm.h).  Once everybody has arrived: cta_batches_tried
-    counts the windows, cta_batches the batches in which both pick orders agree, warp_steps those worked out by iteration."""
+    """What the grouped loop of the last klpm_run on this tree did (see include/klpm.h); what a tree of that kind does not count is 0.
+    cta_batch* and warp_step* are the names that agreed_*, windows and iterated_* go by in programs written before there were windows."""
     v = (_i64 * 16)()
     _check(_lib.rt_debug_counters(tree.handle, ctypes.byref(v)), "rt_debug_counters")
     names = ("careful_steps", "cta_dissolves", "fallback_scans", "fallen_back", "evictions", "cycles_tree", "cycles_scans",
-             "cycles_cta_dissolves", "cta_batches_tried", "cta_batches", "cta_batch_decisions", "warp_steps",
-             "warp_step_decisions", "single_decisions", "cycles_cta_batches", "cycles_warp_steps")
-    return dict(zip(names, [int(x) for x in v]))
+             "cycles_cta_dissolves", "windows", "agreed_batches", "agreed_decisions", "iterated_batches",
+             "iterated_decisions", "single_decisions", "cycles_windows", "cycles_single")
+    c = dict(zip(names, [int(x) for x in v]))
+    c.update(lane_decisions=0, most_grown=0)
+    if tree.budget_tokens == 0:
+        c.update(fallen_back=0, evictions=0, lane_decisions=int(v[3]), most_grown=int(v[4]))
+    for old, new in (("cta_batches_tried", "windows"), ("cta_batches", "agreed_batches"), ("cta_batch_decisions", "agreed_decisions"),
+                     ("warp_steps", "iterated_batches"), ("warp_step_decisions", "iterated_decisions"),
+                     ("cycles_cta_batches", "cycles_windows"), ("cycles_warp_steps", "cycles_single")):
+        c[old] = c[new]
+    return c
 
 
 def klpm_debug_set(name: str, value: int) -> None:

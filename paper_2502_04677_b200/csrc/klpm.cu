@@ -2931,7 +2931,7 @@ struct ListWin {                      // the window, in the scratch of the sorts
     unsigned *EF, *EL;                // needs a step of its own
     unsigned* eq;                     // agreement, one bit per rank
     int32_t* cand; short* cand_p;     // slots in groups found in the window, and their list positions
-    ListLane* lane; ListTaken *taken, *unsorted;       // in the place of `col` once every thread has its meetings
+    ListLane* lane; ListTaken* taken; short* unsorted; // in the place of `col` once every thread has its meetings
 };
 // The prompts of a group of two, and prompts whose key has grown because the other one was processed, are worked out by the same
 // rounds, each by a thread of its own (see `lane_round`).
@@ -2946,7 +2946,7 @@ struct ListTaken { unsigned long long key; int32_t A, o, jr, lane; };
 #define KLPM_LIST_LANES 128           // the first half for grown keys, the second for groups of two
 #define KLPM_LIST_LANE_MIN 8192        // shorter queues make those decisions one at a time: they are few, and lanes lengthen every round (1,000 queries: 65 us, with lanes 121)
 #define KLPM_LIST_CAND 288
-#define KLPM_LIST_TAKEN 80             // guessed to be taken with a grown key at a time, at most (more are not guessed)
+#define KLPM_LIST_TAKEN (KLPM_LIST_LANES / 2 + KLPM_LIST_LANES / 4)      // guessed to be taken with a grown key at a time, at most: every grown key, one of every group
 struct ListShared {
     int32_t n_cand, n_pair, n_grown, n_taken, lane_lim;
     int4 pre[2][4];                              // records of lcp_kernel's pairs for the last four steps found on either side, on their way since then
@@ -2962,7 +2962,8 @@ struct ListShared {
     long long cn[16];                            // what the loop did (FastPost::counters), kept by thread 0: registers are short here
 };
 static_assert(KLPM_LIST_WIN * (4 + 4 + 8 + 4) + KLPM_LIST_THREADS * 8 + 9 * (KLPM_LIST_WIN / 32) * 4 + KLPM_LIST_CAND * 6 <= KLPM_FAST_SORT_CAP * 12, "a window fits the sort scratch");
-static_assert(KLPM_LIST_LANES * sizeof(ListLane) + 2 * KLPM_LIST_TAKEN * sizeof(ListTaken) <= KLPM_LIST_WIN * 4, "the lanes fit the place of the meetings");
+static_assert(KLPM_LIST_LANES * sizeof(ListLane) + KLPM_LIST_TAKEN * (sizeof(ListTaken) + 2) <= KLPM_LIST_WIN * 4, "the lanes fit the place of the meetings");
+static_assert(KLPM_LIST_CAND * 6 <= KLPM_LIST_TAKEN * sizeof(ListTaken), "the candidates' pairs fit the place of the taken");
 
 // first set bit of a bitmap of 64 words, or -1.  One warp.
 __device__ __forceinline__ int32_t list_first(const unsigned* w, int lane) {
@@ -3043,14 +3044,14 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     W.F = reinterpret_cast<uint2*>(W.fw + KLPM_LIST_THREADS); W.L = W.F + WORDS;
     W.LF = reinterpret_cast<unsigned*>(W.L + WORDS); W.LL = W.LF + WORDS; W.EF = W.LL + WORDS; W.EL = W.EF + WORDS; W.eq = W.EL + WORDS;
     W.cand = reinterpret_cast<int32_t*>(W.eq + WORDS); W.cand_p = reinterpret_cast<short*>(W.cand + KLPM_LIST_CAND);
-    W.lane = reinterpret_cast<ListLane*>(W.col); W.taken = reinterpret_cast<ListTaken*>(W.lane + KLPM_LIST_LANES); W.unsorted = W.taken + KLPM_LIST_TAKEN;
+    W.lane = reinterpret_cast<ListLane*>(W.col); W.taken = reinterpret_cast<ListTaken*>(W.lane + KLPM_LIST_LANES); W.unsorted = reinterpret_cast<short*>(W.taken + KLPM_LIST_TAKEN);
     for (int32_t i = tid; i < nb1p + n2p + 32; i += KLPM_LIST_THREADS) R.t1[i] = 0ULL;
     if (tid == 0) {
         s_memcur = n;
         S.head = A.post->head; S.cur = 0; S.root = 0ULL; S.failed = 0; S.job = 0; S.pre_n[0] = 0; S.pre_n[1] = 0; S.n_taken = 0;
         for (int i = 0; i < 16; ++i) S.cn[i] = 0;
     }
-    auto count = [&](int i, long long v) { if (tid == 0) S.cn[i] += v; };
+    auto count = [&](int i, long long v) { if (tid == 0) S.cn[i] += v; __syncwarp(); };      // (together again at once: what follows would run for lane 0 and the others in turn)
     if (A.done_in_smem) for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) R.done[i] = c > 0 ? __ldcg(A.done + i) : 0u;
     for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) {
         R.skip[i] = 0u;                                     // (slots whose key has changed since the sort)
@@ -3381,20 +3382,21 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         if (x == 0) S.n_taken = 0;
         lane_bar();
         int32_t at = -1;
-        if (l.kind && l.taken) {
+        if (l.kind && l.taken) {                            // (never more than there is room for: of a group at most one has grown)
             at = atomicAdd(&S.n_taken, 1);
-            if (at < KLPM_LIST_TAKEN) { ListTaken t; t.key = l.key; t.A = l.A; t.o = l.o; t.jr = l.jr; t.lane = x; W.unsorted[at] = t; }
-            else { l.taken = 0; at = -1; }
+            W.unsorted[at] = (short)x;
         }
         lane_bar();
-        const int32_t nt = S.n_taken < KLPM_LIST_TAKEN ? S.n_taken : KLPM_LIST_TAKEN;
+        const int32_t nt = S.n_taken;
+        if (x == 0 && nt > S.cn[4]) S.cn[4] = nt;
+        __syncwarp();
         if (at >= 0) {
             int32_t rank = 0;
-            for (int32_t u = 0; u < nt; ++u) { const int32_t a = W.unsorted[u].A; rank += a < l.A || (a == l.A && u < at); }
-            W.taken[rank] = W.unsorted[at];
+            for (int32_t u = 0; u < nt; ++u) { const int32_t a = W.lane[W.unsorted[u]].A; rank += a < l.A || (a == l.A && u < at); }
+            ListTaken t; t.key = l.key; t.A = l.A; t.o = l.o; t.jr = l.jr; t.lane = x;
+            W.taken[rank] = t;
         }
         lane_bar();
-        if (x == 0) S.n_taken = nt;
     };
     // A lane's turns from the guesses, and its new guess.  Of a group of two, whoever is reached first is an ordinary pick of either side.
     // The other one's key grows at that moment: A longest-match turns are over by then.  It is taken before the first list entry
@@ -3787,6 +3789,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                     if (l.kind) by = (lane_now & 1u) && lane_tf < B ? 1u : (lane_now & 2u) && lane_tl < B ? 2u : (lane_now & 4u) && l.o < nlb ? 4u : 0u;
                     const int32_t t = by == 1u ? lane_tf : by == 2u ? lane_tl : by == 4u ? l_turn(l.o) : KLPM_LIST_FAR;
                     const int32_t tm = __shfl_xor_sync(FULL_MASK, t, 1);
+                    if (by) atomicAdd(reinterpret_cast<unsigned long long*>(&S.cn[3]), 1ULL);
                     if (by) {                               // its marks on the other sides go (the guesses only once everybody has read them)
                         if (by == 4u) take(l.slot, t);
                         if (by != 1u && l.fi >= 0) { atomicAnd(&W.LF[l.fi >> 5], ~(1u << (l.fi & 31))); gone_f = l.fi; }

@@ -122,3 +122,55 @@ def test_changed_keys_are_looked_for_beside_a_commit(K, smem_kb, k):
         for a, b in zip(got[0], out):
             assert torch.equal(a, b)
     K.rt_destroy(tree)
+
+
+def paired_queue(n, low, share, seed, depth=400):
+    """Match lengths spread over one cached trunk; of the prompts whose length is in the lowest part `low` a part `share` come in pairs that
+    go on together for one to three tokens."""
+    rng = np.random.RandomState(seed)
+    trunk = rng.randint(0, 30000, size=depth).tolist()
+    prompts = []
+    while len(prompts) < n:
+        m, own = rng.randint(1, depth), 100_000 + len(prompts)
+        if m < low * depth and rng.rand() < share / (2 - share):
+            more = [own] + rng.randint(0, 30000, size=rng.randint(0, 3)).tolist()
+            prompts += [trunk[:m] + more + [90_000], trunk[:m] + more + [90_001]]
+        else:
+            prompts.append(trunk[:m] + [own])
+    return trunk + [7], [prompts[i] for i in rng.permutation(len(prompts))[:n]]
+
+
+@pytest.mark.parametrize("n, low, share, ks, smem_kb", [(9000, 0.25, 0.12, (2, 3), 0), (9000, 0.25, 0.1, (3, 4), 52), (20000, 0.1, 0.12, (4, 8), 0),
+                                                        (20000, 0.1, 0.13, (4,), 55), (30000, 0.07, 0.13, (3, 8), 0)])
+@pytest.mark.parametrize("pending", [False, True])
+def test_groups_of_two_inside_the_rounds(K, n, low, share, ks, smem_kb, pending):
+    """Up to 280 prompts of pairs a window: their decisions are made by the rounds.  They sit at the end of the key list, so that keys which
+    have grown wait there in numbers, more at a time than the 64 that find a thread.  `pending`: a fifth of the queue is still to arrive
+    as the loop starts, and the rounds go on from where that leaves the bitmaps.  With less shared memory they live in global memory."""
+    trunk, prompts = paired_queue(n, low, share, n)
+    ct, co = W.to_csr([trunk])
+    qt, qo = W.to_csr(prompts)
+    d_qt, d_qo = qt.cuda(), qo.cuda()
+    late = n // 5 if pending else 0
+    arr = torch.cat([torch.zeros(n - late, dtype=torch.int64), torch.arange(1, late + 1, dtype=torch.int64) // 8]).cuda()
+    tree = K.rt_build(ct.cuda(), co.cuda(), max_nodes=2 * n + 64, max_pool_tokens=ct.numel() + qt.numel() + 8 * n + 64, max_clock=n + 64)
+    K.rt_checkpoint(tree)
+    for k in ks:
+        got = []
+        for one_by_one in (1, 0):
+            K.rt_rollback(tree)
+            out = [torch.full((n,), -1, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.int64, torch.int64)]
+            K.klpm_debug_set("run_one_by_one", one_by_one)
+            K.klpm_debug_set("fast_smem_kb", smem_kb)
+            try:
+                K.klpm_run(tree, d_qt, d_qo, arr, K.make_params(K.POLICY_KLPM, k, 0, 1, 0), *out)
+                assert K.rt_sync_status(tree) == 0
+            finally:
+                K.klpm_debug_set("run_one_by_one", -1)
+                K.klpm_debug_set("fast_smem_kb", -1)
+            got.append(out)
+        for a, b in zip(*got):
+            assert torch.equal(a, b), k
+        c = K.rt_debug_counters(tree)
+        assert c["lane_decisions"] >= 40, c
+    K.rt_destroy(tree)
