@@ -2046,6 +2046,9 @@ group_small_kernel(FastArgs A, GroupTable H) {
 // queue touches few groups, and the others are never dissolved.
 // 120,000 prompts of 256 shared prefixes: 296 us, bound by the 0.9 GB of prefix tokens it compares; eight warps of the loop's
 // CTA, which did the comparing before, took 73 ms for the same (220,000 cycles per group of a shared prefix, now 44,000).
+// PAIRS: what becomes of groups of two is written down too (list mode).  An instance of its own: it takes 57 registers, the other one 48, which
+// is 5 instead of 4 CTAs per SM in a kernel that lives from the loads it has in flight.
+template <bool PAIRS>
 __global__ void __launch_bounds__(256)
 lcp_kernel(FastArgs A, int32_t per, const int32_t* __restrict__ wanted) {
     const int lane = threadIdx.x & 31;
@@ -2084,7 +2087,7 @@ lcp_kernel(FastArgs A, int32_t per, const int32_t* __restrict__ wanted) {
     if (r >= 0) A.lcp[r] = make_int4(ref, e, e < len ? __ldg(A.tok + soff + e) : 0, 0);
     // A group of two is known completely: whoever is processed first, the other one matches e tokens from then on.  (Two slots that share
     // a run by a hash collision are no group.)
-    if (!A.list_mode || count < 2) return;
+    if (!PAIRS || count < 2) return;
     if (count > 2) { A.pair[2LL * r] = make_int4(-2, 0, 0, 0); return; }
     if (other == r) return;                                 // (the other slot's lane writes both)
     if (!cmp) {
@@ -6430,7 +6433,8 @@ static rt_status run_impl(rt_tree* tree, const int32_t* d_q_tokens, const int64_
                 CK(cudaMemsetAsync(wanted, 0, (size_t)n * sizeof(int32_t), s));
                 lcp_wanted_kernel<<<(unsigned)((n_fixed + 255) / 256), 256, 0, s>>>(f, wanted);
             }
-            lcp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(f, (int32_t)per, wanted);
+            if (f.list_mode) lcp_kernel<true><<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(f, (int32_t)per, wanted);
+            else lcp_kernel<false><<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(f, (int32_t)per, wanted);
         }
         if (lru) {                   // per node of the tree: the slots parked in it as the loop starts
             sort_pairs(f.pk, f.pi, np2, s);
