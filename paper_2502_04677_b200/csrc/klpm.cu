@@ -3006,6 +3006,20 @@ __device__ __forceinline__ void list_fetch16(void* dst, const void* src) {
 }
 __device__ __forceinline__ void list_fetch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// The largest key that the tournament holds of leaf block b: of slots that are unprocessed and whose key has changed since the sort, less
+// those (`held`, per bitmap word) whose key a lane has.  One warp.
+template <class Held>
+__device__ __forceinline__ unsigned long long changed_block_max(const FastArgs& A, const FastTour& R, int32_t b, int32_t nwords, int lane, Held held) {
+    const int32_t w0 = b << (A.lb_shift - 5), w1 = (b + 1) << (A.lb_shift - 5);
+    unsigned long long v = 0;
+    for (int32_t w = w0; w < w1 && w < nwords; ++w) {
+        unsigned m = bm_ld(R.skip, w, R.g_bits) & ~bm_ld(R.done, w, R.g_done);
+        if (m) m &= ~held(w);
+        if ((m >> lane) & 1u) { const unsigned long long key = __ldcg(A.key + ((long long)w << 5) + lane); if (key > v) v = key; }
+    }
+    return warp_max64r(v);
+}
+
 template <bool G>
 __global__ void __launch_bounds__(KLPM_LIST_THREADS, 1)
 list_run_kernel(const __grid_constant__ FastArgs A) {
@@ -3494,15 +3508,14 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         }
         __syncwarp();
         if (in_tour) {                                      // its leaf block's largest changed key, without it
-            const int32_t b = j >> A.lb_shift;
-            unsigned long long v = 0;
-            for (int32_t u = 0; u < (1 << A.lb_shift); u += 32) {
-                const long long r = ((long long)b << A.lb_shift) + u + lane;
-                bool in = r < n && bit_of(R.skip, (int32_t)r, gbits) && !bit_of(R.done, (int32_t)r, gdone);
-                for (int32_t l = 0; l < KLPM_LIST_LANES && __any_sync(FULL_MASK, in); ++l) in = in && !(W.lane[l].kind == 1 && W.lane[l].slot == (int32_t)r);      // (a lane's key is not in the tournament)
-                if (in) { const unsigned long long key = __ldcg(A.key + r); if (key > v) v = key; }
-            }
-            root = tour_set(R, b, warp_max64r(v), lane);
+            const bool with_lanes = S.n_pair > 0 || S.n_grown > 0;
+            root = tour_set(R, j >> A.lb_shift, changed_block_max(A, R, j >> A.lb_shift, nwords, lane, [&](int32_t w) -> unsigned {
+                if (!with_lanes) return 0u;
+                unsigned m = 0;
+#pragma unroll
+                for (int u = 0; u < KLPM_LIST_LANES / 32; ++u) { const ListLane& l = W.lane[32 * u + lane]; if (l.kind == 1 && (l.slot >> 5) == w) m |= 1u << (l.slot & 31); }
+                return __reduce_or_sync(FULL_MASK, m);
+            }), lane);
             __syncwarp();
         }
         if (grouped) {
