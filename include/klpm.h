@@ -240,14 +240,16 @@ rt_status klpm_run(rt_tree* tree, const int32_t* d_q_tokens, const int64_t* d_q_
  * outputs. */
 int32_t klpm_run_path(const rt_tree* tree);
 
-/* What the grouped loop of the last klpm_run / klpm_run_ex on this tree did (zeros if it has not run): out16[0] decisions
- * taken by a careful step, [1] groups dissolved by the whole CTA, [2] scans after an eviction of a leaf with queries
- * parked in it, [3] queries that fell back out of evicted leaves, [4] evictions, [5..7] clock cycles spent waiting for
- * tree updates, in those scans, in dissolves by the whole CTA (on a tree without a budget instead: [3] decisions taken by the
- * threads of groups of two and of grown keys, [4] the most of those that were guessed to take one at a time); once everybody had arrived: [8] windows looked at,
- * [9] batches in which both pick orders agree, [10] decisions they made, [11] batches worked out by iteration, [12] decisions
- * they made, [13] decisions made one at a time, [14..15] clock cycles spent on new windows and on single decisions.  A debugging aid; synchronises
- * like rt_stats. */
+/* What the grouped loop of the last klpm_run / klpm_run_ex on this tree did (zeros if it has not run).  out16[0] decisions
+ * taken by a careful step, [1] groups dissolved by the whole CTA, [7] clock cycles spent in those.
+ * On a tree with a budget: [2] scans after an eviction of a leaf with queries parked in it, [3] queries that fell back out of
+ * evicted leaves, [4] evictions, [5..6] clock cycles spent waiting for tree updates and in those scans.
+ * On a tree without one, once everybody had arrived: [2] decisions made in stretches without a window, [3] decisions taken by
+ * the threads of groups of two and of grown keys, [4] the most of those that were guessed to take one at a time, [5] rounds,
+ * [6] clock cycles spent in stretches; [8] windows looked at, [9] batches in which both pick orders agree, [10] decisions they
+ * made, [11] batches worked out by iteration, [12] decisions they made, [13] decisions made one at a time or in a stretch,
+ * [14..15] clock cycles spent on new windows and on decisions made one at a time between batches.
+ * A debugging aid; synchronises like rt_stats. */
 rt_status rt_debug_counters(rt_tree* tree, int64_t* out16);
 
 /* Settings for tests and debugging; process-wide, read when a later call is made; value < 0 restores the default.

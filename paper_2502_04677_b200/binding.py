@@ -343,9 +343,11 @@ def rt_debug_counters(tree: Tree) -> dict:
              "cycles_cta_dissolves", "windows", "agreed_batches", "agreed_decisions", "iterated_batches",
              "iterated_decisions", "single_decisions", "cycles_windows", "cycles_single")
     c = dict(zip(names, [int(x) for x in v]))
-    c.update(lane_decisions=0, most_grown=0)
-    if tree.budget_tokens == 0:
-        c.update(fallen_back=0, evictions=0, lane_decisions=int(v[3]), most_grown=int(v[4]))
+    only_without = ("stretch_decisions", "lane_decisions", "most_grown", "rounds", "cycles_stretches")
+    for i, name in enumerate(only_without):
+        c[name] = 0 if tree.budget_tokens > 0 else int(v[2 + i])
+        if tree.budget_tokens == 0:
+            c[names[2 + i]] = 0
     for old, new in (("cta_batches_tried", "windows"), ("cta_batches", "agreed_batches"), ("cta_batch_decisions", "agreed_decisions"),
                      ("warp_steps", "iterated_batches"), ("warp_step_decisions", "iterated_decisions"),
                      ("cycles_cta_batches", "cycles_windows"), ("cycles_warp_steps", "cycles_single")):

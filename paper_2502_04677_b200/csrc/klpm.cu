@@ -2135,6 +2135,17 @@ __device__ __forceinline__ unsigned long long warp_max64r(unsigned long long v) 
     return ((unsigned long long)mh << 32) | ml;
 }
 
+// position of the k-th set bit of w (k >= 1, at most the number of set bits)
+__device__ __forceinline__ int kth_set_bit(unsigned w, int k) {
+    int pos = 0;
+    int cnt = __popc(w & 0xffffu); if (k > cnt) { k -= cnt; pos += 16; w >>= 16; }
+    cnt = __popc(w & 0xffu);       if (k > cnt) { k -= cnt; pos += 8; w >>= 8; }
+    cnt = __popc(w & 0xfu);        if (k > cnt) { k -= cnt; pos += 4; w >>= 4; }
+    cnt = __popc(w & 0x3u);        if (k > cnt) { k -= cnt; pos += 2; w >>= 2; }
+    if (k > (int)(w & 1u)) pos += 1;
+    return pos;
+}
+
 // ---- the tournament above the leaf blocks (shared memory) ----
 // t1[b] is the largest key of leaf block b among the slots the tournament holds: the arrived, unprocessed slots
 // while arrivals are pending; in list mode (everybody has arrived) only those of them whose key has changed since
@@ -2922,6 +2933,21 @@ fast_run_kernel(FastArgs A) {
 #define KLPM_LIST_ROUNDS 16           // rounds on one state of the window before what is settled is committed
 #define KLPM_LIST_AGREE 24            // stretches shorter than this are left to the rounds
 #define KLPM_LIST_FAR 0x3ffffff
+// When windows are left for a stretch of decisions by one warp (list_stretch), and when they are tried again.  A window is given credit, in
+// units of 100 cycles: what a stretch takes for the decisions of a batch (100 cycles each, 150 where both sides have turns) less what the batch
+// has taken.  Only a batch that ends at a step costs any: without steps a batch is long, or the two orders keep meeting, and then a stretch is
+// the slower way (1,200 cycles a decision on 1,000 prompts of eight prefixes of one length; windows 130).
+#define KLPM_LIST_CREDIT 100           // at its start
+#define KLPM_LIST_CREDIT_MAX 400
+#define KLPM_LIST_PASS 20              // a batch
+#define KLPM_LIST_ROUND 15             // a round; twice that where both sides have turns
+#define KLPM_LIST_STEP 5               // a step (beside what a stretch takes for it as well)
+#define KLPM_LIST_BUILD 100            // a new window after a group that the whole CTA dissolves
+#define KLPM_LIST_TRIAL 64             // decisions after which a stretch ends that has cost half as much again per decision as the windows before it
+#define KLPM_LIST_STRETCH 256          // decisions of a block of a stretch; doubles while the windows after it make fewer than KLPM_LIST_STRETCH_LONG
+#define KLPM_LIST_STRETCH_LONG 4096
+#define KLPM_LIST_STRETCH_MAX 8192     // decisions after which windows are tried again even if most were steps
+#define KLPM_LIST_CALM 48              // a block with fewer steps than one in this many ends the stretch
 struct ListLane;
 struct ListTaken;
 struct ListWin {                      // the window, in the scratch of the sorts
@@ -2962,6 +2988,10 @@ struct ListShared {
     int32_t step_f, step_l, mate_f, mate;        // what a step took (index, position) and changed (index, slot); -1: nothing
     unsigned long long root;
     int32_t w[KLPM_LIST_THREADS / 32];
+    int32_t credit;                              // of the windows (KLPM_LIST_CREDIT)
+    unsigned w_clock; int32_t w_c;               // when and at which decision the first of them was begun
+    int32_t alone, made, stretch_len;            // 1: a stretch (list_stretch) makes the decisions for now; those of its last call; decisions of its blocks
+    int32_t stretch, block, block_steps;         // decisions of the stretch so far; of its block, and those of them that touched a group or a changed key
     long long cn[16];                            // what the loop did (FastPost::counters), kept by thread 0: registers are short here
 };
 static_assert(KLPM_LIST_WIN * (4 + 4 + 8 + 4) + KLPM_LIST_THREADS * 8 + 9 * (KLPM_LIST_WIN / 32) * 4 + KLPM_LIST_CAND * 6 <= KLPM_FAST_SORT_CAP * 12, "a window fits the sort scratch");
@@ -3020,6 +3050,303 @@ __device__ __forceinline__ unsigned long long changed_block_max(const FastArgs& 
     return warp_max64r(v);
 }
 
+// Shared memory of list_run_kernel as in fast_run_kernel: tournament, sort scratch (here also the window), bitmaps.
+template <bool G>
+__device__ __forceinline__ FastTour list_tour(const FastArgs& A, unsigned char* smem, unsigned long long** sort_keys, int32_t** sort_slots) {
+    const int32_t nb1p = (A.nb + 31) & ~31, n2 = nb1p >> 5, n2p = (n2 + 31) & ~31, n3 = n2p >> 5;
+    const int32_t nwords = (A.n + 31) >> 5;
+    FastTour R;
+    R.t1 = reinterpret_cast<unsigned long long*>(smem);
+    R.t2 = R.t1 + nb1p;
+    R.t3 = R.t2 + n2p;
+    R.n2 = n2; R.n3 = n3;
+    *sort_keys = R.t3 + 32;
+    *sort_slots = reinterpret_cast<int32_t*>(*sort_keys + KLPM_FAST_SORT_CAP);
+    unsigned int* s_bits = reinterpret_cast<unsigned int*>(*sort_slots + KLPM_FAST_SORT_CAP);
+    R.g_done = !G || A.done_in_smem ? 0 : 1;
+    R.g_bits = !G || A.bits_in_smem ? 0 : 1;
+    R.done = A.done_in_smem ? s_bits : A.done;
+    R.skip = A.bits_in_smem ? s_bits + nwords : A.gskip;
+    R.gb = A.bits_in_smem ? s_bits + 2 * nwords : A.gbits;
+    R.dirty = nullptr;
+    return R;
+}
+// Slot j of a group of two has been processed, and `rec` (lcp_kernel's pairs) says what becomes of the other prompt: its key grows and goes
+// to the tournament, whose root is returned.  One warp.
+__device__ __forceinline__ unsigned long long list_dissolve_pair(const FastArgs& A, const FastTour& R, int32_t j, const int4& rec, unsigned long long root, int lane) {
+    const int32_t mate = rec.x;
+    const unsigned long long key = (unsigned long long)(unsigned)rec.w << 32 | (unsigned)rec.z;
+    if (lane == 0) {
+        __stcg(reinterpret_cast<int32_t*>(A.dyn + mate) + 2, rec.y);
+        __stcg(A.key + mate, key);
+        atomicOr(R.skip + (mate >> 5), 1u << (mate & 31));
+        atomicAnd(R.gb + (mate >> 5), ~(1u << (mate & 31)));
+        atomicAnd(R.gb + (j >> 5), ~(1u << (j & 31)));
+    }
+    const int32_t b = mate >> A.lb_shift;
+    const unsigned long long p1 = R.t1[b], p2 = R.t2[b >> 5], p3 = R.t3[b >> 10];
+    __syncwarp();
+    R.t1[b] = key > p1 ? key : p1; R.t2[b >> 5] = key > p2 ? key : p2; R.t3[b >> 10] = key > p3 ? key : p3;      // (every lane stores the same)
+    __syncwarp();
+    return key > root ? key : root;
+}
+// Decision `at` took slot j of any other group (d, s: its records).  0: nothing to do; 1: dissolved, anything about the members may have
+// changed; 2: left to the whole CTA, as *job.  One warp.
+__device__ __forceinline__ int list_dissolve_group(const FastArgs& A, const FastTour& R, FastJob* job, int32_t j, int32_t at, const FDyn& d, const FStat& s,
+                                                   unsigned long long* root, int lane) {
+    if (s.len <= d.m || d.gcount <= 1) return 0;
+    FastPick P;
+    P.slot = j; P.m = d.m; P.len = s.len; P.ntok = d.ntok; P.x = A.tok + s.soff; P.pos = d.pos; P.vleaf = A.vbase + ((long long)at << 32);
+    P.admitted = A.n; P.gstart = d.gstart; P.gcount = d.gcount; P.leaf = -1;
+    P.lcp = __ldcg(A.lcp + j);
+    const bool small_ = dissolve_is_small(P);
+    if (small_) *root = dissolve_small(A, P, R, *root, lane);
+    else if (lane == 0) { job->type = FAST_JOB_DISSOLVE; job->pick = P; }
+    __syncwarp();
+    return small_ ? 1 : 2;
+}
+
+// A stretch of decisions by one warp, without a window: for queues, or parts of queues, in which most decisions touch a group or a changed
+// key, and where windows settle little.  Two ways, as often as each pays:
+//   * warp-wide: the next 32 list entries and the next unprocessed slots side by side, interleaved as the policy says, cut before the first
+//     decision that another one could have influenced (a slot in both, a group, a changed key, an entry below the tournament's root): about
+//     3,000 cycles for up to 32 decisions;
+//   * one decision: 900 cycles, 2,500 to 3,500 where a group is dissolved or the tournament changes (two L2 trips).
+// It ends where the whole CTA is needed for a group, after a block of `len` decisions of which few were steps, and after
+// KLPM_LIST_STRETCH_MAX decisions in any case.  Queues of 9,000 prompts in replicas of four: 1.45 us a decision; as steps between batches of a window
+// 3 us.  (A function of its own: inside the kernel its registers would cost the rounds theirs.)
+template <bool G>
+__device__ __noinline__ void list_stretch(const FastArgs& __restrict__ A, ListShared& __restrict__ S, FastJob& __restrict__ job_, int32_t c, int32_t cyc) {
+    extern __shared__ __align__(16) unsigned char fast_smem[];
+    const int lane = threadIdx.x & 31;
+    unsigned long long* sh;
+    int32_t* s_H;
+    const FastTour R = list_tour<G>(A, fast_smem, &sh, &s_H);
+    int32_t* const s_E = s_H + 32;
+    const int gdone = G ? R.g_done : 0, gbits = G ? R.g_bits : 0;
+    const int32_t n = A.n, nwords = (n + 31) >> 5, k = A.k, policy = A.policy;
+    const bool use_l = policy == KLPM_POLICY_LPM || (policy == KLPM_POLICY_KLPM && k >= 2);
+    const long long* const lk = A.lk;
+    const int32_t* const ls = A.ls;
+    int32_t* const order = A.order;
+    const unsigned t0 = (unsigned)clock();
+    int32_t len = S.stretch_len;
+    if (S.stretch == 0) {                                   // a new one
+        __syncwarp();
+        len = c - S.w_c >= KLPM_LIST_STRETCH_LONG ? KLPM_LIST_STRETCH : len < KLPM_LIST_STRETCH_LONG ? 2 * len : len;
+        if (lane == 0) S.stretch_len = len;
+        __syncwarp();
+    }
+    const int32_t c_in = c, before = S.stretch;
+    const unsigned w_cpd = before == 0 ? (t0 - S.w_clock) / (unsigned)(c > S.w_c ? c - S.w_c : 1) : 0u;      // what the windows before it have cost per decision
+    int32_t head = S.head, cur = S.cur, block = S.block, block_steps = S.block_steps, job = 0, groups = 0;
+    unsigned long long root = S.root;
+    bool end = false, trial = before == 0, failed = false;
+    auto bit_of = [&](const unsigned* bm, int32_t slot, int g) -> unsigned { return (bm_ld(bm, slot >> 5, g) >> (slot & 31)) & 1u; };
+    auto stale = [&](int32_t s) -> bool { return (((bm_ld(R.done, s >> 5, gdone) | bm_ld(R.skip, s >> 5, gbits)) >> (s & 31)) & 1u) != 0u; };
+    // the list 32 entries at a time: lane l holds entry (cur & ~31) + l, the next 32 are on their way
+    auto window = [&](int32_t base, long long* wk_, int32_t* ws_) {
+        const long long i = (long long)base + lane;
+        *wk_ = i < n ? __ldg(lk + i) : 0LL;
+        *ws_ = i < n ? __ldg(ls + i) : -1;
+    };
+    long long wk, nk;
+    int32_t ws, ns;
+    window(cur & ~31, &wk, &ws);
+    window((cur & ~31) + 32, &nk, &ns);
+    const int32_t lane_div_k = lane / k;                    // y / k for y = 0..31, looked up by shuffle
+    bool one_next = false;                                  // the last warp-wide step stopped before a decision it could not take
+    int32_t wait = 0, back = 1;                             // decisions until the next warp-wide step is tried; doubles while it makes fewer than two
+    // Up to 32 decisions at once: lane i makes decision c + i.  Returns how many; fewer than two: none, and nothing has changed.
+    auto warp_wide = [&]() -> int32_t {
+        // oldest-first turns among the next x decisions, for x = lane (f_lo) and x = lane + 1 (f_hi)
+        int32_t f_lo, f_hi;
+        if (policy == KLPM_POLICY_FCFS) { f_lo = lane; f_hi = lane + 1; }
+        else if (policy == KLPM_POLICY_LPM) { f_lo = 0; f_hi = 0; }
+        else {
+            const int32_t i0 = cyc == 0 ? 0 : k - cyc;
+            const int32_t y_lo = lane - i0 - 1, y_hi = lane - i0;
+            const int32_t q_lo = __shfl_sync(FULL_MASK, lane_div_k, y_lo > 0 ? y_lo : 0);
+            const int32_t q_hi = __shfl_sync(FULL_MASK, lane_div_k, y_hi > 0 ? y_hi : 0);
+            f_lo = y_lo >= 0 ? q_lo + 1 : 0;
+            f_hi = y_hi >= 0 ? q_hi + 1 : 0;
+        }
+        // the list entries cur .. cur + 31 that still count
+        const int32_t off = (cur & 31) + lane;
+        const long long k0 = __shfl_sync(FULL_MASK, wk, off & 31), k1 = __shfl_sync(FULL_MASK, nk, off & 31);
+        const int32_t s0 = __shfl_sync(FULL_MASK, ws, off & 31), s1 = __shfl_sync(FULL_MASK, ns, off & 31);
+        const long long kk = off < 32 ? k0 : k1;
+        const int32_t es = off < 32 ? s0 : s1;
+        const unsigned mask = __ballot_sync(FULL_MASK, (long long)cur + lane < n && !stale(es));
+        // as many decisions as those entries allow: lane x asks whether x + 1 decisions need no more of them
+        const int32_t B0 = __popc(__ballot_sync(FULL_MASK, c + lane < n && (lane + 1) - f_hi <= __popc(mask)));
+        if (B0 < 2) return 0;
+        const int32_t nF0 = __shfl_sync(FULL_MASK, f_hi, B0 - 1), nL0 = B0 - nF0;
+        // the next nF0 unprocessed slots; limF = how many of them can be taken before one is a step
+        int32_t hs = -1, hmax0 = -1, limF = nF0;
+        if (nF0 > 0) {
+            const int32_t w0 = head >> 5;
+            const int32_t qk = lane < nF0 ? lane : nF0 - 1;           // lane q looks for the q-th unprocessed slot
+            auto free_word = [&](int32_t wi) -> unsigned {            // unprocessed slots of bitmap word wi, from head on
+                unsigned w = wi < nwords ? bm_ld(R.done, wi, gdone) : 0xffffffffu;
+                if (wi == nwords - 1 && (n & 31)) w |= ~((1u << (n & 31)) - 1u);
+                if (wi == w0) w |= (1u << (head & 31)) - 1u;
+                return ~w;
+            };
+            const unsigned f0 = free_word(w0), f1 = free_word(w0 + 1);
+            const int32_t c0 = __popc(f0);
+            if (c0 + __popc(f1) >= nF0) {                             // the usual case: they are all in the first two words
+                hs = qk < c0 ? w0 * 32 + kth_set_bit(f0, qk + 1) : (w0 + 1) * 32 + kth_set_bit(f1, qk - c0 + 1);
+            } else {                                                  // up to 32 words: running counts, then a search per lane
+                const unsigned fr = free_word(w0 + lane);
+                const int32_t cnt = __popc(fr);
+                int32_t inc = cnt;
+#pragma unroll
+                for (int dlt = 1; dlt < 32; dlt <<= 1) { const int32_t o = __shfl_up_sync(FULL_MASK, inc, dlt); if (lane >= dlt) inc += o; }
+                if (__shfl_sync(FULL_MASK, inc, 31) < nF0) return 0;
+                int L = 0;
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1) if (__shfl_sync(FULL_MASK, inc, L + step - 1) <= qk) L += step;
+                const unsigned frL = __shfl_sync(FULL_MASK, fr, L);
+                const int32_t preL = __shfl_sync(FULL_MASK, inc - cnt, L);
+                hs = (w0 + L) * 32 + kth_set_bit(frL, qk - preL + 1);
+            }
+            hmax0 = __shfl_sync(FULL_MASK, hs, nF0 - 1);
+            const unsigned badH = __ballot_sync(FULL_MASK, lane < nF0 && ((((use_l ? bm_ld(R.skip, hs >> 5, gbits) : 0u) | bm_ld(R.gb, hs >> 5, gbits)) >> (hs & 31)) & 1u));
+            if (badH) limF = __ffs(badH) - 1;
+        }
+        // limL = how many list entries can be taken before one is a step, could also be an oldest-first pick of this batch, or lies below the root
+        const bool ok = (mask >> lane) & 1u;
+        const int32_t rank = __popc(mask & ((1u << lane) - 1u));
+        int32_t limL = nL0;
+        int32_t soft = -1;                                  // slot of the entry that stops the batch, if it is only suspected of being an oldest-first pick too
+        {
+            const unsigned long long ek = ~((unsigned long long)kk ^ 0x8000000000000000ULL);
+            const bool hard = ok && (bit_of(R.gb, es, gbits) || root > ek);
+            const unsigned badE = __ballot_sync(FULL_MASK, ok && rank < nL0 && (hard || (es >= head && es <= hmax0)));
+            if (badE) {
+                const int src = __ffs(badE) - 1;
+                limL = __popc(mask & ((1u << src) - 1u));
+                if (!__shfl_sync(FULL_MASK, (int)hard, src)) soft = __shfl_sync(FULL_MASK, es, src);
+            }
+        }
+        int32_t B = __popc(__ballot_sync(FULL_MASK, lane < B0 && f_hi <= limF && (lane + 1) - f_hi <= limL));
+        if (soft >= 0 && B < B0 && B < 32) {
+            // the decision after the batch (lane B's): if it is the longest-match turn that takes that entry and the
+            // oldest-first picks made until then all lie before its slot, it becomes the batch's last decision
+            const int32_t fl = __shfl_sync(FULL_MASK, f_lo, B), fh = __shfl_sync(FULL_MASK, f_hi, B);
+            const int32_t last_h = __shfl_sync(FULL_MASK, hs, fl > 0 ? fl - 1 : 0);
+            if (fh == fl && B - fl == limL && fl <= limF && (fl == 0 || last_h < soft)) { ++B; ++limL; }
+        }
+        if (B < 2) return 0;
+        one_next = B < B0 && soft < 0;
+        const int32_t nF = __shfl_sync(FULL_MASK, f_hi, B - 1), nL = B - nF;
+        const int32_t hmax = nF > 0 ? __shfl_sync(FULL_MASK, hs, nF - 1) : -1;
+        if (lane < nF) s_H[lane] = hs;
+        int32_t consumed = 0;
+        if (nL > 0) {
+            consumed = kth_set_bit(mask, nL) + 1;
+            if (ok && rank < nL) s_E[rank] = es;
+        }
+        __syncwarp();
+        if (lane < B) {
+            const int32_t j = f_hi > f_lo ? s_H[f_lo] : s_E[lane - f_lo];
+            atomicOr(R.done + (j >> 5), 1u << (j & 31));
+            order[c + lane] = j;
+        }
+        __syncwarp();
+        if (consumed) {
+            const int32_t ncur = cur + consumed;
+            if ((ncur >> 5) != (cur >> 5)) { wk = nk; ws = ns; window((ncur & ~31) + 32, &nk, &ns); }
+            cur = ncur;
+        }
+        if (nF > 0) head = next_head(R.done, gdone, nwords, n, hmax, lane);
+        else if (head < n && bit_of(R.done, head, gdone)) head = next_head(R.done, gdone, nwords, n, head, lane);
+        return B;
+    };
+    while (c < n) {
+        int32_t made = 0;
+        if (!one_next && wait <= 0) {
+            made = warp_wide();
+            if (made > 0) back = 1;
+            else { wait = back; back = back < 64 ? 2 * back : 64; }
+        }
+        if (made == 0) {
+            if (!one_next) --wait;
+            one_next = false;
+            made = 1;
+            const bool oldest = policy == KLPM_POLICY_FCFS || (policy == KLPM_POLICY_KLPM && cyc == 0);
+            int32_t j;
+            bool in_tour;
+            if (oldest) {
+                j = head;
+                in_tour = use_l && head < n && bit_of(R.skip, j, gbits) != 0u;
+            } else {
+                unsigned long long ek = 0;                  // next entry of the list that still counts
+                int32_t es = -1;
+                while (cur < n) {                           // (a window's 32 entries are examined at once: stale entries come in runs)
+                    const int32_t wbase = cur & ~31;
+                    const unsigned bal = __ballot_sync(FULL_MASK, lane >= (cur & 31) && (long long)wbase + lane < n && !stale(ws));
+                    if (bal) {
+                        const int src = __ffs(bal) - 1;
+                        cur = wbase + src;
+                        ek = ~((unsigned long long)__shfl_sync(FULL_MASK, wk, src) ^ 0x8000000000000000ULL);
+                        es = __shfl_sync(FULL_MASK, ws, src);
+                        break;
+                    }
+                    cur = wbase + 32; wk = nk; ws = ns; window(cur + 32, &nk, &ns);
+                }
+                if (cur > n) cur = n;
+                in_tour = root > ek;
+                if (in_tour) {
+                    const unsigned rk = 0xffffffffu - (unsigned)(root & 0xffffffffULL);
+                    j = A.pinv ? __ldg(A.pinv + rk) : (int32_t)rk;
+                } else {
+                    j = es;
+                    ++cur;
+                    if ((cur & 31) == 0) { wk = nk; ws = ns; window(cur + 32, &nk, &ns); }
+                }
+            }
+            if (j < 0 || j >= n || bit_of(R.done, j, gdone)) { failed = true; break; }      // cannot happen
+            const bool grouped = bit_of(R.gb, j, gbits) != 0u;
+            FDyn d; FStat s; int4 rec;                      // (asked for before the tournament is brought up to date)
+            if (grouped) { d = ld_dyn(A.dyn + j); s = ld_stat(A.stat + j); rec = __ldg(A.pair + 2LL * j); }
+            __syncwarp();
+            if (lane == 0) { atomicOr(R.done + (j >> 5), 1u << (j & 31)); order[c] = j; }
+            __syncwarp();
+            if (in_tour) {
+                const int32_t b = j >> A.lb_shift;
+                root = tour_set(R, b, changed_block_max(A, R, b, nwords, lane, [](int32_t) -> unsigned { return 0u; }), lane);
+                __syncwarp();
+            }
+            if (j == head) head = next_head(R.done, gdone, nwords, n, j, lane);
+            if (grouped) {
+                ++groups;
+                if (rec.x >= 0) root = list_dissolve_pair(A, R, j, rec, root, lane);
+                else job = list_dissolve_group(A, R, &job_, j, c, d, s, &root, lane);
+            }
+            if (grouped || in_tour) ++block_steps;
+        }
+        c += made;
+        if (policy == KLPM_POLICY_KLPM) cyc = (cyc + made) % k;
+        block += made;
+        if (block >= len) { end = block_steps * KLPM_LIST_CALM <= block || before + (c - c_in) >= KLPM_LIST_STRETCH_MAX; block = 0; block_steps = 0; }
+        if (trial && c - c_in >= KLPM_LIST_TRIAL) {
+            trial = false;
+            const unsigned cy = __shfl_sync(FULL_MASK, (unsigned)clock() - t0, 0);
+            if (2 * (cy / (unsigned)(c - c_in)) > 3 * w_cpd) end = true;
+        }
+        if (job == 2 || end) break;
+    }
+    if (lane == 0) {
+        if (end) { S.credit = KLPM_LIST_CREDIT; S.w_clock = (unsigned)clock(); S.w_c = c; }
+        if (failed) { set_status(A.st, RT_ERR_LIMIT, 107); S.failed = 1; }
+        S.head = head; S.cur = cur < n ? cur : n; S.root = root; S.job = job; S.made = c - c_in; S.alone = !end;
+        S.stretch = before + (c - c_in); S.block = block; S.block_steps = block_steps;
+        S.cn[0] += groups; S.cn[2] += c - c_in; S.cn[13] += c - c_in; S.cn[6] += (unsigned)clock() - t0;
+    }
+}
+
 template <bool G>
 __global__ void __launch_bounds__(KLPM_LIST_THREADS, 1)
 list_run_kernel(const __grid_constant__ FastArgs A) {
@@ -3033,23 +3360,11 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     const int32_t n = A.n;
     int32_t c = A.post->list_c, cyc = A.post->cyc;
     if (c >= n) return;
-    // ---- shared memory as in fast_run_kernel: tournament, sort scratch (here also the window), bitmaps
-    const int32_t nb1p = (A.nb + 31) & ~31, n2 = nb1p >> 5, n2p = (n2 + 31) & ~31, n3 = n2p >> 5;
+    const int32_t nb1p = (A.nb + 31) & ~31, n2p = ((nb1p >> 5) + 31) & ~31;
     const int32_t nwords = (n + 31) >> 5;
-    FastTour R;
-    R.t1 = reinterpret_cast<unsigned long long*>(fast_smem);
-    R.t2 = R.t1 + nb1p;
-    R.t3 = R.t2 + n2p;
-    R.n2 = n2; R.n3 = n3;
-    unsigned long long* sh = R.t3 + 32;
-    int32_t* sr = reinterpret_cast<int32_t*>(sh + KLPM_FAST_SORT_CAP);
-    unsigned int* s_bits = reinterpret_cast<unsigned int*>(sr + KLPM_FAST_SORT_CAP);
-    R.g_done = !G || A.done_in_smem ? 0 : 1;
-    R.g_bits = !G || A.bits_in_smem ? 0 : 1;
-    R.done = A.done_in_smem ? s_bits : A.done;
-    R.skip = A.bits_in_smem ? s_bits + nwords : A.gskip;
-    R.gb = A.bits_in_smem ? s_bits + 2 * nwords : A.gbits;
-    R.dirty = nullptr;
+    unsigned long long* sh;
+    int32_t* sr;
+    const FastTour R = list_tour<G>(A, fast_smem, &sh, &sr);
     const int gdone = G ? R.g_done : 0, gbits = G ? R.g_bits : 0;
     ListWin W;
     W.lk = reinterpret_cast<long long*>(sh);
@@ -3067,6 +3382,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         s_memcur = n;
         S.head = A.post->head; S.cur = 0; S.root = 0ULL; S.failed = 0; S.job = 0; S.pre_n[0] = 0; S.pre_n[1] = 0; S.n_taken = 0;
         for (int i = 0; i < 16; ++i) S.cn[i] = 0;
+        S.alone = 0; S.credit = KLPM_LIST_CREDIT; S.w_clock = (unsigned)clock(); S.w_c = c; S.stretch_len = KLPM_LIST_STRETCH / 2;
     }
     auto count = [&](int i, long long v) { if (tid == 0) S.cn[i] += v; __syncwarp(); };      // (together again at once: what follows would run for lane 0 and the others in turn)
     if (A.done_in_smem) for (int32_t i = tid; i < nwords; i += KLPM_LIST_THREADS) R.done[i] = c > 0 ? __ldcg(A.done + i) : 0u;
@@ -3525,36 +3841,12 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             else rec = __ldg(A.pair + 2LL * j);
             if (rec.x >= 0) {                               // one other prompt, and what becomes of it is known
                 mate_s = rec.x;
-                const unsigned long long key = (unsigned long long)(unsigned)rec.w << 32 | (unsigned)rec.z;
-                if (lane == 0) {
-                    __stcg(reinterpret_cast<int32_t*>(A.dyn + mate_s) + 2, rec.y);
-                    __stcg(A.key + mate_s, key);
-                    atomicOr(R.skip + (mate_s >> 5), 1u << (mate_s & 31));
-                    atomicAnd(R.gb + (mate_s >> 5), ~(1u << (mate_s & 31)));
-                    atomicAnd(R.gb + (j >> 5), ~(1u << (j & 31)));
-                }
                 mate_f = index_of(mate_s);
-                const int32_t b = mate_s >> A.lb_shift;
-                const unsigned long long p1 = R.t1[b], p2 = R.t2[b >> 5], p3 = R.t3[b >> 10];
-                __syncwarp();
-                R.t1[b] = key > p1 ? key : p1; R.t2[b >> 5] = key > p2 ? key : p2; R.t3[b >> 10] = key > p3 ? key : p3;      // (every lane stores the same)
-                root = key > root ? key : root;
-                __syncwarp();
-            } else {
-                const FDyn d = ld_dyn(A.dyn + j);
-                const FStat s = ld_stat(A.stat + j);
-                if (s.len > d.m && d.gcount > 1) {
-                    FastPick P;
-                    P.slot = j; P.m = d.m; P.len = s.len; P.ntok = d.ntok; P.x = A.tok + s.soff; P.pos = d.pos; P.vleaf = A.vbase + ((long long)at << 32);
-                    P.admitted = n; P.gstart = d.gstart; P.gcount = d.gcount; P.leaf = -1;
-                    P.lcp = __ldcg(A.lcp + j);
-                    if (dissolve_is_small(P)) { root = dissolve_small(A, P, R, root, lane); job = 1; }      // (anything about the window's slots may have changed)
-                    else { job = 2; if (lane == 0) { s_job.type = FAST_JOB_DISSOLVE; s_job.pick = P; } }
-                    __syncwarp();
-                }
-            }
+                root = list_dissolve_pair(A, R, j, rec, root, lane);
+            } else job = list_dissolve_group(A, R, &s_job, j, at, ld_dyn(A.dyn + j), ld_stat(A.stat + j), &root, lane);
         }
         if (lane == 0) {
+            if (job == 2) S.credit -= KLPM_LIST_BUILD;
             S.cn[13] += 1; S.cn[0] += grouped; S.cn[15] += (unsigned)clock() - t0;      // (here and not where they happen: a branch of one lane before the dissolve has it run for lane 0 and the others in turn)
             S.root = root; S.job = job; S.step_f = step_f; S.step_l = kind == 1 ? S.ix_l : -1; S.mate_f = mate_f; S.mate = mate_s;
             if (step_f >= 0) { atomicAnd(&W.LF[step_f >> 5], ~(1u << (step_f & 31))); atomicAnd(&W.F[step_f >> 5].x, ~(1u << (step_f & 31))); }
@@ -3586,7 +3878,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
         __syncthreads();
     };
     // Where the two orders stand, for the next window.
-    bool built = false;
+    bool built = false;                                     // there is a window
     auto leave = [&]() {
         if (warp == 0) {
             int32_t head = S.head, cur = S.cur;
@@ -3601,8 +3893,8 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             if (lane == 0) { S.head = head; S.cur = cur; }
         }
         sv_slot = -1;
-        if (laner && built && W.lane[x].kind == 1) { sv_slot = W.lane[x].slot; sv_key = W.lane[x].key; sv_m2 = W.lane[x].m2; }
-        built = true;
+        if (laner && W.lane[x].kind == 1) { sv_slot = W.lane[x].slot; sv_key = W.lane[x].key; sv_m2 = W.lane[x].m2; }
+        built = false;
         __syncthreads();
     };
 
@@ -3610,17 +3902,43 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
     int32_t agree_wait = 0, agree_back = 1;                 // batches until agreement is tried again; doubles while it fails
     int32_t idle = 0;                                       // passes in a row without a decision (a new window, and then one must follow)
     while (c < n) {
+        if (__builtin_expect(S.job == 2, 0)) {              // a group that the whole CTA dissolves: its sorts use the window's memory
+            const unsigned t0 = (unsigned)clock();
+            const FastJob J = s_job;
+            fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
+            if (warp == 0) { const unsigned long long r = tour_top(R, lane); if (lane == 0) { S.root = r; S.job = 0; } }
+            __syncthreads();
+            count(1, 1); count(7, (unsigned)clock() - t0);
+        }
+        if (__builtin_expect(S.alone, 0)) {
+            __syncthreads();                                // (the stretch may take the flag back)
+            if (warp == 0) list_stretch<G>(A, S, s_job, c, cyc);
+            __syncthreads();
+            // (nothing of a window is kept from before a stretch: no register has to hold any of it meanwhile)
+#pragma unroll
+            for (int r = 0; r < PER; ++r) cv[r] = 0u;
+            alive = 0; sv_slot = -1; sv_m2 = 0; sv_key = 0; n_f = 0; n_l = 0; w0 = 0; head0 = 0; list_end = false;
+            built = false; fresh = true; agree = false; agree_wait = 0; agree_back = 1; idle = 0;
+            const int32_t made = S.made;
+            c += made;
+            if (A.policy == KLPM_POLICY_KLPM) cyc = (int32_t)(((long long)cyc + made) % A.k);
+            if (S.failed) break;
+            __syncthreads();
+            continue;
+        }
         if (++idle > 8 || (fresh && S.cn[8] >= A.max_windows)) { if (tid == 0) set_status(A.st, RT_ERR_LIMIT, 118); break; }      // cannot happen (without the debug setting)
         if (fresh) {
             const unsigned t0 = (unsigned)clock();
-            leave();
+            if (built) leave();
             build();
+            built = true;
             count(8, 1); count(14, (unsigned)clock() - t0);
             fresh = false;
         }
         set_i0();
         const int32_t left = n - c;
         int32_t B = 0, kind = -1;                           // decisions of this batch; the step that comes next (-1: none)
+        int32_t rounds = 0;
         bool lanes_on = false;                              // the commit has changed lanes
         int32_t gone_f = -1, gone_l = -1;
         bool spent = false, late = false;                   // the window holds no more; the step comes after the commit
@@ -3700,6 +4018,7 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             if (tid == 0) { S.tstar[0] = KLPM_LIST_FAR; S.tstar[1] = KLPM_LIST_FAR; }
             const bool with_lanes = S.n_pair > 0 || S.n_grown > 0;
             for (int it = 0;; ++it) {
+                rounds = it + 1;
                 ranks();
                 __syncthreads();
                 int32_t best = KLPM_LIST_FAR;
@@ -3825,10 +4144,15 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
                     l.o -= nlb; l.A = l.A > nlb && l.kind == 2 ? l.A - nlb : 0;
                     if (l.o < 0) l.taken = 0;
                 }
-                count(11, 1); count(12, B);
+                count(11, 1); count(12, B); count(5, rounds);
             }
         }
         if (B > 0 || kind >= 0) idle = 0;
+        if (tid == 0) {                                     // has this been worth it?
+            const int32_t credit = S.credit + (kind < 0 ? B : B - KLPM_LIST_PASS - KLPM_LIST_STEP + (use_f && use_l ? B / 2 - 2 * KLPM_LIST_ROUND * rounds : -KLPM_LIST_ROUND * rounds));
+            S.credit = credit < KLPM_LIST_CREDIT_MAX ? credit : KLPM_LIST_CREDIT_MAX;
+        }
+        __syncwarp();
         c += B;
         if (A.policy == KLPM_POLICY_KLPM) cyc = (int32_t)(((long long)cyc + B) % A.k);
         if (c >= n) break;
@@ -3843,20 +4167,24 @@ list_run_kernel(const __grid_constant__ FastArgs A) {
             if (S.failed) break;
             ++c;
             if (A.policy == KLPM_POLICY_KLPM && ++cyc == A.k) cyc = 0;
-            if (S.job == 2) {                               // a group that the whole CTA dissolves: its sorts use the window's memory
-                const unsigned t1 = (unsigned)clock();
+            if (S.job == 2) {
                 refresh();
                 leave();
-                const FastJob J = s_job;
-                fast_job<false>(A, R, J, sh, sr, &s_cnt, &s_memcur);
-                if (warp == 0) { const unsigned long long r = tour_top(R, lane); if (lane == 0) S.root = r; }
-                __syncthreads();
-                if (c < n) build();
-                count(8, 1); count(1, 1); count(7, (unsigned)clock() - t1);
+                fresh = true;
             } else if (S.job == 1) refresh();
             else after_step();
         }
         if (spent) fresh = true;
+        if (__builtin_expect(S.credit < 0, 0)) {            // windows do not pay here
+            __syncthreads();
+            if (built) leave();
+            if (sv_slot >= 0 && !bit_of(R.done, sv_slot, gdone)) {      // a grown key goes to the tournament
+                const int32_t b = sv_slot >> A.lb_shift;
+                atomicMax(R.t1 + b, sv_key); atomicMax(R.t2 + (b >> 5), sv_key); atomicMax(R.t3 + (b >> 10), sv_key); atomicMax(&S.root, sv_key);
+            }
+            if (tid == 0) { S.alone = 1; S.stretch = 0; S.block = 0; S.block_steps = 0; }
+            __syncthreads();
+        }
     }
     list_fetch_wait();
     __syncthreads();

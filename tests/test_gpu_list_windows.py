@@ -218,3 +218,35 @@ def test_a_changed_key_is_taken_without_a_look_at_every_lane(K, k):
     for a, b in zip(got, want):
         assert torch.equal(a, b)
     assert c["single_decisions"] > 1000 and c["cycles_single"] < 10_000 * c["single_decisions"], c
+
+
+@pytest.mark.parametrize("smem_kb", [0, 51, 50])
+@pytest.mark.parametrize("policy, k", [(2, 2), (2, 4), (2, 40), (1, 1), (0, 1)])
+def test_windows_are_left_where_most_decisions_are_steps(K, policy, k, smem_kb):
+    """Prompts that are asked for several times each: most decisions touch a group or a changed key, and one warp makes them one after the
+    other (as steps between batches of a window they took three to ten times as long).  Where such prompts are a part of the queue only,
+    windows are taken up again.  51 and 50 KiB of shared memory: some, all bitmaps in global memory."""
+    n = 3000
+    got, want, c = run_both_ways(K, replicas(n, k, n // 4), [], K.make_params(policy, k), [("fast_smem_kb", smem_kb)])
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    assert c["stretch_decisions"] > n // 2, c
+    rng = np.random.RandomState(k)
+    trunk = rng.randint(0, 30000, size=2000).tolist()
+    plain = [trunk[:rng.randint(100, 1800)] + [100_000 + i] for i in range(5000)]
+    again = [trunk[:m] + [200_000 + i, 7] for i in range(150) for m in [rng.randint(1800, 2000)] for _ in range(4)]      # first in both orders
+    got, want, c = run_both_ways(K, again + plain, [trunk + [3]], K.make_params(policy, k), [("fast_smem_kb", smem_kb)])
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    assert c["windows"] > 1 and c["iterated_decisions"] > 0, c
+
+
+def test_windows_are_kept_where_nothing_is_grouped(K):
+    """The two orders meet all the time on prompts of one match length, which is slow for one warp: without steps windows are never left."""
+    prefixes = [[p] * 40 for p in range(8)]
+    rng = np.random.RandomState(3)
+    prompts = [prefixes[rng.randint(8)] + [1000 + i] for i in range(1000)]
+    got, want, c = run_both_ways(K, prompts, [p + [999] for p in prefixes], K.make_params(K.POLICY_KLPM, 2))
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    assert c["stretch_decisions"] == 0, c
