@@ -397,7 +397,8 @@ def run_ours(args):
         loop_kernel = "list_run_kernel"
         loop_note = ("all decisions in one CTA: once everybody has arrived, longest-match picks come from a presorted list "
                      "of keys and oldest-first picks from a bitmap; windows of 2,048 entries of either order, who takes what is worked out by "
-                     "iteration over prefix sums; picks whose group has other members, and those whose key has changed, are made one at a time; the "
+                     "iteration over prefix sums, groups of two included; other picks whose group has other members, and those whose key has changed, are "
+                     "steps between two batches; where most picks are such, one warp makes the decisions without a window; the "
                      "decisions are charged by a parallel pass after the loop; bound by the barriers of one CTA; the loop starts "
                      "from the records rt_match_batch_ex kept (no query is walked twice); the time includes the sort of the keys "
                      "and the bulk insertion of the processed prompts")
@@ -437,7 +438,7 @@ def run_ours(args):
                                      "capture of scale 0.125 times 8 (the units and the sharing scale alike); null when no "
                                      "capture exists for this workload or the match path's source has changed since"},
         "decision_loop": {"kernel": loop_kernel,
-                          "bound": "latency" if (loop_kernel == "run_kernel" or w.budget_tokens > 0) else "issue",
+                          "bound": "latency",
                           "us_per_decision": 1e6 * t_run / (nq * args.steps), "note": loop_note,
                           "counters": loop_counters},
         "e2e": {"value": world * nq / e2e_match_s, "unit": "queries/s",

@@ -1740,8 +1740,8 @@ run_kernel(TreeDev T, RunArgs A) {
 //     loop get positions from a counter that starts above every real pool index;
 //   * while arrivals are pending, the longest-match pick is the root of a tournament over the keys
 //     (score << 32 | ~rank) of the arrived queries: 32-ary, leaves in global memory, every level above in shared
-//     memory; once everybody has arrived it is the next entry of a list of all keys sorted before the loop, and the
-//     tournament only holds the queries whose key has changed since (see fast_run_kernel);
+//     memory (fast_run_kernel); once everybody has arrived it is the next entry of a list of all keys sorted as they are
+//     then, and the tournament only holds the queries whose key has changed since (list_run_kernel);
 //   * the oldest-first pick is a cursor over a bitmap of processed slots.
 // One CTA runs the whole loop: warp 0 is the sequencer, the other warps wait at a named barrier and join
 // for work that is worth sharing (a large group, a large batch of arrivals).  There is no wait on another
@@ -2919,14 +2919,16 @@ fast_run_kernel(FastArgs A) {
 //   * only where the two orders agree for a stretch (one match length left, ties by arrival) does a round settle just one
 //     or two turns: every guess there hangs on the one before.  But then the next decisions are that common order, whoever
 //     makes them: R decisions, if the unprocessed slots and the live list entries have their first R elements in common.
-// A decision is made outside this scheme only where it changes a key or follows from one (a step): the pick's group has
-// other members, its key sits in the tournament, or the tournament's root beats the list.  The window goes on after it;
-// only a group dissolved by the whole CTA takes its memory.
+// Groups of two and the keys that grow in them take part in the rounds, each prompt by a thread of its own (lane_round), in queues from
+// KLPM_LIST_LANE_MIN on.  Any other decision that changes a key or follows from a changed one is a step of warp 0, beside the commit of the
+// batch before it: the pick's group has other members, its key sits in the tournament, or the tournament's root beats the list.  The window
+// goes on after it; only a group dissolved by the whole CTA takes its memory.  Where most decisions are steps, windows are left for
+// stretches in which one warp makes the decisions (list_stretch).
 // Decisions are recorded as slots in `order`; the charge pass after the loop computes their outputs.
-// What bounds it: the barriers and shared-memory round trips of one CTA: about 1,500 cycles per round, 6,000 per step with the
-// batch before it, 8,000 per window.  klpm_run of 32,768 / 65,536 / 262,144 waiting queries (medium, hierarchical, adversarial): 0.64 / 2.6 /
-// 3.0 ms in this kernel; batches of up to 1,024 decisions cut at every decision that touches a group, whose meetings one
-// warp resolved one after the other (or played through decision by decision), took 1.39 / 4.1 / 3.9.
+// What bounds it: the barriers and shared-memory round trips of one CTA: 1,500 cycles per round, twice that where the two orders meet a lot,
+// 3,000 to 6,800 per step beside its batch, 4,000 to 13,000 per window.  klpm_run of 32,768
+// waiting medium queries, k = 4: 1.00 ms in all; 2.05 with batches of up to 1,024 decisions cut at every decision that touches a group.
+// It has 128 registers, which 512 threads leave it, and spills some 200 bytes around the call of list_stretch.
 // G: some of the loop's bitmaps live in global memory (queues too long for shared memory).
 #define KLPM_LIST_THREADS 512
 #define KLPM_LIST_WIN 2048            // (4 per thread, 64 words of one bit each: two per lane of a warp)
@@ -2973,7 +2975,7 @@ struct alignas(16) ListLane {
 };
 struct ListTaken { unsigned long long key; int32_t A, o, jr, lane; };
 #define KLPM_LIST_LANES 128           // the first half for grown keys, the second for groups of two
-#define KLPM_LIST_LANE_MIN 8192        // shorter queues make those decisions one at a time: they are few, and lanes lengthen every round (1,000 queries: 65 us, with lanes 121)
+#define KLPM_LIST_LANE_MIN 8192        // shorter queues make those decisions as steps: 1,000 queries 65 us, with lanes 121 (where between that and 32,768 the line lies best was not looked for)
 #define KLPM_LIST_CAND 288
 #define KLPM_LIST_TAKEN (KLPM_LIST_LANES / 2 + KLPM_LIST_LANES / 4)      // guessed to be taken with a grown key at a time, at most: every grown key, one of every group
 struct ListShared {

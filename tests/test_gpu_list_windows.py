@@ -18,8 +18,8 @@ def K():
 @pytest.mark.parametrize("n", [2047, 2049, 8191, 8193, 12288])
 @pytest.mark.parametrize("own", [900, 40_000])
 def test_windows_against_the_one_by_one_loop(K, n, own):
-    """`own` different continuations of 12 prefixes (two of one length): about 40 prompts of a prefix share theirs at 900, few at 40,000.
-    Queues of 8,192 and more work groups of two out inside the rounds."""
+    """`own` different continuations of 12 prefixes (two of one length): at 900 two thirds of the prompts share theirs with one or two others,
+    more to a window than are looked at for groups of two; at 40,000 few do, and queues of 8,192 and more work them out inside the rounds."""
     rng = np.random.RandomState(n + own)
     prefixes = [rng.randint(0, 1000, size=ln).tolist() for ln in (3, 9, 17, 17, 25, 33, 40, 41, 50, 64, 80, 90)]
     prompts = [prefixes[rng.randint(12)] + [2000 + int(rng.randint(own))] + rng.randint(0, 9, size=rng.randint(0, 4)).tolist() for _ in range(n)]
